@@ -107,8 +107,6 @@ struct DecodeParams {
   int hold;       // 1: Algorithm 1 stops after step 3; lengths and lists stay as they are
   int evict_every;   // m >= 1: step 4 waits until a head is m entries over its budget, then removes them all
   int literal;    // 1: Algorithm 1 is skipped for a head below its budget (its first line as printed)
-  int rows_absent;   // 1: the heads' entries are only metadata so far (a prompt being scored before its
-                     //    survivors' rows are stored): nothing touches pool pages
   int plan_append;   // what the plan the LRFU kernel leaves behind is for: 1 = a decode step, 0 = a scoring pass
   int plan_warps;    // warps of the attention grid the plan is made for
   int plan_grid;     // CTAs of that grid

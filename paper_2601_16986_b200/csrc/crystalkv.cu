@@ -25,6 +25,7 @@
 #include "aux_kernels.cuh"
 #include "lrfu_kernel.cuh"
 #include "plan.cuh"
+#include "prefill_kernels.cuh"
 
 using namespace ckv;
 
@@ -588,11 +589,10 @@ static int prefill_common(crystalkv_t* h, int layer, const void* k, const void* 
   const crystalkv_config_t& c = h->cfg;
   const bool evict = c.mode == CRYSTALKV_MODE_EVICT;
   if (P < 1) return fail(h, CRYSTALKV_EINVAL, "P must be >= 1");
-  // A prompt beyond the budget is scored from the caller's tensors and only its survivors are
+  // With a last query only, a prompt is scored from the caller's tensors and only its survivors are
   // stored; with an observation window the whole prompt must fit the pool for a moment (the
   // window's attention outputs need the values).
-  const bool score_first = evict && W == 0 && P > (c.budget_ratio > 0.f ? ratio_budget(c, P) : c.budget_per_head);
-  if (evict && !score_first && P > c.budget_per_head + c.max_answer_tokens)
+  if (evict && W > 0 && P > c.budget_per_head + c.max_answer_tokens)
     return fail(h, CRYSTALKV_EINVAL, "prompt with an observation window longer than budget_per_head + max_answer_tokens");
   if (evict && P + 1 > h->cap) return fail(h, CRYSTALKV_EINVAL, "prompt longer than the heads' list capacity (max_budget + evict_every + max_answer_tokens)");
   if (P >= c.max_context) return fail(h, CRYSTALKV_EINVAL, "prompt reaches max_context");
@@ -601,45 +601,56 @@ static int prefill_common(crystalkv_t* h, int layer, const void* k, const void* 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   rc = join_side(h, s);   // the insertion takes pages; no LRFU kernel may take or return any meanwhile
   if (rc) return rc;
+  const auto* kb = static_cast<const unsigned char*>(k);
+  const auto* vb = static_cast<const unsigned char*>(v);
+  // CTAs per head of the row copy: a page per warp and turn, up to eight CTAs per SM in all
+  const int per_head = std::max(1, std::min((P / GRP + NW) / NW, (8 * h->num_sms + h->U - 1) / h->U));
+  h->prev_layer = -1;
+  if (evict && W == 0) {
+    // Algorithm 1 with the last query over scores and metadata only, then the survivors' rows; every
+    // kernel on `s`, which has joined the internal streams, so any scratch set is free
+    DecodeParams p = make_params(h, layer);
+    const int chunk = score_chunk(P, h->U), chunks = (P + chunk - 1) / chunk;
+    const size_t sm = (size_t)P * sizeof(float) <= SEL_SMEM ? (size_t)P * sizeof(float) : 0;
+    if (sm > 32 * 1024)
+      CK(h, cudaFuncSetAttribute(prefill_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SEL_SMEM));
+    prefill_score_kernel<<<dim3(chunks, h->U), NT, 0, s>>>(p.sc, static_cast<const __nv_bfloat16*>(k),
+                                                           static_cast<const __nv_bfloat16*>(q), c.n_kv_heads, P, h->G,
+                                                           chunk, p.scale, p.scale_log2);
+    CK(h, cudaGetLastError());
+    prefill_select_kernel<<<h->U, SEL_NT, sm, s>>>(h->st, p.sc, layer, P, h->G, chunks, c.top_p, c.evict_every,
+                                                   c.literal_return, c.budget_ratio > 0.f ? ratio_budget(c, P) : 0, sm > 0);
+    CK(h, cudaGetLastError());
+    prefill_rows_kernel<<<1 + h->U * per_head, NT, 0, s>>>(h->st, h->plans[layer], layer, kb, vb, P, ROWS_SURVIVORS, per_head,
+                                                           1, 0, h->grid * NW, h->grid);
+    CK(h, cudaGetLastError());
+    h->t_layer[layer] = P - 1;
+    return CRYSTALKV_OK;
+  }
   if (evict && c.budget_ratio > 0.f) {   // the prompt's share of the context
     fill_layer_budget_kernel<<<(h->U + NT - 1) / NT, NT, 0, s>>>(h->st, layer, ratio_budget(c, P));
     CK(h, cudaGetLastError());
   }
-  if (score_first) {
-    // Algorithm 1 with the last query over metadata and logits only; every kernel on `s`, which has
-    // joined the internal stream, so any scratch set is free
-    DecodeParams p = make_params(h, layer);
-    p.q = static_cast<const __nv_bfloat16*>(q);
-    p.t = P - 1;
-    p.append = 0; p.track = 1; p.release = 1; p.rows_absent = 1; p.plan_append = 1;
-    prefill_score_kernel<<<h->U, NT, 0, s>>>(h->st, p.sc, layer, static_cast<const __nv_bfloat16*>(k), p.q, P, h->G,
-                                             p.scale, p.scale_log2);
-    CK(h, cudaGetLastError());
-    CK(h, lrfu_dispatch(h->G, p, h->U, s));
-    prefill_rows_kernel<<<h->U, NT, 0, s>>>(h->st, layer, static_cast<const __nv_bfloat16*>(k),
-                                            static_cast<const __nv_bfloat16*>(v), P);
-    CK(h, cudaGetLastError());
-    h->prev_layer = -1;
-    h->t_layer[layer] = P - 1;
-    return CRYSTALKV_OK;
-  }
-  prefill_insert_kernel<<<h->U, NT, 0, s>>>(h->st, layer, static_cast<const __nv_bfloat16*>(k),
-                                            static_cast<const __nv_bfloat16*>(v), P, W > 0 ? 1 : 0);
+  // the whole prompt is stored; the plan written beside the copy serves the window's first pass or,
+  // in full-cache mode, the first decode step
+  prefill_take_kernel<<<h->U, NT, 0, s>>>(h->st, layer, P);
+  CK(h, cudaGetLastError());
+  prefill_rows_kernel<<<1 + h->U * per_head, NT, 0, s>>>(h->st, h->plans[layer], layer, kb, vb, P,
+                                                         W > 0 ? ROWS_ALL_POS : ROWS_ALL_LAST, per_head, evict ? 0 : 1,
+                                                         evict && W > 1 ? P - W + 1 : 0, h->grid * NW, h->grid);
   CK(h, cudaGetLastError());
   if (evict) {
-    const int passes = W > 0 ? W : 1;
     const size_t qn = (size_t)c.batch * c.n_q_heads * HD;
-    int planned_groups = -1;
-    for (int i = 0; i < passes; ++i) {
+    int planned_groups = (P - W + 1 + GRP - 1) / GRP;   // written beside the copy
+    for (int i = 0; i < W; ++i) {
       // Algorithm 1 with the query of token t: steps 1-3 for every query, step 4 (down to the
       // budget, emptied pages back to the free list) after the last one
-      const int t = P - passes + i;
-      const bool last = i == passes - 1;
+      const int t = P - W + i;
+      const bool last = i == W - 1;
       // a scoring pass over the first t + 1 entries; a plan serves the passes that follow it until
       // their heads are two groups longer (pieces take their bounds from the lengths at launch)
       const int groups = (t + 1 + GRP - 1) / GRP;
-      const bool planned = planned_groups < 0 || groups >= planned_groups + 2;
-      if (planned) {
+      if (groups >= planned_groups + 2) {
         rc = replan(h, layer, 1, 0, last ? 0 : t + 1, s);
         if (rc) return rc;
         planned_groups = groups;
@@ -658,10 +669,6 @@ static int prefill_common(crystalkv_t* h, int layer, const void* k, const void* 
     }
     rc = join_side(h, s);
     if (rc) return rc;
-  } else {
-    rc = replan(h, layer, 1, 1, 0, s);
-    if (rc) return rc;
-    h->prev_layer = -1;
   }
   h->t_layer[layer] = P - 1;
   return CRYSTALKV_OK;

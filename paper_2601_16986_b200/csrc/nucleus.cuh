@@ -1,0 +1,213 @@
+// The top-p threshold of one head, found exactly: the value theta of pbar such that the entries
+// above it (and the earliest of those equal to it) are the smallest descending-pbar prefix whose
+// exclusive mass is below p.  One histogram of 1024 bins of 1/64 octave around 1/n locates theta's
+// bin, the few entries of that bin are ranked against one another; a bin outside the window or
+// with more than 64 entries falls back to four 8-bit radix passes over all bits.
+// The mass walk uses 2^-40 fixed-point integers so it is exact and order independent; the
+// threshold is relative to the integer total, so a common factor on pbar changes nothing.
+#pragma once
+#include "common.cuh"
+
+namespace ckv {
+
+constexpr int HIST_BINS = 1024;   // shared histogram size: the fine pass uses all of it, a radix pass 256
+constexpr float MASS_ONE = 1099511627776.0f;   // 2^40
+
+constexpr int FINE_BINS = 1024;   // fast path: bins of 2^17 key steps = 1/64 octave, 16 octaves wide
+constexpr int FINE_SHIFT = 17;
+constexpr int MAX_CAND = 64;
+
+template <int NTH>
+struct NucleusSmem {
+  unsigned hist_lo[HIST_BINS];   // per-bin mass, low 16 bits of every term
+  unsigned hist_hi[HIST_BINS];   // per-bin mass, the bits above
+  unsigned long long redu[NTH / 32 + 1];
+  unsigned cand[MAX_CAND];       // keys of the entries in the threshold's bin
+  unsigned long long A_theta;    // fast path result: mass strictly above the threshold key
+  unsigned theta;                //                   the threshold key
+  int cnt_theta;                 //                   entries that carry it
+  int ncand;
+  int star;
+  int eq[NTH / 32];
+};
+
+struct Nucleus {
+  uint32_t theta;             // the threshold's key (bits of pbar); 0xffffffff: nothing is a hit
+  int cnt_eq;                 // entries that carry it
+  unsigned long long A;       // mass of the entries above it
+  unsigned long long Pthr;    // the mass below which an entry's predecessors must stay
+  bool found;
+};
+
+__device__ __forceinline__ unsigned long long mass_of(float pm) { return (unsigned long long)(pm * MASS_ONE); }
+
+// Inclusive suffix sum over the lanes of a warp (higher lane = higher bins).
+__device__ __forceinline__ unsigned long long warp_suffix(unsigned long long v, int lane) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long x = __shfl_down_sync(0xffffffffu, v, o);
+    if (lane + o < 32) v += x;
+  }
+  return v;
+}
+
+// All NTH threads of a CTA call it; `each(f)` calls f(pbar) for every entry the calling thread owns.
+template <int NTH, class Each>
+__device__ __forceinline__ Nucleus nucleus_search(int n, float top_p, NucleusSmem<NTH>& sh, int* errword, Each each) {
+  constexpr int WARPS = NTH / 32;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  // ---- fast path, pass over all entries: histogram of mass in fine bins around 1/n
+  //      bin(key) = clamp((key >> 17) - base, 0, 1023), monotone in key
+  const int fbase = (int)(__float_as_uint(1.0f / (256.0f * (float)n)) >> FINE_SHIFT);
+  auto fbin = [&](uint32_t key) { return min(FINE_BINS - 1, max(0, (int)(key >> FINE_SHIFT) - fbase)); };
+  for (int b = tid; b < FINE_BINS; b += NTH) { sh.hist_lo[b] = 0u; sh.hist_hi[b] = 0u; }
+  if (tid == 0) { sh.star = -1; sh.ncand = 0; sh.theta = 0xffffffffu; sh.cnt_theta = 0; }
+  __syncthreads();
+  each([&](float pm) {
+    const unsigned long long m = mass_of(pm);
+    const int b = fbin(__float_as_uint(pm));
+    atomicAdd(&sh.hist_lo[b], (unsigned)(m & 0xffffu));
+    atomicAdd(&sh.hist_hi[b], (unsigned)(m >> 16));
+  });
+  __syncthreads();
+  Nucleus r;
+  unsigned long long W = 0, A = 0;   // A: mass of keys strictly above the threshold's bin / prefix range
+  {
+    // suffix sums from the top bin: thread k owns bins [PER k, PER (k + 1))
+    constexpr int PER = FINE_BINS / NTH;
+    unsigned long long hb[PER], loc = 0;
+#pragma unroll
+    for (int b = 0; b < PER; ++b) {
+      hb[b] = ((unsigned long long)sh.hist_hi[tid * PER + b] << 16) + sh.hist_lo[tid * PER + b];
+      loc += hb[b];
+    }
+    const unsigned long long suf = warp_suffix(loc, lane);
+    if (lane == 0) sh.redu[w] = suf;
+    __syncthreads();
+    unsigned long long above = 0;
+    for (int x = 0; x < WARPS; ++x) {
+      const unsigned long long v = sh.redu[x];
+      W += v;
+      if (x > w) above += v;
+    }
+    // hit  <=>  mass strictly before the entry  <  p * W
+    r.Pthr = (unsigned long long)ceil((double)top_p * (double)W);
+    unsigned long long sab = above + (suf - loc);   // mass above this thread's top bin
+#pragma unroll
+    for (int b = PER - 1; b >= 0; --b) {
+      if (sab < r.Pthr && r.Pthr <= sab + hb[b]) {
+        sh.star = tid * PER + b;
+        sh.redu[WARPS] = sab;
+      }
+      sab += hb[b];
+    }
+    __syncthreads();
+  }
+  const unsigned long long Pthr = r.Pthr;
+  uint32_t theta = 0xffffffffu;
+  int cnt_eq = 0;
+  bool found = false;
+  const int bstar = sh.star;
+  if (bstar > 0 && bstar < FINE_BINS - 1) {   // inside the window: rank the bin's entries exactly
+    A = sh.redu[WARPS];
+    each([&](float pm) {
+      const uint32_t key = __float_as_uint(pm);
+      if (fbin(key) == bstar) {
+        const int x = atomicAdd(&sh.ncand, 1);
+        if (x < MAX_CAND) sh.cand[x] = key;
+      }
+    });
+    __syncthreads();
+    const int c = sh.ncand;
+    if (c <= MAX_CAND) {
+      // candidate x carries the threshold iff  A + mass(keys above it) < Pthr <= that + mass(keys equal)
+      if (tid < c) {
+        const uint32_t mine = sh.cand[tid];
+        const unsigned long long wm = mass_of(__uint_as_float(mine));
+        unsigned long long gt = 0;
+        int eqc = 0;
+        for (int x = 0; x < c; ++x) {
+          const uint32_t kx = sh.cand[x];
+          if (kx > mine) gt += mass_of(__uint_as_float(kx));
+          eqc += (kx == mine);
+        }
+        if (A + gt < Pthr && Pthr <= A + gt + (unsigned long long)eqc * wm) {
+          sh.theta = mine;            // every carrier writes the same three values
+          sh.A_theta = A + gt;
+          sh.cnt_theta = eqc;
+        }
+      }
+      __syncthreads();
+      if (sh.cnt_theta > 0) {
+        theta = sh.theta;
+        A = sh.A_theta;
+        cnt_eq = sh.cnt_theta;
+        found = true;
+      }
+    }
+  }
+  if (!found) {
+    // ---- general path: MSB-first radix passes over the fp32 bits of pbar, 8 bits each
+    A = 0;
+    uint32_t prefix = 0;
+    found = true;
+    for (int pass = 0; pass < 4; ++pass) {
+      const int sft = 24 - 8 * pass;
+      constexpr int NB = 256;
+      __syncthreads();
+      for (int b = tid; b < NB; b += NTH) { sh.hist_lo[b] = 0u; sh.hist_hi[b] = 0u; }
+      if (tid == 0) sh.star = -1;
+      __syncthreads();
+      each([&](float pm) {
+        const uint32_t key = __float_as_uint(pm);
+        const bool match = (pass == 0) || ((key >> (sft + 8)) == (prefix >> (sft + 8)));
+        if (match) {
+          const unsigned long long m = mass_of(pm);
+          const int b = (key >> sft) & (NB - 1);
+          atomicAdd(&sh.hist_lo[b], (unsigned)(m & 0xffffu));
+          atomicAdd(&sh.hist_hi[b], (unsigned)(m >> 16));
+        }
+      });
+      __syncthreads();
+      // suffix sums from the top bin: thread k < 256 owns bin k
+      static_assert(NTH >= NB, "one bin per thread");
+      const unsigned long long hb =
+          tid < NB ? ((unsigned long long)sh.hist_hi[tid] << 16) + sh.hist_lo[tid] : 0ull;
+      const unsigned long long suf = warp_suffix(hb, lane);
+      if (lane == 0) sh.redu[w] = suf;
+      __syncthreads();
+      unsigned long long above = 0;
+      for (int x = w + 1; x < WARPS; ++x) above += sh.redu[x];
+      const unsigned long long sab = A + above + (suf - hb);   // mass above this thread's bin
+      if (tid < NB && sab < Pthr && Pthr <= sab + hb) {
+        sh.star = tid;
+        sh.redu[WARPS] = sab;
+      }
+      __syncthreads();
+      const int dstar = sh.star;
+      if (dstar < 0) { found = false; break; }
+      prefix |= (uint32_t)dstar << sft;
+      A = sh.redu[WARPS];
+    }
+    __syncthreads();
+    if (!found) {
+      if (tid == 0) atomicOr(errword, ERR_NUCLEUS);
+      prefix = 0xffffffffu;  // nothing is a hit
+    }
+    // entries whose pbar equals the threshold key share one mass; the earliest positions win
+    theta = prefix;
+    int eq = 0;
+    each([&](float pm) { eq += (__float_as_uint(pm) == theta); });
+    eq = warp_sum_i(eq);
+    if (lane == 0) sh.eq[w] = eq;
+    __syncthreads();
+    for (int x = 0; x < WARPS; ++x) cnt_eq += sh.eq[x];
+  }
+  r.theta = theta;
+  r.cnt_eq = cnt_eq;
+  r.A = A;
+  r.found = found;
+  return r;
+}
+
+}  // namespace ckv

@@ -148,6 +148,43 @@ def test_prompt_far_longer_than_the_budget_needs_no_reserve(prompt, budget):
     ls.close()
 
 
+@pytest.mark.parametrize("prompt,budget,G", [(1, 4, 1), (15, 7, 5), (16, 16, 3), (17, 16, 8), (127, 200, 2), (129, 128, 4),
+                                             (513, 512, 7), (1025, 300, 6), (2049, 2048, 5)])
+def test_prompt_sizes_around_tiles_and_chunks(prompt, budget, G):
+    """Lengths one off the 16-key tiles, the chunks of the scoring kernel and the select kernel's 1024
+    threads, below and above the budget, for every group size."""
+    wl = Workload(name=f"edge{prompt}", seed=900 + prompt, n_layers=2, n_q_heads=3 * G, n_kv_heads=3, batch=2, prompt=prompt,
+                  think_steps=3, budget_per_head=budget, outlier="flat", outlier_frac=0.05)
+    ls = LockStep(wl, [0, 1], max_budget=max(4 * budget, prompt))
+    ls.prefill()
+    for _ in range(wl.think_steps):
+        ls.step()
+    ls.gpu.check()
+    ls.assert_clean()
+    ls.close()
+
+
+@pytest.mark.parametrize("prompt,budget", [(100, 40), (41003, 100)])
+def test_prompt_of_equal_keys_keeps_the_latest_hits(prompt, budget):
+    """All scores equal: token i is a hit iff i / P < p, misses leave first, then the earliest hits.  The
+    longer prompt's probabilities do not fit shared memory."""
+    from paper_2601_16986_b200 import Config, CrystalKV
+    kv = CrystalKV(Config(n_layers=1, n_q_heads=4, n_kv_heads=2, batch=1, budget_per_head=budget, max_context=prompt + 8,
+                          max_budget=prompt))
+    g = torch.Generator("cuda").manual_seed(3)
+    k = torch.randn(1, 1, 2, 128, device="cuda", generator=g).to(torch.bfloat16).expand(1, prompt, 2, 128).contiguous()
+    q = torch.randn(1, 4, 128, device="cuda", generator=g).to(torch.bfloat16)
+    kv.prefill(0, k, k, q)
+    hits = int(np.ceil(float(np.float32(0.9)) * prompt))
+    for h in range(2):
+        rec = kv.export_state(0, 0, h)
+        assert (rec[:, 0] == np.arange(hits - budget, hits)).all()
+        assert (rec[:, 1].view(np.float32) == 1.0).all() and (rec[:, 2] == prompt - 1).all()
+    kv.check()
+    kv.validate()
+    kv.close()
+
+
 def test_ratio_budgets_follow_the_context():
     """Ratio budgets: the prompt's share at prefill (heads evict down to it), then Algorithm 2 over a
     total that grows with the context at every reallocation; budgets, retained sets and CRF state
