@@ -1,5 +1,5 @@
-// Algorithm 1 step 4 for the cases in which several entries leave a head at once (a prompt longer
-// than the budget, a budget that shrank, a buffered eviction cadence): pick the k entries lowest
+// Algorithm 1 step 4 for the cases in which several entries leave a head at once (a prompt
+// with an observation window, a budget that shrank, a buffered eviction cadence): pick the k entries lowest
 // under (CRF decayed to now, tau, position) by a radix select, then close the gaps they leave by
 // moving at most k entries from the end of the list into them (their rows and their metadata), so
 // that the list is dense again and the pages past its end can go back to the sequence's free
