@@ -278,6 +278,19 @@ int replan(crystalkv_t* h, int layer0, int count, int append, int n_limit, cudaS
   return CRYSTALKV_OK;
 }
 
+// Brings the heads of `count` layers down to their budgets, on `s`, which has joined the internal
+// streams (no launch uses a logit set meanwhile).
+int shrink_layers(crystalkv_t* h, int layer0, int count, int t_last, cudaStream_t s) {
+  ShrinkScratch sc;
+  for (int i = 0; i < NSETS; ++i) sc.area[i] = reinterpret_cast<int*>(h->sc_logits[i]);
+  sc.cap_s = h->cap_s;
+  for (int l = 0; l < count; l += SHRINK_LAYERS) {
+    shrink_kernel<<<dim3(h->U, std::min(SHRINK_LAYERS, count - l)), NT, 0, s>>>(h->st, layer0 + l, t_last, sc);
+    CK(h, cudaGetLastError());
+  }
+  return CRYSTALKV_OK;
+}
+
 // Makes `s` wait for every LRFU kernel launched so far.
 int join_side(crystalkv_t* h, cudaStream_t s) {
   h->prev_layer = -1;
@@ -806,10 +819,7 @@ int crystalkv_rebudget(crystalkv_t* h, void* stream) {
   const long long B_total = (long long)(c.budget_ratio > 0.f ? ratio_budget(c, t_last + 1) : c.budget_per_head) * N;
   alg2_kernel<<<c.batch, NT, sm, s>>>(h->Asum, h->st.budget, c.n_layers, c.n_kv_heads, B_total, c.min_budget, c.max_budget);
   CK(h, cudaGetLastError());
-  for (int l = 0; l < c.n_layers; ++l) {
-    shrink_kernel<<<h->U, NT, 0, s>>>(h->st, l, t_last, reinterpret_cast<int*>(h->sc_pbar[0]), h->cap_s);
-    CK(h, cudaGetLastError());
-  }
+  if (int sr = shrink_layers(h, 0, c.n_layers, t_last, s)) return sr;
   // heads changed length: every layer's next decode step needs a new plan
   return replan(h, 0, c.n_layers, 1, 0, s);
 }
@@ -827,8 +837,7 @@ int crystalkv_set_budget(crystalkv_t* h, int layer, int seq, int kv_head, int32_
   CK(h, cudaMemcpyAsync(h->st.budget + uid, &budget, sizeof(int), cudaMemcpyHostToDevice, s));
   CK(h, cudaStreamSynchronize(s));
   if (h->t_layer[layer] >= 0) {
-    shrink_kernel<<<h->U, NT, 0, s>>>(h->st, layer, h->t_layer[layer], reinterpret_cast<int*>(h->sc_pbar[0]), h->cap_s);
-    CK(h, cudaGetLastError());
+    if (int sr = shrink_layers(h, layer, 1, h->t_layer[layer], s)) return sr;
     return replan(h, layer, 1, 1, 0, s);
   }
   return CRYSTALKV_OK;
