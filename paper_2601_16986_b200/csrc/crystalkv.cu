@@ -46,7 +46,6 @@ struct crystalkv {
   float* sc_partials[2] = {};
   int* sc_ticket[2] = {};
   float* sc_pbar[2] = {};          // one per internal stream
-  int* piece_ctr = nullptr;
   int cap_s = 0, pmax = 0;
   long long nA = 0;                // attention launches so far
   std::vector<int> t_layer;        // per layer: time of the last step
@@ -75,7 +74,7 @@ struct crystalkv {
   unsigned char* io_rows = nullptr;
   int* io_n = nullptr;
   float* tab = nullptr;
-  std::vector<void*> allocs;
+  void* arena = nullptr;           // the one device allocation all of the above point into
   std::string err;
   bool cuda_dead = false;
 };
@@ -127,19 +126,31 @@ struct DeviceScope {
   DeviceScope dev_scope_((h)->cfg.device); \
   CK((h), dev_scope_.err)
 
-template <typename T>
-int dalloc(crystalkv_t* h, T** p, size_t count) {
-  void* q = nullptr;
-  cudaError_t e = cudaMalloc(&q, std::max<size_t>(count, 1) * sizeof(T));
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return fail(h, e == cudaErrorMemoryAllocation ? CRYSTALKV_ENOMEM : CRYSTALKV_ECUDA,
-                std::string("cudaMalloc: ") + cudaGetErrorString(e));
+// A handle's device arrays are parts of one allocation.  Some 330 separate ones (staging sets, logit
+// sets, lists) cost a handle of the 8B shape (5.5 GB) 16 ms to take and 16 ms to give back, against
+// 0.5 and 2.3 ms for one of the same total size.
+struct Arena {
+  struct Part { void** where; size_t at; };
+  std::vector<Part> parts;
+  size_t bytes = 0;
+  template <typename T>
+  void add(T** p, size_t count) {
+    parts.push_back({reinterpret_cast<void**>(p), bytes});
+    bytes += (std::max<size_t>(count, 1) * sizeof(T) + 255) / 256 * 256;   // every array starts on a 256-byte boundary
   }
-  h->allocs.push_back(q);
-  *p = static_cast<T*>(q);
-  return CRYSTALKV_OK;
-}
+  int take(crystalkv_t* h) {
+    void* base = nullptr;
+    cudaError_t e = cudaMalloc(&base, bytes);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return fail(h, e == cudaErrorMemoryAllocation ? CRYSTALKV_ENOMEM : CRYSTALKV_ECUDA,
+                  std::string("cudaMalloc: ") + cudaGetErrorString(e));
+    }
+    h->arena = base;
+    for (const Part& x : parts) *x.where = static_cast<unsigned char*>(base) + x.at;
+    return CRYSTALKV_OK;
+  }
+};
 
 __global__ void init_free_stack_kernel(int* stack, int* top, long long pages_per_seq, int batch) {
   const long long total = pages_per_seq * batch;
@@ -396,7 +407,7 @@ int crystalkv_destroy(crystalkv_t* h) {
     if (e) cudaEventDestroy(e);
   for (cudaEvent_t e : h->evF)
     if (e) cudaEventDestroy(e);
-  for (void* p : h->allocs) cudaFree(p);
+  if (h->arena) cudaFree(h->arena);
   delete h;
   return CRYSTALKV_OK;
 }
@@ -450,17 +461,9 @@ int crystalkv_create(const crystalkv_config_t* cfg, crystalkv_t** out) {
       CREATE_FAIL(CRYSTALKV_ECUDA);                                            \
     }                                                                          \
   } while (0)
-#define DA(ptr, count)                                   \
-  do {                                                   \
-    int r_ = dalloc(h, ptr, (size_t)(count));            \
-    if (r_) CREATE_FAIL(r_);                             \
-  } while (0)
-
   DeviceScope scope(c.device);
   CKC(scope.err);
-  cudaDeviceProp prop;
-  CKC(cudaGetDeviceProperties(&prop, c.device));
-  h->num_sms = prop.multiProcessorCount;
+  CKC(cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, c.device));
   // ring stages, one mbarrier per stage, every warp's queue of fetched pieces: the same for every
   // handle (the attribute belongs to the function, so no handle may lower it under another)
   h->smem = RING_BYTES + NW * STAGES * 8 + NW * FIFO * sizeof(int);
@@ -493,67 +496,73 @@ int crystalkv_create(const crystalkv_config_t* cfg, crystalkv_t** out) {
   State& st = h->st;
   st.batch = c.batch; st.L = c.n_layers; st.H = c.n_kv_heads; st.cap = h->cap; st.capg = h->cap / GRP;
   st.pages_per_seq = h->pages_per_seq;
-  DA(&st.pool, (size_t)c.batch * h->pages_per_seq * PAGE_BYTES);
-  DA(&st.free_stack, (size_t)c.batch * h->pages_per_seq);
-  DA(&st.free_top, c.batch);
-  DA(&st.ptab, (size_t)h->units * st.capg);
-  DA(&st.meta_pos, (size_t)h->units * h->cap);
-  DA(&st.meta_tau, (size_t)h->units * h->cap);
-  DA(&st.meta_crf, (size_t)h->units * h->cap);
-  DA(&st.n_cur, h->units);
-  DA(&st.hole, h->units);
-  DA(&st.npages, h->units);
-  DA(&st.budget, h->units);
   // launch plans, one per layer: at most one piece per warp and one more per head
-  {
-    const int nWarps = h->grid * NW, pd_cap = nWarps + h->U;
-    int4* desc = nullptr; int4* wr = nullptr; int *npc = nullptr, *gpl = nullptr, *hdr = nullptr;
-    DA(&desc, (size_t)c.n_layers * pd_cap);
-    DA(&wr, (size_t)c.n_layers * nWarps);
-    DA(&npc, (size_t)c.n_layers * h->U);
-    DA(&gpl, (size_t)c.n_layers * h->U);
-    DA(&hdr, (size_t)c.n_layers * 4);
-    CKC(cudaMemset(hdr, 0, (size_t)c.n_layers * 4 * sizeof(int)));
-    h->plans.resize(c.n_layers);
-    for (int l = 0; l < c.n_layers; ++l)
-      h->plans[l] = Plan{desc + (size_t)l * pd_cap, wr + (size_t)l * nWarps, npc + (size_t)l * h->U, gpl + (size_t)l * h->U,
-                         hdr + (size_t)l * 4};
-    DA(&h->d_plans, c.n_layers);
-    CKC(cudaMemcpy(h->d_plans, h->plans.data(), (size_t)c.n_layers * sizeof(Plan), cudaMemcpyHostToDevice));
-    DA(&h->done_ctr, 4);   // per internal stream: finished CTAs of its running LRFU kernel; whether the layer's plan went stale
-    CKC(cudaMemset(h->done_ctr, 0, 4 * sizeof(int)));
-  }
-  DA(&h->tab, (size_t)c.max_context + 1);
-  st.tab = h->tab;
-  DA(&st.errword, 1);
-  DA(&st.counters, 4);
-  DA(&h->Asum, h->units);
+  const int nWarps = h->grid * NW, pd_cap = nWarps + h->U;
+  int4 *desc = nullptr, *wr = nullptr;
+  int *npc = nullptr, *gpl = nullptr, *hdr = nullptr;
   const int capgroups = (h->cap + GRP - 1) / GRP;
   h->cap_s = evict ? h->cap : 4;   // whole 128-byte lines of logit rows per unit (cap is a multiple of 16)
   h->pmax = capgroups / GMIN + 2;
-  for (int i = 0; i < NSETS; ++i) {
-    DA(&h->sc_logits[i], (size_t)h->U * h->cap_s * QH);
-    DA(&h->sc_mfin[i], (size_t)h->U * 2 * QH);
-  }
-  for (int i = 0; i < 2; ++i) {
-    DA(&h->sc_partials[i], (size_t)h->U * h->pmax * (16 + h->G * HD));
-    DA(&h->sc_ticket[i], h->U);
-    CKC(cudaMemset(h->sc_ticket[i], 0, (size_t)h->U * sizeof(int)));
-  }
-  for (int i = 0; i < 2; ++i) DA(&h->sc_pbar[i], (size_t)h->U * h->cap_s);
-  DA(&h->piece_ctr, 4);
-  CKC(cudaMemset(h->piece_ctr, 0, 4 * sizeof(int)));
   const size_t qn = (size_t)c.batch * c.n_q_heads * HD, kn = (size_t)c.batch * c.n_kv_heads * HD;
-  for (int i = 0; i < crystalkv::HOST_RING; ++i) { DA(&h->dq[i], qn); DA(&h->dout[i], qn); DA(&h->dk[i], kn); DA(&h->dv[i], kn); }
-  DA(&h->dummy_out, qn);
-  DA(&h->io_rec, (size_t)3 * h->cap);
-  DA(&h->io_rows, (size_t)2 * h->cap * ROW_BYTES);
-  DA(&h->io_n, 1);
+  {
+    Arena a;
+    a.add(&st.pool, (size_t)c.batch * h->pages_per_seq * PAGE_BYTES);
+    a.add(&st.free_stack, (size_t)c.batch * h->pages_per_seq);
+    a.add(&st.free_top, c.batch);
+    a.add(&st.ptab, (size_t)h->units * st.capg);
+    a.add(&st.meta_pos, (size_t)h->units * h->cap);
+    a.add(&st.meta_tau, (size_t)h->units * h->cap);
+    a.add(&st.meta_crf, (size_t)h->units * h->cap);
+    a.add(&st.n_cur, h->units);
+    a.add(&st.hole, h->units);
+    a.add(&st.npages, h->units);
+    a.add(&st.budget, h->units);
+    a.add(&desc, (size_t)c.n_layers * pd_cap);
+    a.add(&wr, (size_t)c.n_layers * nWarps);
+    a.add(&npc, (size_t)c.n_layers * h->U);
+    a.add(&gpl, (size_t)c.n_layers * h->U);
+    a.add(&hdr, (size_t)c.n_layers * 4);
+    a.add(&h->d_plans, c.n_layers);
+    a.add(&h->done_ctr, 4);   // per internal stream: finished CTAs of its running LRFU kernel; whether the layer's plan went stale
+    a.add(&h->tab, (size_t)c.max_context + 1);
+    a.add(&st.errword, 1);
+    a.add(&st.counters, 4);
+    a.add(&h->Asum, h->units);
+    for (int i = 0; i < NSETS; ++i) {
+      a.add(&h->sc_logits[i], (size_t)h->U * h->cap_s * QH);
+      a.add(&h->sc_mfin[i], (size_t)h->U * 2 * QH);
+    }
+    for (int i = 0; i < 2; ++i) {
+      a.add(&h->sc_partials[i], (size_t)h->U * h->pmax * (16 + h->G * HD));
+      a.add(&h->sc_ticket[i], h->U);
+      a.add(&h->sc_pbar[i], (size_t)h->U * h->cap_s);
+    }
+    for (int i = 0; i < crystalkv::HOST_RING; ++i) {
+      a.add(&h->dq[i], qn); a.add(&h->dout[i], qn); a.add(&h->dk[i], kn); a.add(&h->dv[i], kn);
+    }
+    a.add(&h->dummy_out, qn);
+    a.add(&h->io_rec, (size_t)3 * h->cap);
+    a.add(&h->io_rows, (size_t)2 * h->cap * ROW_BYTES);
+    a.add(&h->io_n, 1);
+    if (int r = a.take(h)) CREATE_FAIL(r);
+  }
+  st.tab = h->tab;
+  CKC(cudaMemset(hdr, 0, (size_t)c.n_layers * 4 * sizeof(int)));
+  CKC(cudaMemset(h->done_ctr, 0, 4 * sizeof(int)));
+  for (int i = 0; i < 2; ++i) CKC(cudaMemset(h->sc_ticket[i], 0, (size_t)h->U * sizeof(int)));
+  h->plans.resize(c.n_layers);
+  for (int l = 0; l < c.n_layers; ++l)
+    h->plans[l] = Plan{desc + (size_t)l * pd_cap, wr + (size_t)l * nWarps, npc + (size_t)l * h->U, gpl + (size_t)l * h->U,
+                       hdr + (size_t)l * 4};
+  CKC(cudaMemcpy(h->d_plans, h->plans.data(), (size_t)c.n_layers * sizeof(Plan), cudaMemcpyHostToDevice));
 
   // lambda^D as fp32 from an fp64 pow; pow(0, 0) = 1 keeps same-step hits when lambda = 0
   {
     std::vector<float> tab((size_t)c.max_context + 1);
-    for (int D = 0; D <= c.max_context; ++D) tab[D] = (float)std::pow((double)c.lambda, (double)D);
+    for (int D = 0; D <= c.max_context; ++D) {
+      tab[D] = (float)std::pow((double)c.lambda, (double)D);
+      if (tab[D] == 0.0f && D > 0) break;   // powers of lambda < 1 do not grow again: the rest is 0
+    }
     CKC(cudaMemcpy(h->tab, tab.data(), tab.size() * sizeof(float), cudaMemcpyHostToDevice));
   }
   init_free_stack_kernel<<<1024, 256>>>(st.free_stack, st.free_top, h->pages_per_seq, c.batch);
@@ -571,7 +580,6 @@ int crystalkv_create(const crystalkv_config_t* cfg, crystalkv_t** out) {
   return CRYSTALKV_OK;
 #undef CREATE_FAIL
 #undef CKC
-#undef DA
 }
 
 int crystalkv_set_stage(crystalkv_t* h, int stage) {
