@@ -228,7 +228,7 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
   asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");   // made visible to the copy engine
   __syncthreads();
   const int4 range = __ldg(p.plan.wrange + blockIdx.x * NW + w);   // (requested together with the header)
-  if (__ldg(p.plan.hdr + 2) != (int)gridDim.x * NW || __ldg(p.plan.hdr + 3) != p.append) {   // a plan made for another launch
+  if (__ldg(p.plan.hdr + 2) != (int)gridDim.x * NW) {   // a plan made for another launch
     if (tid == 0 && blockIdx.x == 0) atomicOr(st.errword, ERR_PLAN);
     return;
   }
@@ -253,9 +253,7 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
   const int* pt = st.ptab;
   auto entries_of = [&](int u) {   // entries of head u that take part in this launch
     const int uid = ((u / st.H) * st.L + p.layer) * st.H + (u % st.H);
-    int n = __ldg(st.n_cur + uid);
-    if (p.n_limit > 0) n = min(n, p.n_limit);
-    return n + p.append;
+    return __ldg(st.n_cur + uid) + 1;
   };
   // the descriptor of the warp's first piece came with its range
   const int4 dd_first = range.z >= 0 ? make_int4(range.z, range.w & 4095, (range.w >> 12) & 4095, range.w >> 24)
@@ -337,7 +335,7 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
     const int n_tot = entries_of(u);
     const unsigned g_u = (unsigned)(n_tot + GRP - 1) / GRP;
     const int lo = (int)(g_u * (unsigned)piece / (unsigned)npieces), hi = (int)(g_u * (unsigned)(piece + 1) / (unsigned)npieces);
-    const int hole = p.append ? __ldg(st.hole + uid) : -1;   // where the arriving token goes
+    const int hole = __ldg(st.hole + uid);   // where the arriving token goes
     // A head whose pieces all belong to consecutive warps of this CTA, each warp holding nothing else
     // (the plan marks it), is merged through shared memory.
     // (A head of more than eight pieces is placed in runs of eight, whole CTAs and one shorter run:

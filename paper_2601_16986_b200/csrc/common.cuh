@@ -71,7 +71,7 @@ struct Plan {
                      // a second dependent read, or z = -1: read desc[x]
   int* npc;          // [U] pieces per head
   int* gplan;        // [U] groups per head the plan was made for
-  int* hdr;          // [4] pieces in total, groups in total, warps the plan was made for, append it was made for
+  int* hdr;          // [4] pieces in total, groups in total, warps the plan was made for, 1
 };
 
 // scratch of one launch pair (attention kernel, then LRFU kernel), assembled per launch: the
@@ -98,16 +98,11 @@ struct DecodeParams {
   int layer;
   int G;          // query heads per kv head
   int t;          // time of this step
-  int append;     // 1: decode (a new entry arrives); 0: scoring pass over the prompt
   int track;      // 1: Algorithm 1 runs (hits, CRF, eviction) in the LRFU kernel that follows
-  int release;    // 1: pages a head no longer needs go back to the free list (no pops in this launch)
   int early;      // 1: the lists and rows of this layer are final, so the attention kernel may read them
                   //    before the kernel ahead of it in the stream has completed
-  int n_limit;    // > 0: only the first n_limit entries of every head take part (a prompt token's causal view)
-  int hold;       // 1: Algorithm 1 stops after step 3; lengths and lists stay as they are
   int evict_every;   // m >= 1: step 4 waits until a head is m entries over its budget, then removes them all
   int literal;    // 1: Algorithm 1 is skipped for a head below its budget (its first line as printed)
-  int plan_append;   // what the plan the LRFU kernel leaves behind is for: 1 = a decode step, 0 = a scoring pass
   int plan_warps;    // warps of the attention grid the plan is made for
   int plan_grid;     // CTAs of that grid
   float scale;    // logit scale
@@ -197,10 +192,10 @@ __device__ __forceinline__ void back_position(const State& st, int uid, int seq,
 }
 
 // A head keeps all n entries of a step: the next arrival goes behind them.
-__device__ __forceinline__ void keep_all(const State& st, int uid, int seq, int n, bool will_append) {
+__device__ __forceinline__ void keep_all(const State& st, int uid, int seq, int n) {
   st.n_cur[uid] = n;
   st.hole[uid] = n;
-  if (will_append) back_position(st, uid, seq, n);
+  back_position(st, uid, seq, n);
 }
 
 // List position of the i-th live entry of a head (i in [0, n)) given its hole.

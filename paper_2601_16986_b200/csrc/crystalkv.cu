@@ -26,6 +26,7 @@
 #include "lrfu_kernel.cuh"
 #include "plan.cuh"
 #include "prefill_kernels.cuh"
+#include "window_kernels.cuh"
 
 using namespace ckv;
 
@@ -69,7 +70,6 @@ struct crystalkv {
   cudaEvent_t evIn[HOST_RING] = {}, evUse[HOST_RING] = {}, evOut[HOST_RING] = {};
   long long outJoined = -1;   // newest host step whose copy back the caller's stream has waited for
   long long nHost = 0;             // host-buffer steps so far
-  __nv_bfloat16* dummy_out = nullptr;
   int* io_rec = nullptr;           // staging for export / import of one head: records, rows, count
   unsigned char* io_rows = nullptr;
   int* io_n = nullptr;
@@ -276,15 +276,14 @@ DecodeParams make_params(crystalkv_t* h, int layer) {
   p.top_p = h->cfg.top_p;
   p.evict_every = h->cfg.evict_every;
   p.literal = h->cfg.literal_return;
-  p.plan_append = -1;
   p.plan_warps = h->grid * NW;
   p.plan_grid = h->grid;
   return p;
 }
 
 // Writes the launch plans of `count` layers from their heads' current lengths, on `s`.
-int replan(crystalkv_t* h, int layer0, int count, int append, int n_limit, cudaStream_t s) {
-  plan_kernel<<<count, NT, 0, s>>>(h->st, h->d_plans, layer0, append, n_limit, h->grid * NW, h->grid);
+int replan(crystalkv_t* h, int layer0, int count, cudaStream_t s) {
+  plan_kernel<<<count, NT, 0, s>>>(h->st, h->d_plans, layer0, h->grid * NW, h->grid);
   CK(h, cudaGetLastError());
   return CRYSTALKV_OK;
 }
@@ -314,20 +313,16 @@ int join_side(crystalkv_t* h, cudaStream_t s) {
 
 // One attention launch on `s` and its follow-up (Algorithm 1 when it runs, the heads' new lengths
 // and the layer's next plan) on the internal stream.
-// chain: this launch scores the same, unchanged lists as the layer's previous launch (a window of
-// prompt queries): its attention kernel need not wait for that launch's LRFU kernel, only its own
-// LRFU kernel must run behind it.
-int launch_step(crystalkv_t* h, DecodeParams& p, int layer, cudaStream_t s, bool chain = false) {
-  const bool track = true;   // every launch has a follow-up that uses a scratch set
+int launch_step(crystalkv_t* h, DecodeParams& p, int layer, cudaStream_t s) {
   const long long k = h->kF;
-  if (track) {
+  {
     // launch k reuses the scratch of launch k - NSETS and continues the state its layer's
     // previous LRFU launch wrote; each internal stream runs in order, so the events of two
     // consecutive launches cover everything before them
     // A wait on the caller's stream costs several microseconds (the attention kernel behind it
     // no longer starts early), so one wait covers as many launches as the sets allow: it targets
     // the newest LRFU launch that has had two attention kernels' time to finish.
-    const long long need = chain ? k - NSETS : std::max(k - NSETS, h->lastF[layer]);
+    const long long need = std::max(k - NSETS, h->lastF[layer]);
     if (need >= 0 && need > h->joined) {
       const long long target = std::max(need, k - 3);
       CK(h, cudaStreamWaitEvent(s, h->evF[target % crystalkv::EV_RING], 0));
@@ -356,14 +351,13 @@ int launch_step(crystalkv_t* h, DecodeParams& p, int layer, cudaStream_t s, bool
     CK(h, cudaLaunchKernelEx(&lc, attn_kernel, p));
   }
   h->prev_layer = layer;
-  if (track) {
+  {
     const int si = (int)(k & 1);
     cudaEvent_t ea = h->evA[k % crystalkv::EV_RING];
     p.sc.pbar = h->sc_pbar[si];
     p.done_ctr = h->done_ctr + 2 * si;
     CK(h, cudaEventRecord(ea, s));
     CK(h, cudaStreamWaitEvent(h->side[si], ea, 0));
-    if (chain && k > 0) CK(h, cudaStreamWaitEvent(h->side[si], h->evF[(k - 1) % crystalkv::EV_RING], 0));   // (the other internal stream)
     CK(h, lrfu_dispatch(h->G, p, h->U, h->side[si]));
     CK(h, cudaEventRecord(h->evF[k % crystalkv::EV_RING], h->side[si]));
     h->lastF[layer] = k;
@@ -528,10 +522,8 @@ int crystalkv_create(const crystalkv_config_t* cfg, crystalkv_t** out) {
     a.add(&st.errword, 1);
     a.add(&st.counters, 4);
     a.add(&h->Asum, h->units);
-    for (int i = 0; i < NSETS; ++i) {
-      a.add(&h->sc_logits[i], (size_t)h->U * h->cap_s * QH);
-      a.add(&h->sc_mfin[i], (size_t)h->U * 2 * QH);
-    }
+    for (int i = 0; i < NSETS; ++i) a.add(&h->sc_logits[i], (size_t)h->U * h->cap_s * QH);   // one block: no padding between sets
+    for (int i = 0; i < NSETS; ++i) a.add(&h->sc_mfin[i], (size_t)h->U * 2 * QH);
     for (int i = 0; i < 2; ++i) {
       a.add(&h->sc_partials[i], (size_t)h->U * h->pmax * (16 + h->G * HD));
       a.add(&h->sc_ticket[i], h->U);
@@ -540,7 +532,6 @@ int crystalkv_create(const crystalkv_config_t* cfg, crystalkv_t** out) {
     for (int i = 0; i < crystalkv::HOST_RING; ++i) {
       a.add(&h->dq[i], qn); a.add(&h->dout[i], qn); a.add(&h->dk[i], kn); a.add(&h->dv[i], kn);
     }
-    a.add(&h->dummy_out, qn);
     a.add(&h->io_rec, (size_t)3 * h->cap);
     a.add(&h->io_rows, (size_t)2 * h->cap * ROW_BYTES);
     a.add(&h->io_n, 1);
@@ -600,6 +591,46 @@ int crystalkv_time(crystalkv_t* h, int layer) {
   return h->t_layer[layer];
 }
 
+// Algorithm 1 with the queries of the prompt's last W tokens, in as many launches as the scratch
+// asks for (usually one): steps 1-3 for every query, step 4 after the last one.  Everything runs on
+// `s`, which has joined the internal streams: the logit sets, one block of the arena, hold the
+// window's logits, the partials its softmax references, the first pbar area the hit bits.
+static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, const unsigned char* v, const unsigned char* q,
+                         int P, int W, __nv_bfloat16* out, cudaStream_t s) {
+  const crystalkv_config_t& c = h->cfg;
+  WindowParams p{};
+  p.k = k; p.v = v;
+  p.logits = h->sc_logits[0];
+  p.ml = h->sc_partials[0];
+  p.hits = reinterpret_cast<unsigned*>(h->sc_pbar[0]);
+  p.H = c.n_kv_heads; p.G = h->G; p.U = h->U; p.P = P;
+  p.Ps = (P + 7) / 8 * 8;   // rows of logits start on 32-byte sectors
+  p.words = (P + 31) / 32;
+  p.scale = c.sm_scale;
+  p.scale_log2 = c.sm_scale * 1.44269504088896340736f;
+  // queries of one launch: what the logit sets, the partials and the pbar area have room for
+  const long long fit = std::min<long long>((long long)NSETS * h->cap_s * QH / ((long long)h->G * p.Ps),
+                                            std::min<long long>((long long)h->pmax * (16 + h->G * HD) / 16, h->cap_s / p.words));
+  const size_t sm = (size_t)P * sizeof(float) <= WIN_SMEM ? (size_t)P * sizeof(float) : 0;
+  const auto attn = out ? window_attn_kernel<true> : window_attn_kernel<false>;
+  CK(h, cudaFuncSetAttribute(attn, cudaFuncAttributeMaxDynamicSharedMemorySize, WA_SMEM));
+  const size_t qn = (size_t)c.batch * c.n_q_heads * HD;
+  for (int w0 = 0; w0 < W; w0 += p.W) {
+    p.W = (int)std::min<long long>(W - w0, std::max<long long>(1, fit));
+    p.t0 = P - W + w0;
+    p.q = q + (size_t)w0 * qn * sizeof(__nv_bfloat16);
+    p.out = out ? out + (size_t)w0 * qn : nullptr;
+    attn<<<dim3((p.W * p.G + WA_ROWS - 1) / WA_ROWS, h->U), WA_WARPS * 32, WA_SMEM, s>>>(p);
+    CK(h, cudaGetLastError());
+    window_hits_kernel<<<dim3(p.W, h->U), NT, sm, s>>>(h->st, p, layer, c.top_p, c.literal_return, sm > 0);
+    CK(h, cudaGetLastError());
+    window_apply_kernel<<<h->U, NT, 0, s>>>(h->st, p, layer, w0 + p.W == W, c.evict_every, reinterpret_cast<int*>(h->sc_pbar[1]),
+                                            h->cap_s);
+    CK(h, cudaGetLastError());
+  }
+  return replan(h, layer, 1, s);
+}
+
 // Prompt insertion and the Algorithm 1 passes that seed CRF/tau: one pass with the last query
 // (W = 0) or a replay of the last W queries, each over the tokens up to its own.
 static int prefill_common(crystalkv_t* h, int layer, const void* k, const void* v, const void* q,
@@ -643,7 +674,7 @@ static int prefill_common(crystalkv_t* h, int layer, const void* k, const void* 
                                                    c.literal_return, c.budget_ratio > 0.f ? ratio_budget(c, P) : 0, sm > 0);
     CK(h, cudaGetLastError());
     prefill_rows_kernel<<<1 + h->U * per_head, NT, 0, s>>>(h->st, h->plans[layer], layer, kb, vb, P, ROWS_SURVIVORS, per_head,
-                                                           1, 0, h->grid * NW, h->grid);
+                                                           h->grid * NW, h->grid);
     CK(h, cudaGetLastError());
     h->t_layer[layer] = P - 1;
     return CRYSTALKV_OK;
@@ -652,43 +683,15 @@ static int prefill_common(crystalkv_t* h, int layer, const void* k, const void* 
     fill_layer_budget_kernel<<<(h->U + NT - 1) / NT, NT, 0, s>>>(h->st, layer, ratio_budget(c, P));
     CK(h, cudaGetLastError());
   }
-  // the whole prompt is stored; the plan written beside the copy serves the window's first pass or,
-  // in full-cache mode, the first decode step
+  // the whole prompt is stored; in full-cache mode the first step's plan is written beside the copy
   prefill_take_kernel<<<h->U, NT, 0, s>>>(h->st, layer, P);
   CK(h, cudaGetLastError());
   prefill_rows_kernel<<<1 + h->U * per_head, NT, 0, s>>>(h->st, h->plans[layer], layer, kb, vb, P,
-                                                         W > 0 ? ROWS_ALL_POS : ROWS_ALL_LAST, per_head, evict ? 0 : 1,
-                                                         evict && W > 1 ? P - W + 1 : 0, h->grid * NW, h->grid);
+                                                         W > 0 ? ROWS_ALL_POS : ROWS_ALL_LAST, per_head,
+                                                         evict ? 0 : h->grid * NW, h->grid);
   CK(h, cudaGetLastError());
   if (evict) {
-    const size_t qn = (size_t)c.batch * c.n_q_heads * HD;
-    int planned_groups = (P - W + 1 + GRP - 1) / GRP;   // written beside the copy
-    for (int i = 0; i < W; ++i) {
-      // Algorithm 1 with the query of token t: steps 1-3 for every query, step 4 (down to the
-      // budget, emptied pages back to the free list) after the last one
-      const int t = P - W + i;
-      const bool last = i == W - 1;
-      // a scoring pass over the first t + 1 entries; a plan serves the passes that follow it until
-      // their heads are two groups longer (pieces take their bounds from the lengths at launch)
-      const int groups = (t + 1 + GRP - 1) / GRP;
-      if (groups >= planned_groups + 2) {
-        rc = replan(h, layer, 1, 0, last ? 0 : t + 1, s);
-        if (rc) return rc;
-        planned_groups = groups;
-      }
-      DecodeParams p = make_params(h, layer);
-      p.q = static_cast<const __nv_bfloat16*>(q) + (size_t)i * qn;
-      p.k_new = p.v_new = nullptr;
-      p.out = out_window ? static_cast<__nv_bfloat16*>(out_window) + (size_t)i * qn : h->dummy_out;
-      p.t = t;
-      p.append = 0; p.track = 1; p.release = 1;
-      if (!last) { p.n_limit = t + 1; p.hold = 1; }
-      else p.plan_append = 1;   // the layer's first decode step
-      h->prev_layer = -1;       // the plan kernel ahead writes what the attention kernel reads at once
-      rc = launch_step(h, p, layer, s, i > 0);
-      if (rc) return rc;
-    }
-    rc = join_side(h, s);
+    rc = replay_window(h, layer, kb, vb, static_cast<const unsigned char*>(q), P, W, static_cast<__nv_bfloat16*>(out_window), s);
     if (rc) return rc;
   }
   h->t_layer[layer] = P - 1;
@@ -728,8 +731,7 @@ int crystalkv_decode_step(crystalkv_t* h, int layer, const void* q, const void* 
   p.v_new = static_cast<const __nv_bfloat16*>(v_new);
   p.out = static_cast<__nv_bfloat16*>(out);
   p.t = t;
-  p.append = 1; p.track = track ? 1 : 0; p.release = 0;
-  p.plan_append = 1;
+  p.track = track ? 1 : 0;
   rc = launch_step(h, p, layer, static_cast<cudaStream_t>(stream));
   if (rc) return rc;
   h->t_layer[layer] = t;
@@ -829,7 +831,7 @@ int crystalkv_rebudget(crystalkv_t* h, void* stream) {
   CK(h, cudaGetLastError());
   if (int sr = shrink_layers(h, 0, c.n_layers, t_last, s)) return sr;
   // heads changed length: every layer's next decode step needs a new plan
-  return replan(h, 0, c.n_layers, 1, 0, s);
+  return replan(h, 0, c.n_layers, s);
 }
 
 int crystalkv_set_budget(crystalkv_t* h, int layer, int seq, int kv_head, int32_t budget, void* stream) {
@@ -846,7 +848,7 @@ int crystalkv_set_budget(crystalkv_t* h, int layer, int seq, int kv_head, int32_
   CK(h, cudaStreamSynchronize(s));
   if (h->t_layer[layer] >= 0) {
     if (int sr = shrink_layers(h, layer, 1, h->t_layer[layer], s)) return sr;
-    return replan(h, layer, 1, 1, 0, s);
+    return replan(h, layer, 1, s);
   }
   return CRYSTALKV_OK;
 }
@@ -978,7 +980,7 @@ int crystalkv_import_state(crystalkv_t* h, int layer, int seq, int kv_head, cons
   CK(h, cudaStreamSynchronize(s));   // the host buffers and the staging area are free again
   h->t_layer[layer] = t;
   h->prev_layer = -1;
-  return replan(h, layer, 1, 1, 0, s);
+  return replan(h, layer, 1, s);
 }
 
 int crystalkv_get_counters(crystalkv_t* h, uint64_t* entries_attended, uint64_t* hits,

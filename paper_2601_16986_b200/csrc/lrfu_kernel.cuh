@@ -186,7 +186,7 @@ __device__ int lrfu_unit(const DecodeParams& p, int u, int uid, int seq, int n, 
 
   // ---- steps 2-3: CRF/tau update; step 4 candidates
   // step 4 runs once the head is evict_every entries over its budget, and then for all of them
-  const int k_evict = (!p.hold && n - fr.budget >= p.evict_every) ? n - fr.budget : 0;
+  const int k_evict = (n - fr.budget >= p.evict_every) ? n - fr.budget : 0;
   uint32_t bk0 = 0xffffffffu, bk1 = 0xffffffffu, bk2 = 0xffffffffu;
   int bidx = -1, nhit = 0;
   auto update = [&](int i, float pm, int pos_i, int tau, float crf, float dec) {
@@ -281,11 +281,11 @@ __device__ int lrfu_unit(const DecodeParams& p, int u, int uid, int seq, int n, 
     n_after = n - 1;
   } else if (k_evict > 1) {
     __syncthreads();
-    if (p.append && k_evict > p.evict_every && tid == 0) atomicOr(st.errword, ERR_OVER_EVICT);
-    evict_many(st, uid, seq, n, min(k_evict, n - 1), p.t, p.release != 0, sh.ev, reinterpret_cast<int*>(pbar));
+    if (k_evict > p.evict_every && tid == 0) atomicOr(st.errword, ERR_OVER_EVICT);
+    evict_many(st, uid, seq, n, min(k_evict, n - 1), p.t, false, sh.ev, reinterpret_cast<int*>(pbar));
     n_after = n - min(k_evict, n - 1);
   }
-  if (n_after == n && tid == 0 && !p.hold) keep_all(st, uid, seq, n, p.append != 0);
+  if (n_after == n && tid == 0) keep_all(st, uid, seq, n);
   return n_after;   // the head's length after the step
 }
 
@@ -297,10 +297,8 @@ __global__ void __launch_bounds__(NT, 5) lrfu_kernel(const DecodeParams p) {
   const int uid = (seq * st.L + p.layer) * st.H + head;
   // one batch of requests: the length, the budget, the softmax reference, and the logit rows the
   // common path needs (requested for a full thread's worth, clamped to the scratch)
-  int n_raw = ld_i32(st.n_cur + uid);
-  const int g_plan = (threadIdx.x == 0 && p.plan_append >= 0) ? ld_i32(p.plan.gplan + u) : 0;   // used at the very end
-  if (p.n_limit > 0) n_raw = min(n_raw, p.n_limit);
-  const int n = n_raw + p.append;
+  const int n = ld_i32(st.n_cur + uid) + 1;
+  const int g_plan = threadIdx.x == 0 ? ld_i32(p.plan.gplan + u) : 0;   // used at the very end
   int n_new = n;   // the head's length after this launch
   if (p.track) {
     Front<G> fr;
@@ -320,10 +318,10 @@ __global__ void __launch_bounds__(NT, 5) lrfu_kernel(const DecodeParams p) {
       }
     }
     if (n <= 0) {
-      if (threadIdx.x == 0 && !p.hold) { st.n_cur[uid] = 0; st.hole[uid] = 0; }
+      if (threadIdx.x == 0) { st.n_cur[uid] = 0; st.hole[uid] = 0; }
       n_new = 0;
     } else if (p.literal && n < fr.budget) {   // Algorithm 1's first line as printed: nothing runs below the budget
-      if (threadIdx.x == 0 && !p.hold) keep_all(st, uid, seq, n, p.append != 0);
+      if (threadIdx.x == 0) keep_all(st, uid, seq, n);
     } else if (n <= FRONT * NT) {
       n_new = lrfu_unit<G, FRONT>(p, u, uid, seq, n, sh, fr);
     } else if (n <= 10 * NT) {
@@ -334,10 +332,9 @@ __global__ void __launch_bounds__(NT, 5) lrfu_kernel(const DecodeParams p) {
       n_new = lrfu_unit<G, 0>(p, u, uid, seq, n, sh, fr);
     }
   } else if (threadIdx.x == 0) {
-    keep_all(st, uid, seq, n, p.append != 0);   // no Algorithm 1: the head keeps its new entry
+    keep_all(st, uid, seq, n);   // no Algorithm 1: the head keeps its new entry
   }
   if (threadIdx.x == 0) atomicAdd(&st.counters[0], (unsigned long long)max(n, 0));
-  if (p.plan_append < 0) return;
   // ---- The layer's plan names pieces by (head, j of k), so it stays correct while heads grow or
   // shrink a little; a head whose group count has drifted from the planned one by an eighth (at
   // least two), or a next launch of another kind than this one, marks it stale, and the CTA that
@@ -345,8 +342,8 @@ __global__ void __launch_bounds__(NT, 5) lrfu_kernel(const DecodeParams p) {
   // entry arrives, one leaves) nothing is written.  Thread 0 wrote the head's new length itself,
   // so the release of its count makes that length visible to whoever acquires the last count.
   if (threadIdx.x == 0) {
-    const int g_new = (n_new + p.plan_append + GRP - 1) / GRP;
-    if (abs(g_new - g_plan) >= max(2, g_plan >> 3) || p.append != p.plan_append) atomicOr(p.done_ctr + 1, 1);
+    const int g_new = (n_new + 1 + GRP - 1) / GRP;
+    if (abs(g_new - g_plan) >= max(2, g_plan >> 3)) atomicOr(p.done_ctr + 1, 1);
     int done;
     asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;\n" : "=r"(done) : "l"(p.done_ctr) : "memory");
     int last = (done == (int)gridDim.x - 1);
@@ -358,7 +355,7 @@ __global__ void __launch_bounds__(NT, 5) lrfu_kernel(const DecodeParams p) {
   }
   __syncthreads();
   if (!sh.is_last) return;
-  write_plan(st, p.plan, p.layer, p.plan_append, 0, p.plan_warps, p.plan_grid, reinterpret_cast<int*>(&sh), sh.ev);
+  write_plan(st, p.plan, p.layer, p.plan_warps, p.plan_grid, reinterpret_cast<int*>(&sh), sh.ev);
 }
 
 }  // namespace ckv

@@ -51,18 +51,16 @@ __host__ __device__ __forceinline__ int ctas_needed(int full, const int (&cnt)[8
 }
 
 // Called by all NT threads of one CTA.  `gs` is shared memory for U + 1 ints, `red` for 320.
-// append: the plan is for a decode step (every head one entry longer than now); n_limit > 0: for
-// a scoring pass over the first n_limit entries of every head.
-__device__ __forceinline__ void write_plan(const State& st, const Plan& pl, int layer, int append, int n_limit, int nWarps,
-                                        int grid, int* gs, int* red) {
+// The plan is for a decode step: every head one entry longer than now.
+__device__ __forceinline__ void write_plan(const State& st, const Plan& pl, int layer, int nWarps, int grid,
+                                        int* gs, int* red) {
   const int U = st.batch * st.H, tid = threadIdx.x, lane = tid & 31;
   // ---- groups per head
   int mine = 0, gmax = 0, empty = 0;
   for (int u = tid; u < U; u += NT) {
     const int uid = ((u / st.H) * st.L + layer) * st.H + (u % st.H);
-    int n = __ldcg(st.n_cur + uid);   // (other CTAs of the calling kernel may just have written it: not from L1)
-    if (n_limit > 0) n = min(n, n_limit);
-    const int g = (n + append + GRP - 1) / GRP;
+    const int n = __ldcg(st.n_cur + uid);   // (other CTAs of the calling kernel may just have written it: not from L1)
+    const int g = (n + 1 + GRP - 1) / GRP;
     gs[u] = g;
     mine += g;
     gmax = max(gmax, g);
@@ -264,17 +262,16 @@ __device__ __forceinline__ void write_plan(const State& st, const Plan& pl, int 
     pl.hdr[0] = pieces;
     pl.hdr[1] = Gtot;
     pl.hdr[2] = nWarps;   // (-1 after a failed placement: no launch accepts the plan)
-    pl.hdr[3] = append;
+    pl.hdr[3] = 1;
   }
 }
 
 // The plan as a kernel of its own: one CTA per layer of `layers` consecutive layers starting at
 // layer0 (after a prompt insertion, a reallocation, or any edit of a head's state from the host).
-__global__ void __launch_bounds__(NT) plan_kernel(State st, const Plan* plans, int layer0, int append, int n_limit,
-                                                  int nWarps, int grid) {
+__global__ void __launch_bounds__(NT) plan_kernel(State st, const Plan* plans, int layer0, int nWarps, int grid) {
   __shared__ int s_gs[MAX_UNITS_PER_CALL + 1];
   __shared__ int s_red[320];
-  write_plan(st, plans[layer0 + blockIdx.x], layer0 + blockIdx.x, append, n_limit, nWarps, grid, s_gs, s_red);
+  write_plan(st, plans[layer0 + blockIdx.x], layer0 + blockIdx.x, nWarps, grid, s_gs, s_red);
 }
 
 }  // namespace ckv

@@ -299,18 +299,18 @@ constexpr int ROWS_ALL_LAST = 1;    // entry i is token i: metadata written here
 constexpr int ROWS_ALL_POS = 2;     // ... tau = i, the token's own arrival time (its queries are replayed)
 
 // The rows of a layer's entries into their pages.  k, v: [batch][P][H][128].  CTA 0 writes the
-// layer's launch plan meanwhile (plan.append >= 0); the others, `per_head` for every head, copy a
+// layer's launch plan meanwhile (plan_warps > 0); the others, `per_head` for every head, copy a
 // page per warp and turn, eight rows of 512 bytes in flight.  Bound: HBM, 1 KB moved per entry, or
 // the plan's serial placement when there is little to copy: 64 heads x 935 entries in 16.8 us (one
 // CTA per head: 85 us), 128 heads x 512 entries in 21.5 us (insertion, plan kernel and a scoring
 // pass of the attention kernel: 81 us).
 __global__ void __launch_bounds__(NT) prefill_rows_kernel(State st, Plan plan, int layer, const unsigned char* __restrict__ k,
                                                           const unsigned char* __restrict__ v, int P, int mode, int per_head,
-                                                          int plan_append, int plan_limit, int plan_warps, int plan_grid) {
+                                                          int plan_warps, int plan_grid) {
   __shared__ int s_gs[MAX_UNITS_PER_CALL + 1];
   __shared__ int s_red[320];
   if (blockIdx.x == 0) {
-    write_plan(st, plan, layer, plan_append, plan_limit, plan_warps, plan_grid, s_gs, s_red);
+    if (plan_warps > 0) write_plan(st, plan, layer, plan_warps, plan_grid, s_gs, s_red);
     return;
   }
   const int u = (blockIdx.x - 1) / per_head, b = (blockIdx.x - 1) % per_head, seq = u / st.H, head = u % st.H;

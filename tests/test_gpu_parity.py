@@ -653,6 +653,47 @@ def test_observation_window_prefill(W, prompt, budget):
     ls.close()
 
 
+@pytest.mark.parametrize("W,prompt,budget,G", [(1, 1, 4, 2), (13, 63, 70, 5), (64, 64, 64, 1), (9, 65, 80, 7), (16, 129, 100, 8),
+                                               (40, 300, 300, 8), (33, 257, 256, 3)])
+def test_window_sizes_around_tiles_and_launches(W, prompt, budget, G):
+    """W x G rows around the 64 of a CTA, prompts around the 64-key tiles, and (40 x 8 rows on lists with no
+    room to spare) windows that take several launches."""
+    wl = Workload(name=f"win{W}_{prompt}", seed=950 + W, n_layers=1, n_q_heads=3 * G, n_kv_heads=3, batch=2, prompt=prompt,
+                  think_steps=3, budget_per_head=budget, outlier="flat", outlier_frac=0.05)
+    ls = LockStep(wl, [0, 1], max_budget=budget, max_answer_tokens=max(0, prompt - budget))
+    ls.prefill_window(W)
+    ls.compare()
+    for _ in range(wl.think_steps):
+        ls.step()
+    ls.gpu.check()
+    ls.assert_clean()
+    ls.close()
+
+
+@pytest.mark.parametrize("prompt", [97, 8213])
+def test_window_over_equal_keys_takes_the_earlier_position(prompt):
+    """All scores of a query equal: the hits are its earliest entries; without `out_window`, and with a
+    prompt whose probabilities do not fit shared memory."""
+    from oracle import Oracle, OracleConfig
+    from paper_2601_16986_b200 import Config, CrystalKV
+    W, budget = 4, prompt - 7
+    shape = dict(n_layers=1, n_q_heads=4, n_kv_heads=2, batch=1, budget_per_head=budget, max_context=prompt + 8,
+                 max_budget=2 * prompt)
+    kv = CrystalKV(Config(**shape, max_answer_tokens=8))
+    ora = Oracle(OracleConfig(**shape, min_budget=max(16, budget // 8)))
+    g = torch.Generator("cuda").manual_seed(4)
+    k = torch.randn(1, 1, 2, 128, device="cuda", generator=g).to(torch.bfloat16).expand(1, prompt, 2, 128).contiguous()
+    q = torch.randn(W, 1, 4, 128, device="cuda", generator=g).to(torch.bfloat16)
+    kv.prefill_window(0, k, k, q)
+    ora.prefill_window(0, k.cpu(), k.cpu(), q.cpu())
+    for h in range(2):
+        assert (kv.export_state(0, 0, h) == ora.export_state(0, 0, h)).all()
+    kv.check()
+    kv.validate()
+    kv.close()
+    ora.close()
+
+
 @pytest.mark.parametrize("m,literal,prompt,budget", [(8, 0, 83, 53), (16, 0, 40, 64), (3, 1, 30, 64), (1, 1, 83, 53),
                                                      (64, 0, 300, 256)])
 def test_buffered_cadence_and_literal_return(m, literal, prompt, budget):
