@@ -102,6 +102,7 @@ struct DecodeParams {
   int early;      // 1: the lists and rows of this layer are final, so the attention kernel may read them
                   //    before the kernel ahead of it in the stream has completed
   int evict_every;   // m >= 1: step 4 waits until a head is m entries over its budget, then removes them all
+  int front;      // LRFU kernel: logit rows of a head requested before its length is known
   int literal;    // 1: Algorithm 1 is skipped for a head below its budget (its first line as printed)
   int plan_warps;    // warps of the attention grid the plan is made for
   int plan_grid;     // CTAs of that grid
@@ -141,8 +142,9 @@ __device__ __forceinline__ int warp_sum_i(int v) {
   return v;
 }
 
-// Exclusive scan of one int per thread across the block; returns this thread's prefix and
-// the block total.  `red` needs NW+1 ints.  Contains two __syncthreads().
+// Exclusive scan of one int per thread across the block of NTH threads; returns this thread's
+// prefix and the block total.  `red` needs NTH / 32 ints.  Contains two __syncthreads().
+template <int NTH = NT>
 __device__ __forceinline__ int block_excl_scan(int v, int* red, int& total) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int inc = v;
@@ -156,7 +158,7 @@ __device__ __forceinline__ int block_excl_scan(int v, int* red, int& total) {
   __syncthreads();
   int base = 0, tot = 0;
 #pragma unroll
-  for (int i = 0; i < NW; ++i) {
+  for (int i = 0; i < NTH / 32; ++i) {
     int x = red[i];
     if (i < w) base += x;
     tot += x;

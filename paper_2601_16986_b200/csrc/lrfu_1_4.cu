@@ -1,0 +1,16 @@
+// Algorithm 1's kernel with CTAs of eight warps, up to four query heads per kv head.
+#include "lrfu_kernel.cuh"
+
+namespace ckv {
+
+cudaError_t lrfu_launch_1_4(int G, const DecodeParams& p, int heads, cudaStream_t s) {
+  switch (G) {
+    case 1: return launch_lrfu<1, NT>(p, heads, s);
+    case 2: return launch_lrfu<2, NT>(p, heads, s);
+    case 3: return launch_lrfu<3, NT>(p, heads, s);
+    case 4: return launch_lrfu<4, NT>(p, heads, s);
+  }
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace ckv

@@ -1,0 +1,37 @@
+// Launching Algorithm 1's kernel (lrfu_kernel.cuh): its launch shape, and the instantiations by group
+// size, which are compiled in units of their own.
+#pragma once
+#include "common.cuh"
+
+namespace ckv {
+
+constexpr int MAX_DEVICES = 64;   // device ordinals this library keeps per-device state for
+
+constexpr int FRONT = 5;   // entries per thread whose logit rows are requested before n is known
+constexpr int LRFU_SMALL = 64;   // threads of the CTAs for short heads
+constexpr int LRFU_LARGE = 512;  // ... for long ones
+
+// Threads of a head's CTA.  hint: entries of a head if all are alike (uniform), else about the mean.
+//  * Heads of at most 5 x 64 entries take CTAs of two warps once there are more heads than SMs: six
+//    of them fit beside an attention CTA instead of two of eight warps, most of which idle in the
+//    block-wide steps.  128 sequences of 8 heads of 257 entries: 26 us a layer instead of 38.6.
+//  * Heads longer than 5 x 256 entries take CTAs of sixteen warps (one of which fits beside an attention
+//    CTA) while every head finds an SM of its own: half the rounds of loads per thread.  64 heads of
+//    4097 entries: 32.0 us a layer instead of 34.3; 128 heads of 1024 .. 3072: 29.5 instead of 31.1.
+inline int lrfu_threads(int U, int hint, bool uniform, int num_sms) {
+  if (uniform && hint <= FRONT * LRFU_SMALL && U > num_sms) return LRFU_SMALL;
+  return hint > FRONT * NT && U <= num_sms ? LRFU_LARGE : NT;
+}
+
+// Launches the kernel for `heads` heads; threads: LRFU_SMALL, NT or LRFU_LARGE.
+cudaError_t lrfu_launch_small(int G, const DecodeParams& p, int heads, cudaStream_t s);
+cudaError_t lrfu_launch_large(int G, const DecodeParams& p, int heads, cudaStream_t s);
+cudaError_t lrfu_launch_1_4(int G, const DecodeParams& p, int heads, cudaStream_t s);
+cudaError_t lrfu_launch_5_8(int G, const DecodeParams& p, int heads, cudaStream_t s);
+inline cudaError_t lrfu_launch(int threads, int G, const DecodeParams& p, int heads, cudaStream_t s) {
+  if (threads == LRFU_SMALL) return lrfu_launch_small(G, p, heads, s);
+  if (threads == LRFU_LARGE) return lrfu_launch_large(G, p, heads, s);
+  return G <= 4 ? lrfu_launch_1_4(G, p, heads, s) : lrfu_launch_5_8(G, p, heads, s);
+}
+
+}  // namespace ckv

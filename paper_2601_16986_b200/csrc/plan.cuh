@@ -22,7 +22,7 @@ namespace ckv {
 // pieces are packed best fit, longest first.  A run goes to the open CTA with the fewest free
 // warps that still holds it, so a CTA with c free warps takes c / s runs of length s one after the
 // other: the loop below moves whole classes of CTAs at once and counts exactly what the
-// run-by-run placement in write_plan() does.
+// run-by-run placement does; place_runs() below walks the same classes and says where each run goes.
 __host__ __device__ __forceinline__ int ctas_needed(int full, const int (&cnt)[8]) {
   int open[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};   // open[c]: CTAs with c free warps
   int ctas = full;
@@ -50,14 +50,69 @@ __host__ __device__ __forceinline__ int ctas_needed(int full, const int (&cnt)[8
   return ctas;
 }
 
-// Called by all NT threads of one CTA.  `gs` is shared memory for U + 1 ints, `red` for 320.
+// Where the runs go: the same walk as ctas_needed() over ranges of consecutive CTAs instead of counts.
+// An entry says: the runs [r0, r0 + n) of length s (in head order) fill CTAs base, base + 1, ... with q
+// runs each, from warp `off` on.  A range of CTAs visited for a length is cut into at most a consumed, a
+// partly consumed and an untouched part, so no more than 13 ranges and 35 entries arise.
+constexpr int PL_SCRATCH = 320;   // ints of shared scratch that write_plan() wants
+constexpr int PL_ENTRIES = 40, PL_RANGES = 16;
+struct Placement {
+  int first[9];                  // entries of length s: [first[s], first[s - 1]), s = 7 .. 1
+  int r0[PL_ENTRIES], n[PL_ENTRIES], base[PL_ENTRIES], qoff[PL_ENTRIES];   // qoff = q | off << 8
+  int rb[PL_RANGES], rn[PL_RANGES], rc[PL_RANGES];   // ranges of open CTAs: first, count, free warps
+};
+static_assert(sizeof(Placement) <= (PL_SCRATCH - 64) * sizeof(int), "the placement lives in the planner's scratch");
+// cnt[s]: runs of length s; full: CTAs taken whole (the first ones).  One thread.  False if they do not fit.
+__host__ __device__ inline bool place_runs(int full, const int* cnt, int grid, Placement& p) {
+  int ne = 0, nr = 0, fresh = full;
+  p.first[8] = p.first[7] = 0;
+  for (int s = 7; s >= 1; --s) {
+    p.first[s] = ne;
+    int todo = cnt[s], done = 0;
+    for (int c = s; c <= 8 && todo > 0; ++c) {
+      const int q = c / s, live = nr;   // (ranges made while this length is placed have fewer than s warps left or one run's)
+      for (int x = 0; x < (c == 8 ? 1 : live) && todo > 0; ++x) {
+        int base, have;
+        if (c == 8) {
+          base = fresh; have = (todo + q - 1) / q;
+          if (fresh + have > grid) return false;
+          fresh += have;
+        } else {
+          if (p.rc[x] != c || p.rn[x] == 0) continue;
+          base = p.rb[x]; have = p.rn[x];
+        }
+        const int wholes = todo / q < have ? todo / q : have;
+        const int rest = wholes < have ? (todo - wholes * q < q ? todo - wholes * q : 0) : 0;
+        const int used = wholes + (rest > 0 ? 1 : 0), runs = wholes * q + rest;
+        if (ne >= PL_ENTRIES || nr + 2 > PL_RANGES) return false;
+        p.r0[ne] = done; p.n[ne] = runs; p.base[ne] = base; p.qoff[ne] = q | ((8 - c) << 8);
+        ++ne;
+        done += runs;
+        todo -= runs;
+        if (c < 8) { p.rb[x] += used; p.rn[x] -= used; }
+        if (wholes > 0 && c - q * s > 0) { p.rb[nr] = base; p.rn[nr] = wholes; p.rc[nr] = c - q * s; ++nr; }
+        if (rest > 0) { p.rb[nr] = base + wholes; p.rn[nr] = 1; p.rc[nr] = c - rest * s; ++nr; }
+      }
+    }
+    if (todo > 0) return false;
+    int keep = 0;   // drop emptied ranges
+    for (int x = 0; x < nr; ++x)
+      if (p.rn[x] > 0) { p.rb[keep] = p.rb[x]; p.rn[keep] = p.rn[x]; p.rc[keep] = p.rc[x]; ++keep; }
+    nr = keep;
+  }
+  p.first[0] = ne;
+  return true;
+}
+
+// Called by all NTH threads of one CTA.  `gs` is memory for U + 1 ints, `red` shared memory for 320.
 // The plan is for a decode step: every head one entry longer than now.
+template <int NTH = NT>
 __device__ __forceinline__ void write_plan(const State& st, const Plan& pl, int layer, int nWarps, int grid,
                                         int* gs, int* red) {
   const int U = st.batch * st.H, tid = threadIdx.x, lane = tid & 31;
   // ---- groups per head
   int mine = 0, gmax = 0, empty = 0;
-  for (int u = tid; u < U; u += NT) {
+  for (int u = tid; u < U; u += NTH) {
     const int uid = ((u / st.H) * st.L + layer) * st.H + (u % st.H);
     const int n = __ldcg(st.n_cur + uid);   // (other CTAs of the calling kernel may just have written it: not from L1)
     const int g = (n + 1 + GRP - 1) / GRP;
@@ -67,13 +122,13 @@ __device__ __forceinline__ void write_plan(const State& st, const Plan& pl, int 
     empty |= (g == 0);
   }
   int Gtot;
-  block_excl_scan(mine, red, Gtot);
+  block_excl_scan<NTH>(mine, red, Gtot);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) gmax = max(gmax, __shfl_xor_sync(0xffffffffu, gmax, o));
   __syncthreads();
   if (lane == 0) red[tid >> 5] = gmax;
   __syncthreads();
-  for (int x = 0; x < NW; ++x) gmax = max(gmax, red[x]);
+  for (int x = 0; x < NTH / 32; ++x) gmax = max(gmax, red[x]);
   empty = __syncthreads_or(empty);
   if (empty) {   // a head without entries cannot be attended: nothing is planned
     if (tid == 0) atomicOr(st.errword, ERR_PLAN);
@@ -97,10 +152,10 @@ __device__ __forceinline__ void write_plan(const State& st, const Plan& pl, int 
     // first feasible bound among Tfirst .. Tfirst + 31, or -1
     auto first_that_packs = [&](int Tfirst) {
       const int Tc = Tfirst + lane;
-      if (tid < 128) hist[tid] = 0;
+      for (int x = tid; x < 128; x += NTH) hist[x] = 0;
       __syncthreads();
       unsigned h4[4] = {0u, 0u, 0u, 0u};
-      for (int u = tid >> 5; u < U; u += NW) {
+      for (int u = tid >> 5; u < U; u += NTH / 32) {
         const int k = (gs[u] + Tc - 1) / Tc;
         const int r = k & 7;   // 0: nothing beyond whole CTAs
 #pragma unroll
@@ -151,22 +206,27 @@ __device__ __forceinline__ void write_plan(const State& st, const Plan& pl, int 
     while (lo < hi) {
       const int mid = (lo + hi) >> 1;
       int cnt = 0;
-      for (int u = tid; u < U; u += NT) cnt += (gs[u] + mid - 1) / mid;
+      for (int u = tid; u < U; u += NTH) cnt += (gs[u] + mid - 1) / mid;
       int tot;
-      block_excl_scan(cnt, red, tot);
+      block_excl_scan<NTH>(cnt, red, tot);
       __syncthreads();
       if (tot <= nWarps) hi = mid; else lo = mid + 1;
     }
     T = max(lo, min(GMIN, gmax));
   }
-  // ---- pieces per head, their prefix sums, the descriptors
-  int pieces = 0;
-  for (int b0 = 0; b0 < U; b0 += NT) {
+  // ---- pieces per head, their prefix sums, the descriptors; when packing, also the CTAs a head takes
+  // whole and its place among the runs of its length
+  Placement& place = *reinterpret_cast<Placement*>(red + 64);
+  int pieces = 0, wholes = 0;
+  int runs[8] = {0, 0, 0, 0, 0, 0, 0, 0};   // runs of each length among the heads so far
+  if (packed)
+    for (int pw = tid; pw < nWarps; pw += NTH) pl.wrange[pw] = make_int4(0, 0, -1, 0);
+  for (int b0 = 0; b0 < U; b0 += NTH) {
     const int u = b0 + tid;
     const int g = (u < U && Gtot > 0) ? gs[u] : 0;
     const int k = g == 0 ? 0 : (T == 0x7fffffff ? 1 : (g + T - 1) / T);
     int tot;
-    const int start = pieces + block_excl_scan(k, red, tot);
+    const int start = pieces + block_excl_scan<NTH>(k, red, tot);
     pieces += tot;
     if (u < U) {
       pl.npc[u] = k;
@@ -175,79 +235,53 @@ __device__ __forceinline__ void write_plan(const State& st, const Plan& pl, int 
       // nothing else to stream; 2 when they sit that way in runs of eight (whole CTAs) and one shorter run
       const int together = k <= 1 ? 0 : (packed ? (k <= NW ? 1 : 2) : ((start & (NW - 1)) + k <= NW ? 1 : 0));
       for (int j = 0; j < k; ++j) pl.desc[start + j] = make_int4(u, j, k, together);
-      if (packed) gs[u] = (start << 12) | k;
+    }
+    if (packed) {
+      const int f = k >> 3, s = k & 7;
+      const int c0 = wholes + block_excl_scan<NTH>(f, red, tot);
+      wholes += tot;
+      if ((c0 + f) * NW <= nWarps)
+        for (int x = 0; x < f * NW; ++x)
+          pl.wrange[c0 * NW + x] = make_int4(start + x, start + x + 1, u, x | (k << 12) | ((k <= NW ? 1 : 2) << 24));
+      int r = 0;   // this head's place among the runs of its length: two lengths per scan
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        const int v = (x > 0 && s == 2 * x ? 1 : 0) | (s == 2 * x + 1 ? 0x10000 : 0);
+        const int e = block_excl_scan<NTH>(v, red, tot);
+        if (x > 0 && s == 2 * x) r = runs[2 * x] + (e & 0xffff);
+        if (s == 2 * x + 1) r = runs[2 * x + 1] + (e >> 16);
+        runs[2 * x] += tot & 0xffff;
+        runs[2 * x + 1] += tot >> 16;
+      }
+      if (u < U) gs[u] = (start << 12) | r;   // (both below 4096: packing wants fewer pieces than 4096 warps)
     }
   }
   if (packed) {
-    for (int pw = tid; pw < nWarps; pw += NT) pl.wrange[pw] = make_int4(0, 0, -1, 0);
-    __syncthreads();
-    if (tid < 32) {
-      // every lane keeps the same books; the lanes share the stores
-      int* nxt = red + 16;   // [grid] next CTA in the list of its class
-      int next_cta = 0, over = 0;
-      for (int b0 = 0; b0 < U && !over; b0 += 32) {   // whole CTAs first
-        const int v = (b0 + lane < U) ? gs[b0 + lane] : 0;
-        unsigned m = __ballot_sync(0xffffffffu, (v & 4095) >= NW);
-        while (m) {
-          const int b = __ffs(m) - 1;
-          m &= m - 1;
-          const int vv = __shfl_sync(0xffffffffu, v, b);
-          const int start = vv >> 12, kk = vv & 4095, nw = (kk >> 3) * NW;
-          if (next_cta * NW + nw > nWarps) { over = 1; break; }
-          for (int x = lane; x < nw; x += 32)
-            pl.wrange[next_cta * NW + x] = make_int4(start + x, start + x + 1, b0 + b, x | (kk << 12) | ((kk <= NW ? 1 : 2) << 24));
-          next_cta += nw / NW;
-        }
-      }
-      int head[8] = {-1, -1, -1, -1, -1, -1, -1, -1};   // head[c]: first of the CTAs with c free warps
-#pragma unroll
-      for (int s = 7; s >= 1; --s) {
-        for (int b0 = 0; b0 < U && !over; b0 += 32) {
-          const int v = (b0 + lane < U) ? gs[b0 + lane] : 0;
-          unsigned m = __ballot_sync(0xffffffffu, (v & 7) == s);
-          while (m) {
-            const int b = __ffs(m) - 1;
-            m &= m - 1;
-            const int vv = __shfl_sync(0xffffffffu, v, b);
-            const int start = vv >> 12, k = vv & 4095;
-            int cta = -1, c = 8;
-#pragma unroll
-            for (int cc = s; cc <= 7; ++cc)
-              if (cta < 0 && head[cc] >= 0) {
-                cta = head[cc];
-                head[cc] = nxt[cta];
-                c = cc;
-              }
-            if (cta < 0) {
-              if (next_cta >= grid) { over = 1; break; }
-              cta = next_cta++;
-            }
-            const int left = c - s;
-#pragma unroll
-            for (int dd = 1; dd <= 7; ++dd)
-              if (left == dd) {
-                nxt[cta] = head[dd];
-                head[dd] = cta;
-              }
-            __syncwarp();
-            const int j0 = k - s;   // the pieces before these took whole CTAs
-            if (lane < s)
-              pl.wrange[cta * NW + (NW - c) + lane] = make_int4(start + j0 + lane, start + j0 + lane + 1, b0 + b,
-                                                                (j0 + lane) | (k << 12) | ((k <= 1 ? 0 : (k <= NW ? 1 : 2)) << 24));
-          }
-        }
-      }
-      if (over && lane == 0) {   // cannot happen while ctas_needed() counts what this loop does; never leave half a plan
-        atomicOr(st.errword, ERR_PLAN);
-        nWarps = -1;
-      }
-      nWarps = __shfl_sync(0xffffffffu, nWarps, 0);
+    // One thread walks the classes of CTAs, then every head looks its run up.  (A
+    // plan of 128 heads takes 9 us; one warp placing the runs one by one took it to 26.)
+    if (tid == 0) {
+      const bool ok = wholes <= grid && place_runs(wholes, runs, grid, place);
+      place.first[8] = ok;
+      if (!ok) atomicOr(st.errword, ERR_PLAN);   // cannot happen while ctas_needed() counts the same walk
     }
+    __syncthreads();   // (also: the empty ranges above are written)
+    const bool ok = place.first[8] != 0;
+    for (int u = tid; u < U && ok; u += NTH) {
+      const int k = pl.npc[u], s = k & 7, start = gs[u] >> 12, r = gs[u] & 4095, j0 = k - s;   // the pieces before took whole CTAs
+      if (s == 0) continue;
+      int e = place.first[s];
+      while (e + 1 < place.first[s - 1] && r >= place.r0[e] + place.n[e]) ++e;
+      const int q = place.qoff[e] & 255, off = place.qoff[e] >> 8, d = r - place.r0[e];
+      int4* w = pl.wrange + (place.base[e] + d / q) * NW + off + (d % q) * s;
+      for (int x = 0; x < s; ++x)
+        w[x] = make_int4(start + j0 + x, start + j0 + x + 1, u, (j0 + x) | (k << 12) | ((k <= 1 ? 0 : (k <= NW ? 1 : 2)) << 24));
+    }
+    if (!ok) nWarps = -1;   // no launch accepts the plan
   } else {
     // heads end to end: consecutive pieces go to consecutive warps; with more pieces than warps
     // every warp takes a run of consecutive pieces
     const int per = (pieces + nWarps - 1) / max(nWarps, 1);
-    for (int pw = tid; pw < nWarps; pw += NT) {
+    for (int pw = tid; pw < nWarps; pw += NTH) {
       int4 r = make_int4(0, 0, -1, 0);
       if (pieces <= nWarps) {
         if (pw < pieces) r = make_int4(pw, pw + 1, -1, 0);
@@ -264,14 +298,6 @@ __device__ __forceinline__ void write_plan(const State& st, const Plan& pl, int 
     pl.hdr[2] = nWarps;   // (-1 after a failed placement: no launch accepts the plan)
     pl.hdr[3] = 1;
   }
-}
-
-// The plan as a kernel of its own: one CTA per layer of `layers` consecutive layers starting at
-// layer0 (after a prompt insertion, a reallocation, or any edit of a head's state from the host).
-__global__ void __launch_bounds__(NT) plan_kernel(State st, const Plan* plans, int layer0, int nWarps, int grid) {
-  __shared__ int s_gs[MAX_UNITS_PER_CALL + 1];
-  __shared__ int s_red[320];
-  write_plan(st, plans[layer0 + blockIdx.x], layer0 + blockIdx.x, nWarps, grid, s_gs, s_red);
 }
 
 }  // namespace ckv

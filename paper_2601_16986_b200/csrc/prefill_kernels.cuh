@@ -10,6 +10,14 @@
 
 namespace ckv {
 
+// The plan as a kernel of its own: one CTA per layer of `layers` consecutive layers starting at
+// layer0 (after a prompt insertion, a reallocation, or any edit of a head's state from the host).
+__global__ void __launch_bounds__(NT) plan_kernel(State st, const Plan* plans, int layer0, int nWarps, int grid) {
+  __shared__ int s_gs[MAX_UNITS_PER_CALL + 1];
+  __shared__ int s_red[320];
+  write_plan(st, plans[layer0 + blockIdx.x], layer0 + blockIdx.x, nWarps, grid, s_gs, s_red);
+}
+
 constexpr int SEL_NT = 1024;            // threads of prefill_select_kernel
 constexpr int SEL_SMEM = 160 * 1024;    // pbar of up to this many bytes stays in shared memory
 
