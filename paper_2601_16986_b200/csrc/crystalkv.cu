@@ -662,15 +662,13 @@ static int prefill_common(crystalkv_t* h, int layer, const void* k, const void* 
     // Algorithm 1 with the last query over scores and metadata only, then the survivors' rows; every
     // kernel on `s`, which has joined the internal streams, so any scratch set is free
     DecodeParams p = make_params(h, layer);
-    const int chunk = score_chunk(P, h->U), chunks = (P + chunk - 1) / chunk;
+    const int chunks = (P + SCORE_KEYS - 1) / SCORE_KEYS;
     const size_t sm = (size_t)P * sizeof(float) <= SEL_SMEM ? (size_t)P * sizeof(float) : 0;
     if (sm > 32 * 1024)
       CK(h, cudaFuncSetAttribute(prefill_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SEL_SMEM));
-    prefill_score_kernel<<<dim3(chunks, h->U), NT, 0, s>>>(p.sc, static_cast<const __nv_bfloat16*>(k),
-                                                           static_cast<const __nv_bfloat16*>(q), c.n_kv_heads, P, h->G,
-                                                           chunk, p.scale, p.scale_log2);
-    CK(h, cudaGetLastError());
-    prefill_select_kernel<<<h->U, SEL_NT, sm, s>>>(h->st, p.sc, layer, P, h->G, chunks, c.top_p, c.evict_every,
+    CK(h, score_dispatch(h->G, p.sc, static_cast<const __nv_bfloat16*>(k), static_cast<const __nv_bfloat16*>(q), h->U,
+                         c.n_kv_heads, P, p.scale, p.scale_log2, s));
+    prefill_select_kernel<<<h->U, SEL_NT, sm, s>>>(h->st, p.sc, layer, P, h->G, chunks, p.scale_log2 / p.scale, c.top_p, c.evict_every,
                                                    c.literal_return, c.budget_ratio > 0.f ? ratio_budget(c, P) : 0, sm > 0);
     CK(h, cudaGetLastError());
     prefill_rows_kernel<<<1 + h->U * per_head, NT, 0, s>>>(h->st, h->plans[layer], layer, kb, vb, P, ROWS_SURVIVORS, per_head,

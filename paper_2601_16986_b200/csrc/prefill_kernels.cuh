@@ -21,111 +21,112 @@ __global__ void __launch_bounds__(NT) plan_kernel(State st, const Plan* plans, i
 constexpr int SEL_NT = 1024;            // threads of prefill_select_kernel
 constexpr int SEL_SMEM = 160 * 1024;    // pbar of up to this many bytes stays in shared memory
 
-// Keys per CTA of prefill_score_kernel: long enough that a CTA's start (its queries) is paid for by
-// several groups per warp, short enough for four CTAs per SM (two are resident) to be there at all.
-__host__ __device__ __forceinline__ int score_chunk(int P, int U) {
-  int chunk = 512;
-  while (chunk > 128 && (long long)U * ((P + chunk - 1) / chunk) < 592) chunk >>= 1;
-  return chunk;
-}
-
-__device__ __forceinline__ void score_mma(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
-               : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
+constexpr int SCORE_NT = 256;           // threads of prefill_score_kernel, one key each
+constexpr int SCORE_KEYS = SCORE_NT;
 
 // The scaled logits of the last query's G heads against the prompt's keys, and per CTA the softmax
-// reference point (log2 domain) and normaliser of its chunk of keys.
-//   k: [batch][P][H][128]   q_last: [batch][Hq][128]   part: [U][chunks][16] = m[8], l[8]
-// Bound: HBM (the keys are read once, 256 bytes each).  A warp takes 16 keys at a time straight
-// from global memory into MMA fragments: which channels form a k-step is free as long as both
-// operands agree, so lane tig of a row takes the 16-byte pieces tig, tig + 4, ... (two whole sectors
-// per row and load), and the next 16 keys are requested before the current ones are used.
-// 64 heads x 9350 tokens (153 MB): 37.6 us, 4.1 TB/s; one CTA per head with a thread per key and
-// fp32 multiply-adds took 252 us.  128 heads x 512 tokens: 9.6 us.
-__global__ void __launch_bounds__(NT, 2) prefill_score_kernel(Scratch sc, const __nv_bfloat16* __restrict__ k,
-                                                              const __nv_bfloat16* __restrict__ q_last, int H, int P, int G,
-                                                              int chunk, float scale, float scale_log2) {
-  __shared__ float s_m[NW][QH], s_l[NW][QH];
+// reference point (log2 domain) of its keys.  grid: (chunks of SCORE_KEYS keys, U).
+//   k: [batch][P][H][128]   q_last: [batch][Hq][128]   partials: [U][chunks][8] = m
+// Every logit is one chain of fp32 multiply-adds over the channels in order, by one thread: which
+// entries of a prompt survive hangs on the last bits of the logits, so their rounding is part of the
+// result.  Bound: HBM and, close behind, the multiply-adds (G x 128 per key).  A CTA brings its 64 KB
+// of keys into shared memory with 16-byte asynchronous copies (chunk c of key i at c ^ (i & 7): the
+// threads of a quarter warp read eight different bank groups) and then computes; three CTAs share an
+// SM, so that the others' copies run beside one's arithmetic.  64 heads x 9350 tokens (153 MB): 46 us,
+// 3.3 TB/s (two keys a thread, half the warps: 55 us; one CTA per head with a thread per row of
+// global memory: 252 us; MMA fragments straight from global memory: 38 us, but other roundings, and a
+// head in some thousands then kept another entry at the hit boundary).  128 heads x 512 tokens: 9.6 us.
+template <int G>
+__global__ void __launch_bounds__(SCORE_NT, 3) prefill_score_kernel(Scratch sc, const __nv_bfloat16* __restrict__ k,
+                                                                    const __nv_bfloat16* __restrict__ q_last, int H, int P,
+                                                                    float scale, float scale_log2) {
+  extern __shared__ __align__(128) unsigned char s_keys[];
+  __shared__ __align__(16) float s_q[G * HD];
+  __shared__ float s_m[SCORE_NT / 32][G];
   const int u = blockIdx.y, seq = u / H, head = u % H;
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, gid = lane >> 2, tig = lane & 3;
-  const int end = min(P, (int)(blockIdx.x + 1) * chunk);
-  // queries as B fragments: k-step 2 j + h of lane tig holds channels 8 (tig + 4 j) + 4 h .. + 3
-  uint32_t qb[8][2];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int i0 = blockIdx.x * SCORE_KEYS, n = min(SCORE_KEYS, P - i0);
   {
-    const unsigned short* q16 = reinterpret_cast<const unsigned short*>(q_last) + ((size_t)u * G + gid) * HD;
-#pragma unroll
-    for (int s = 0; s < 8; ++s) {
-      const int c = 8 * (tig + 4 * (s >> 1)) + 4 * (s & 1);
-#pragma unroll
-      for (int x = 0; x < 2; ++x)
-        qb[s][x] = gid < G ? (uint32_t)q16[c + 2 * x] | ((uint32_t)q16[c + 2 * x + 1] << 16) : 0u;
-    }
+    const size_t row = (size_t)H * ROW_BYTES;
+    const unsigned char* src = reinterpret_cast<const unsigned char*>(k) + (((size_t)seq * P + i0) * H + head) * ROW_BYTES + (tid & 15) * 16;
+    const uint32_t dst = smem_u32(s_keys);
+    for (int i = tid >> 4; i < n; i += SCORE_NT / 16)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n"
+                   ::"r"(dst + i * ROW_BYTES + (((tid & 15) ^ (i & 7)) << 4)), "l"(src + (size_t)i * row) : "memory");
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
   }
-  const size_t row = (size_t)H * HD * 2;   // bytes from one token's key of this head to the next one's
-  const unsigned char* kb = reinterpret_cast<const unsigned char*>(k) + ((size_t)seq * P * H + head) * (HD * 2) + tig * 16;
-  auto load = [&](int i0, uint4 (&a)[4], uint4 (&b)[4]) {
-    const unsigned char* pa = kb + (size_t)min(i0 + gid, P - 1) * row;
-    const unsigned char* pb = kb + (size_t)min(i0 + gid + 8, P - 1) * row;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      a[j] = __ldg(reinterpret_cast<const uint4*>(pa + 64 * j));
-      b[j] = __ldg(reinterpret_cast<const uint4*>(pb + 64 * j));
-    }
-  };
-  float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;
-  float* S = sc.logits + (size_t)u * sc.cap_s * QH + 2 * tig;
-  uint4 a[4], b[4];
-  int i0 = blockIdx.x * chunk + w * GRP;
-  if (i0 < end) load(i0, a, b);
-#pragma unroll 1
-  for (; i0 < end; i0 += NW * GRP) {
-    uint4 na[4], nb[4];
-    if (i0 + NW * GRP < end) load(i0 + NW * GRP, na, nb);
-    float s[4] = {0.f, 0.f, 0.f, 0.f}, s2[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      score_mma(s, a[j].x, b[j].x, a[j].y, b[j].y, qb[2 * j][0], qb[2 * j][1]);
-      score_mma(s2, a[j].z, b[j].z, a[j].w, b[j].w, qb[2 * j + 1][0], qb[2 * j + 1][1]);
-    }
-#pragma unroll
-    for (int x = 0; x < 4; ++x) s[x] += s2[x];
-    const bool v0 = i0 + gid < end, v1 = i0 + gid + 8 < end;
-    float* lr = S + (size_t)(i0 + gid) * QH;
-    if (v0) *reinterpret_cast<float2*>(lr) = make_float2(__fmul_rn(s[0], scale), __fmul_rn(s[1], scale));
-    if (v1) *reinterpret_cast<float2*>(lr + 8 * QH) = make_float2(__fmul_rn(s[2], scale), __fmul_rn(s[3], scale));
-    const float t0 = v0 ? s[0] * scale_log2 : -INFINITY, t1 = v0 ? s[1] * scale_log2 : -INFINITY;
-    const float t2 = v1 ? s[2] * scale_log2 : -INFINITY, t3 = v1 ? s[3] * scale_log2 : -INFINITY;
-    const float c0 = fmaxf(t0, t2), c1 = fmaxf(t1, t3);
-    if (c0 > m0) { l0 *= ex2(m0 - c0); m0 = c0; }
-    if (c1 > m1) { l1 *= ex2(m1 - c1); m1 = c1; }
-    if (v0) { l0 += ex2(t0 - m0); l1 += ex2(t1 - m1); }
-    if (v1) { l0 += ex2(t2 - m0); l1 += ex2(t3 - m1); }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) { a[j] = na[j]; b[j] = nb[j]; }
-  }
-  // over the lanes that hold the same two heads, then over the warps
-  auto reduce = [&](float m, float l, int g) {
-    float mm = m;
-#pragma unroll
-    for (int x = 4; x < 32; x <<= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, x));
-    float ll = m > -INFINITY ? l * ex2(m - mm) : 0.f;
-#pragma unroll
-    for (int x = 4; x < 32; x <<= 1) ll += __shfl_xor_sync(0xffffffffu, ll, x);
-    if (gid == 0) { s_m[w][g] = mm; s_l[w][g] = ll; }
-  };
-  reduce(m0, l0, 2 * tig);
-  reduce(m1, l1, 2 * tig + 1);
+  for (int x = tid; x < G * HD; x += SCORE_NT) s_q[x] = __bfloat162float(q_last[(size_t)u * G * HD + x]);
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
   __syncthreads();
-  if (tid < QH) {
-    float m = s_m[0][tid], l = 0.f;
-    for (int x = 1; x < NW; ++x) m = fmaxf(m, s_m[x][tid]);
-    for (int x = 0; x < NW; ++x) l += s_m[x][tid] > -INFINITY ? s_l[x][tid] * ex2(s_m[x][tid] - m) : 0.f;
-    float* pp = sc.partials + ((size_t)u * gridDim.x + blockIdx.x) * 16;
-    pp[tid] = m;
-    pp[8 + tid] = l;
+  float acc[G];
+#pragma unroll
+  for (int g = 0; g < G; ++g) acc[g] = 0.f;
+  const unsigned char* ra = s_keys + tid * ROW_BYTES;   // (rows past the prompt's end hold anything; their results are dropped)
+#pragma unroll 2
+  for (int c = 0; c < HD / 8; ++c) {
+    const uint4 va = *reinterpret_cast<const uint4*>(ra + ((c ^ (tid & 7)) << 4));
+    const uint32_t ua[4] = {va.x, va.y, va.z, va.w};
+    float ka[8];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {   // a bf16 is the upper half of its fp32
+      ka[2 * x] = __uint_as_float(ua[x] << 16); ka[2 * x + 1] = __uint_as_float(ua[x] & 0xffff0000u);
+    }
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      const float4 q0 = *reinterpret_cast<const float4*>(s_q + g * HD + c * 8), q1 = *reinterpret_cast<const float4*>(s_q + g * HD + c * 8 + 4);
+      const float q[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
+#pragma unroll
+      for (int x = 0; x < 8; ++x) acc[g] = fmaf(q[x], ka[x], acc[g]);
+    }
   }
+  float* S = sc.logits + ((size_t)u * sc.cap_s + i0) * QH;
+  float mx[G];
+#pragma unroll
+  for (int g = 0; g < G; ++g) mx[g] = -INFINITY;
+  if (tid < n) {
+    float out[QH];
+#pragma unroll
+    for (int g = 0; g < QH; ++g) out[g] = g < G ? __fmul_rn(acc[g < G ? g : 0], scale) : 0.f;
+    *reinterpret_cast<float4*>(S + (size_t)tid * QH) = make_float4(out[0], out[1], out[2], out[3]);
+    if (G > 4) *reinterpret_cast<float4*>(S + (size_t)tid * QH + 4) = make_float4(out[4], out[5], out[6], out[7]);
+#pragma unroll
+    for (int g = 0; g < G; ++g) mx[g] = acc[g] * scale_log2;
+  }
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    const float m = warp_max(mx[g]);
+    if (lane == 0) s_m[w][g] = m;
+  }
+  __syncthreads();
+  if (tid < G) {
+    float m = s_m[0][tid];
+    for (int x = 1; x < SCORE_NT / 32; ++x) m = fmaxf(m, s_m[x][tid]);
+    sc.partials[((size_t)u * gridDim.x + blockIdx.x) * QH + tid] = m;
+  }
+}
+
+template <int G>
+cudaError_t launch_score(const Scratch& sc, const __nv_bfloat16* k, const __nv_bfloat16* q, int U, int H, int P, float scale,
+                         float scale_log2, cudaStream_t s) {
+  const int sm = SCORE_KEYS * ROW_BYTES;
+  cudaError_t e = cudaFuncSetAttribute(prefill_score_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  if (e != cudaSuccess) return e;
+  prefill_score_kernel<G><<<dim3((P + SCORE_KEYS - 1) / SCORE_KEYS, U), SCORE_NT, sm, s>>>(sc, k, q, H, P, scale, scale_log2);
+  return cudaGetLastError();
+}
+inline cudaError_t score_dispatch(int G, const Scratch& sc, const __nv_bfloat16* k, const __nv_bfloat16* q, int U, int H, int P,
+                                  float scale, float scale_log2, cudaStream_t s) {
+  switch (G) {
+    case 1: return launch_score<1>(sc, k, q, U, H, P, scale, scale_log2, s);
+    case 2: return launch_score<2>(sc, k, q, U, H, P, scale, scale_log2, s);
+    case 3: return launch_score<3>(sc, k, q, U, H, P, scale, scale_log2, s);
+    case 4: return launch_score<4>(sc, k, q, U, H, P, scale, scale_log2, s);
+    case 5: return launch_score<5>(sc, k, q, U, H, P, scale, scale_log2, s);
+    case 6: return launch_score<6>(sc, k, q, U, H, P, scale, scale_log2, s);
+    case 7: return launch_score<7>(sc, k, q, U, H, P, scale, scale_log2, s);
+    case 8: return launch_score<8>(sc, k, q, U, H, P, scale, scale_log2, s);
+  }
+  return cudaErrorInvalidValue;
 }
 
 // Exclusive scan of one int per thread over the SEL_NT threads; red: SEL_NT / 32 ints.
@@ -182,14 +183,14 @@ __device__ __forceinline__ bool take_pages(const State& st, int uid, int seq, in
 // fixed_budget > 0 sets the heads' budget first.
 // Bound: latency (a few block-wide steps over 36 bytes per token); 1024 threads keep a prompt of
 // 10 000 tokens at ten entries per thread, pbar in shared memory up to SEL_SMEM bytes.
-// 64 heads x 9350 tokens cut to 935: 34.8 us; the decode step's Algorithm 1 kernel with its radix
-// select over 96-bit keys in global memory took 286 us.  128 heads x 512 tokens: 10.1 us.
+// 64 heads x 9350 tokens cut to 935: 40.7 us; the decode step's Algorithm 1 kernel with its radix
+// select over 96-bit keys in global memory took 286 us.  128 heads x 512 tokens: 10.9 us.
 __global__ void __launch_bounds__(SEL_NT) prefill_select_kernel(State st, Scratch sc, int layer, int P, int G, int chunks,
-                                                                float top_p, int evict_every, int literal,
+                                                                float to_log2, float top_p, int evict_every, int literal,
                                                                 int fixed_budget, int in_smem) {
   extern __shared__ float s_pbar[];
   __shared__ NucleusSmem<SEL_NT> s_nu;
-  __shared__ float s_m[QH], s_il[QH];
+  __shared__ float s_m[QH], s_il[QH], s_l[8][QH];
   __shared__ int s_red[SEL_NT / 32];
   __shared__ int s_top;
   const int u = blockIdx.x, seq = u / st.H, head = u % st.H;
@@ -198,27 +199,47 @@ __global__ void __launch_bounds__(SEL_NT) prefill_select_kernel(State st, Scratc
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int B = fixed_budget > 0 ? fixed_budget : st.budget[uid];
   if (fixed_budget > 0 && tid == 0) st.budget[uid] = fixed_budget;
-  if (w < G) {   // warp g merges query head g's chunks
-    const float* pp = sc.partials + (size_t)u * chunks * 16;
-    float m = -INFINITY, l = 0.f;
-    for (int c = lane; c < chunks; c += 32) m = fmaxf(m, pp[c * 16 + w]);
+  const float* S = sc.logits + (size_t)u * sc.cap_s * QH;
+  if (w < G) {   // warp g: query head g's reference point
+    const float* pp = sc.partials + (size_t)u * chunks * QH;
+    float m = -INFINITY;
+    for (int c = lane; c < chunks; c += 32) m = fmaxf(m, pp[c * QH + w]);
     m = warp_max(m);
-    for (int c = lane; c < chunks; c += 32) l += pp[c * 16 + 8 + w] * ex2(pp[c * 16 + w] - m);
-    l = warp_sum(l);
-    if (lane == 0) {
-      s_m[w] = m * 0.693147180559945309f;   // log2 domain -> natural log
-      s_il[w] = 1.0f / (l * (float)G);
+    if (lane == 0) s_m[w] = m;
+  }
+  __syncthreads();
+  // normalisers: 256 threads to a pair of query heads, thread t over tokens t, t + 256, ..; then the
+  // lanes of a warp, then the eight warps in order (an order the results hang on, like the logits')
+  {
+    const int g = 2 * (tid >> 8), t = tid & 255;
+    float s0 = 0.f, s1 = 0.f;
+    if (g < G) {
+      const float m0 = s_m[g], m1 = s_m[min(g + 1, G - 1)];
+#pragma unroll 4
+      for (int i = t; i < P; i += 256) {
+        const float2 x = *reinterpret_cast<const float2*>(S + (size_t)i * QH + g);
+        s0 += ex2(x.x * to_log2 - m0);
+        s1 += ex2(x.y * to_log2 - m1);
+      }
     }
+    s0 = warp_sum(s0);
+    s1 = warp_sum(s1);
+    if (lane == 0) { s_l[w & 7][g] = s0; s_l[w & 7][g + 1] = s1; }
+  }
+  __syncthreads();
+  if (tid < G) {
+    float l = 0.f;
+    for (int x = 0; x < 8; ++x) l += s_l[x][tid];
+    s_il[tid] = 1.0f / (l * (float)G);
   }
   __syncthreads();
   // ---- step 1: pbar_i = mean_g exp(s_gi - m_g) / l_g
   float mx[QH], il[QH];
 #pragma unroll
   for (int g = 0; g < QH; ++g) {
-    mx[g] = g < G ? s_m[g] : 0.f;
+    mx[g] = g < G ? s_m[g] * 0.693147180559945309f : 0.f;   // log2 domain -> natural log
     il[g] = g < G ? s_il[g] : 0.f;
   }
-  const float* S = sc.logits + (size_t)u * sc.cap_s * QH;
   float* pb = in_smem ? s_pbar : sc.pbar + (size_t)u * sc.cap_s;
   for (int i0 = tid; i0 < P; i0 += 2 * SEL_NT) {   // two rows requested together
     float4 ra[2], rb[2];
@@ -309,8 +330,8 @@ constexpr int ROWS_ALL_POS = 2;     // ... tau = i, the token's own arrival time
 // The rows of a layer's entries into their pages.  k, v: [batch][P][H][128].  CTA 0 writes the
 // layer's launch plan meanwhile (plan_warps > 0); the others, `per_head` for every head, copy a
 // page per warp and turn, eight rows of 512 bytes in flight.  Bound: HBM, 1 KB moved per entry, or
-// the plan's serial placement when there is little to copy: 64 heads x 935 entries in 16.8 us (one
-// CTA per head: 85 us), 128 heads x 512 entries in 21.5 us (insertion, plan kernel and a scoring
+// the plan when there is little to copy: 64 heads x 935 entries in 10 us (one
+// CTA per head: 85 us), 128 heads x 512 entries in 11 us (insertion, plan kernel and a scoring
 // pass of the attention kernel: 81 us).
 __global__ void __launch_bounds__(NT) prefill_rows_kernel(State st, Plan plan, int layer, const unsigned char* __restrict__ k,
                                                           const unsigned char* __restrict__ v, int P, int mode, int per_head,
