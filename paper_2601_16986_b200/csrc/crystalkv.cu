@@ -23,7 +23,7 @@
 
 #include "attn_kernel.cuh"
 #include "aux_kernels.cuh"
-#include "lrfu_kernel.cuh"
+#include "lrfu_launch.cuh"
 #include "plan.cuh"
 #include "prefill_kernels.cuh"
 #include "window_kernels.cuh"
@@ -61,6 +61,8 @@ struct crystalkv {
   int prev_layer = -1;             // layer of the launch pair issued last, -1 after any other call
   int stage = CRYSTALKV_STAGE_THINK;
   int answer_steps = 0;
+  bool uniform = true;             // no head's budget or length has been set apart from the others'
+  int len_hint = 0;                // entries of a head in a decode step: of every head while uniform, else about the mean
   long long* Asum = nullptr;
   // host I/O: HOST_RING staging sets; inputs go up on one internal stream and results come
   // down on another, so the copies of other layers run beside the attention kernels
@@ -82,7 +84,6 @@ struct crystalkv {
 namespace {
 
 thread_local std::string g_create_err;
-constexpr int MAX_DEVICES = 64;   // device ordinals this library keeps per-device state for
 
 int fail(crystalkv_t* h, int code, const std::string& msg) {
   if (h) h->err = msg;
@@ -166,40 +167,6 @@ __global__ void init_free_stack_kernel(int* stack, int* top, long long pages_per
 __global__ void fill_int_kernel(int* p, long long n, int v) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     p[i] = v;
-}
-
-template <int G>
-cudaError_t launch_lrfu(const DecodeParams& p, int grid, cudaStream_t s) {
-  // the same shared-memory carve-out as the attention kernel, so that CTAs of both can be
-  // resident on one SM at the same time
-  // (function attributes are kept per device)
-  static std::atomic<bool> prepared[MAX_DEVICES] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= MAX_DEVICES) return cudaErrorInvalidDevice;
-  if (!prepared[dev].load(std::memory_order_acquire)) {
-    e = cudaFuncSetAttribute(lrfu_kernel<G>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    prepared[dev].store(true, std::memory_order_release);
-  }
-  lrfu_kernel<G><<<grid, NT, 0, s>>>(p);
-  return cudaGetLastError();
-}
-
-cudaError_t lrfu_dispatch(int G, const DecodeParams& p, int grid, cudaStream_t s) {
-  switch (G) {
-    case 1: return launch_lrfu<1>(p, grid, s);
-    case 2: return launch_lrfu<2>(p, grid, s);
-    case 3: return launch_lrfu<3>(p, grid, s);
-    case 4: return launch_lrfu<4>(p, grid, s);
-    case 5: return launch_lrfu<5>(p, grid, s);
-    case 6: return launch_lrfu<6>(p, grid, s);
-    case 7: return launch_lrfu<7>(p, grid, s);
-    case 8: return launch_lrfu<8>(p, grid, s);
-  }
-  return cudaErrorInvalidValue;
 }
 
 int validate(const crystalkv_config_t* c, std::string& why) {
@@ -358,7 +325,9 @@ int launch_step(crystalkv_t* h, DecodeParams& p, int layer, cudaStream_t s) {
     p.done_ctr = h->done_ctr + 2 * si;
     CK(h, cudaEventRecord(ea, s));
     CK(h, cudaStreamWaitEvent(h->side[si], ea, 0));
-    CK(h, lrfu_dispatch(h->G, p, h->U, h->side[si]));
+    const int threads = p.track ? lrfu_threads(h->U, h->len_hint, h->uniform, h->num_sms) : LRFU_SMALL;
+    p.front = std::min(h->cap_s, h->uniform ? h->len_hint : FRONT * threads);
+    CK(h, lrfu_launch(threads, h->G, p, h->U, h->side[si]));
     CK(h, cudaEventRecord(h->evF[k % crystalkv::EV_RING], h->side[si]));
     h->lastF[layer] = k;
     h->kF = k + 1;
@@ -422,6 +391,7 @@ int crystalkv_create(const crystalkv_config_t* cfg, crystalkv_t** out) {
   if (c.max_budget == 0) c.max_budget = 4 * c.budget_per_head;
   if (c.evict_every < 1) c.evict_every = 1;
   const bool evict = c.mode == CRYSTALKV_MODE_EVICT;
+  h->len_hint = c.budget_per_head + c.evict_every;
   h->G = c.n_q_heads / c.n_kv_heads;
   h->U = c.batch * c.n_kv_heads;
   h->units = h->U * c.n_layers;
@@ -658,6 +628,7 @@ static int prefill_common(crystalkv_t* h, int layer, const void* k, const void* 
   // CTAs per head of the row copy: a page per warp and turn, up to eight CTAs per SM in all
   const int per_head = std::max(1, std::min((P / GRP + NW) / NW, (8 * h->num_sms + h->U - 1) / h->U));
   h->prev_layer = -1;
+  if (evict && c.budget_ratio > 0.f) h->len_hint = ratio_budget(c, P) + c.evict_every;
   if (evict && W == 0) {
     // Algorithm 1 with the last query over scores and metadata only, then the survivors' rows; every
     // kernel on `s`, which has joined the internal streams, so any scratch set is free
@@ -827,6 +798,8 @@ int crystalkv_rebudget(crystalkv_t* h, void* stream) {
   const long long B_total = (long long)(c.budget_ratio > 0.f ? ratio_budget(c, t_last + 1) : c.budget_per_head) * N;
   alg2_kernel<<<c.batch, NT, sm, s>>>(h->Asum, h->st.budget, c.n_layers, c.n_kv_heads, B_total, c.min_budget, c.max_budget);
   CK(h, cudaGetLastError());
+  h->uniform = false;
+  h->len_hint = (int)(B_total / N) + c.evict_every;
   if (int sr = shrink_layers(h, 0, c.n_layers, t_last, s)) return sr;
   // heads changed length: every layer's next decode step needs a new plan
   return replan(h, 0, c.n_layers, s);
@@ -841,6 +814,7 @@ int crystalkv_set_budget(crystalkv_t* h, int layer, int seq, int kv_head, int32_
   ON_DEVICE(h);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (int jr = join_side(h, s)) return jr;
+  h->uniform = false;
   const int uid = (seq * c.n_layers + layer) * c.n_kv_heads + kv_head;
   CK(h, cudaMemcpyAsync(h->st.budget + uid, &budget, sizeof(int), cudaMemcpyHostToDevice, s));
   CK(h, cudaStreamSynchronize(s));
@@ -976,6 +950,7 @@ int crystalkv_import_state(crystalkv_t* h, int layer, int seq, int kv_head, cons
   import_unit_kernel<<<1, NT, 0, s>>>(h->st, uid, seq, h->io_rec, h->io_rows, h->io_rows + (size_t)h->cap * ROW_BYTES, n_rec, b);
   CK(h, cudaGetLastError());
   CK(h, cudaStreamSynchronize(s));   // the host buffers and the staging area are free again
+  h->uniform = false;
   h->t_layer[layer] = t;
   h->prev_layer = -1;
   return replan(h, layer, 1, s);

@@ -44,6 +44,7 @@ __device__ __forceinline__ void move_entry(const State& st, int uid, int seq, si
 
 // The pages a head owns beyond those that back list positions 0 .. n_new return to the
 // sequence's free list.  Only called from launches in which no head takes a page.
+template <int NTH = NT>
 __device__ __forceinline__ void release_pages(const State& st, int uid, int seq, int n_new, int* s_base) {
   const int need = n_new / GRP + 1;   // position n_new (the hole) stays backed
   const int have = st.npages[uid];
@@ -53,22 +54,23 @@ __device__ __forceinline__ void release_pages(const State& st, int uid, int seq,
   __syncthreads();
   const int base = *s_base;
   int* stack = st.free_stack + (size_t)seq * st.pages_per_seq;
-  for (int r = threadIdx.x; r < cnt; r += NT) stack[base + r] = st.ptab[(size_t)uid * st.capg + need + r];
+  for (int r = threadIdx.x; r < cnt; r += NTH) stack[base + r] = st.ptab[(size_t)uid * st.capg + need + r];
   __syncthreads();
   if (threadIdx.x == 0) st.npages[uid] = need;
 }
 
 // Removes the k lowest entries (1 <= k < n) of head `uid` at time t; the head's n entries must be
 // dense (list positions 0 .. n-1).  `sh` is >= 1.2 KB (300 ints) of shared scratch, `tmp` a global
-// int scratch of >= n words.  All NT threads call it.
+// int scratch of >= n words.  All NTH threads call it.
+template <int NTH = NT>
 __device__ void evict_many(const State& st, int uid, int seq, int n, int k, int t, bool release, int* sh, int* tmp) {
   const size_t mb = (size_t)uid * st.cap;
   int* hist = sh;             // 256
   int* s_kw = sh + 256;       // 3 words of the k-th key
   int* s_krem = sh + 259;
-  int* red = sh + 260;        // NW + 1
+  int* red = sh + 260;        // NTH / 32
   const int tid = threadIdx.x;
-  int* s_done = sh + 260 + NW + 1;
+  int* s_done = sh + 260 + NTH / 32;
   if (tid < 3) s_kw[tid] = 0;
   if (tid == 0) { *s_krem = k; *s_done = 0; }
   __syncthreads();
@@ -77,11 +79,11 @@ __device__ void evict_many(const State& st, int uid, int seq, int n, int k, int 
   // prefix followed by all ones then separates the same set as the k-th key itself.
   for (int word = 0; word < 3 && !*s_done; ++word) {
     for (int shift = 24; shift >= 0 && !*s_done; shift -= 8) {
-      for (int b = tid; b < 256; b += NT) hist[b] = 0;
+      for (int b = tid; b < 256; b += NTH) hist[b] = 0;
       __syncthreads();
       const uint32_t k0 = s_kw[0], k1 = s_kw[1], k2 = s_kw[2];
       const uint32_t kw[3] = {k0, k1, k2};
-      for (int i = tid; i < n; i += NT) {
+      for (int i = tid; i < n; i += NTH) {
         const Key96 key = entry_key(st, mb, i, t);
         bool match = true;
         for (int x = 0; x < word; ++x) match = match && (key.w[x] == kw[x]);
@@ -127,34 +129,34 @@ __device__ void evict_many(const State& st, int uid, int seq, int n, int k, int 
   const int nk = n - k;
   // gaps: leaving entries inside the surviving range [0, nk)
   int gaps = 0;
-  for (int base = 0; base < nk; base += NT) {
+  for (int base = 0; base < nk; base += NTH) {
     const int i = base + tid;
     const int flag = (i < nk) && key_le(entry_key(st, mb, i, t), kth);
     int tot;
-    const int r = block_excl_scan(flag, red, tot);
+    const int r = block_excl_scan<NTH>(flag, red, tot);
     if (flag) tmp[gaps + r] = i;
     gaps += tot;
   }
   // movers: staying entries in the tail [nk, n), as many as there are gaps
   int movers = 0;
-  for (int base = nk; base < n; base += NT) {
+  for (int base = nk; base < n; base += NTH) {
     const int i = base + tid;
     const int flag = (i < n) && !key_le(entry_key(st, mb, i, t), kth);
     int tot;
-    const int r = block_excl_scan(flag, red, tot);
+    const int r = block_excl_scan<NTH>(flag, red, tot);
     if (flag) tmp[gaps + movers + r] = i;
     movers += tot;
   }
   __syncthreads();
   // every mover fills one gap, in order; rows and metadata travel together
-  for (int j = tid >> 5; j < min(gaps, movers); j += NW) move_entry(st, uid, seq, mb, tmp[j], tmp[gaps + j], tid & 31);
+  for (int j = tid >> 5; j < min(gaps, movers); j += NTH / 32) move_entry(st, uid, seq, mb, tmp[j], tmp[gaps + j], tid & 31);
   __syncthreads();
   if (tid == 0) {
     st.n_cur[uid] = nk;
     st.hole[uid] = nk;
     atomicAdd(&st.counters[2], (unsigned long long)k);
   }
-  if (release) release_pages(st, uid, seq, nk, s_krem);
+  if (release) release_pages<NTH>(st, uid, seq, nk, s_krem);
 }
 
 }  // namespace ckv

@@ -12,21 +12,30 @@
 // A launch without Algorithm 1 (answer stage, full-cache mode) only lets every head keep its new
 // entry.  Either way the CTA that finishes last writes the layer's next launch plan (plan.cuh) when
 // a head's length has drifted from the one the current plan was made for.
+//
+// Bound: latency, a chain of a dozen block-wide steps and dependent reads beside an attention kernel
+// that saturates HBM.  (Sharing long heads among the CTAs of a cluster did not help: two to four
+// CTAs for heads of 4097 entries took 48 us beside the attention kernel instead of 56, and the layer
+// 36.3 us instead of 34.4; for heads of 1025 entries 17 us instead of 11.)
 #pragma once
-#include "common.cuh"
+#include <atomic>
+#include <cstddef>
+
 #include "evict.cuh"
+#include "lrfu_launch.cuh"
 #include "nucleus.cuh"
 #include "plan.cuh"
 
 namespace ckv {
 
+template <int NTH>
 struct LrfuSmem {
-  NucleusSmem<NT> nu;
-  int amin[NW * 4];
+  NucleusSmem<NTH> nu;
+  int amin[NTH / 32 * 4];
   int ev[320];
   int is_last;
 };
-static_assert(sizeof(LrfuSmem) >= (MAX_UNITS_PER_CALL + 1) * sizeof(int) + 321 * sizeof(int), "the planner's prefix sums reuse this memory");
+static_assert(offsetof(LrfuSmem<NT>, ev) >= (MAX_UNITS_PER_CALL + 1) * sizeof(int), "the planner's list of lengths reuses this memory");
 
 // Loads the compiler must leave where they are written: the kernel is bound by the latency of
 // its dependent global reads (several microseconds each while the attention kernel saturates
@@ -47,27 +56,28 @@ __device__ __forceinline__ float4 ld_f32x4(const float* p) {
   return v;
 }
 
-constexpr int FRONT = 5;   // entries per thread whose logit rows are requested before n is known
-
 // What the kernel requests before it knows the head's length.
 template <int G>
 struct Front {
-  float4 ra[FRONT], rb[FRONT];   // logit rows of entries tid, tid + NT, ... (index clamped to the scratch)
+  float4 ra[FRONT], rb[FRONT];   // logit rows of this thread's first entries (index clamped to p.front)
   float m[G], l[G];              // merged reference point (log2 domain) and normaliser per query head
   int budget;
 };
 
-// EPT > 0: every thread keeps the pbar of its entries tid, tid + NT, ... (at most EPT) in
-// registers; EPT == 0: they live in the global scratch and any n is allowed.
-template <int G, int EPT>
-__device__ int lrfu_unit(const DecodeParams& p, int u, int uid, int seq, int n, LrfuSmem& sh, const Front<G>& fr) {
+// EPT > 0: every thread keeps the pbar of its entries tid, tid + NTH, ... (at most EPT) in
+// registers; EPT == 0: they live in the global scratch and any n is allowed.  A single leaver's place
+// becomes the head's hole; returns the number of entries that leave, of which the caller removes more
+// than one.
+template <int G, int NTH, int EPT>
+__device__ int lrfu_unit(const DecodeParams& p, int u, int uid, int seq, int n, LrfuSmem<NTH>& sh, const Front<G>& fr) {
   constexpr int R = EPT > 0 ? EPT : 1;
+  constexpr int WARPS = NTH / 32;
   const State& st = p.st;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const size_t mb = (size_t)uid * st.cap;
   const float* S = p.sc.logits + (size_t)u * p.sc.cap_s * QH;
   float* pbar = p.sc.pbar + (size_t)u * p.sc.cap_s;
-  const int kmax = EPT > 0 ? (n + NT - 1) / NT : 0;
+  const int kmax = EPT > 0 ? (n + NTH - 1) / NTH : 0;
 
   // ---- step 1: pbar_i = mean_g exp(s_gi - m_g) / l_g
   float mx[G], invl[G];
@@ -87,6 +97,24 @@ __device__ int lrfu_unit(const DecodeParams& p, int u, int uid, int seq, int n, 
     return pm;
   };
   float pmr[R];
+  // Once every thread holds its entries' pbar in registers the logit rows are dead: their L2 lines are
+  // dropped instead of being written back to DRAM later.  Four 32-byte rows share a 128-byte line;
+  // units start on line boundaries (cap_s is a multiple of four).
+  // The barrier takes a value computed from every pbar, so no thread passes it with a row
+  // load still in flight.
+  auto drop_rows = [&]() {
+    int unordered = 0;
+#pragma unroll
+    for (int k = 0; k < R; ++k) unordered |= (pmr[k] != pmr[k]);
+    (void)__syncthreads_or(unordered);
+    if ((tid & 3) == 0) {
+#pragma unroll
+      for (int k = 0; k < R; ++k) {
+        const int i = tid + k * NTH;
+        if (i < n) asm volatile("discard.global.L2 [%0], 128;\n" ::"l"(S + (size_t)i * QH) : "memory");
+      }
+    }
+  };
   // stored state of this thread's entries, requested as soon as the logits are consumed so that
   // the reads complete under the threshold search (EPT == FRONT only)
   int pos_r[R], tau_r[R];
@@ -98,32 +126,16 @@ __device__ int lrfu_unit(const DecodeParams& p, int u, int uid, int seq, int n, 
       float pm = 0.f;
 #pragma unroll
       for (int g = 0; g < G; ++g) pm = fmaf(expf(sv[g] - mx[g]), invl[g], pm);
-      pmr[k] = (tid + k * NT < n) ? pm : 0.f;
+      pmr[k] = (tid + k * NTH < n) ? pm : 0.f;
     }
 #pragma unroll
     for (int k = 0; k < R; ++k) {
-      const size_t i = mb + min(tid + k * NT, n - 1);
+      const size_t i = mb + min(tid + k * NTH, n - 1);
       pos_r[k] = ld_i32(st.meta_pos + i);
       tau_r[k] = ld_i32(st.meta_tau + i);
       crf_r[k] = ld_f32(st.meta_crf + i);
     }
-    // The logit rows are dead now (every thread holds its own in registers since before the
-    // kernel learnt n, and nothing reads them again): drop their L2 lines instead of letting
-    // them be written back to DRAM later.  Four 32-byte rows share a 128-byte line; units start
-    // on line boundaries (cap_s is a multiple of four).
-    // The barrier takes a value computed from every pbar, so no thread passes it with a row
-    // load still in flight.
-    int unordered = 0;
-#pragma unroll
-    for (int k = 0; k < R; ++k) unordered |= (pmr[k] != pmr[k]);
-    (void)__syncthreads_or(unordered);
-    if ((tid & 3) == 0) {
-#pragma unroll
-      for (int k = 0; k < R; ++k) {
-        const int i = tid + k * NT;
-        if (i < n) asm volatile("discard.global.L2 [%0], 128;\n" ::"l"(S + (size_t)i * QH) : "memory");
-      }
-    }
+    drop_rows();
   } else if (EPT > 0) {
     // batches of BR entries whose rows are requested together (clamped index, no branch): while the
     // attention kernel saturates HBM every dependent round of loads costs this CTA microseconds, so
@@ -138,7 +150,7 @@ __device__ int lrfu_unit(const DecodeParams& p, int u, int uid, int seq, int n, 
         float rb[BR][4];
 #pragma unroll
         for (int j = 0; j < BR; ++j) {
-          const int i = min(tid + (k0 + j) * NT, n - 1);
+          const int i = min(tid + (k0 + j) * NTH, n - 1);
           ra[j] = ld_f32x4(S + (size_t)i * QH);
           if (G == 5) {
             rb[j][0] = ld_f32(S + (size_t)i * QH + 4);
@@ -155,21 +167,22 @@ __device__ int lrfu_unit(const DecodeParams& p, int u, int uid, int seq, int n, 
             float pm = 0.f;
 #pragma unroll
             for (int g = 0; g < G; ++g) pm = fmaf(expf(sv[g] - mx[g]), invl[g], pm);
-            pmr[k0 + j] = (tid + (k0 + j) * NT < n) ? pm : 0.f;
+            pmr[k0 + j] = (tid + (k0 + j) * NTH < n) ? pm : 0.f;
           }
         }
       }
     }
+    drop_rows();
   } else {
-    for (int i = tid; i < n; i += NT) pbar[i] = pbar_of(i);
+    for (int i = tid; i < n; i += NTH) pbar[i] = pbar_of(i);
   }
-  const Nucleus nu = nucleus_search<NT>(n, p.top_p, sh.nu, st.errword, [&](auto f) {
+  const Nucleus nu = nucleus_search<NTH>(n, p.top_p, sh.nu, st.errword, [&](auto f) {
     if (EPT > 0) {
 #pragma unroll
       for (int k = 0; k < R; ++k)
-        if (k < kmax && tid + k * NT < n) f(pmr[k]);
+        if (k < kmax && tid + k * NTH < n) f(pmr[k]);
     } else {
-      for (int i = tid; i < n; i += NT) f(pbar[i]);
+      for (int i = tid; i < n; i += NTH) f(pbar[i]);
     }
   });
   const uint32_t theta = nu.theta;
@@ -179,9 +192,9 @@ __device__ int lrfu_unit(const DecodeParams& p, int u, int uid, int seq, int n, 
   if (EPT > 0 && cnt_eq > 1) {   // the rank among equal keys needs every entry's key: spill them
 #pragma unroll
     for (int k = 0; k < R; ++k)
-      if (k < kmax && tid + k * NT < n) pbar[tid + k * NT] = pmr[k];
-    __syncthreads();
+      if (k < kmax && tid + k * NTH < n) pbar[tid + k * NTH] = pmr[k];
   }
+  if (cnt_eq > 1) __syncthreads();
   const unsigned long long w_theta = mass_of(__uint_as_float(theta));
 
   // ---- steps 2-3: CRF/tau update; step 4 candidates
@@ -193,11 +206,11 @@ __device__ int lrfu_unit(const DecodeParams& p, int u, int uid, int seq, int n, 
     const uint32_t key = __float_as_uint(pm);
     bool hit = key > theta && found_all;
     if (key == theta && found_all) {
-      unsigned long long rank = 0;
+      unsigned long long before = 0;
       if (cnt_eq > 1)
         for (int x = 0; x < n; ++x)
-          rank += (__float_as_uint(pbar[x]) == theta) && (st.meta_pos[mb + x] < pos_i);
-      hit = (A + rank * w_theta) < Pthr;
+          before += (__float_as_uint(__ldcg(pbar + x)) == theta) && (st.meta_pos[mb + x] < pos_i);
+      hit = (A + before * w_theta) < Pthr;
     }
     float ct = __fmul_rn(dec, crf);
     if (hit) {
@@ -221,7 +234,7 @@ __device__ int lrfu_unit(const DecodeParams& p, int u, int uid, int seq, int n, 
         float crf4[8], dec4[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          const size_t i = mb + min(tid + (k0 + j) * NT, n - 1);
+          const size_t i = mb + min(tid + (k0 + j) * NTH, n - 1);
           pos4[j] = ld_i32(st.meta_pos + i);
           tau4[j] = ld_i32(st.meta_tau + i);
           crf4[j] = ld_f32(st.meta_crf + i);
@@ -230,7 +243,7 @@ __device__ int lrfu_unit(const DecodeParams& p, int u, int uid, int seq, int n, 
         for (int j = 0; j < 8; ++j) dec4[j] = __ldg(st.tab + (p.t - min(tau4[j], p.t)));
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          const int i = tid + (k0 + j) * NT;
+          const int i = tid + (k0 + j) * NTH;
           if (k0 + j < R && i < n) update(i, pmr[k0 + j < R ? k0 + j : 0], pos4[j], tau4[j], crf4[j], dec4[j]);
         }
       }
@@ -241,20 +254,19 @@ __device__ int lrfu_unit(const DecodeParams& p, int u, int uid, int seq, int n, 
     for (int k = 0; k < R; ++k) dec_r[k] = __ldg(st.tab + (p.t - min(tau_r[k], p.t)));
 #pragma unroll
     for (int k = 0; k < R; ++k) {
-      const int i = tid + k * NT;
+      const int i = tid + k * NTH;
       if (i < n) update(i, pmr[k], pos_r[k], tau_r[k], crf_r[k], dec_r[k]);
     }
   } else {
-    for (int i = tid; i < n; i += NT) {
+    for (int i = tid; i < n; i += NTH) {
       const int tau = st.meta_tau[mb + i];
       update(i, pbar[i], st.meta_pos[mb + i], tau, st.meta_crf[mb + i], st.tab[p.t - tau]);
     }
   }
   nhit = warp_sum_i(nhit);
   if (lane == 0 && nhit) atomicAdd(&st.counters[1], (unsigned long long)nhit);
-  int n_after = n;
-  if (k_evict == 1) {
-    // block argmin of (CRF_temp, tau, pos)
+  // the lowest (CRF_temp, tau, pos) of the warp, then (the first warp) of all warps
+  auto least = [&]() {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       const uint32_t o0 = __shfl_xor_sync(0xffffffffu, bk0, o), o1 = __shfl_xor_sync(0xffffffffu, bk1, o),
@@ -263,40 +275,34 @@ __device__ int lrfu_unit(const DecodeParams& p, int u, int uid, int seq, int n, 
       const bool less = (o0 != bk0) ? (o0 < bk0) : ((o1 != bk1) ? (o1 < bk1) : (o2 < bk2));
       if (less) { bk0 = o0; bk1 = o1; bk2 = o2; bidx = oi; }
     }
+  };
+  if (k_evict == 1) {
+    least();
     if (lane == 0) { sh.amin[w * 4] = (int)bk0; sh.amin[w * 4 + 1] = (int)bk1; sh.amin[w * 4 + 2] = (int)bk2; sh.amin[w * 4 + 3] = bidx; }
     __syncthreads();
-    if (tid == 0) {
-      uint32_t a0 = (uint32_t)sh.amin[0], a1 = (uint32_t)sh.amin[1], a2 = (uint32_t)sh.amin[2];
-      int ai = sh.amin[3];
-      for (int x = 1; x < NW; ++x) {
-        const uint32_t o0 = (uint32_t)sh.amin[x * 4], o1 = (uint32_t)sh.amin[x * 4 + 1], o2 = (uint32_t)sh.amin[x * 4 + 2];
-        const bool less = (o0 != a0) ? (o0 < a0) : ((o1 != a1) ? (o1 < a1) : (o2 < a2));
-        if (less) { a0 = o0; a1 = o1; a2 = o2; ai = sh.amin[x * 4 + 3]; }
+    if (w == 0) {
+      const int* a = sh.amin + min(lane, WARPS - 1) * 4;
+      bk0 = (uint32_t)a[0]; bk1 = (uint32_t)a[1]; bk2 = (uint32_t)a[2]; bidx = a[3];
+      least();
+      if (lane == 0) {
+        // the leaving entry's place is where the next arriving token is written
+        st.hole[uid] = bidx;
+        st.n_cur[uid] = n - 1;
+        atomicAdd(&st.counters[2], 1ull);
       }
-      // the leaving entry's place is where the next arriving token is written
-      st.hole[uid] = ai;
-      st.n_cur[uid] = n - 1;
-      atomicAdd(&st.counters[2], 1ull);
     }
-    n_after = n - 1;
-  } else if (k_evict > 1) {
-    __syncthreads();
-    if (k_evict > p.evict_every && tid == 0) atomicOr(st.errword, ERR_OVER_EVICT);
-    evict_many(st, uid, seq, n, min(k_evict, n - 1), p.t, false, sh.ev, reinterpret_cast<int*>(pbar));
-    n_after = n - min(k_evict, n - 1);
   }
-  if (n_after == n && tid == 0) keep_all(st, uid, seq, n);
-  return n_after;   // the head's length after the step
+  return k_evict;
 }
 
-template <int G>
-__global__ void __launch_bounds__(NT, 5) lrfu_kernel(const DecodeParams p) {
-  __shared__ LrfuSmem sh;
+template <int G, int NTH>
+__global__ void __maxnreg__(48) lrfu_kernel(const __grid_constant__ DecodeParams p) {
+  __shared__ LrfuSmem<NTH> sh;
   const State& st = p.st;
   const int u = blockIdx.x, seq = u / st.H, head = u % st.H;
   const int uid = (seq * st.L + p.layer) * st.H + head;
   // one batch of requests: the length, the budget, the softmax reference, and the logit rows the
-  // common path needs (requested for a full thread's worth, clamped to the scratch)
+  // common path needs (requested for a full thread's worth, clamped to the expected length)
   const int n = ld_i32(st.n_cur + uid) + 1;
   const int g_plan = threadIdx.x == 0 ? ld_i32(p.plan.gplan + u) : 0;   // used at the very end
   int n_new = n;   // the head's length after this launch
@@ -312,24 +318,28 @@ __global__ void __launch_bounds__(NT, 5) lrfu_kernel(const DecodeParams p) {
       const float* S = p.sc.logits + (size_t)u * p.sc.cap_s * QH;
 #pragma unroll
       for (int k = 0; k < FRONT; ++k) {
-        const int i = min((int)threadIdx.x + k * NT, p.sc.cap_s - 1);
+        const int i = min((int)threadIdx.x + k * NTH, p.front - 1);
         fr.ra[k] = ld_f32x4(S + (size_t)i * QH);
         fr.rb[k] = (G > 4) ? ld_f32x4(S + (size_t)i * QH + 4) : make_float4(0.f, 0.f, 0.f, 0.f);
       }
     }
-    if (n <= 0) {
-      if (threadIdx.x == 0) { st.n_cur[uid] = 0; st.hole[uid] = 0; }
-      n_new = 0;
-    } else if (p.literal && n < fr.budget) {   // Algorithm 1's first line as printed: nothing runs below the budget
-      if (threadIdx.x == 0) keep_all(st, uid, seq, n);
-    } else if (n <= FRONT * NT) {
-      n_new = lrfu_unit<G, FRONT>(p, u, uid, seq, n, sh, fr);
-    } else if (n <= 10 * NT) {
-      n_new = lrfu_unit<G, 10>(p, u, uid, seq, n, sh, fr);
-    } else if (n <= 17 * NT) {
-      n_new = lrfu_unit<G, 17>(p, u, uid, seq, n, sh, fr);
-    } else {
-      n_new = lrfu_unit<G, 0>(p, u, uid, seq, n, sh, fr);
+    int leave = 0;
+    if (n > 0 && !(p.literal && n < fr.budget)) {   // (Algorithm 1's first line as printed: nothing runs below the budget)
+      if (n <= min(FRONT * NTH, p.front)) leave = lrfu_unit<G, NTH, FRONT>(p, u, uid, seq, n, sh, fr);
+      else if (NTH >= NT && n <= 10 * NTH) leave = lrfu_unit<G, NTH, NTH >= NT ? 10 : 0>(p, u, uid, seq, n, sh, fr);
+      else if (NTH == NT && n <= 17 * NTH) leave = lrfu_unit<G, NTH, NTH == NT ? 17 : 0>(p, u, uid, seq, n, sh, fr);
+      else leave = lrfu_unit<G, NTH, 0>(p, u, uid, seq, n, sh, fr);
+    }
+    if (leave > 1) {
+      __syncthreads();   // every thread's CRFs are written
+      if (leave > p.evict_every && threadIdx.x == 0) atomicOr(st.errword, ERR_OVER_EVICT);
+      leave = min(leave, n - 1);
+      evict_many<NTH>(st, uid, seq, n, leave, p.t, false, sh.ev, reinterpret_cast<int*>(p.sc.pbar + (size_t)u * p.sc.cap_s));
+    }
+    n_new = max(n - leave, 0);
+    if (leave == 0 && threadIdx.x == 0) {
+      if (n > 0) keep_all(st, uid, seq, n);
+      else { st.n_cur[uid] = 0; st.hole[uid] = 0; }
     }
   } else if (threadIdx.x == 0) {
     keep_all(st, uid, seq, n);   // no Algorithm 1: the head keeps its new entry
@@ -337,10 +347,10 @@ __global__ void __launch_bounds__(NT, 5) lrfu_kernel(const DecodeParams p) {
   if (threadIdx.x == 0) atomicAdd(&st.counters[0], (unsigned long long)max(n, 0));
   // ---- The layer's plan names pieces by (head, j of k), so it stays correct while heads grow or
   // shrink a little; a head whose group count has drifted from the planned one by an eighth (at
-  // least two), or a next launch of another kind than this one, marks it stale, and the CTA that
-  // finishes last (it then knows every head's new length) writes a new one.  In steady state (one
-  // entry arrives, one leaves) nothing is written.  Thread 0 wrote the head's new length itself,
-  // so the release of its count makes that length visible to whoever acquires the last count.
+  // least two) marks it stale, and the head that finishes last (its CTA then knows every head's new
+  // length) writes a new one.  In steady state (one entry arrives, one leaves) nothing is written.
+  // Thread 0 wrote the head's new length itself, so the release of its count makes that length
+  // visible to whoever acquires the last count.
   if (threadIdx.x == 0) {
     const int g_new = (n_new + 1 + GRP - 1) / GRP;
     if (abs(g_new - g_plan) >= max(2, g_plan >> 3)) atomicOr(p.done_ctr + 1, 1);
@@ -355,7 +365,30 @@ __global__ void __launch_bounds__(NT, 5) lrfu_kernel(const DecodeParams p) {
   }
   __syncthreads();
   if (!sh.is_last) return;
-  write_plan(st, p.plan, p.layer, p.plan_warps, p.plan_grid, reinterpret_cast<int*>(&sh), sh.ev);
+  // the planner's list of lengths takes the place of the histogram or, where that is too small, of
+  // this launch's pbar area, with which all heads are through
+  write_plan<NTH>(st, p.plan, p.layer, p.plan_warps, p.plan_grid,
+                  NTH >= NT ? reinterpret_cast<int*>(&sh) : reinterpret_cast<int*>(p.sc.pbar), sh.ev);
+}
+
+template <int G, int NTH>
+cudaError_t launch_lrfu(const DecodeParams& p, int heads, cudaStream_t s) {
+  // the same shared-memory carve-out as the attention kernel, so that CTAs of both can be
+  // resident on one SM at the same time
+  // (function attributes are kept per device)
+  static std::atomic<bool> prepared[MAX_DEVICES] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= MAX_DEVICES) return cudaErrorInvalidDevice;
+  if (!prepared[dev].load(std::memory_order_acquire)) {
+    e = cudaFuncSetAttribute(lrfu_kernel<G, NTH>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             (int)cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
+    prepared[dev].store(true, std::memory_order_release);
+  }
+  lrfu_kernel<G, NTH><<<heads, NTH, 0, s>>>(p);
+  return cudaGetLastError();
 }
 
 }  // namespace ckv

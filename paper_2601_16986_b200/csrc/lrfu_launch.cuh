@@ -6,7 +6,6 @@
 namespace ckv {
 
 constexpr int MAX_DEVICES = 64;   // device ordinals this library keeps per-device state for
-
 constexpr int FRONT = 5;   // entries per thread whose logit rows are requested before n is known
 constexpr int LRFU_SMALL = 64;   // threads of the CTAs for short heads
 constexpr int LRFU_LARGE = 512;  // ... for long ones

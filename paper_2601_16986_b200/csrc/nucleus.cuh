@@ -1,8 +1,9 @@
 // The top-p threshold of one head, found exactly: the value theta of pbar such that the entries
 // above it (and the earliest of those equal to it) are the smallest descending-pbar prefix whose
-// exclusive mass is below p.  One histogram of 1024 bins of 1/64 octave around 1/n locates theta's
-// bin, the few entries of that bin are ranked against one another; a bin outside the window or
-// with more than 64 entries falls back to four 8-bit radix passes over all bits.
+// exclusive mass is below p.  One histogram of 1024 bins of 1/64 octave around 1/n (256 of 1/16 for
+// CTAs of 64 threads) locates theta's bin, the few entries of that bin are ranked against one
+// another; a bin outside the window or with more than 64 entries falls back to four 8-bit radix
+// passes over all bits.
 // The mass walk uses 2^-40 fixed-point integers so it is exact and order independent; the
 // threshold is relative to the integer total, so a common factor on pbar changes nothing.
 #pragma once
@@ -10,17 +11,17 @@
 
 namespace ckv {
 
-constexpr int HIST_BINS = 1024;   // shared histogram size: the fine pass uses all of it, a radix pass 256
 constexpr float MASS_ONE = 1099511627776.0f;   // 2^40
-
-constexpr int FINE_BINS = 1024;   // fast path: bins of 2^17 key steps = 1/64 octave, 16 octaves wide
-constexpr int FINE_SHIFT = 17;
 constexpr int MAX_CAND = 64;
+
+// fine bins of CTAs of NTH threads and the key bits below a bin: 16 octaves in all
+__host__ __device__ constexpr int fine_bins(int nth) { return nth < 256 ? 256 : 1024; }
+__host__ __device__ constexpr int fine_shift(int nth) { return nth < 256 ? 19 : 17; }
 
 template <int NTH>
 struct NucleusSmem {
-  unsigned hist_lo[HIST_BINS];   // per-bin mass, low 16 bits of every term
-  unsigned hist_hi[HIST_BINS];   // per-bin mass, the bits above
+  unsigned hist_lo[fine_bins(NTH)];   // per-bin mass, low 16 bits of every term
+  unsigned hist_hi[fine_bins(NTH)];   // per-bin mass, the bits above
   unsigned long long redu[NTH / 32 + 1];
   unsigned cand[MAX_CAND];       // keys of the entries in the threshold's bin
   unsigned long long A_theta;    // fast path result: mass strictly above the threshold key
@@ -54,10 +55,10 @@ __device__ __forceinline__ unsigned long long warp_suffix(unsigned long long v, 
 // All NTH threads of a CTA call it; `each(f)` calls f(pbar) for every entry the calling thread owns.
 template <int NTH, class Each>
 __device__ __forceinline__ Nucleus nucleus_search(int n, float top_p, NucleusSmem<NTH>& sh, int* errword, Each each) {
-  constexpr int WARPS = NTH / 32;
+  constexpr int WARPS = NTH / 32, FINE_BINS = fine_bins(NTH), FINE_SHIFT = fine_shift(NTH);
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   // ---- fast path, pass over all entries: histogram of mass in fine bins around 1/n
-  //      bin(key) = clamp((key >> 17) - base, 0, 1023), monotone in key
+  //      bin(key) = clamp((key >> FINE_SHIFT) - base, 0, FINE_BINS - 1), monotone in key
   const int fbase = (int)(__float_as_uint(1.0f / (256.0f * (float)n)) >> FINE_SHIFT);
   auto fbin = [&](uint32_t key) { return min(FINE_BINS - 1, max(0, (int)(key >> FINE_SHIFT) - fbase)); };
   for (int b = tid; b < FINE_BINS; b += NTH) { sh.hist_lo[b] = 0u; sh.hist_hi[b] = 0u; }
@@ -77,10 +78,9 @@ __device__ __forceinline__ Nucleus nucleus_search(int n, float top_p, NucleusSme
     constexpr int PER = FINE_BINS / NTH;
     unsigned long long hb[PER], loc = 0;
 #pragma unroll
-    for (int b = 0; b < PER; ++b) {
-      hb[b] = ((unsigned long long)sh.hist_hi[tid * PER + b] << 16) + sh.hist_lo[tid * PER + b];
-      loc += hb[b];
-    }
+    for (int b = 0; b < PER; ++b) hb[b] = ((unsigned long long)sh.hist_hi[tid * PER + b] << 16) + sh.hist_lo[tid * PER + b];
+#pragma unroll
+    for (int b = 0; b < PER; ++b) loc += hb[b];
     const unsigned long long suf = warp_suffix(loc, lane);
     if (lane == 0) sh.redu[w] = suf;
     __syncthreads();
@@ -153,7 +153,7 @@ __device__ __forceinline__ Nucleus nucleus_search(int n, float top_p, NucleusSme
     found = true;
     for (int pass = 0; pass < 4; ++pass) {
       const int sft = 24 - 8 * pass;
-      constexpr int NB = 256;
+      constexpr int NB = 256, PER = NB > NTH ? NB / NTH : 1;
       __syncthreads();
       for (int b = tid; b < NB; b += NTH) { sh.hist_lo[b] = 0u; sh.hist_hi[b] = 0u; }
       if (tid == 0) sh.star = -1;
@@ -169,19 +169,27 @@ __device__ __forceinline__ Nucleus nucleus_search(int n, float top_p, NucleusSme
         }
       });
       __syncthreads();
-      // suffix sums from the top bin: thread k < 256 owns bin k
-      static_assert(NTH >= NB, "one bin per thread");
-      const unsigned long long hb =
-          tid < NB ? ((unsigned long long)sh.hist_hi[tid] << 16) + sh.hist_lo[tid] : 0ull;
-      const unsigned long long suf = warp_suffix(hb, lane);
+      // suffix sums from the top bin: thread k owns bins [PER k, PER (k + 1))
+      unsigned long long hb[PER], loc = 0;
+#pragma unroll
+      for (int b = 0; b < PER; ++b) {
+        const int bin = tid * PER + b;
+        hb[b] = bin < NB ? ((unsigned long long)sh.hist_hi[bin] << 16) + sh.hist_lo[bin] : 0ull;
+        loc += hb[b];
+      }
+      const unsigned long long suf = warp_suffix(loc, lane);
       if (lane == 0) sh.redu[w] = suf;
       __syncthreads();
       unsigned long long above = 0;
       for (int x = w + 1; x < WARPS; ++x) above += sh.redu[x];
-      const unsigned long long sab = A + above + (suf - hb);   // mass above this thread's bin
-      if (tid < NB && sab < Pthr && Pthr <= sab + hb) {
-        sh.star = tid;
-        sh.redu[WARPS] = sab;
+      unsigned long long sab = A + above + (suf - loc);   // mass above this thread's top bin
+#pragma unroll
+      for (int b = PER - 1; b >= 0; --b) {
+        if (sab < Pthr && Pthr <= sab + hb[b]) {
+          sh.star = tid * PER + b;
+          sh.redu[WARPS] = sab;
+        }
+        sab += hb[b];
       }
       __syncthreads();
       const int dstar = sh.star;

@@ -2,7 +2,7 @@
 // already stored.  Which entries a query hits depends on its scores alone, not on what earlier
 // queries of the window marked, so the window is one attention kernel over all (query, head) rows,
 // one threshold search per (head, query), and one kernel that walks an entry through its queries.
-// 128 heads x 1024 tokens, 32 queries of 5 heads: 83 + 49 + 21 us a layer; a decode-step launch pair
+// 128 heads x 1024 tokens, 32 queries of 5 heads: 83 + 49 + 21 us a layer (and 9 for the plan); a decode-step launch pair
 // per query, each reading the prompt's rows again, took 720 us.
 #pragma once
 #include "attn_kernel.cuh"

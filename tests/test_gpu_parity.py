@@ -483,6 +483,60 @@ def test_very_long_heads_use_the_general_lrfu_path():
     ls.close()
 
 
+@pytest.mark.parametrize("batch,H,G,budget,m", [(8, 8, 5, 2047, 16), (75, 8, 4, 130, 1), (160, 1, 1, 319, 1), (160, 1, 8, 300, 16),
+                                                (38, 4, 2, 320, 1), (1, 2, 8, 4352, 64),
+                                                (18, 8, 4, 1300, 1), (1, 1, 2, 5200, 1)])
+def test_launch_shapes_of_the_algorithm_1_kernel(batch, H, G, budget, m):
+    """CTAs of 64 threads (many heads of at most 320 entries), of 256 and of 512 (long heads) at the ends of their ranges, with one and
+    with many entries leaving at once; then a reallocation, after which heads of different lengths go
+    back to CTAs of 256 threads."""
+    wl = Workload(name=f"shape{batch}_{budget}", seed=1200 + budget, n_layers=1, n_q_heads=H * G, n_kv_heads=H, batch=batch,
+                  prompt=budget, think_steps=2 * m + 6, budget_per_head=budget, outlier="perhead")
+    ls = LockStep(wl, [0, batch - 1], max_budget=3 * budget, evict_every=m)
+    ls.prefill()
+    for _ in range(2 * m + 3):
+        ls.step()
+    ls.rebudget()
+    for _ in range(3):
+        ls.step()
+    ls.gpu.check()
+    ls.assert_clean()
+    ls.close()
+
+
+@pytest.mark.parametrize("batch,budget,spread", [(1, 1100, 0.0), (200, 200, 0.0), (1, 1100, 1e4), (200, 200, 1e4)])
+def test_equal_and_extreme_scores_in_every_launch_shape(batch, budget, spread):
+    """Equal keys (every entry carries the threshold's value: positions decide) and logits so far apart that the
+    threshold lies outside the histogram's window, for CTAs of 256 and of 64 threads."""
+    from oracle import Oracle, OracleConfig
+    from paper_2601_16986_b200 import Config, CrystalKV
+    shape = dict(n_layers=1, n_q_heads=8, n_kv_heads=2, batch=batch, budget_per_head=budget, max_context=budget + 8)
+    kv = CrystalKV(Config(**shape))
+    ora = Oracle(OracleConfig(**dict(shape, batch=1), min_budget=min(budget, max(16, budget // 8)), max_budget=4 * budget))
+    g = torch.Generator("cuda").manual_seed(5)
+    row = torch.randn(1, 1, 2, 128, device="cuda", generator=g)
+    k = row.expand(1, budget + 3, 2, 128).clone()
+    if spread:
+        k[:, 3:] *= -1.0          # three entries hold all the mass, the others' weights underflow
+        k *= spread ** 0.25
+    k = k.to(torch.bfloat16)
+    q = row.repeat_interleave(4, 2)[:, 0].to(torch.bfloat16).expand(batch, 8, 128).contiguous()
+    kb = k.expand(batch, budget + 3, 2, 128)
+    kv.prefill(0, kb[:, :budget].contiguous(), kb[:, :budget].contiguous(), q)
+    ora.prefill(0, k[:, :budget].cpu(), k[:, :budget].cpu(), q[:1].cpu())
+    for i in range(3):
+        new = kb[:, budget + i].contiguous()
+        kv.decode_step(0, q, new, new)
+        ora.decode_step(0, q[:1].cpu(), new[:1].cpu(), new[:1].cpu())
+        for h in range(2):
+            assert (kv.export_state(0, 0, h) == ora.export_state(0, 0, h)).all()
+            assert (kv.export_state(0, batch - 1, h) == ora.export_state(0, 0, h)).all()
+    kv.check()
+    kv.validate()
+    kv.close()
+    ora.close()
+
+
 def test_host_buffer_steps_match_device_steps():
     """crystalkv_decode_step_host with pinned buffers (the kernel reads them over PCIe) and with
     pageable buffers (staged copies) gives the outputs and the state of the device-pointer call."""
