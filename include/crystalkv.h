@@ -291,7 +291,7 @@ int crystalkv_debug_set_page(crystalkv_t* h, int layer, int seq, int kv_head, in
  * {head index seq * n_kv_heads + kv_head, j, k, together} of piece i: the j-th of the head's k
  * pieces, `together` = 1 when the k pieces sit in consecutive warps of one CTA, 2 when they sit
  * that way in runs of eight (pieces 8 r .. 8 r + 7 in the eight warps of one CTA) and one shorter
- * run, 0 otherwise.  warps_cap and pieces_cap are the capacities of the two arrays in warps and
+ * run, 3 when they are dealt evenly to the CTAs of a cluster that shares the head, 0 otherwise.  warps_cap and pieces_cap are the capacities of the two arrays in warps and
  * in pieces; EINVAL unless warps_cap >= 8 x SMs and pieces_cap >= 8 x SMs + batch x n_kv_heads.
  * Synchronises `stream`.
  */

@@ -14,7 +14,9 @@
 // its (m, l, O) partial in its idle ring stages, the head's warps meet at a named barrier and
 // share the query heads.  A head of more than eight pieces is merged that way run by run (whole
 // CTAs and one shorter run) and its runs' partials through global memory: the warp whose ticket
-// completes the head merges them into `out`; so is a head that the plan could not keep together
+// completes the head merges them into `out`.  When there are few heads, a cluster of two or four
+// CTAs shares each of them: the CTAs merge their pieces as above and then one another's partials
+// through distributed shared memory.  Global memory also carries a head that the plan could not keep together
 // (after the warp's own pieces, if it has more).  The arriving token is written into the head's hole (the place
 // an evicted entry left, or the end of the list) by the warp that streams that group.  The scaled
 // logits of the step are left in the scratch for the LRFU kernel, which marks hits from the final
@@ -113,6 +115,8 @@ __device__ __forceinline__ void bar_sync(int id, int nthreads) {
 __device__ __forceinline__ void bar_arrive(int id, int nthreads) {
   asm volatile("bar.arrive %0, %1;\n" ::"r"(id), "r"(nthreads) : "memory");
 }
+
+constexpr int MAX_CLUSTER = 4;   // CTAs that may share a head
 
 constexpr float LAZY = 8.0f;   // the running maximum (log2 domain) may trail the true one by this much
 
@@ -232,7 +236,10 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
     if (tid == 0 && blockIdx.x == 0) atomicOr(st.errword, ERR_PLAN);
     return;
   }
-  if (range.x >= range.y) return;   // no run for this warp
+  if (range.x >= range.y) {   // no run for this warp
+    if (p.cl > 1) { cluster_sync(); cluster_sync(); }   // (the two barriers of the CTAs that share the head)
+    return;
+  }
 
   const int G = p.G, PS = 16 + G * HD;
   const uint32_t ring_u32 = smem_u32(smem) + w * (STAGES * PAGE_BYTES);
@@ -340,9 +347,11 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
     // (the plan marks it), is merged through shared memory.
     // (A head of more than eight pieces is placed in runs of eight, whole CTAs and one shorter run:
     // every run is merged in its CTA, and only one partial per run goes through global memory.)
-    const bool runs = dd.w == 2;
-    const int jr = runs ? (piece & (NW - 1)) : piece;                       // this piece's place in its run
-    const int rl = runs ? min(NW, npieces - (piece & ~(NW - 1))) : npieces;   // pieces in the run
+    const bool runs = dd.w == 2, shared_head = dd.w == 3;
+    const int j_cta = shared_head ? shared_first(npieces, cluster_rank(), p.cl) : 0;   // (a shared head's pieces before this CTA's)
+    const int jr = runs ? (piece & (NW - 1)) : piece - j_cta;               // this piece's place in its run
+    const int rl = runs ? min(NW, npieces - (piece & ~(NW - 1)))            // pieces in the run
+                        : shared_head ? shared_first(npieces, cluster_rank() + 1, p.cl) - j_cta : npieces;
     const int first_w = w - jr;
     const bool local = dd.w != 0 && npieces > 1 && range.y - range.x == 1 && first_w >= 0 && first_w + rl <= NW;
     // the G queries as B fragments, running softmax state, O^T accumulators
@@ -370,6 +379,8 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
         for (int s = 0; s < STAGES; ++s)
           if (s != csi) mbar_wait_bounded(bar0 + s * 8, (phases >> s) & 1u);
         if (local) bar_arrive(1 + first_w, 32 * rl);   // the run's other warps must not wait for this one
+        __syncwarp();
+        if (p.cl > 1) { cluster_sync(); cluster_sync(); }
         return;
       }
       phases ^= 1u << csi;
@@ -513,6 +524,8 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
       bar_sync(1 + first_w, 32 * rl);
       const unsigned char* base = smem + first_w * WSTRIDE;
       float* rpart = p.sc.partials + ((size_t)u * p.sc.pmax + (piece >> 3)) * PS;   // the run's partial (runs only)
+      constexpr int SHARE_AT = 8192, SHARE = (HD + 4) * 4;   // a shared head's partial of this CTA, query head g: at
+                                                             // SHARE_AT + g SHARE of the ring of warp g % rl
       for (int g = jr; g < G; g += rl) {
         float pm[NW], pl[NW];
         float4 v[NW];
@@ -534,6 +547,12 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
           a.x = fmaf(v[j].x, c, a.x); a.y = fmaf(v[j].y, c, a.y);
           a.z = fmaf(v[j].z, c, a.z); a.w = fmaf(v[j].w, c, a.w);
         }
+        if (shared_head) {
+          unsigned char* to = smem + w * WSTRIDE + SHARE_AT + g * SHARE;
+          *reinterpret_cast<float4*>(to + lane * 16) = a;
+          if (lane == 0) *reinterpret_cast<float2*>(to + HD * 4) = make_float2(m, L);
+          continue;
+        }
         if (runs) {   // the run's share of the head, not normalised
           *reinterpret_cast<float4*>(rpart + 16 + g * HD + lane * 4) = a;
           if (lane == 0) { rpart[g] = m; rpart[8 + g] = L; }
@@ -548,6 +567,50 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
           p.sc.mfin[u * (2 * QH) + g] = m;
           p.sc.mfin[u * (2 * QH) + QH + g] = L;
         }
+      }
+      if (shared_head) {
+        // every CTA's partials are written; query head g is put together by CTA g % (those that have pieces)
+        __syncwarp();
+        cluster_sync();
+        const int ctas = min(npieces, p.cl);
+        for (int g = cluster_rank() + ctas * jr; g < G; g += ctas * rl) {
+          float4 v[MAX_CLUSTER];
+          float2 ml[MAX_CLUSTER];
+          float m = -INFINITY;
+#pragma unroll
+          for (int x = 0; x < MAX_CLUSTER; ++x) {
+            ml[x] = make_float2(-INFINITY, 0.f);
+            v[x] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (x < ctas) {
+              const int n = shared_first(npieces, x + 1, p.cl) - shared_first(npieces, x, p.cl);   // pieces of CTA x
+              const uint32_t from = peer_addr(smem_u32(smem) + (g % n) * WSTRIDE + SHARE_AT + g * SHARE, x);
+              v[x] = peer_f32x4(from + lane * 16);
+              ml[x] = peer_f32x2(from + HD * 4);
+            }
+            m = fmaxf(m, ml[x].x);
+          }
+          float L = 0.f;
+          float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int x = 0; x < MAX_CLUSTER; ++x) {
+            const float c = (ml[x].x > -INFINITY) ? ex2(ml[x].x - m) : 0.f;
+            L = fmaf(ml[x].y, c, L);
+            a.x = fmaf(v[x].x, c, a.x); a.y = fmaf(v[x].y, c, a.y);
+            a.z = fmaf(v[x].z, c, a.z); a.w = fmaf(v[x].w, c, a.w);
+          }
+          const float iv = 1.0f / L;
+          uint2 pk;
+          pk.x = pack_bf16(a.x * iv, a.y * iv);
+          pk.y = pack_bf16(a.z * iv, a.w * iv);
+          *reinterpret_cast<uint2*>(p.out + ((size_t)(u * G + g)) * HD + lane * 4) = pk;
+          if (lane == 0 && p.track) {
+            p.sc.mfin[u * (2 * QH) + g] = m;
+            p.sc.mfin[u * (2 * QH) + QH + g] = L;
+          }
+        }
+        __syncwarp();
+        cluster_sync();   // nobody reads this CTA's shared memory any more
+        return;           // (a warp has one piece of a shared head and nothing else)
       }
       if (!runs) continue;
       // every warp of the head counts itself once its share of its run's partial is written; the
@@ -598,6 +661,8 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
   }
   if (defer0 >= 0) merge_head(p, defer0, __ldg(p.plan.npc + defer0), lane);
   if (defer1 >= 0) merge_head(p, defer1, __ldg(p.plan.npc + defer1), lane);
+  __syncwarp();
+  if (p.cl > 1) { cluster_sync(); cluster_sync(); }   // (a head that is one piece)
 }
 
 }  // namespace ckv

@@ -106,6 +106,7 @@ struct DecodeParams {
   int literal;    // 1: Algorithm 1 is skipped for a head below its budget (its first line as printed)
   int plan_warps;    // warps of the attention grid the plan is made for
   int plan_grid;     // CTAs of that grid
+  int cl;            // attention kernel: CTAs (a cluster) that share a head; 1: the plan places heads anywhere
   float scale;    // logit scale
   float scale_log2;
   float top_p;
@@ -139,6 +140,37 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v)
 __device__ __forceinline__ int warp_sum_i(int v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Pieces of a head of k that the CTAs before CTA x of a cluster of cl take: k dealt evenly, longer shares
+// first (the first min(k, cl) CTAs get at least one).
+__host__ __device__ __forceinline__ int shared_first(int k, int x, int cl) { return k / cl * x + (x < k % cl ? x : k % cl); }
+
+// ---- thread-block clusters (a launch without the attribute is a cluster of one)
+__device__ __forceinline__ int cluster_rank() {
+  int r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(r));
+  return r;
+}
+// The cluster's threads that have not exited meet; what they wrote to shared memory before is visible to all.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+// The shared::cluster address of CTA `rank`'s counterpart of this CTA's shared address.
+__device__ __forceinline__ uint32_t peer_addr(uint32_t addr, int rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(addr), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ float4 peer_f32x4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];\n" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ float2 peer_f32x2(uint32_t addr) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0,%1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
   return v;
 }
 

@@ -367,7 +367,7 @@ __global__ void __maxnreg__(48) lrfu_kernel(const __grid_constant__ DecodeParams
   if (!sh.is_last) return;
   // the planner's list of lengths takes the place of the histogram or, where that is too small, of
   // this launch's pbar area, with which all heads are through
-  write_plan<NTH>(st, p.plan, p.layer, p.plan_warps, p.plan_grid,
+  write_plan<NTH>(st, p.plan, p.layer, p.plan_warps, p.plan_grid, p.cl,
                   NTH >= NT ? reinterpret_cast<int*>(&sh) : reinterpret_cast<int*>(p.sc.pbar), sh.ev);
 }
 

@@ -107,7 +107,7 @@ __host__ __device__ inline bool place_runs(int full, const int* cnt, int grid, P
 // Called by all NTH threads of one CTA.  `gs` is memory for U + 1 ints, `red` shared memory for 320.
 // The plan is for a decode step: every head one entry longer than now.
 template <int NTH = NT>
-__device__ __forceinline__ void write_plan(const State& st, const Plan& pl, int layer, int nWarps, int grid,
+__device__ __forceinline__ void write_plan(const State& st, const Plan& pl, int layer, int nWarps, int grid, int cl,
                                         int* gs, int* red) {
   const int U = st.batch * st.H, tid = threadIdx.x, lane = tid & 31;
   // ---- groups per head
@@ -142,7 +142,11 @@ __device__ __forceinline__ void write_plan(const State& st, const Plan& pl, int 
   int T = 0x7fffffff;
   bool packed = false;
   int* hist = red + 16;   // [32][4]: counts of two run lengths per word, 16 bits each (U < 65536)
-  if (Gtot > 0 && U <= nWarps && grid * NW == nWarps && grid <= 256 && nWarps < 4096) {
+  if (cl > 1) {
+    // few heads: the cl CTAs of a cluster share each of them, in pieces of nearly equal length (at least
+    // two groups) dealt evenly to the CTAs
+    T = max(2, (gmax + NW * cl - 1) / (NW * cl));
+  } else if (Gtot > 0 && U <= nWarps && grid * NW == nWarps && grid <= 256 && nWarps < 4096) {
     // A launch with few groups per warp is bound by the steps a head's result goes through, not by
     // bytes: pieces are then made long enough (up to GLAT groups) for the longest head to stay inside
     // one CTA, whose merge is one barrier instead of a trip through global memory.
@@ -200,7 +204,7 @@ __device__ __forceinline__ void write_plan(const State& st, const Plan& pl, int 
       }
     }
   }
-  if (!packed && Gtot > 0 && U <= nWarps) {
+  if (!packed && cl == 1 && Gtot > 0 && U <= nWarps) {
     // fallback: the smallest T for which sum ceil(g_u / T) <= nWarps, heads laid over the warps end to end
     int lo = max(1, (Gtot + nWarps - 1) / nWarps), hi = max(lo, gmax);   // feasible at hi: one piece per head
     while (lo < hi) {
@@ -233,9 +237,10 @@ __device__ __forceinline__ void write_plan(const State& st, const Plan& pl, int 
       pl.gplan[u] = g;
       // the last word: 1 when the head's k pieces sit in consecutive warps of one CTA, each warp with
       // nothing else to stream; 2 when they sit that way in runs of eight (whole CTAs) and one shorter run
-      const int together = k <= 1 ? 0 : (packed ? (k <= NW ? 1 : 2) : ((start & (NW - 1)) + k <= NW ? 1 : 0));
+      const int together = k <= 1 ? 0 : cl > 1 ? 3 : (packed ? (k <= NW ? 1 : 2) : ((start & (NW - 1)) + k <= NW ? 1 : 0));
       for (int j = 0; j < k; ++j) pl.desc[start + j] = make_int4(u, j, k, together);
     }
+    if (cl > 1 && u < U) gs[u] = start;
     if (packed) {
       const int f = k >> 3, s = k & 7;
       const int c0 = wholes + block_excl_scan<NTH>(f, red, tot);
@@ -277,6 +282,15 @@ __device__ __forceinline__ void write_plan(const State& st, const Plan& pl, int 
         w[x] = make_int4(start + j0 + x, start + j0 + x + 1, u, (j0 + x) | (k << 12) | ((k <= 1 ? 0 : (k <= NW ? 1 : 2)) << 24));
     }
     if (!ok) nWarps = -1;   // no launch accepts the plan
+  } else if (cl > 1) {
+    __syncthreads();   // (every head's pieces and first piece are known)
+    // head u belongs to CTAs u cl .. u cl + cl - 1; CTA x of them takes the pieces from shared_first(k, x, cl) on
+    for (int pw = tid; pw < nWarps; pw += NTH) {
+      const int cta = pw / NW, u = cta / cl, x = cta % cl, k = u < U ? pl.npc[u] : 0;
+      const int j = shared_first(k, x, cl) + (pw & (NW - 1));
+      const bool mine = j < shared_first(k, x + 1, cl);
+      pl.wrange[pw] = mine ? make_int4(gs[u] + j, gs[u] + j + 1, u, j | (k << 12) | ((k <= 1 ? 0 : 3) << 24)) : make_int4(0, 0, -1, 0);
+    }
   } else {
     // heads end to end: consecutive pieces go to consecutive warps; with more pieces than warps
     // every warp takes a run of consecutive pieces

@@ -12,10 +12,10 @@ namespace ckv {
 
 // The plan as a kernel of its own: one CTA per layer of `layers` consecutive layers starting at
 // layer0 (after a prompt insertion, a reallocation, or any edit of a head's state from the host).
-__global__ void __launch_bounds__(NT) plan_kernel(State st, const Plan* plans, int layer0, int nWarps, int grid) {
+__global__ void __launch_bounds__(NT) plan_kernel(State st, const Plan* plans, int layer0, int nWarps, int grid, int cl) {
   __shared__ int s_gs[MAX_UNITS_PER_CALL + 1];
   __shared__ int s_red[320];
-  write_plan(st, plans[layer0 + blockIdx.x], layer0 + blockIdx.x, nWarps, grid, s_gs, s_red);
+  write_plan(st, plans[layer0 + blockIdx.x], layer0 + blockIdx.x, nWarps, grid, cl, s_gs, s_red);
 }
 
 constexpr int SEL_NT = 1024;            // threads of prefill_select_kernel
@@ -335,11 +335,11 @@ constexpr int ROWS_ALL_POS = 2;     // ... tau = i, the token's own arrival time
 // pass of the attention kernel: 81 us).
 __global__ void __launch_bounds__(NT) prefill_rows_kernel(State st, Plan plan, int layer, const unsigned char* __restrict__ k,
                                                           const unsigned char* __restrict__ v, int P, int mode, int per_head,
-                                                          int plan_warps, int plan_grid) {
+                                                          int plan_warps, int plan_grid, int plan_cl) {
   __shared__ int s_gs[MAX_UNITS_PER_CALL + 1];
   __shared__ int s_red[320];
   if (blockIdx.x == 0) {
-    if (plan_warps > 0) write_plan(st, plan, layer, plan_warps, plan_grid, s_gs, s_red);
+    if (plan_warps > 0) write_plan(st, plan, layer, plan_warps, plan_grid, plan_cl, s_gs, s_red);
     return;
   }
   const int u = (blockIdx.x - 1) / per_head, b = (blockIdx.x - 1) % per_head, seq = u / st.H, head = u % st.H;

@@ -347,6 +347,33 @@ def test_launch_plans_after_reallocations_are_all_inside_ctas():
     kv.close()
 
 
+@pytest.mark.parametrize("batch,H,G,budget", [(1, 1, 8, 16), (1, 2, 4, 33), (3, 2, 2, 53), (2, 8, 5, 500), (5, 7, 1, 130), (37, 1, 7, 97),
+                                              (19, 2, 3, 250), (9, 8, 6, 700)])
+def test_heads_shared_by_the_ctas_of_a_cluster(batch, H, G, budget):
+    """Few heads: two or four CTAs share each (one piece, fewer pieces than CTAs, uneven shares, every group
+    size).  Outputs and state against the oracle while the lists fill, through a reallocation, and after a
+    budget was set by hand (plans go back to placing heads anywhere)."""
+    wl = Workload(name=f"cl{batch}_{budget}", seed=1500 + budget, n_layers=2, n_q_heads=H * G, n_kv_heads=H, batch=batch,
+                  prompt=max(1, budget - 5), think_steps=24, budget_per_head=budget, outlier="perhead")
+    ls = LockStep(wl, [0, batch - 1] if batch > 1 else [0])
+    ls.prefill()
+    for s in range(20):
+        ls.step()
+        if s == 4:
+            hdr, wrange, desc = ls.gpu.debug_plan(1)
+            assert hdr[2] % (16 * batch * H) == 0 and set(desc[:hdr[0], 3]) <= {0, 3}
+        if s == 11:
+            ls.rebudget()
+        if s == 15:
+            ls.gpu.set_budget(0, 0, 0, max(1, budget // 2))
+            ls.ora.set_budget(0, 0, 0, max(1, budget // 2))
+            assert ls.gpu.debug_plan(1)[0][2] == ls.gpu.debug_plan(1)[1].shape[0]
+            ls.compare()
+    ls.gpu.check()
+    ls.assert_clean()
+    ls.close()
+
+
 # ------------------------------------------------------------------ full-size shapes, sampled
 def _run_sampled(name, sample, n_steps, cmp_every, answer=0, max_answer=0):
     wl = WORKLOADS[name]
