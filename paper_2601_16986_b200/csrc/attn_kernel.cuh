@@ -20,8 +20,7 @@
 // (after the warp's own pieces, if it has more).  The arriving token is written into the head's hole (the place
 // an evicted entry left, or the end of the list) by the warp that streams that group.  The scaled
 // logits of the step are left in the scratch for the LRFU kernel, which marks hits from the final
-// softmax weights without reading the cache again; the lines of the metadata that kernel will
-// read are asked into L2 on the way.
+// softmax weights without reading the cache again.
 #pragma once
 #include "common.cuh"
 
@@ -287,19 +286,6 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
     }
     const int f_uid = (f_seq * st.L + p.layer) * st.H + (u % st.H);
     pt = st.ptab + (size_t)f_uid * st.capg;
-    if (p.track) {
-      // The LRFU kernel that follows reads position, tau and CRF of these entries while the next
-      // layer's attention saturates HBM, and every round trip to DRAM costs it microseconds then:
-      // their lines are asked into L2 now (12 bytes per entry against the 512 streamed here).
-      const size_t e0 = (size_t)f_uid * st.cap + (size_t)f_next * GRP, e1 = (size_t)f_uid * st.cap + (size_t)f_hi * GRP;
-      const char* bases[3] = {reinterpret_cast<const char*>(st.meta_pos), reinterpret_cast<const char*>(st.meta_tau),
-                              reinterpret_cast<const char*>(st.meta_crf)};
-      const int nl = (int)(((e1 * 4 + 127) >> 7) - ((e0 * 4) >> 7));   // 128-byte lines per array (arrays are 256-byte aligned)
-      for (int x = lane; x < 3 * nl; x += 32) {
-        const char* a = bases[x / nl] + (((e0 * 4) >> 7) + (x % nl)) * 128;
-        asm volatile("prefetch.global.L2::evict_last [%0];\n" ::"l"(a));
-      }
-    }
     idbase = f_next;
     ids = (f_next + lane < f_hi) ? __ldg(pt + f_next + lane) : 0;   // page ids of groups f_next + lane
     if (lane == 0) fifo[fq_tail & (FIFO - 1)] = pi;

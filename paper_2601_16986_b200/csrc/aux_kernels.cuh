@@ -333,4 +333,23 @@ __global__ void __launch_bounds__(NT) import_unit_kernel(State st, int uid, int 
   if (tid == 0) { st.n_cur[uid] = n; st.hole[uid] = n; st.budget[uid] = budget; }
 }
 
+// The counters of the whole handle: out[0..2] = entries attended, hits, evictions.  One CTA of 1024 threads.
+__global__ void __launch_bounds__(1024) sum_counters_kernel(State st, int units, unsigned long long* out) {
+  __shared__ unsigned long long s_sum[32][3];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  unsigned long long a[3] = {0, 0, 0};
+  for (int i = tid; i < units; i += 1024)
+    for (int x = 0; x < 3; ++x) a[x] += st.ucount[(size_t)i * 4 + x];
+  for (int x = 0; x < 3; ++x) {
+    a[x] = warp_sum_u64(a[x]);
+    if (lane == 0) s_sum[w][x] = a[x];
+  }
+  __syncthreads();
+  if (tid < 3) {
+    unsigned long long v = st.counters[tid];
+    for (int x = 0; x < 32; ++x) v += s_sum[x][tid];
+    out[tid] = v;
+  }
+}
+
 }  // namespace ckv

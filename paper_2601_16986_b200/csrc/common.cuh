@@ -56,7 +56,8 @@ struct State {
   int* budget;       // [units] == [batch][L][H]
   const float* tab;  // lambda^D, D in [0, max_context]
   int* errword;
-  unsigned long long* counters;  // entries attended, hits, evictions
+  unsigned long long* counters;  // entries attended, hits, evictions of prompts and of evictions of several entries at once
+  unsigned long long* ucount;    // [units][4] the same of decode steps, per head
   int batch, L, H, cap, capg;
 };
 
@@ -230,10 +231,20 @@ __device__ __forceinline__ bool back_position(const State& st, int uid, int seq,
 
 // A head keeps all n entries of a step: the next arrival goes behind them, or, when that place cannot be
 // backed (the error word says so), takes the place of the last one.
-__device__ __forceinline__ void keep_all(const State& st, int uid, int seq, int n) {
+__device__ __forceinline__ int keep_all(const State& st, int uid, int seq, int n) {   // (its length from now on)
   if (!back_position(st, uid, seq, n)) --n;
   st.n_cur[uid] = n;
   st.hole[uid] = n;
+  return n;
+}
+
+// A decode step's counts for one head, kept per head: one launch's heads adding to the same three words held up one
+// another (1024 heads of 257 entries: 0.5 us a layer).
+__device__ __forceinline__ void count_unit(const State& st, int uid, int entries, int hits, int evictions) {
+  ulonglong2* c = reinterpret_cast<ulonglong2*>(st.ucount + (size_t)uid * 4);
+  ulonglong2 a = c[0], b = c[1];
+  a.x += entries; a.y += hits; b.x += evictions;
+  c[0] = a; c[1] = b;
 }
 
 // List position of the i-th live entry of a head (i in [0, n)) given its hole.

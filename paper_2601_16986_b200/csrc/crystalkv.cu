@@ -83,6 +83,7 @@ struct crystalkv {
   int* io_rec = nullptr;           // staging for export / import of one head: records, rows, count
   unsigned char* io_rows = nullptr;
   int* io_n = nullptr;
+  unsigned long long* io_sum = nullptr;   // ... and for the counters
   float* tab = nullptr;
   void* arena = nullptr;           // the one device allocation all of the above point into
   std::string err;
@@ -398,7 +399,8 @@ int launch_step(crystalkv_t* h, DecodeParams& p, int layer, cudaStream_t s) {
     CK(h, cudaStreamWaitEvent(h->side[si], ea, 0));
     const int threads = p.track ? lrfu_threads(h->U, entries, h->uniform, h->num_sms) : LRFU_SMALL;
     p.front = std::min(h->cap_s, h->uniform ? entries : std::min(p.t + 1, FRONT * threads));
-    CK(h, lrfu_launch(threads, std::min(h->cap, p.t + 1), h->G, p, h->U, h->side[si]));
+    const int npb = std::min(std::min(h->cap, p.t + 1), pbar_room(threads, h->U, entries, h->num_sms));
+    CK(h, lrfu_launch(threads, npb, h->G, p, h->U, h->side[si]));
     CK(h, cudaEventRecord(h->evF[k % crystalkv::EV_RING], h->side[si]));
     h->lastF[layer] = k;
     h->kF = k + 1;
@@ -567,6 +569,7 @@ int crystalkv_create(const crystalkv_config_t* cfg, crystalkv_t** out) {
     a.add(&h->tab, (size_t)c.max_context + 1);
     a.add(&st.errword, 1);
     a.add(&st.counters, 4);
+    a.add(&st.ucount, (size_t)h->units * 4);
     a.add(&h->Asum, h->units);
     for (int i = 0; i < NSETS; ++i) a.add(&h->sc_logits[i], (size_t)h->U * h->cap_s * QH);   // one block: no padding between sets
     for (int i = 0; i < NSETS; ++i) a.add(&h->sc_mfin[i], (size_t)h->U * 2 * QH);
@@ -581,6 +584,7 @@ int crystalkv_create(const crystalkv_config_t* cfg, crystalkv_t** out) {
     a.add(&h->io_rec, (size_t)3 * h->cap);
     a.add(&h->io_rows, (size_t)2 * h->cap * ROW_BYTES);
     a.add(&h->io_n, 1);
+    a.add(&h->io_sum, 4);
     if (int r = a.take(h)) CREATE_FAIL(r);
   }
   st.tab = h->tab;
@@ -609,6 +613,7 @@ int crystalkv_create(const crystalkv_config_t* cfg, crystalkv_t** out) {
   CKC(cudaMemset(st.npages, 0, (size_t)h->units * sizeof(int)));
   CKC(cudaMemset(st.errword, 0, sizeof(int)));
   CKC(cudaMemset(st.counters, 0, 4 * sizeof(unsigned long long)));
+  CKC(cudaMemset(st.ucount, 0, (size_t)h->units * 4 * sizeof(unsigned long long)));
   CKC(cudaGetLastError());
   CKC(cudaDeviceSynchronize());
   h->t_layer.assign(c.n_layers, -1);
@@ -1041,8 +1046,10 @@ int crystalkv_get_counters(crystalkv_t* h, uint64_t* entries_attended, uint64_t*
   ON_DEVICE(h);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (int jr = join_side(h, s)) return jr;
-  unsigned long long v[4];
-  CK(h, cudaMemcpyAsync(v, h->st.counters, sizeof(v), cudaMemcpyDeviceToHost, s));
+  unsigned long long v[3];
+  sum_counters_kernel<<<1, 1024, 0, s>>>(h->st, h->units, h->io_sum);
+  CK(h, cudaGetLastError());
+  CK(h, cudaMemcpyAsync(v, h->io_sum, sizeof(v), cudaMemcpyDeviceToHost, s));
   CK(h, cudaStreamSynchronize(s));
   if (entries_attended) *entries_attended = v[0];
   if (hits) *hits = v[1];

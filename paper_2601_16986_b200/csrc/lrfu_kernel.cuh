@@ -19,7 +19,6 @@
 // 36.3 us instead of 34.4; for heads of 1025 entries 17 us instead of 11.)
 #pragma once
 #include <atomic>
-#include <cstddef>
 
 #include "evict.cuh"
 #include "lrfu_launch.cuh"
@@ -31,11 +30,13 @@ namespace ckv {
 template <int NTH>
 struct LrfuSmem {
   NucleusSmem<NTH> nu;
-  int amin[NTH / 32 * 4];
-  int ev[320];
+  alignas(16) uint32_t least[NTH / 32][4];   // per warp: the lowest (CRF_temp, tau, position) and its list position
+  int hits[NTH / 32];
   int is_last;
 };
-static_assert(offsetof(LrfuSmem<NT>, ev) >= (MAX_UNITS_PER_CALL + 1) * sizeof(int), "the planner's list of lengths reuses this memory");
+static_assert(sizeof(LrfuSmem<NT>) >= (MAX_UNITS_PER_CALL + 1) * sizeof(int), "the planner's list of lengths reuses this memory");
+// Dynamic shared memory: pbar of the head's entries, and once they are dead the scratch of evict_many and of the planner.
+static_assert(PL_SCRATCH >= 300, "evict_many wants 300 ints");
 
 // Loads the compiler must leave where they are written: the kernel is bound by the latency of
 // its dependent global reads (several microseconds each while the attention kernel saturates
@@ -56,161 +57,153 @@ __device__ __forceinline__ float4 ld_f32x4(const float* p) {
   return v;
 }
 
+// A row's logits of G query heads (only those are loaded).
+template <int G>
+struct Row {
+  float4 a;
+  float b[G > 4 ? G - 4 : 1];
+  __device__ __forceinline__ void load(const float* r) {
+    a = ld_f32x4(r);
+    if (G == 5) {
+      b[0] = ld_f32(r + 4);
+    } else if (G > 5) {
+      const float4 t = ld_f32x4(r + 4);
+      const float v[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+      for (int g = 4; g < G; ++g) b[g - 4] = v[g - 4];
+    }
+  }
+  // Mean over the query heads of 2^(s_g log2(e) - m_g) / l_g  (invl: 1 / (l_g G)).  One rounding in the exponent: against
+  // 64 bits pbar is off by no more than with expf(s_g - m_g ln 2), which rounds the reference point as well.
+  __device__ __forceinline__ float pbar(const float (&m)[G], const float (&invl)[G]) const {
+    const float v[4] = {a.x, a.y, a.z, a.w};
+    float pm = 0.f;
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+      pm = fmaf(ex2(fmaf(g < 4 ? v[g < 4 ? g : 0] : b[g < 4 ? 0 : g - 4], 1.44269504088896340736f, -m[g])), invl[g], pm);
+    return pm;
+  }
+};
+
 // What the kernel requests before it knows the head's length.
 template <int G>
 struct Front {
-  float4 ra[FRONT], rb[FRONT];   // logit rows of this thread's first entries (index clamped to p.front)
+  Row<G> row[FRONT];             // logit rows of this thread's first entries (index clamped to p.front)
   float m[G], l[G];              // merged reference point (log2 domain) and normaliser per query head
   int budget;
 };
 
-// EPT > 0: every thread keeps the pbar of its entries tid, tid + NTH, ... (at most EPT) in
-// registers; EPT == 0: they live in the global scratch and any n is allowed.  A single leaver's place
-// becomes the head's hole; returns the number of entries that leave, of which the caller removes more
-// than one.
-template <int G, int NTH, int EPT>
-__device__ int lrfu_unit(const DecodeParams& p, int u, int uid, int seq, int n, LrfuSmem<NTH>& sh, const Front<G>& fr) {
-  constexpr int R = EPT > 0 ? EPT : 1;
+// The head's length after this launch, the page that backs its next entry, and the count of finished heads.
+// The layer's plan names pieces by (head, j of k), so it stays correct while heads grow or
+// shrink a little; a head whose group count has drifted from the planned one by an eighth (at
+// least two) marks it stale, and the head that is counted last (its CTA then knows every head's new
+// length) writes a new one.  In steady state (one entry arrives, one leaves) nothing is written.
+// One thread calls it, once it is known how many entries leave and all threads have read n_cur: the count's release
+// makes the length visible to whoever acquires the last count.
+__device__ __forceinline__ bool settle_length(const DecodeParams& p, int uid, int seq, int n, int leave, int g_plan) {
+  const State& st = p.st;
+  int n_new = n - leave;
+  if (n <= 1) n_new = n;                                     // (a head without entries stays as it is)
+  else if (leave == 0) n_new = keep_all(st, uid, seq, n);
+  else st.n_cur[uid] = n_new;
+  const int g_new = (n_new + 1 + GRP - 1) / GRP;
+  if (abs(g_new - g_plan) >= max(2, g_plan >> 3)) atomicOr(p.done_ctr + 1, 1);
+  int done;
+  asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;\n" : "=r"(done) : "l"(p.done_ctr) : "memory");
+  if (done != (int)gridDim.x - 1) return false;
+  *p.done_ctr = 0;
+  return atomicExch(p.done_ctr + 1, 0) != 0;   // stale?
+}
+
+// Algorithm 1 for a head of n entries, n > 1.  pbar lives in shared memory (room for npb entries) or, for longer heads,
+// in the global scratch.  Returns the number of entries that leave; a single leaver's place becomes the head's
+// hole, more than one are left to the caller.  The head's length is settled on the way (sh.is_last).
+template <int G, int NTH>
+__device__ __forceinline__ int lrfu_unit(const DecodeParams& p, int u, int uid, int seq, int n, int g_plan, float* s_pb, int npb,
+                                         LrfuSmem<NTH>& sh, const Front<G>& fr) {
   constexpr int WARPS = NTH / 32;
   const State& st = p.st;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const size_t mb = (size_t)uid * st.cap;
   const float* S = p.sc.logits + (size_t)u * p.sc.cap_s * QH;
-  float* pbar = p.sc.pbar + (size_t)u * p.sc.cap_s;
-  const int kmax = EPT > 0 ? (n + NTH - 1) / NTH : 0;
+  float* pb = n <= npb ? s_pb : p.sc.pbar + (size_t)u * p.sc.cap_s;
 
-  // ---- step 1: pbar_i = mean_g exp(s_gi - m_g) / l_g
-  float mx[G], invl[G];
+  // ---- step 1: pbar_i = mean_g exp(s_gi - m_g) / l_g, and the histogram of its mass
+  const int base = nucleus_base<NTH>(n);
+  {
+    float m[G], invl[G];
 #pragma unroll
-  for (int g = 0; g < G; ++g) {
-    mx[g] = fr.m[g] * 0.693147180559945309f;   // log2 domain -> natural log
-    invl[g] = 1.0f / (fr.l[g] * (float)G);
+    for (int g = 0; g < G; ++g) {
+      m[g] = fr.m[g];
+      invl[g] = 1.0f / (fr.l[g] * (float)G);
+    }
+    auto put = [&](int i, float pm) {
+      pb[i] = pm;
+      nucleus_add<NTH>(sh.nu, base, pm);
+    };
+    const int nf = min(n, min(FRONT * NTH, p.front));   // entries whose rows were requested up front
+#pragma unroll
+    for (int k = 0; k < FRONT; ++k)
+      if (tid + k * NTH < nf) put(tid + k * NTH, fr.row[k].pbar(m, invl));
+    // the others in batches whose rows are requested together (clamped index, no branch): while the
+    // attention kernel saturates HBM every dependent round of loads costs this CTA microseconds
+    constexpr int BR = G <= 5 ? 5 : 4;
+#pragma unroll 1
+    for (int i0 = nf; i0 < n; i0 += BR * NTH) {
+      Row<G> row[BR];
+#pragma unroll
+      for (int j = 0; j < BR; ++j) row[j].load(S + (size_t)min(i0 + j * NTH + tid, n - 1) * QH);
+#pragma unroll
+      for (int j = 0; j < BR; ++j)
+        if (i0 + j * NTH + tid < n) put(i0 + j * NTH + tid, row[j].pbar(m, invl));
+    }
   }
-  auto pbar_of = [&](int i) {
-    const float4 a = *reinterpret_cast<const float4*>(S + (size_t)i * QH);
-    float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (G > 4) b = *reinterpret_cast<const float4*>(S + (size_t)i * QH + 4);
-    const float sv[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-    float pm = 0.f;
+  // stored state of this thread's first entries: the reads complete under the threshold search
+  int pos_r[FRONT], tau_r[FRONT];
+  float crf_r[FRONT], dec_r[FRONT];
 #pragma unroll
-    for (int g = 0; g < G; ++g) pm = fmaf(expf(sv[g] - mx[g]), invl[g], pm);
-    return pm;
-  };
-  float pmr[R];
-  // Once every thread holds its entries' pbar in registers the logit rows are dead: their L2 lines are
-  // dropped instead of being written back to DRAM later.  Four 32-byte rows share a 128-byte line;
-  // units start on line boundaries (cap_s is a multiple of four).
-  // The barrier takes a value computed from every pbar, so no thread passes it with a row
-  // load still in flight.
-  auto drop_rows = [&]() {
-    int unordered = 0;
-#pragma unroll
-    for (int k = 0; k < R; ++k) unordered |= (pmr[k] != pmr[k]);
-    (void)__syncthreads_or(unordered);
-    if ((tid & 3) == 0) {
-#pragma unroll
-      for (int k = 0; k < R; ++k) {
-        const int i = tid + k * NTH;
-        if (i < n) asm volatile("discard.global.L2 [%0], 128;\n" ::"l"(S + (size_t)i * QH) : "memory");
-      }
-    }
-  };
-  // stored state of this thread's entries, requested as soon as the logits are consumed so that
-  // the reads complete under the threshold search (EPT == FRONT only)
-  int pos_r[R], tau_r[R];
-  float crf_r[R];
-  if (EPT == FRONT) {
-#pragma unroll
-    for (int k = 0; k < R; ++k) {
-      const float sv[8] = {fr.ra[k].x, fr.ra[k].y, fr.ra[k].z, fr.ra[k].w, fr.rb[k].x, fr.rb[k].y, fr.rb[k].z, fr.rb[k].w};
-      float pm = 0.f;
-#pragma unroll
-      for (int g = 0; g < G; ++g) pm = fmaf(expf(sv[g] - mx[g]), invl[g], pm);
-      pmr[k] = (tid + k * NTH < n) ? pm : 0.f;
-    }
-#pragma unroll
-    for (int k = 0; k < R; ++k) {
-      const size_t i = mb + min(tid + k * NTH, n - 1);
-      pos_r[k] = ld_i32(st.meta_pos + i);
-      tau_r[k] = ld_i32(st.meta_tau + i);
-      crf_r[k] = ld_f32(st.meta_crf + i);
-    }
-    drop_rows();
-  } else if (EPT > 0) {
-    // batches of BR entries whose rows are requested together (clamped index, no branch): while the
-    // attention kernel saturates HBM every dependent round of loads costs this CTA microseconds, so
-    // a batch is as large as the registers allow (only the G logits of a row are loaded)
-    constexpr int BR = G <= 5 ? 8 : 4;
-#pragma unroll
-    for (int k = 0; k < R; ++k) pmr[k] = 0.f;
-#pragma unroll
-    for (int k0 = 0; k0 < R; k0 += BR) {
-      if (k0 < kmax) {
-        float4 ra[BR];
-        float rb[BR][4];
-#pragma unroll
-        for (int j = 0; j < BR; ++j) {
-          const int i = min(tid + (k0 + j) * NTH, n - 1);
-          ra[j] = ld_f32x4(S + (size_t)i * QH);
-          if (G == 5) {
-            rb[j][0] = ld_f32(S + (size_t)i * QH + 4);
-          } else if (G > 5) {
-            const float4 t4 = ld_f32x4(S + (size_t)i * QH + 4);
-            rb[j][0] = t4.x; rb[j][1] = t4.y; rb[j][2] = t4.z; rb[j][3] = t4.w;
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < BR; ++j) {
-          if (k0 + j < R) {
-            const float sv[8] = {ra[j].x, ra[j].y, ra[j].z, ra[j].w, G > 4 ? rb[j][0] : 0.f, G > 5 ? rb[j][1] : 0.f,
-                                 G > 6 ? rb[j][2] : 0.f, G > 7 ? rb[j][3] : 0.f};
-            float pm = 0.f;
-#pragma unroll
-            for (int g = 0; g < G; ++g) pm = fmaf(expf(sv[g] - mx[g]), invl[g], pm);
-            pmr[k0 + j] = (tid + (k0 + j) * NTH < n) ? pm : 0.f;
-          }
-        }
-      }
-    }
-    drop_rows();
-  } else {
-    for (int i = tid; i < n; i += NTH) pbar[i] = pbar_of(i);
+  for (int k = 0; k < FRONT; ++k) {
+    const size_t i = mb + min(tid + k * NTH, n - 1);
+    tau_r[k] = ld_i32(st.meta_tau + i);
+    crf_r[k] = ld_f32(st.meta_crf + i);
+    pos_r[k] = ld_i32(st.meta_pos + i);
   }
-  const Nucleus nu = nucleus_search<NTH>(n, p.top_p, sh.nu, st.errword, [&](auto f) {
-    if (EPT > 0) {
+  __syncthreads();
+  // The logit rows are dead (every thread has used what it loaded): their L2 lines are dropped instead of being written
+  // back to DRAM later.  Four 32-byte rows share a 128-byte line; units start on line boundaries (cap_s is a
+  // multiple of four).
+  for (int x = tid; x * 4 < n; x += NTH) asm volatile("discard.global.L2 [%0], 128;\n" ::"l"(S + (size_t)x * (4 * QH)) : "memory");
+  const Nucleus nu = nucleus_find<NTH>(
+      base, p.top_p, sh.nu, st.errword,
+      [&](auto f) {
+#pragma unroll 4
+        for (int i = tid; i < n; i += NTH) f(pb[i]);
+      },
+      [&] {
 #pragma unroll
-      for (int k = 0; k < R; ++k)
-        if (k < kmax && tid + k * NTH < n) f(pmr[k]);
-    } else {
-      for (int i = tid; i < n; i += NTH) f(pbar[i]);
-    }
-  });
+        for (int k = 0; k < FRONT; ++k) dec_r[k] = __ldg(st.tab + (p.t - min(tau_r[k], p.t)));
+      });
   const uint32_t theta = nu.theta;
-  const int cnt_eq = nu.cnt_eq;
-  const unsigned long long A = nu.A, Pthr = nu.Pthr;
-  const bool found_all = nu.found;
-  if (EPT > 0 && cnt_eq > 1) {   // the rank among equal keys needs every entry's key: spill them
-#pragma unroll
-    for (int k = 0; k < R; ++k)
-      if (k < kmax && tid + k * NTH < n) pbar[tid + k * NTH] = pmr[k];
-  }
-  if (cnt_eq > 1) __syncthreads();
   const unsigned long long w_theta = mass_of(__uint_as_float(theta));
 
   // ---- steps 2-3: CRF/tau update; step 4 candidates
   // step 4 runs once the head is evict_every entries over its budget, and then for all of them
   const int k_evict = (n - fr.budget >= p.evict_every) ? n - fr.budget : 0;
+  // (every thread has read the head's length: the count's round trip runs under the update)
+  if (tid == NTH - 32) sh.is_last = settle_length(p, uid, seq, n, min(k_evict, n - 1), g_plan);
   uint32_t bk0 = 0xffffffffu, bk1 = 0xffffffffu, bk2 = 0xffffffffu;
   int bidx = -1, nhit = 0;
-  auto update = [&](int i, float pm, int pos_i, int tau, float crf, float dec) {
+  auto update = [&](int i, int pos_i, int tau, float crf, float dec) {
+    const float pm = pb[i];
     const uint32_t key = __float_as_uint(pm);
-    bool hit = key > theta && found_all;
-    if (key == theta && found_all) {
+    bool hit = key > theta && nu.found;
+    if (key == theta && nu.found) {
       unsigned long long before = 0;
-      if (cnt_eq > 1)
+      if (nu.cnt_eq > 1)
+#pragma unroll 1
         for (int x = 0; x < n; ++x)
-          before += (__float_as_uint(__ldcg(pbar + x)) == theta) && (st.meta_pos[mb + x] < pos_i);
-      hit = (A + before * w_theta) < Pthr;
+          before += (__float_as_uint(pb[x]) == theta) && (st.meta_pos[mb + x] < pos_i);
+      hit = (nu.A + before * w_theta) < nu.Pthr;
     }
     float ct = __fmul_rn(dec, crf);
     if (hit) {
@@ -220,94 +213,76 @@ __device__ int lrfu_unit(const DecodeParams& p, int u, int uid, int seq, int n, 
       st.meta_tau[mb + i] = tau;
       ++nhit;
     }
-    if (k_evict == 1) {
-      const uint32_t c0 = __float_as_uint(ct), c1 = (uint32_t)tau, c2 = (uint32_t)pos_i;
-      const bool less = (c0 != bk0) ? (c0 < bk0) : ((c1 != bk1) ? (c1 < bk1) : (c2 < bk2));
-      if (less) { bk0 = c0; bk1 = c1; bk2 = c2; bidx = i; }
-    }
+    const uint32_t c0 = __float_as_uint(ct), c1 = (uint32_t)tau, c2 = (uint32_t)pos_i;
+    const bool less = (c0 != bk0) ? (c0 < bk0) : ((c1 != bk1) ? (c1 < bk1) : (c2 < bk2));
+    if (less) { bk0 = c0; bk1 = c1; bk2 = c2; bidx = i; }
   };
-  if (EPT > 8) {   // many entries per thread: eight at a time, their stored state requested together
 #pragma unroll
-    for (int k0 = 0; k0 < R; k0 += 8) {
-      if (k0 < kmax) {
-        int pos4[8], tau4[8];
-        float crf4[8], dec4[8];
+  for (int k = 0; k < FRONT; ++k)
+    if (tid + k * NTH < n) update(tid + k * NTH, pos_r[k], tau_r[k], crf_r[k], dec_r[k]);
+#pragma unroll 1
+  for (int i0 = FRONT * NTH; i0 < n; i0 += FRONT * NTH) {   // a long head: the next FRONT entries of every thread
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const size_t i = mb + min(tid + (k0 + j) * NTH, n - 1);
-          pos4[j] = ld_i32(st.meta_pos + i);
-          tau4[j] = ld_i32(st.meta_tau + i);
-          crf4[j] = ld_f32(st.meta_crf + i);
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) dec4[j] = __ldg(st.tab + (p.t - min(tau4[j], p.t)));
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int i = tid + (k0 + j) * NTH;
-          if (k0 + j < R && i < n) update(i, pmr[k0 + j < R ? k0 + j : 0], pos4[j], tau4[j], crf4[j], dec4[j]);
-        }
-      }
+    for (int k = 0; k < FRONT; ++k) {
+      const size_t i = mb + min(i0 + tid + k * NTH, n - 1);
+      tau_r[k] = ld_i32(st.meta_tau + i);
+      crf_r[k] = ld_f32(st.meta_crf + i);
+      pos_r[k] = ld_i32(st.meta_pos + i);
     }
-  } else if (EPT > 0) {
-    float dec_r[R];
 #pragma unroll
-    for (int k = 0; k < R; ++k) dec_r[k] = __ldg(st.tab + (p.t - min(tau_r[k], p.t)));
+    for (int k = 0; k < FRONT; ++k) dec_r[k] = __ldg(st.tab + (p.t - min(tau_r[k], p.t)));
 #pragma unroll
-    for (int k = 0; k < R; ++k) {
-      const int i = tid + k * NTH;
-      if (i < n) update(i, pmr[k], pos_r[k], tau_r[k], crf_r[k], dec_r[k]);
-    }
-  } else {
-    for (int i = tid; i < n; i += NTH) {
-      const int tau = st.meta_tau[mb + i];
-      update(i, pbar[i], st.meta_pos[mb + i], tau, st.meta_crf[mb + i], st.tab[p.t - tau]);
-    }
+    for (int k = 0; k < FRONT; ++k)
+      if (i0 + tid + k * NTH < n) update(i0 + tid + k * NTH, pos_r[k], tau_r[k], crf_r[k], dec_r[k]);
   }
-  nhit = warp_sum_i(nhit);
-  if (lane == 0 && nhit) atomicAdd(&st.counters[1], (unsigned long long)nhit);
-  // the lowest (CRF_temp, tau, pos) of the warp, then (the first warp) of all warps
+  // the lowest (CRF_temp, tau, position) of a warp's lanes, word by word (positions are unique)
   auto least = [&]() {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const uint32_t o0 = __shfl_xor_sync(0xffffffffu, bk0, o), o1 = __shfl_xor_sync(0xffffffffu, bk1, o),
-                     o2 = __shfl_xor_sync(0xffffffffu, bk2, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bidx, o);
-      const bool less = (o0 != bk0) ? (o0 < bk0) : ((o1 != bk1) ? (o1 < bk1) : (o2 < bk2));
-      if (less) { bk0 = o0; bk1 = o1; bk2 = o2; bidx = oi; }
-    }
+    const uint32_t m0 = __reduce_min_sync(0xffffffffu, bk0);
+    const uint32_t m1 = __reduce_min_sync(0xffffffffu, bk0 == m0 ? bk1 : 0xffffffffu);
+    const uint32_t m2 = __reduce_min_sync(0xffffffffu, bk0 == m0 && bk1 == m1 ? bk2 : 0xffffffffu);
+    bidx = (int)__reduce_min_sync(0xffffffffu, bk0 == m0 && bk1 == m1 && bk2 == m2 ? (uint32_t)bidx : 0xffffffffu);
+    bk0 = m0; bk1 = m1; bk2 = m2;
   };
-  if (k_evict == 1) {
+  least();
+  nhit = __reduce_add_sync(0xffffffffu, nhit);
+  if (lane == 0) {
+    *reinterpret_cast<uint4*>(sh.least[w]) = make_uint4(bk0, bk1, bk2, (uint32_t)bidx);
+    sh.hits[w] = nhit;
+  }
+  __syncthreads();
+  if (w == 0) {
+    const uint4 a = *reinterpret_cast<const uint4*>(sh.least[min(lane, WARPS - 1)]);
+    bk0 = a.x; bk1 = a.y; bk2 = a.z; bidx = (int)a.w;
     least();
-    if (lane == 0) { sh.amin[w * 4] = (int)bk0; sh.amin[w * 4 + 1] = (int)bk1; sh.amin[w * 4 + 2] = (int)bk2; sh.amin[w * 4 + 3] = bidx; }
-    __syncthreads();
-    if (w == 0) {
-      const int* a = sh.amin + min(lane, WARPS - 1) * 4;
-      bk0 = (uint32_t)a[0]; bk1 = (uint32_t)a[1]; bk2 = (uint32_t)a[2]; bidx = a[3];
-      least();
-      if (lane == 0) {
-        // the leaving entry's place is where the next arriving token is written
-        st.hole[uid] = bidx;
-        st.n_cur[uid] = n - 1;
-        atomicAdd(&st.counters[2], 1ull);
-      }
+    nhit = __reduce_add_sync(0xffffffffu, lane < WARPS ? sh.hits[min(lane, WARPS - 1)] : 0);
+    if (lane == 0) {
+      if (k_evict == 1) st.hole[uid] = bidx;   // the leaving entry's place is where the next arriving token is written
+      count_unit(st, uid, n, nhit, k_evict == 1 ? 1 : 0);
     }
   }
   return k_evict;
 }
 
-// LONG: heads of more than ten entries per thread have a path with seventeen in registers.
-template <int G, int NTH, bool LONG>
-__global__ void __maxnreg__(48) lrfu_kernel(const __grid_constant__ DecodeParams p) {
-  __shared__ LrfuSmem<NTH> sh;
+template <int G, int NTH>
+__global__ void __maxnreg__(48) lrfu_kernel(const __grid_constant__ DecodeParams p, int npb) {
+  extern __shared__ __align__(16) float s_pb[];
+  __shared__ __align__(16) LrfuSmem<NTH> sh;
   const State& st = p.st;
   const int u = blockIdx.x, seq = u / st.H, head = u % st.H;
   const int uid = (seq * st.L + p.layer) * st.H + head;
   // one batch of requests: the length, the budget, the softmax reference, and the logit rows the
   // common path needs (requested for a full thread's worth, clamped to the expected length)
   const int n = ld_i32(st.n_cur + uid) + 1;
-  const int g_plan = threadIdx.x == 0 ? ld_i32(p.plan.gplan + u) : 0;   // used at the very end
-  int n_new = n;   // the head's length after this launch
+  const int g_plan = threadIdx.x == NTH - 32 ? ld_i32(p.plan.gplan + u) : 0;
+  bool settled = false;
   if (p.track) {
+    // the stored state is asked into L2: every round trip to DRAM costs microseconds beside a saturated HBM
+    for (int x = threadIdx.x; x * 32 < p.front; x += NTH) {
+      const size_t at = (size_t)uid * st.cap + x * 32;
+      asm volatile("prefetch.global.L2 [%0];\n" ::"l"(st.meta_tau + at));
+      asm volatile("prefetch.global.L2 [%0];\n" ::"l"(st.meta_crf + at));
+      asm volatile("prefetch.global.L2 [%0];\n" ::"l"(st.meta_pos + at));
+    }
     Front<G> fr;
     fr.budget = ld_i32(st.budget + uid);
 #pragma unroll
@@ -318,63 +293,36 @@ __global__ void __maxnreg__(48) lrfu_kernel(const __grid_constant__ DecodeParams
     {
       const float* S = p.sc.logits + (size_t)u * p.sc.cap_s * QH;
 #pragma unroll
-      for (int k = 0; k < FRONT; ++k) {
-        const int i = min((int)threadIdx.x + k * NTH, p.front - 1);
-        fr.ra[k] = ld_f32x4(S + (size_t)i * QH);
-        fr.rb[k] = (G > 4) ? ld_f32x4(S + (size_t)i * QH + 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int k = 0; k < FRONT; ++k) fr.row[k].load(S + (size_t)min((int)threadIdx.x + k * NTH, p.front - 1) * QH);
+    }
+    nucleus_clear<NTH>(sh.nu);
+    __syncthreads();
+    if (n > 1 && !(p.literal && n < fr.budget)) {   // (Algorithm 1's first line as printed: nothing runs below the budget)
+      int leave = lrfu_unit<G, NTH>(p, u, uid, seq, n, g_plan, s_pb, npb, sh, fr);
+      settled = true;
+      if (leave > 1) {
+        __syncthreads();   // every thread's CRFs are written, pbar is dead
+        if (leave > p.evict_every && threadIdx.x == 0) atomicOr(st.errword, ERR_OVER_EVICT);
+        leave = min(leave, n - 1);
+        evict_many<NTH>(st, uid, seq, n, leave, p.t, false, reinterpret_cast<int*>(s_pb), reinterpret_cast<int*>(p.sc.pbar + (size_t)u * p.sc.cap_s));
       }
     }
-    int leave = 0;
-    if (n > 1 && !(p.literal && n < fr.budget)) {   // (Algorithm 1's first line as printed: nothing runs below the budget)
-      if (n <= min(FRONT * NTH, p.front)) leave = lrfu_unit<G, NTH, FRONT>(p, u, uid, seq, n, sh, fr);
-      else if (NTH >= NT && n <= 10 * NTH) leave = lrfu_unit<G, NTH, NTH >= NT ? 10 : 0>(p, u, uid, seq, n, sh, fr);
-      else if (LONG && n <= 17 * NTH) leave = lrfu_unit<G, NTH, LONG ? 17 : 0>(p, u, uid, seq, n, sh, fr);
-      else leave = lrfu_unit<G, NTH, 0>(p, u, uid, seq, n, sh, fr);
-    }
-    if (leave > 1) {
-      __syncthreads();   // every thread's CRFs are written
-      if (leave > p.evict_every && threadIdx.x == 0) atomicOr(st.errword, ERR_OVER_EVICT);
-      leave = min(leave, n - 1);
-      evict_many<NTH>(st, uid, seq, n, leave, p.t, false, sh.ev, reinterpret_cast<int*>(p.sc.pbar + (size_t)u * p.sc.cap_s));
-    }
-    n_new = n - leave;
-    if (leave == 0 && n > 1 && threadIdx.x == 0) keep_all(st, uid, seq, n);
-  } else if (n > 1 && threadIdx.x == 0) {
-    keep_all(st, uid, seq, n);   // no Algorithm 1: the head keeps its new entry
   }
-  if (threadIdx.x == 0) {
-    if (n > 1) atomicAdd(&st.counters[0], (unsigned long long)n);
+  if (!settled && threadIdx.x == NTH - 32) {   // no Algorithm 1: the head keeps its new entry
+    if (n > 1) count_unit(st, uid, n, 0, 0);
     else atomicOr(st.errword, ERR_EMPTY);   // the head has no entries and no page: nothing was attended
-  }
-  // ---- The layer's plan names pieces by (head, j of k), so it stays correct while heads grow or
-  // shrink a little; a head whose group count has drifted from the planned one by an eighth (at
-  // least two) marks it stale, and the head that finishes last (its CTA then knows every head's new
-  // length) writes a new one.  In steady state (one entry arrives, one leaves) nothing is written.
-  // Thread 0 wrote the head's new length itself, so the release of its count makes that length
-  // visible to whoever acquires the last count.
-  if (threadIdx.x == 0) {
-    const int g_new = (n_new + 1 + GRP - 1) / GRP;
-    if (abs(g_new - g_plan) >= max(2, g_plan >> 3)) atomicOr(p.done_ctr + 1, 1);
-    int done;
-    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;\n" : "=r"(done) : "l"(p.done_ctr) : "memory");
-    int last = (done == (int)gridDim.x - 1);
-    if (last) {
-      *p.done_ctr = 0;
-      last = atomicExch(p.done_ctr + 1, 0);   // stale?
-    }
-    sh.is_last = last;
+    sh.is_last = settle_length(p, uid, seq, n, 0, g_plan);
   }
   __syncthreads();
   if (!sh.is_last) return;
   // The planner's list of lengths takes the place of this CTA's histogram or, where that is too small, a
-  // place of its own.  (Not the pbar area: a CTA counts itself as soon as its thread 0 is through, and its other
-  // warps may still be reading pbar then.)
+  // place of its own.  (Not the pbar scratch: other heads' CTAs may still be reading theirs.)
   write_plan<NTH>(st, p.plan, p.layer, p.plan_warps, p.plan_grid, p.cl,
-                  NTH >= NT ? reinterpret_cast<int*>(&sh) : p.plan_len, sh.ev);
+                  NTH >= NT ? reinterpret_cast<int*>(&sh) : p.plan_len, reinterpret_cast<int*>(s_pb));
 }
 
-template <int G, int NTH, bool LONG = false>
-cudaError_t launch_lrfu(const DecodeParams& p, int heads, cudaStream_t s) {
+template <int G, int NTH>
+cudaError_t launch_lrfu(const DecodeParams& p, int npb, int heads, cudaStream_t s) {
   // the same shared-memory carve-out as the attention kernel, so that CTAs of both can be
   // resident on one SM at the same time
   // (function attributes are kept per device)
@@ -384,12 +332,12 @@ cudaError_t launch_lrfu(const DecodeParams& p, int heads, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= MAX_DEVICES) return cudaErrorInvalidDevice;
   if (!prepared[dev].load(std::memory_order_acquire)) {
-    e = cudaFuncSetAttribute(lrfu_kernel<G, NTH, LONG>, cudaFuncAttributePreferredSharedMemoryCarveout,
+    e = cudaFuncSetAttribute(lrfu_kernel<G, NTH>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              (int)cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
     prepared[dev].store(true, std::memory_order_release);
   }
-  lrfu_kernel<G, NTH, LONG><<<heads, NTH, 0, s>>>(p);
+  lrfu_kernel<G, NTH><<<heads, NTH, std::max(npb, PL_SCRATCH) * sizeof(float), s>>>(p, npb);
   return cudaGetLastError();
 }
 

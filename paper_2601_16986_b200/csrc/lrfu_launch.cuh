@@ -8,35 +8,34 @@ namespace ckv {
 constexpr int MAX_DEVICES = 64;   // device ordinals this library keeps per-device state for
 constexpr int FRONT = 5;   // entries per thread whose logit rows are requested before n is known
 constexpr int LRFU_SMALL = 64;   // threads of the CTAs for short heads
-constexpr int LRFU_LARGE = 512;  // ... for long ones
 
 // Threads of a head's CTA.  hint: entries of a head in this step if all are alike (uniform), else about
 // the mean (crystalkv::entries; it follows heads that fill).
 //  * Heads of at most 5 x 64 entries take CTAs of two warps once there are more heads than SMs: six
 //    of them fit beside an attention CTA instead of two of eight warps, most of which idle in the
 //    block-wide steps.  128 sequences of 8 heads of 257 entries: 27.8 us a layer instead of 38.7.
-//  * Heads longer than 5 x 256 entries take CTAs of sixteen warps (one of which fits beside an attention
-//    CTA) while every head finds an SM of its own: half the rounds of loads per thread.  128 heads of
-//    1024 .. 3072 entries: 30.0 us a layer instead of 31.1; 64 heads of 4097: 33.1 instead of 34.3, no more
-//    than runs of one side differ by.
+//  * All other heads take CTAs of eight warps, two of which fit beside an attention CTA.  (Sixteen for heads of more than
+//    1280 entries make the kernel shorter and the layer longer, 64 heads of 4097 entries 33.0 us instead of 32.4,
+//    128 heads of 1024 .. 3072 entries 29.1 instead of 28.85: what counts is how hard a CTA presses on the attention
+//    warps of its SM.)
 inline int lrfu_threads(int U, int hint, bool uniform, int num_sms) {
-  if (uniform && hint <= FRONT * LRFU_SMALL && U > num_sms) return LRFU_SMALL;
-  return hint > FRONT * NT && U <= num_sms ? LRFU_LARGE : NT;
+  return uniform && hint <= FRONT * LRFU_SMALL && U > num_sms ? LRFU_SMALL : NT;
 }
 
-// Launches the kernel for `heads` heads of at most `most` entries; threads: LRFU_SMALL, NT or LRFU_LARGE.  Where no
-// head can hold more than ten entries per thread, CTAs of NT threads run an instantiation without the path for
-// seventeen, whose registers cost the others: 718 bytes of spill stores per thread in one, 256 in the other.
-cudaError_t lrfu_launch_small(int G, const DecodeParams& p, int heads, cudaStream_t s);
-cudaError_t lrfu_launch_large(int G, const DecodeParams& p, int heads, cudaStream_t s);
-cudaError_t lrfu_launch_mid(int G, const DecodeParams& p, int heads, cudaStream_t s);
-cudaError_t lrfu_launch_1_4(int G, const DecodeParams& p, int heads, cudaStream_t s);
-cudaError_t lrfu_launch_5_8(int G, const DecodeParams& p, int heads, cudaStream_t s);
-inline cudaError_t lrfu_launch(int threads, int most, int G, const DecodeParams& p, int heads, cudaStream_t s) {
-  if (threads == LRFU_SMALL) return lrfu_launch_small(G, p, heads, s);
-  if (threads == LRFU_LARGE) return lrfu_launch_large(G, p, heads, s);
-  if (most <= 10 * NT) return lrfu_launch_mid(G, p, heads, s);
-  return G <= 4 ? lrfu_launch_1_4(G, p, heads, s) : lrfu_launch_5_8(G, p, heads, s);
+// Entries whose pbar a CTA keeps in shared memory (longer heads use the global scratch).  Beside an attention CTA an SM
+// has 34 KB left: room for six CTAs of LRFU_SMALL, two of NT, or one of NT where heads are long and find an SM each or so few
+// that two launches' heads do.
+constexpr int PBAR_TWO = 1792, PBAR_ONE = 5632;
+inline int pbar_room(int threads, int U, int hint, int num_sms) {
+  if (threads == LRFU_SMALL) return FRONT * LRFU_SMALL;
+  return 2 * U <= num_sms || (hint > PBAR_TWO && U <= num_sms) ? PBAR_ONE : PBAR_TWO;
+}
+
+// Launches the kernel for `heads` heads; threads: LRFU_SMALL or NT; npb: entries whose pbar fits shared memory.
+cudaError_t lrfu_launch_small(int G, const DecodeParams& p, int npb, int heads, cudaStream_t s);
+cudaError_t lrfu_launch_mid(int G, const DecodeParams& p, int npb, int heads, cudaStream_t s);
+inline cudaError_t lrfu_launch(int threads, int npb, int G, const DecodeParams& p, int heads, cudaStream_t s) {
+  return threads == LRFU_SMALL ? lrfu_launch_small(G, p, npb, heads, s) : lrfu_launch_mid(G, p, npb, heads, s);
 }
 
 }  // namespace ckv

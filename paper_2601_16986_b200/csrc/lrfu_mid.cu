@@ -1,18 +1,18 @@
-// Algorithm 1's kernel with CTAs of eight warps for heads of at most ten entries per thread, every group size.
+// Algorithm 1's kernel with CTAs of eight warps, every group size.
 #include "lrfu_kernel.cuh"
 
 namespace ckv {
 
-cudaError_t lrfu_launch_mid(int G, const DecodeParams& p, int heads, cudaStream_t s) {
+cudaError_t lrfu_launch_mid(int G, const DecodeParams& p, int npb, int heads, cudaStream_t s) {
   switch (G) {
-    case 1: return launch_lrfu<1, NT>(p, heads, s);
-    case 2: return launch_lrfu<2, NT>(p, heads, s);
-    case 3: return launch_lrfu<3, NT>(p, heads, s);
-    case 4: return launch_lrfu<4, NT>(p, heads, s);
-    case 5: return launch_lrfu<5, NT>(p, heads, s);
-    case 6: return launch_lrfu<6, NT>(p, heads, s);
-    case 7: return launch_lrfu<7, NT>(p, heads, s);
-    case 8: return launch_lrfu<8, NT>(p, heads, s);
+    case 1: return launch_lrfu<1, NT>(p, npb, heads, s);
+    case 2: return launch_lrfu<2, NT>(p, npb, heads, s);
+    case 3: return launch_lrfu<3, NT>(p, npb, heads, s);
+    case 4: return launch_lrfu<4, NT>(p, npb, heads, s);
+    case 5: return launch_lrfu<5, NT>(p, npb, heads, s);
+    case 6: return launch_lrfu<6, NT>(p, npb, heads, s);
+    case 7: return launch_lrfu<7, NT>(p, npb, heads, s);
+    case 8: return launch_lrfu<8, NT>(p, npb, heads, s);
   }
   return cudaErrorInvalidValue;
 }

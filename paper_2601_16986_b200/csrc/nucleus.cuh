@@ -28,7 +28,8 @@ struct NucleusSmem {
   unsigned hist_lo[fine_bins(NTH)];   // per-bin mass, low bits of every term
   unsigned hist_hi[fine_bins(NTH)];   // per-bin mass, the bits above
   unsigned long long redu[NTH / 32 + 1];
-  unsigned cand[MAX_CAND];       // keys of the entries in the threshold's bin
+  unsigned long long cmass[MAX_CAND];   // masses and keys of the entries in the threshold's bin
+  unsigned cand[MAX_CAND];
   unsigned long long A_theta;    // fast path result: mass strictly above the threshold key
   unsigned theta;                //                   the threshold key
   int cnt_theta;                 //                   entries that carry it
@@ -57,25 +58,32 @@ __device__ __forceinline__ unsigned long long warp_suffix(unsigned long long v, 
   return v;
 }
 
-// All NTH threads of a CTA call it; `each(f)` calls f(pbar) for every entry the calling thread owns.
-template <int NTH, class Each>
-__device__ __forceinline__ Nucleus nucleus_search(int n, float top_p, NucleusSmem<NTH>& sh, int* errword, Each each) {
-  constexpr int WARPS = NTH / 32, FINE_BINS = fine_bins(NTH), FINE_SHIFT = fine_shift(NTH);
+// The search in three parts, all called by the NTH threads of a CTA: nucleus_clear, a barrier, nucleus_add for every
+// entry (a histogram of mass in fine bins around 1/n: bin(key) = clamp((key >> FINE_SHIFT) - base, 0, FINE_BINS - 1),
+// monotone in key), a barrier, nucleus_find.
+template <int NTH>
+__device__ __forceinline__ void nucleus_clear(NucleusSmem<NTH>& sh) {
+  for (int b = threadIdx.x; b < fine_bins(NTH); b += NTH) { sh.hist_lo[b] = 0u; sh.hist_hi[b] = 0u; }
+  if (threadIdx.x == 0) { sh.star = -1; sh.ncand = 0; sh.theta = 0xffffffffu; sh.cnt_theta = 0; }
+}
+template <int NTH>
+__device__ __forceinline__ int nucleus_base(int n) {
+  return (int)(__float_as_uint(1.0f / (256.0f * (float)n)) >> fine_shift(NTH));
+}
+template <int NTH>
+__device__ __forceinline__ void nucleus_add(NucleusSmem<NTH>& sh, int base, float pm) {
+  const unsigned long long m = mass_of(pm);
+  const int b = min(fine_bins(NTH) - 1, max(0, (int)(__float_as_uint(pm) >> fine_shift(NTH)) - base));
+  atomicAdd(&sh.hist_lo[b], (unsigned)m & LOW_MASK);
+  atomicAdd(&sh.hist_hi[b], (unsigned)(m >> LOW_BITS));
+}
+
+// `each(f)` calls f(pbar) for every entry the calling thread owns; `mid()` is called once on the way, where the search
+// waits for other threads (a caller's loads that should be under way by then).
+template <int NTH, class Each, class Mid>
+__device__ __forceinline__ Nucleus nucleus_find(int base, float top_p, NucleusSmem<NTH>& sh, int* errword, Each each, Mid mid) {
+  constexpr int WARPS = NTH / 32, FINE_BINS = fine_bins(NTH);
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  // ---- fast path, pass over all entries: histogram of mass in fine bins around 1/n
-  //      bin(key) = clamp((key >> FINE_SHIFT) - base, 0, FINE_BINS - 1), monotone in key
-  const int fbase = (int)(__float_as_uint(1.0f / (256.0f * (float)n)) >> FINE_SHIFT);
-  auto fbin = [&](uint32_t key) { return min(FINE_BINS - 1, max(0, (int)(key >> FINE_SHIFT) - fbase)); };
-  for (int b = tid; b < FINE_BINS; b += NTH) { sh.hist_lo[b] = 0u; sh.hist_hi[b] = 0u; }
-  if (tid == 0) { sh.star = -1; sh.ncand = 0; sh.theta = 0xffffffffu; sh.cnt_theta = 0; }
-  __syncthreads();
-  each([&](float pm) {
-    const unsigned long long m = mass_of(pm);
-    const int b = fbin(__float_as_uint(pm));
-    atomicAdd(&sh.hist_lo[b], (unsigned)m & LOW_MASK);
-    atomicAdd(&sh.hist_hi[b], (unsigned)(m >> LOW_BITS));
-  });
-  __syncthreads();
   Nucleus r;
   unsigned long long W = 0, A = 0;   // A: mass of keys strictly above the threshold's bin / prefix range
   {
@@ -89,6 +97,7 @@ __device__ __forceinline__ Nucleus nucleus_search(int n, float top_p, NucleusSme
     const unsigned long long suf = warp_suffix(loc, lane);
     if (lane == 0) sh.redu[w] = suf;
     __syncthreads();
+    mid();
     unsigned long long above = 0;
     for (int x = 0; x < WARPS; ++x) {
       const unsigned long long v = sh.redu[x];
@@ -117,9 +126,9 @@ __device__ __forceinline__ Nucleus nucleus_search(int n, float top_p, NucleusSme
     A = sh.redu[WARPS];
     each([&](float pm) {
       const uint32_t key = __float_as_uint(pm);
-      if (fbin(key) == bstar) {
+      if ((int)(key >> fine_shift(NTH)) == bstar + base) {   // (no bin at the window's ends)
         const int x = atomicAdd(&sh.ncand, 1);
-        if (x < MAX_CAND) sh.cand[x] = key;
+        if (x < MAX_CAND) { sh.cand[x] = key; sh.cmass[x] = mass_of(pm); }
       }
     });
     __syncthreads();
@@ -128,12 +137,13 @@ __device__ __forceinline__ Nucleus nucleus_search(int n, float top_p, NucleusSme
       // candidate x carries the threshold iff  A + mass(keys above it) < Pthr <= that + mass(keys equal)
       if (tid < c) {
         const uint32_t mine = sh.cand[tid];
-        const unsigned long long wm = mass_of(__uint_as_float(mine));
+        const unsigned long long wm = sh.cmass[tid];
         unsigned long long gt = 0;
         int eqc = 0;
+#pragma unroll 4
         for (int x = 0; x < c; ++x) {
           const uint32_t kx = sh.cand[x];
-          if (kx > mine) gt += mass_of(__uint_as_float(kx));
+          if (kx > mine) gt += sh.cmass[x];
           eqc += (kx == mine);
         }
         if (A + gt < Pthr && Pthr <= A + gt + (unsigned long long)eqc * wm) {
@@ -221,6 +231,16 @@ __device__ __forceinline__ Nucleus nucleus_search(int n, float top_p, NucleusSme
   r.A = A;
   r.found = found;
   return r;
+}
+
+template <int NTH, class Each>
+__device__ __forceinline__ Nucleus nucleus_search(int n, float top_p, NucleusSmem<NTH>& sh, int* errword, Each each) {
+  const int base = nucleus_base<NTH>(n);
+  nucleus_clear<NTH>(sh);
+  __syncthreads();
+  each([&](float pm) { nucleus_add<NTH>(sh, base, pm); });
+  __syncthreads();
+  return nucleus_find<NTH>(base, top_p, sh, errword, each, [] {});
 }
 
 }  // namespace ckv
