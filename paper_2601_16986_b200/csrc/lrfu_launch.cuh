@@ -23,12 +23,12 @@ inline int lrfu_threads(int U, int hint, bool uniform, int num_sms) {
 }
 
 // Entries whose pbar a CTA keeps in shared memory (longer heads use the global scratch).  Beside an attention CTA an SM
-// has 34 KB left: room for six CTAs of LRFU_SMALL, two of NT, or one of NT where heads are long and find an SM each or so few
-// that two launches' heads do.
-constexpr int PBAR_TWO = 1792, PBAR_ONE = 5632;
+// has 34 KB left: room for six CTAs of LRFU_SMALL, two of NT, or one of NT for long heads that find an SM each.
+// (One of NT for few heads of any length: 64 heads of 128 .. 2000 entries 11.55 us a layer instead of 11.3.)
+constexpr int PBAR_TWO = 1856, PBAR_ONE = 5632;
 inline int pbar_room(int threads, int U, int hint, int num_sms) {
   if (threads == LRFU_SMALL) return FRONT * LRFU_SMALL;
-  return 2 * U <= num_sms || (hint > PBAR_TWO && U <= num_sms) ? PBAR_ONE : PBAR_TWO;
+  return hint > PBAR_TWO && U <= num_sms ? PBAR_ONE : PBAR_TWO;
 }
 
 // Launches the kernel for `heads` heads; threads: LRFU_SMALL or NT; npb: entries whose pbar fits shared memory.

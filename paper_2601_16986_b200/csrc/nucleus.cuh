@@ -2,7 +2,7 @@
 // above it (and the earliest of those equal to it) are the smallest descending-pbar prefix whose
 // exclusive mass is below p.  One histogram of 1024 bins of 1/64 octave around 1/n (256 of 1/16 for
 // CTAs of 64 threads) locates theta's bin, the few entries of that bin are ranked against one
-// another; a bin outside the window or with more than 64 entries falls back to four 8-bit radix
+// another; a bin outside the window or with more entries than max_cand() falls back to four 8-bit radix
 // passes over all bits.
 // The mass walk uses 2^-40 fixed-point integers so it is exact and order independent; the
 // threshold is relative to the integer total, so a common factor on pbar changes nothing.
@@ -12,7 +12,6 @@
 namespace ckv {
 
 constexpr float MASS_ONE = 1099511627776.0f;   // 2^40
-constexpr int MAX_CAND = 64;
 // A bin's mass is summed in two 32-bit words: the low LOW_BITS of every term, and the bits above.  The masses
 // of a head add up to 2^40, so the upper word stays below 2^31, and the lower one holds 2^22 terms (with 16
 // low bits it wrapped at 2^16 terms of one bin: a prompt of 100 003 equal keys lost 351 hits).
@@ -22,14 +21,16 @@ constexpr unsigned LOW_MASK = (1u << LOW_BITS) - 1u;
 // fine bins of CTAs of NTH threads and the key bits below a bin: 16 octaves in all
 __host__ __device__ constexpr int fine_bins(int nth) { return nth < 256 ? 256 : 1024; }
 __host__ __device__ constexpr int fine_shift(int nth) { return nth < 256 ? 19 : 17; }
+// Entries of the threshold's bin that are ranked against one another; they take the histogram's place (12 bytes each).
+// (With room for 64 a head of 5000 entries fell back to the radix passes in some steps and not in others, a prompt of
+// 9350 tokens in all: 18 of its selection's 40 us.)
+__host__ __device__ constexpr int max_cand(int nth) { return nth < 256 ? 128 : 512; }
 
 template <int NTH>
 struct NucleusSmem {
-  unsigned hist_lo[fine_bins(NTH)];   // per-bin mass, low bits of every term
+  alignas(8) unsigned hist_lo[fine_bins(NTH)];   // per-bin mass, low bits of every term
   unsigned hist_hi[fine_bins(NTH)];   // per-bin mass, the bits above
   unsigned long long redu[NTH / 32 + 1];
-  unsigned long long cmass[MAX_CAND];   // masses and keys of the entries in the threshold's bin
-  unsigned cand[MAX_CAND];
   unsigned long long A_theta;    // fast path result: mass strictly above the threshold key
   unsigned theta;                //                   the threshold key
   int cnt_theta;                 //                   entries that carry it
@@ -124,26 +125,30 @@ __device__ __forceinline__ Nucleus nucleus_find(int base, float top_p, NucleusSm
   const int bstar = sh.star;
   if (bstar > 0 && bstar < FINE_BINS - 1) {   // inside the window: rank the bin's entries exactly
     A = sh.redu[WARPS];
+    constexpr int MAX_CAND = max_cand(NTH);
+    static_assert(MAX_CAND * 12 <= FINE_BINS * 8, "the candidates take the histogram's place");
+    unsigned long long* cmass = reinterpret_cast<unsigned long long*>(sh.hist_lo);   // (every thread has read its bins)
+    unsigned* cand = reinterpret_cast<unsigned*>(cmass + MAX_CAND);
     each([&](float pm) {
       const uint32_t key = __float_as_uint(pm);
       if ((int)(key >> fine_shift(NTH)) == bstar + base) {   // (no bin at the window's ends)
         const int x = atomicAdd(&sh.ncand, 1);
-        if (x < MAX_CAND) { sh.cand[x] = key; sh.cmass[x] = mass_of(pm); }
+        if (x < MAX_CAND) { cand[x] = key; cmass[x] = mass_of(pm); }
       }
     });
     __syncthreads();
     const int c = sh.ncand;
     if (c <= MAX_CAND) {
       // candidate x carries the threshold iff  A + mass(keys above it) < Pthr <= that + mass(keys equal)
-      if (tid < c) {
-        const uint32_t mine = sh.cand[tid];
-        const unsigned long long wm = sh.cmass[tid];
+      for (int y = tid; y < c; y += NTH) {
+        const uint32_t mine = cand[y];
+        const unsigned long long wm = cmass[y];
         unsigned long long gt = 0;
         int eqc = 0;
 #pragma unroll 4
         for (int x = 0; x < c; ++x) {
-          const uint32_t kx = sh.cand[x];
-          if (kx > mine) gt += sh.cmass[x];
+          const uint32_t kx = cand[x];
+          if (kx > mine) gt += cmass[x];
           eqc += (kx == mine);
         }
         if (A + gt < Pthr && Pthr <= A + gt + (unsigned long long)eqc * wm) {

@@ -197,6 +197,7 @@ __global__ void __launch_bounds__(SEL_NT) prefill_select_kernel(State st, Scratc
   const int uid = (seq * st.L + layer) * st.H + head;
   const size_t mb = (size_t)uid * st.cap;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  nucleus_clear<SEL_NT>(s_nu);   // (a barrier follows long before the histogram is filled)
   const int B = fixed_budget > 0 ? fixed_budget : st.budget[uid];
   if (fixed_budget > 0 && tid == 0) st.budget[uid] = fixed_budget;
   const float* S = sc.logits + (size_t)u * sc.cap_s * QH;
@@ -215,7 +216,7 @@ __global__ void __launch_bounds__(SEL_NT) prefill_select_kernel(State st, Scratc
     float s0 = 0.f, s1 = 0.f;
     if (g < G) {
       const float m0 = s_m[g], m1 = s_m[min(g + 1, G - 1)];
-#pragma unroll 4
+#pragma unroll 8
       for (int i = t; i < P; i += 256) {
         const float2 x = *reinterpret_cast<const float2*>(S + (size_t)i * QH + g);
         s0 += ex2(x.x * to_log2 - m0);
@@ -241,33 +242,39 @@ __global__ void __launch_bounds__(SEL_NT) prefill_select_kernel(State st, Scratc
     il[g] = g < G ? s_il[g] : 0.f;
   }
   float* pb = in_smem ? s_pbar : sc.pbar + (size_t)u * sc.cap_s;
-  for (int i0 = tid; i0 < P; i0 += 2 * SEL_NT) {   // two rows requested together
-    float4 ra[2], rb[2];
+  const bool track = !(literal && P < B);   // Algorithm 1's first line as printed: nothing runs below the budget
+  const int base = nucleus_base<SEL_NT>(P);
+  constexpr int BR = 3;                       // rows requested together
+  for (int i0 = tid; i0 < P; i0 += BR * SEL_NT) {
+    float4 ra[BR], rb[BR];
 #pragma unroll
-    for (int x = 0; x < 2; ++x) {
+    for (int x = 0; x < BR; ++x) {
       const float* r = S + (size_t)min(i0 + x * SEL_NT, P - 1) * QH;
       ra[x] = *reinterpret_cast<const float4*>(r);
       rb[x] = G > 4 ? *reinterpret_cast<const float4*>(r + 4) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 #pragma unroll
-    for (int x = 0; x < 2; ++x) {
+    for (int x = 0; x < BR; ++x) {
       const int i = i0 + x * SEL_NT;
       const float sv[8] = {ra[x].x, ra[x].y, ra[x].z, ra[x].w, rb[x].x, rb[x].y, rb[x].z, rb[x].w};
       float pm = 0.f;
 #pragma unroll
       for (int g = 0; g < QH; ++g)
         if (g < G) pm = fmaf(expf(sv[g] - mx[g]), il[g], pm);
-      if (i < P) pb[i] = pm;
+      if (i < P) {
+        pb[i] = pm;
+        if (track) nucleus_add<SEL_NT>(s_nu, base, pm);
+      }
     }
   }
-  const bool track = !(literal && P < B);   // Algorithm 1's first line as printed: nothing runs below the budget
+  __syncthreads();
   Nucleus nu{};
   nu.theta = 0xffffffffu;
   if (track)
-    nu = nucleus_search<SEL_NT>(P, top_p, s_nu, st.errword, [&](auto f) {
+    nu = nucleus_find<SEL_NT>(base, top_p, s_nu, st.errword, [&](auto f) {
+#pragma unroll 4
       for (int i = tid; i < P; i += SEL_NT) f(pb[i]);
-    });
-  __syncthreads();
+    }, [] {});
   // ---- hits and survivors: every thread owns a run of consecutive tokens (of odd length: the
   // threads of a warp then read different banks)
   const int per = ((P + SEL_NT - 1) / SEL_NT) | 1, lo = min(P, tid * per), hi = min(P, lo + per);
