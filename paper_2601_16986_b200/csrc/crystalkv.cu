@@ -283,13 +283,18 @@ int find_clusters(crystalkv_t* h) {
 // has one layer (a launch that cannot start early gains the whole difference).  Below that the wider merge and the
 // launch of clusters cost more than they save.  us a layer, shared and not: 48 layers of 32 heads, four CTAs: of 29
 // groups 7.9 and 6.65, of 41 groups 8.1 and 8.8, of 65 groups 9.9 and 11.2; 64 heads, two CTAs: of 41 groups 9.3 and
-// 9.3, of 57 groups 10.5 and 12.0, of 257 groups 32.9 and 32.0.  One layer of 2 heads, four CTAs: of 29 groups 10.8
-// and 10.95, of 33 groups 10.7 and 11.4.
+// 9.3, of 57 groups 10.5 and 12.0.  One layer of 2 heads, four CTAs: of 29 groups 10.8 and 10.95, of 33 groups 10.7 and
+// 11.4.
+// Longer heads of one length gain from two CTAs where one could not hold them without pieces twice as long
+// as a chain-bound launch takes: their other choice is more than eight pieces and a merge through global memory
+// at the end of the launch (4 us for 64 heads of 257 groups).  64 heads of 193 groups 24.3 and 28.2, of 257 32.5 and
+// 32.4; 72 of 257 34.9 and 39.7; 60 of 257 30.7 and 30.9; 48 of 257 27.3 and 27.8.
 int share_heads(crystalkv_t* h, int entries) {
   const int g = (entries + GRP - 1) / GRP, alone = (g + NW - 1) / NW;
   for (int cl = MAX_CLUSTER; cl > 1; cl /= 2) {
     const int per = (g + NW * cl - 1) / (NW * cl);
-    if (h->share_ok[cl] && per <= GLAT && alone - per >= (h->cfg.n_layers > 1 ? 4 : 3)) return cl;
+    const bool chain = per <= GLAT, merge = cl == 2 && h->uniform && 10 * h->U >= 3 * h->num_sms && alone > 2 * GLAT && per <= 2 * GLAT;
+    if (h->share_ok[cl] && (chain || merge) && alone - per >= (h->cfg.n_layers > 1 ? 4 : 3)) return cl;
   }
   return 1;
 }
