@@ -659,7 +659,7 @@ static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, cons
   p.logits = h->sc_logits[0];
   p.ml = h->sc_partials[0];
   p.hits = reinterpret_cast<unsigned*>(h->sc_pbar[0]);
-  p.H = c.n_kv_heads; p.G = h->G; p.U = h->U; p.P = P;
+  p.H = c.n_kv_heads; p.G = h->G; p.U = h->U; p.P = P; p.layer = layer;
   p.Ps = (P + 7) / 8 * 8;   // rows of logits start on 32-byte sectors
   p.words = (P + 31) / 32;
   p.scale = c.sm_scale;
@@ -669,6 +669,9 @@ static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, cons
                                             std::min<long long>((long long)h->pmax * (16 + h->G * HD) / 16, h->cap_s / p.words));
   const size_t sm = (size_t)P * sizeof(float) <= WIN_SMEM ? (size_t)P * sizeof(float) : 0;
   const auto attn = out ? window_attn_kernel<true> : window_attn_kernel<false>;
+  const bool small = P <= WH_SMALL;
+  const auto hits = small ? window_hits_kernel<64> : window_hits_kernel<NT>;
+  const int plan_grid = h->plan_grid(layer);
   CK(h, cudaFuncSetAttribute(attn, cudaFuncAttributeMaxDynamicSharedMemorySize, WA_SMEM));
   const size_t qn = (size_t)c.batch * c.n_q_heads * HD;
   for (int w0 = 0; w0 < W; w0 += p.W) {
@@ -676,15 +679,18 @@ static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, cons
     p.t0 = P - W + w0;
     p.q = q + (size_t)w0 * qn * sizeof(__nv_bfloat16);
     p.out = out ? out + (size_t)w0 * qn : nullptr;
-    attn<<<dim3((p.W * p.G + WA_ROWS - 1) / WA_ROWS, h->U), WA_WARPS * 32, WA_SMEM, s>>>(p);
+    const bool last = w0 + p.W == W;
+    p.store = last;
+    attn<<<dim3((p.W * p.G + WA_ROWS - 1) / WA_ROWS, h->U), WA_WARPS * 32, WA_SMEM, s>>>(h->st, p);
     CK(h, cudaGetLastError());
-    window_hits_kernel<<<dim3(p.W, h->U), NT, sm, s>>>(h->st, p, layer, c.top_p, c.literal_return, sm > 0);
+    // (the plan is for the heads' lengths after the last query's step 4, known from their budgets)
+    hits<<<dim3(p.W, h->U + 1), small ? 64 : NT, std::max(sm, PL_SCRATCH * sizeof(int)), s>>>(h->st, p, c.top_p, c.literal_return, sm > 0, h->plans[layer],
+                                                          last ? plan_grid : 0, h->cl[layer], c.evict_every, h->plan_len);
     CK(h, cudaGetLastError());
-    window_apply_kernel<<<h->U, NT, 0, s>>>(h->st, p, layer, w0 + p.W == W, c.evict_every, reinterpret_cast<int*>(h->sc_pbar[1]),
-                                            h->cap_s);
+    window_apply_kernel<<<h->U, NT, 0, s>>>(h->st, p, last, c.evict_every, reinterpret_cast<int*>(h->sc_pbar[1]), h->cap_s);
     CK(h, cudaGetLastError());
   }
-  return replan(h, layer, 1, s);
+  return CRYSTALKV_OK;
 }
 
 // Prompt insertion and the Algorithm 1 passes that seed CRF/tau: one pass with the last query
@@ -740,13 +746,15 @@ static int prefill_common(crystalkv_t* h, int layer, const void* k, const void* 
     fill_layer_budget_kernel<<<(h->U + NT - 1) / NT, NT, 0, s>>>(h->st, layer, ratio_budget(c, P));
     CK(h, cudaGetLastError());
   }
-  // the whole prompt is stored; in full-cache mode the first step's plan is written beside the copy
-  prefill_take_kernel<<<h->U, NT, 0, s>>>(h->st, layer, P);
+  // the whole prompt is stored; in full-cache mode the first step's plan is written beside the copy, and a replayed window
+  // copies the rows in its attention kernel where that reads all of them (it has outputs)
+  prefill_take_kernel<<<h->U, NT, 0, s>>>(h->st, layer, P, W > 0 ? 1 : 0);
   CK(h, cudaGetLastError());
-  prefill_rows_kernel<<<1 + h->U * per_head, NT, 0, s>>>(h->st, h->plans[layer], layer, kb, vb, P,
-                                                         W > 0 ? ROWS_ALL_POS : ROWS_ALL_LAST, per_head,
-                                                         evict ? 0 : plan_grid * NW, plan_grid, h->cl[layer]);
-  CK(h, cudaGetLastError());
+  if (!evict || !out_window) {
+    prefill_rows_kernel<<<1 + h->U * per_head, NT, 0, s>>>(h->st, h->plans[layer], layer, kb, vb, P, W > 0 ? ROWS_ALL : ROWS_ALL_LAST,
+                                                           per_head, evict ? 0 : plan_grid * NW, plan_grid, h->cl[layer]);
+    CK(h, cudaGetLastError());
+  }
   if (evict) {
     rc = replay_window(h, layer, kb, vb, static_cast<const unsigned char*>(q), P, W, static_cast<__nv_bfloat16*>(out_window), s);
     if (rc) return rc;

@@ -113,20 +113,22 @@ __host__ __device__ __forceinline__ int run_warp(const Placement& p, int s, int 
 }
 
 // Called by all NTH threads of one CTA.  `gs` is memory for U + 1 ints, `red` shared memory for 320.
-// The plan is for a decode step: every head one entry longer than now.
+// The plan is for a decode step: every head one entry longer than now, or, with shrink > 0, than once the heads that are
+// `shrink` or more entries over their budgets have come down to them.
 // A function of its own: inlined at the end of the LRFU kernel (48 registers) its counts and placement cost the
 // kernel's common path registers.  14B shape with unequal budgets 27.95 us a layer instead of 28.1, 8B shape 29.0
 // instead of 30.1, 64 heads of 4097 entries 31.5 instead of 32.9.  The kernels that call it take the state as a
 // __grid_constant__, so that its address is passed without a copy on the stack.
 template <int NTH = NT>
 __device__ __noinline__ void write_plan(const State& st, const Plan& pl, int layer, int nWarps, int grid, int cl,
-                                        int* gs, int* red) {
+                                        int* gs, int* red, int shrink = 0) {
   const int U = st.batch * st.H, tid = threadIdx.x, lane = tid & 31;
   // ---- groups per head
   int mine = 0, gmax = 0;
   for (int u = tid; u < U; u += NTH) {
     const int uid = ((u / st.H) * st.L + layer) * st.H + (u % st.H);
-    const int n = __ldcg(st.n_cur + uid);   // (other CTAs of the calling kernel may just have written it: not from L1)
+    int n = __ldcg(st.n_cur + uid);   // (other CTAs of the calling kernel may just have written it: not from L1)
+    if (shrink > 0 && n > 1 && n - __ldcg(st.budget + uid) >= shrink) n = max(1, __ldcg(st.budget + uid));
     // A head without entries (an insertion that found no pages, a head that is yet to be imported) has no page
     // to read: it gets no pieces.  The LRFU kernel flags it when a step meets it.
     const int g = n > 0 ? (n + 1 + GRP - 1) / GRP : 0;

@@ -323,16 +323,25 @@ __global__ void __launch_bounds__(SEL_NT) prefill_select_kernel(State st, Scratc
 }
 
 // A prompt that is kept as it is: the pages that back list positions 0 .. P (the P entries and the
-// place of the next arrival), one CTA per head.
-__global__ void __launch_bounds__(NT) prefill_take_kernel(State st, int layer, int P) {
+// place of the next arrival), one CTA per head.  meta: the entries' stored state as well, tau = the token's own arrival
+// time (its queries are replayed).
+__global__ void __launch_bounds__(NT) prefill_take_kernel(State st, int layer, int P, int meta) {
   __shared__ int s_top;
-  const int u = blockIdx.x, seq = u / st.H;
-  take_pages(st, (seq * st.L + layer) * st.H + u % st.H, seq, P / GRP + 1, P, NT, &s_top);
+  const int u = blockIdx.x, seq = u / st.H, uid = (seq * st.L + layer) * st.H + u % st.H;
+  if (meta) {
+    const size_t mb = (size_t)uid * st.cap;
+    for (int i = threadIdx.x; i < P; i += NT) {
+      st.meta_pos[mb + i] = i;
+      st.meta_tau[mb + i] = i;
+      st.meta_crf[mb + i] = 0.0f;
+    }
+  }
+  take_pages(st, uid, seq, P / GRP + 1, P, NT, &s_top);
 }
 
 constexpr int ROWS_SURVIVORS = 0;   // entries are listed in the metadata (their token positions)
 constexpr int ROWS_ALL_LAST = 1;    // entry i is token i: metadata written here, tau = P - 1
-constexpr int ROWS_ALL_POS = 2;     // ... tau = i, the token's own arrival time (its queries are replayed)
+constexpr int ROWS_ALL = 2;         // ... metadata written before
 
 // The rows of a layer's entries into their pages.  k, v: [batch][P][H][128].  CTA 0 writes the
 // layer's launch plan meanwhile (plan_warps > 0); the others, `per_head` for every head, copy a
@@ -364,9 +373,9 @@ __global__ void __launch_bounds__(NT) prefill_rows_kernel(const __grid_constant_
     int tok = i;
     if (mode == ROWS_SURVIVORS) {
       tok = min(max(st.meta_pos[mb + i], 0), P - 1);
-    } else if (lane < cnt) {
+    } else if (mode == ROWS_ALL_LAST && lane < cnt) {
       st.meta_pos[mb + i] = i;
-      st.meta_tau[mb + i] = mode == ROWS_ALL_POS ? i : P - 1;
+      st.meta_tau[mb + i] = P - 1;
       st.meta_crf[mb + i] = 0.0f;
     }
     unsigned char* dst = poolseq + (size_t)page * PAGE_BYTES;

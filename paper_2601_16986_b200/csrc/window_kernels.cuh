@@ -8,6 +8,7 @@
 #include "attn_kernel.cuh"
 #include "evict.cuh"
 #include "nucleus.cuh"
+#include "plan.cuh"
 
 namespace ckv {
 
@@ -17,6 +18,7 @@ constexpr int WA_KEYS = 64;                   // keys per tile
 constexpr int WA_TILE = WA_KEYS * ROW_BYTES;  // bytes of a K (or V) tile
 constexpr int WA_SMEM = 4 * WA_TILE;          // K and V, two stages
 constexpr int WIN_SMEM = 32 * 1024;           // pbar of up to this many bytes stays in shared memory
+constexpr int WH_SMALL = 1280;                // entries up to which window_hits_kernel takes CTAs of two warps
 
 struct WindowParams {
   const unsigned char* k;      // [batch][P][H][128]
@@ -28,6 +30,7 @@ struct WindowParams {
   unsigned* hits;              // [U][W][words] hit bits, bit i % 32 of word i / 32
   int H, G, U, P, Ps, words;
   int W, t0;                   // queries of this launch, time of the first
+  int layer, store;            // store: the prompt's rows go to the heads' pages (the launch with the last query)
   float scale, scale_log2;
 };
 
@@ -41,9 +44,12 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
 // decode kernel) and the logits written.  Keys on the MMA N dimension, rows on M; a row's channels
 // are contracted in the order in which 16-byte pieces of it load (lane tig: pieces tig, tig + 4, ..),
 // which makes every K fragment one 16-byte shared load.  Q, S and O live in registers, K and V tiles
-// of 64 keys in two cp.async stages; three CTAs fit an SM.
+// of 64 keys in two cp.async stages; three CTAs fit an SM.  (Two CTAs of five warps for 160 rows, without idle rows but with
+// ten warps an SM instead of twelve: 92 us instead of 82.)
+// The tiles are also what the heads' pages are filled from (store): the CTAs of a head take its tiles in turn, a tile that
+// only the last one sees in full falls to that one.  (A copy kernel of its own read the prompt again: 20 us.)
 template <bool OUT>
-__global__ void __launch_bounds__(WA_WARPS * 32, 3) window_attn_kernel(const WindowParams p) {
+__global__ void __launch_bounds__(WA_WARPS * 32, 3) window_attn_kernel(const __grid_constant__ State st, const WindowParams p) {
   extern __shared__ __align__(1024) unsigned char smem[];
   const int u = blockIdx.y, seq = u / p.H, head = u % p.H;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, gid = lane >> 2, tig = lane & 3;
@@ -52,7 +58,8 @@ __global__ void __launch_bounds__(WA_WARPS * 32, 3) window_attn_kernel(const Win
   const bool va = ra < R, vb = rb < R;
   const int wa = min(ra, R - 1) / p.G, ga = min(ra, R - 1) % p.G, wb = min(rb, R - 1) / p.G, gb = min(rb, R - 1) % p.G;
   const int ta = p.t0 + wa, tb = p.t0 + wb;                 // times: keys 0 .. t take part
-  const int n_keys = p.t0 + min(R - 1, r_lo + WA_ROWS - 1) / p.G + 1;   // the block's last query sees these
+  auto keys_of = [&](int b) { return p.t0 + min(R - 1, (b + 1) * WA_ROWS - 1) / p.G + 1; };   // block b's last query sees these
+  const int n_keys = keys_of(blockIdx.x);
   const int ntiles = (n_keys + WA_KEYS - 1) / WA_KEYS;
   const size_t qstride = (size_t)p.U * p.G * ROW_BYTES;     // one query of the window to the next
   uint32_t qa[8][4];
@@ -92,6 +99,8 @@ __global__ void __launch_bounds__(WA_WARPS * 32, 3) window_attn_kernel(const Win
   float ma = -INFINITY, mb = -INFINITY, la = 0.f, lb = 0.f;
   float* lga = p.logits + (((size_t)u * p.W + wa) * p.G + ga) * p.Ps + 2 * tig;
   float* lgb = p.logits + (((size_t)u * p.W + wb) * p.G + gb) * p.Ps + 2 * tig;
+  const int uid = (seq * st.L + p.layer) * st.H + head;
+  const bool store = OUT && p.store && st.n_cur[uid] == p.P;   // (a head that found no pages stays empty)
   fetch(0, 0);
 #pragma unroll 1
   for (int tile = 0; tile < ntiles; ++tile) {
@@ -104,6 +113,21 @@ __global__ void __launch_bounds__(WA_WARPS * 32, 3) window_attn_kernel(const Win
     }
     __syncthreads();
     const uint32_t ks = s0 + stage * 2 * WA_TILE, vs = ks + WA_TILE;
+    if (store) {
+      const int last = gridDim.x - 1, turn = tile % gridDim.x;
+      if (blockIdx.x == ((tile + 1) * WA_KEYS <= keys_of(turn) ? turn : last)) {   // an entry per warp and turn, lane c its chunk c
+        const int* pt = st.ptab + (size_t)uid * st.capg + tile * (WA_KEYS / GRP);
+        unsigned char* pool = st.pool + (size_t)seq * st.pages_per_seq * PAGE_BYTES;
+#pragma unroll 4
+        for (int key = w; key < min(WA_KEYS, p.P - tile * WA_KEYS); key += WA_WARPS) {
+          const uint32_t at = lane < 16 ? ks + key * ROW_BYTES + ((lane ^ ((key & 1) << 2)) << 4)
+                                        : vs + key * ROW_BYTES + (((lane - 16) ^ (key & 7)) << 4);
+          uint4 x;
+          asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];\n" : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w) : "r"(at));
+          *reinterpret_cast<uint4*>(pool + (size_t)__ldg(pt + key / GRP) * PAGE_BYTES + chunk_offset(key & (GRP - 1), lane)) = x;
+        }
+      }
+    }
     float s[8][4];
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
@@ -204,20 +228,30 @@ __global__ void __launch_bounds__(WA_WARPS * 32, 3) window_attn_kernel(const Win
 }
 
 // The hit bits of one (query, head): Algorithm 1 step 1 with the query of time t over its t + 1 entries.
-// grid: (W, U).  Bound: latency of a dozen block-wide steps; eight CTAs fit an SM.
+// grid: (W, U + 1); one CTA of the last row writes the layer's launch plan meanwhile.
+// Bound: issue slots (some hundred instructions per warp beside those per entry) and the latency of a dozen block-wide
+// steps: short prompts take CTAs of two warps (WH_SMALL).
 // pbar lives in shared memory or, for long prompts, in the place of the first query head's logits.
-__global__ void __launch_bounds__(NT) window_hits_kernel(State st, const WindowParams p, int layer, float top_p, int literal,
-                                                         int in_smem) {
-  extern __shared__ float s_pbar[];
-  __shared__ NucleusSmem<NT> s_nu;
-  __shared__ int s_cnt[NW];
+template <int NTH>
+__global__ void __launch_bounds__(NTH) window_hits_kernel(const __grid_constant__ State st, const WindowParams p, float top_p, int literal,
+                                                          int in_smem, const __grid_constant__ Plan plan, int plan_grid, int plan_cl,
+                                                          int shrink, int* plan_len) {
+  constexpr int WARPS = NTH / 32;
+  extern __shared__ __align__(16) float s_pbar[];   // (the planner's scratch in its CTA)
+  __shared__ NucleusSmem<NTH> s_nu;
+  __shared__ int s_cnt[WARPS];
   const int u = blockIdx.y, q = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  if (u == p.U) {
+    if (q == 0 && plan_grid > 0)
+      write_plan<NTH>(st, plan, p.layer, plan_grid * NW, plan_grid, plan_cl, plan_len, reinterpret_cast<int*>(s_pbar), shrink);
+    return;
+  }
   const int n = p.t0 + q + 1;
   unsigned* bits = p.hits + ((size_t)u * p.W + q) * p.words;
   if (literal) {   // Algorithm 1's first line as printed: nothing runs below the budget
-    const int uid = ((u / st.H) * st.L + layer) * st.H + u % st.H;
+    const int uid = ((u / st.H) * st.L + p.layer) * st.H + u % st.H;
     if (n < st.budget[uid]) {
-      for (int x = tid; x < p.words; x += NT) bits[x] = 0u;
+      for (int x = tid; x < p.words; x += NTH) bits[x] = 0u;
       return;
     }
   }
@@ -230,22 +264,36 @@ __global__ void __launch_bounds__(NT) window_hits_kernel(State st, const WindowP
     mx[g] = g < p.G ? ml[g] * 0.693147180559945309f : 0.f;   // log2 domain -> natural log
     il[g] = g < p.G ? 1.0f / (ml[8 + g] * (float)p.G) : 0.f;
   }
-  for (int i = tid; i < n; i += NT) {
-    float sv[QH];
+  const int base = nucleus_base<NTH>(n);
+  nucleus_clear<NTH>(s_nu);
+  __syncthreads();
+  constexpr int BR = 4;   // entries requested together
+  for (int i0 = tid; i0 < n; i0 += BR * NTH) {
+    float sv[BR][QH];
 #pragma unroll
-    for (int g = 0; g < QH; ++g) sv[g] = g < p.G ? S[(size_t)g * p.Ps + i] : 0.f;
-    float pm = 0.f;
+    for (int x = 0; x < BR; ++x)
 #pragma unroll
-    for (int g = 0; g < QH; ++g)
-      if (g < p.G) pm = fmaf(expf(sv[g] - mx[g]), il[g], pm);
-    pb[i] = pm;
+      for (int g = 0; g < QH; ++g) sv[x][g] = g < p.G ? S[(size_t)g * p.Ps + min(i0 + x * NTH, n - 1)] : 0.f;
+#pragma unroll
+    for (int x = 0; x < BR; ++x) {
+      float pm = 0.f;
+#pragma unroll
+      for (int g = 0; g < QH; ++g)
+        if (g < p.G) pm = fmaf(expf(sv[x][g] - mx[g]), il[g], pm);
+      if (i0 + x * NTH < n) {
+        pb[i0 + x * NTH] = pm;   // (in the place of its own logit, which has been read)
+        nucleus_add<NTH>(s_nu, base, pm);
+      }
+    }
   }
-  const Nucleus nu = nucleus_search<NT>(n, top_p, s_nu, st.errword, [&](auto f) {
-    for (int i = tid; i < n; i += NT) f(pb[i]);
-  });
+  __syncthreads();
+  const Nucleus nu = nucleus_find<NTH>(base, top_p, s_nu, st.errword, [&](auto f) {
+#pragma unroll 4
+    for (int i = tid; i < n; i += NTH) f(pb[i]);
+  }, [] {});
   const unsigned long long w_theta = mass_of(__uint_as_float(nu.theta));
   int eq_before = 0;   // entries of earlier rounds that carry the threshold's value
-  for (int i0 = 0; i0 < n; i0 += NT) {   // (uniform: a round may hold a barrier)
+  for (int i0 = 0; i0 < n; i0 += NTH) {   // (uniform: a round may hold a barrier)
     const int i = i0 + tid;
     const uint32_t key = i < n ? __float_as_uint(pb[i]) : 0u;
     bool hit = i < n && nu.found && key > nu.theta;
@@ -255,7 +303,7 @@ __global__ void __launch_bounds__(NT) window_hits_kernel(State st, const WindowP
       if (lane == 0) s_cnt[w] = __popc(m);
       __syncthreads();
       int r = eq_before + __popc(m & ((1u << lane) - 1u));
-      for (int x = 0; x < NW; ++x) {
+      for (int x = 0; x < WARPS; ++x) {
         if (x < w) r += s_cnt[x];
         eq_before += s_cnt[x];
       }
@@ -273,30 +321,37 @@ __global__ void __launch_bounds__(NT) window_hits_kernel(State st, const WindowP
 // on; its CRF and tau only depend on its own hits), and after the last query (last != 0) step 4: the
 // head comes down to its budget.  One CTA per head; tmp: U x tmp_stride ints.
 // Bound: latency (W dependent multiply-adds per entry).
-__global__ void __launch_bounds__(NT) window_apply_kernel(State st, const WindowParams p, int layer, int last, int evict_every,
+__global__ void __launch_bounds__(NT) window_apply_kernel(State st, const WindowParams p, int last, int evict_every,
                                                           int* tmp, int tmp_stride) {
   __shared__ int sh[300];
   const int u = blockIdx.x, seq = u / st.H, tid = threadIdx.x;
-  const int uid = (seq * st.L + layer) * st.H + u % st.H;
+  const int uid = (seq * st.L + p.layer) * st.H + u % st.H;
   if (st.n_cur[uid] != p.P) return;   // the prompt found no pages: the head is empty
   const size_t mb = (size_t)uid * st.cap;
   int nhit = 0;
-  for (int i = tid; i < p.P; i += NT) {
-    float crf = st.meta_crf[mb + i];
-    int tau = st.meta_tau[mb + i];
-    const unsigned* bits = p.hits + (size_t)u * p.W * p.words + (i >> 5);
-#pragma unroll 8
-    for (int q = 0; q < p.W; ++q) {
-      const unsigned m = bits[(size_t)q * p.words];
-      const int t = p.t0 + q;
-      if (i <= t && ((m >> (i & 31)) & 1u)) {
-        crf = __fadd_rn(__fmul_rn(st.tab[t - tau], crf), 1.0f);
-        tau = t;
-        ++nhit;
+  const int lane = tid & 31;
+  for (int i0 = tid - lane; i0 < p.P; i0 += NT) {   // a warp takes 32 entries: one word of hit bits per query, a word per lane
+    const int i = i0 + lane, e = min(i, p.P - 1);
+    float crf = st.meta_crf[mb + e];
+    int tau = st.meta_tau[mb + e];
+    const unsigned* bits = p.hits + (size_t)u * p.W * p.words + (i0 >> 5);
+    for (int q0 = 0; q0 < p.W; q0 += 32) {
+      const unsigned mine = q0 + lane < p.W ? bits[(size_t)(q0 + lane) * p.words] : 0u;
+      const int qs = min(32, p.W - q0);
+      for (int q = 0; q < qs; ++q) {
+        const unsigned m = __shfl_sync(0xffffffffu, mine, q);
+        const int t = p.t0 + q0 + q;
+        if (i <= t && ((m >> lane) & 1u)) {   // (entries past the prompt's end are later than any query)
+          crf = __fadd_rn(__fmul_rn(__ldg(st.tab + (t - tau)), crf), 1.0f);
+          tau = t;
+          ++nhit;
+        }
       }
     }
-    st.meta_crf[mb + i] = crf;
-    st.meta_tau[mb + i] = tau;
+    if (i < p.P) {
+      st.meta_crf[mb + i] = crf;
+      st.meta_tau[mb + i] = tau;
+    }
   }
   nhit = warp_sum_i(nhit);
   if ((tid & 31) == 0 && nhit) atomicAdd(&st.counters[1], (unsigned long long)nhit);
