@@ -681,7 +681,7 @@ static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, cons
   const size_t sm = (size_t)P * sizeof(float) <= WIN_SMEM ? (size_t)P * sizeof(float) : 0;
   const auto attn = out ? window_attn_kernel<true> : window_attn_kernel<false>;
   const bool small = P <= WH_SMALL;
-  const auto hits = small ? window_hits_kernel<64> : window_hits_kernel<NT>;
+  const WindowHits hits = small ? window_hits_of<64>(h->G) : window_hits_of<NT>(h->G);
   const int plan_grid = h->plan_grid(layer);
   CK(h, cudaFuncSetAttribute(attn, cudaFuncAttributeMaxDynamicSharedMemorySize, WA_SMEM));
   const size_t qn = (size_t)c.batch * c.n_q_heads * HD;

@@ -1,7 +1,7 @@
 // Algorithm 1 for the heads of one layer, one CTA per head, from the scaled logits the
 // attention kernel left in the scratch (the cache itself is not read again):
 //   step 1   softmax weights per query head from the logits, the attention kernel's merged
-//            reference point and normaliser (accurate expf), group-mean probability pbar,
+//            reference point and normaliser, group-mean probability pbar,
 //            hit mask = smallest descending-pbar prefix whose exclusive mass is below p
 //            (equal pbar: ascending position; nucleus.cuh);
 //   step 2-3 hits: CRF <- lambda^(t - tau) CRF + 1, tau <- t; misses only get the decayed
@@ -14,9 +14,13 @@
 // a head's length has drifted from the one the current plan was made for.
 //
 // Bound: latency, a chain of a dozen block-wide steps and dependent reads beside an attention kernel
-// that saturates HBM.  (Sharing long heads among the CTAs of a cluster did not help: two to four
+// that saturates HBM; the attention warps of the same SM feel its issue slots and loads.  256 heads of 512 .. 1536
+// entries: 22 us beside the attention kernel and 26.6 us a layer; with pbar in register arrays, a spilling path for
+// heads of more than ten entries per thread, counters shared by all heads and the heads counted last, 28 and 27.3.
+// (Sharing long heads among the CTAs of a cluster did not help: two to four
 // CTAs for heads of 4097 entries took 48 us beside the attention kernel instead of 56, and the layer
-// 36.3 us instead of 34.4; for heads of 1025 entries 17 us instead of 11.)
+// 36.3 us instead of 34.4; for heads of 1025 entries 17 us instead of 11.  Nor did fewer instructions by predicated loads at
+// fixed offsets: 27.0 us a layer instead of 26.4.)
 #pragma once
 #include <atomic>
 
@@ -74,7 +78,8 @@ struct Row {
     }
   }
   // Mean over the query heads of 2^(s_g log2(e) - m_g) / l_g  (invl: 1 / (l_g G)).  One rounding in the exponent: against
-  // 64 bits pbar is off by no more than with expf(s_g - m_g ln 2), which rounds the reference point as well.
+  // 64 bits pbar is off by no more (6.0e-7 rms over logits of deviation 0.5 .. 8 and 1 .. 8 query heads) than with
+  // expf(s_g - m_g ln 2) (6.3e-7), which rounds the reference point as well.
   __device__ __forceinline__ float pbar(const float (&m)[G], const float (&invl)[G]) const {
     const float v[4] = {a.x, a.y, a.z, a.w};
     float pm = 0.f;

@@ -183,7 +183,8 @@ __device__ __forceinline__ bool take_pages(const State& st, int uid, int seq, in
 // fixed_budget > 0 sets the heads' budget first.
 // Bound: latency (a few block-wide steps over 36 bytes per token); 1024 threads keep a prompt of
 // 10 000 tokens at ten entries per thread, pbar in shared memory up to SEL_SMEM bytes.
-// 64 heads x 9350 tokens cut to 935: 40.7 us; the decode step's Algorithm 1 kernel with its radix
+// 64 heads x 9350 tokens cut to 935: 25.9 us (40.6 while the threshold search fell back to its radix passes);
+// the decode step's Algorithm 1 kernel with its radix
 // select over 96-bit keys in global memory took 286 us.  128 heads x 512 tokens: 10.9 us.
 __global__ void __launch_bounds__(SEL_NT) prefill_select_kernel(State st, Scratch sc, int layer, int P, int G, int chunks,
                                                                 float to_log2, float top_p, int evict_every, int literal,

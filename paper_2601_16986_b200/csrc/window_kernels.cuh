@@ -2,7 +2,8 @@
 // already stored.  Which entries a query hits depends on its scores alone, not on what earlier
 // queries of the window marked, so the window is one attention kernel over all (query, head) rows,
 // one threshold search per (head, query), and one kernel that walks an entry through its queries.
-// 128 heads x 1024 tokens, 32 queries of 5 heads: 83 + 49 + 21 us a layer (and 9 for the plan); a decode-step launch pair
+// 128 heads x 1024 tokens, 32 queries of 5 heads: 92 + 41 + 14 us a layer, the pages and the launch plan included (as kernels
+// of their own they took 20 and 9 us, the three others 83 + 49 + 21); a decode-step launch pair
 // per query, each reading the prompt's rows again, took 720 us.
 #pragma once
 #include "attn_kernel.cuh"
@@ -229,10 +230,11 @@ __global__ void __launch_bounds__(WA_WARPS * 32, 3) window_attn_kernel(const __g
 
 // The hit bits of one (query, head): Algorithm 1 step 1 with the query of time t over its t + 1 entries.
 // grid: (W, U + 1); one CTA of the last row writes the layer's launch plan meanwhile.
-// Bound: issue slots (some hundred instructions per warp beside those per entry) and the latency of a dozen block-wide
-// steps: short prompts take CTAs of two warps (WH_SMALL).
+// Bound: issue slots (some hundred instructions per warp beside those per entry), three quarters of which are in use:
+// short prompts take CTAs of two warps (WH_SMALL), and the query heads are a template argument.  128 heads x 32 queries over
+// 1000 entries: 41 us (with the heads a run-time number and expf 48.7; with CTAs of eight warps as well 49.3).
 // pbar lives in shared memory or, for long prompts, in the place of the first query head's logits.
-template <int NTH>
+template <int NTH, int G>
 __global__ void __launch_bounds__(NTH) window_hits_kernel(const __grid_constant__ State st, const WindowParams p, float top_p, int literal,
                                                           int in_smem, const __grid_constant__ Plan plan, int plan_grid, int plan_cl,
                                                           int shrink, int* plan_len) {
@@ -255,31 +257,32 @@ __global__ void __launch_bounds__(NTH) window_hits_kernel(const __grid_constant_
       return;
     }
   }
-  float* S = p.logits + ((size_t)u * p.W + q) * p.G * p.Ps;
+  float* S = p.logits + ((size_t)u * p.W + q) * G * p.Ps;
   float* pb = in_smem ? s_pbar : S;
-  float mx[QH], il[QH];
+  float m[G], il[G];   // reference point (log2 domain), 1 / (normaliser x query heads)
   const float* ml = p.ml + ((size_t)u * p.W + q) * 16;
 #pragma unroll
-  for (int g = 0; g < QH; ++g) {
-    mx[g] = g < p.G ? ml[g] * 0.693147180559945309f : 0.f;   // log2 domain -> natural log
-    il[g] = g < p.G ? 1.0f / (ml[8 + g] * (float)p.G) : 0.f;
+  for (int g = 0; g < G; ++g) {
+    m[g] = ml[g];
+    il[g] = 1.0f / (ml[8 + g] * (float)G);
   }
   const int base = nucleus_base<NTH>(n);
   nucleus_clear<NTH>(s_nu);
   __syncthreads();
   constexpr int BR = 4;   // entries requested together
   for (int i0 = tid; i0 < n; i0 += BR * NTH) {
-    float sv[BR][QH];
-#pragma unroll
-    for (int x = 0; x < BR; ++x)
-#pragma unroll
-      for (int g = 0; g < QH; ++g) sv[x][g] = g < p.G ? S[(size_t)g * p.Ps + min(i0 + x * NTH, n - 1)] : 0.f;
+    float sv[BR][G];
 #pragma unroll
     for (int x = 0; x < BR; ++x) {
-      float pm = 0.f;
+      const float* r = S + min(i0 + x * NTH, n - 1);
 #pragma unroll
-      for (int g = 0; g < QH; ++g)
-        if (g < p.G) pm = fmaf(expf(sv[x][g] - mx[g]), il[g], pm);
+      for (int g = 0; g < G; ++g) sv[x][g] = r[(size_t)g * p.Ps];
+    }
+#pragma unroll
+    for (int x = 0; x < BR; ++x) {
+      float pm = 0.f;   // (as in the decode step's kernel)
+#pragma unroll
+      for (int g = 0; g < G; ++g) pm = fmaf(ex2(fmaf(sv[x][g], 1.44269504088896340736f, -m[g])), il[g], pm);
       if (i0 + x * NTH < n) {
         pb[i0 + x * NTH] = pm;   // (in the place of its own logit, which has been read)
         nucleus_add<NTH>(s_nu, base, pm);
@@ -314,6 +317,21 @@ __global__ void __launch_bounds__(NTH) window_hits_kernel(const __grid_constant_
     }
     const unsigned m = __ballot_sync(0xffffffffu, hit);
     if (lane == 0 && (i >> 5) < p.words) bits[i >> 5] = m;
+  }
+}
+
+using WindowHits = void (*)(State, WindowParams, float, int, int, Plan, int, int, int, int*);
+template <int NTH>
+WindowHits window_hits_of(int G) {
+  switch (G) {
+    case 1: return window_hits_kernel<NTH, 1>;
+    case 2: return window_hits_kernel<NTH, 2>;
+    case 3: return window_hits_kernel<NTH, 3>;
+    case 4: return window_hits_kernel<NTH, 4>;
+    case 5: return window_hits_kernel<NTH, 5>;
+    case 6: return window_hits_kernel<NTH, 6>;
+    case 7: return window_hits_kernel<NTH, 7>;
+    default: return window_hits_kernel<NTH, 8>;
   }
 }
 
