@@ -342,24 +342,6 @@ int join_side(crystalkv_t* h, cudaStream_t s) {
   return CRYSTALKV_OK;
 }
 
-// The streams and events of steps from and to host memory, made by a handle's first such step: two streams and 192
-// events cost every other handle 0.35 ms to make and give back.
-int open_host_io(crystalkv_t* h) {
-  if (h->copy_out) return CRYSTALKV_OK;
-  // (another stream of the caller may be in a capture that would refuse a new stream)
-  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-  CK(h, cudaThreadExchangeStreamCaptureMode(&mode));
-  cudaError_t e = cudaSuccess;
-  for (int i = 0; i < crystalkv::HOST_RING; ++i)
-    for (cudaEvent_t* x : {&h->evIn[i], &h->evUse[i], &h->evOut[i]})
-      if (e == cudaSuccess && !*x) e = cudaEventCreateWithFlags(x, cudaEventDisableTiming);
-  if (e == cudaSuccess && !h->copy_in) e = cudaStreamCreateWithFlags(&h->copy_in, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->copy_out, cudaStreamNonBlocking);
-  CK(h, cudaThreadExchangeStreamCaptureMode(&mode));
-  CK(h, e);
-  return CRYSTALKV_OK;
-}
-
 // One attention launch on `s` and its follow-up (Algorithm 1 when it runs, the heads' new lengths
 // and the layer's next plan) on the internal stream.
 int launch_step(crystalkv_t* h, DecodeParams& p, int layer, cudaStream_t s) {
@@ -546,6 +528,13 @@ int crystalkv_create(const crystalkv_config_t* cfg, crystalkv_t** out) {
     int least = 0, greatest = 0;
     CKC(cudaDeviceGetStreamPriorityRange(&least, &greatest));
     for (cudaStream_t& x : h->side) CKC(cudaStreamCreateWithPriority(&x, cudaStreamNonBlocking, greatest));
+  }
+  CKC(cudaStreamCreateWithFlags(&h->copy_in, cudaStreamNonBlocking));
+  CKC(cudaStreamCreateWithFlags(&h->copy_out, cudaStreamNonBlocking));
+  for (int i = 0; i < crystalkv::HOST_RING; ++i) {
+    CKC(cudaEventCreateWithFlags(&h->evIn[i], cudaEventDisableTiming));
+    CKC(cudaEventCreateWithFlags(&h->evUse[i], cudaEventDisableTiming));
+    CKC(cudaEventCreateWithFlags(&h->evOut[i], cudaEventDisableTiming));
   }
   for (cudaEvent_t& e : h->evA) CKC(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   for (cudaEvent_t& e : h->evF) CKC(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
@@ -825,8 +814,6 @@ int crystalkv_decode_step_host(crystalkv_t* h, int layer, const void* q_host, co
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const size_t qb = (size_t)c.batch * c.n_q_heads * HD * 2, kb = (size_t)c.batch * c.n_kv_heads * HD * 2;
   if (h->t_layer[layer] < 0) return fail(h, CRYSTALKV_ESTATE, "decode before prefill");
-  rc = open_host_io(h);
-  if (rc) return rc;
   // Staging set j was last used HOST_RING host steps ago.  Page-locked inputs that the GPU can
   // address are fetched by one small kernel in the caller's stream; anything else (pageable
   // memory, 16-byte misalignment) goes up by three copies on the copy-in stream, for which the
