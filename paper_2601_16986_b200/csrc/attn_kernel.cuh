@@ -255,7 +255,7 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
   const uint32_t ring_u32 = smem_u32(smem) + w * (STAGES * PAGE_BYTES);
   const uint32_t bar0 = bars_u32 + w * (STAGES * 8);
   const int gid = lane >> 2, tig = lane & 3, mi = lane >> 3, r8 = lane & 7;
-  const uint64_t pol_stream = policy_evict_first(), pol_keep = policy_evict_last();
+  const uint64_t pol_stream = policy_evict_first();
   // ldmatrix row addresses inside a stage: entry row r, 16-byte chunk c at 512 r + 16 (c ^ (r & 7))
   const uint32_t krow = (uint32_t)(((mi & 1) * 8 + r8) * SLOT_BYTES), khalf = (uint32_t)(mi >> 1);
   const uint32_t vrow = (uint32_t)(((mi >> 1) * 8 + r8) * SLOT_BYTES), vhalf = (uint32_t)(mi & 1);
@@ -421,6 +421,7 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
       const bool v0 = gid < valid, v1 = gid + 8 < valid;
       if (p.track) {
         float* lrow = lrow0 + (size_t)base * QH;
+        const uint64_t pol_keep = policy_evict_last();   // (one instruction: kept over the loop it cost a spilled register)
         if (v0) st_f32x2_hint(lrow, __fmul_rn(s[0], p.scale), __fmul_rn(s[1], p.scale), pol_keep);
         if (v1) st_f32x2_hint(lrow + 8 * QH, __fmul_rn(s[2], p.scale), __fmul_rn(s[3], p.scale), pol_keep);
       }
