@@ -77,16 +77,12 @@ struct Row {
       for (int g = 4; g < G; ++g) b[g - 4] = v[g - 4];
     }
   }
-  // Mean over the query heads of 2^(s_g log2(e) - m_g) / l_g  (invl: 1 / (l_g G)).  One rounding in the exponent: against
-  // 64 bits pbar is off by no more (6.0e-7 rms over logits of deviation 0.5 .. 8 and 1 .. 8 query heads) than with
-  // expf(s_g - m_g ln 2) (6.3e-7), which rounds the reference point as well.
   __device__ __forceinline__ float pbar(const float (&m)[G], const float (&invl)[G]) const {
     const float v[4] = {a.x, a.y, a.z, a.w};
-    float pm = 0.f;
+    float s[G];
 #pragma unroll
-    for (int g = 0; g < G; ++g)
-      pm = fmaf(ex2(fmaf(g < 4 ? v[g < 4 ? g : 0] : b[g < 4 ? 0 : g - 4], 1.44269504088896340736f, -m[g])), invl[g], pm);
-    return pm;
+    for (int g = 0; g < G; ++g) s[g] = g < 4 ? v[g < 4 ? g : 0] : b[g < 4 ? 0 : g - 4];
+    return group_mean(s, m, invl);
   }
 };
 
@@ -139,7 +135,7 @@ __device__ __forceinline__ int lrfu_unit(const DecodeParams& p, int u, int uid, 
     float m[G], invl[G];
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-      m[g] = fr.m[g];
+      m[g] = to_natural(fr.m[g]);
       invl[g] = 1.0f / (fr.l[g] * (float)G);
     }
     auto put = [&](int i, float pm) {

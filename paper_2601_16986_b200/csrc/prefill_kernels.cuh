@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(SEL_NT) prefill_select_kernel(State st, Scratc
   float mx[QH], il[QH];
 #pragma unroll
   for (int g = 0; g < QH; ++g) {
-    mx[g] = g < G ? s_m[g] * 0.693147180559945309f : 0.f;   // log2 domain -> natural log
+    mx[g] = g < G ? to_natural(s_m[g]) : 0.f;
     il[g] = g < G ? s_il[g] : 0.f;
   }
   float* pb = in_smem ? s_pbar : sc.pbar + (size_t)u * sc.cap_s;
@@ -258,10 +258,7 @@ __global__ void __launch_bounds__(SEL_NT) prefill_select_kernel(State st, Scratc
     for (int x = 0; x < BR; ++x) {
       const int i = i0 + x * SEL_NT;
       const float sv[8] = {ra[x].x, ra[x].y, ra[x].z, ra[x].w, rb[x].x, rb[x].y, rb[x].z, rb[x].w};
-      float pm = 0.f;
-#pragma unroll
-      for (int g = 0; g < QH; ++g)
-        if (g < G) pm = fmaf(expf(sv[g] - mx[g]), il[g], pm);
+      const float pm = group_mean(sv, mx, il, G);
       if (i < P) {
         pb[i] = pm;
         if (track) nucleus_add<SEL_NT>(s_nu, base, pm);

@@ -259,11 +259,11 @@ __global__ void __launch_bounds__(NTH) window_hits_kernel(const __grid_constant_
   }
   float* S = p.logits + ((size_t)u * p.W + q) * G * p.Ps;
   float* pb = in_smem ? s_pbar : S;
-  float m[G], il[G];   // reference point (log2 domain), 1 / (normaliser x query heads)
+  float m[G], il[G];   // reference point, 1 / (normaliser x query heads)
   const float* ml = p.ml + ((size_t)u * p.W + q) * 16;
 #pragma unroll
   for (int g = 0; g < G; ++g) {
-    m[g] = ml[g];
+    m[g] = to_natural(ml[g]);
     il[g] = 1.0f / (ml[8 + g] * (float)G);
   }
   const int base = nucleus_base<NTH>(n);
@@ -280,9 +280,7 @@ __global__ void __launch_bounds__(NTH) window_hits_kernel(const __grid_constant_
     }
 #pragma unroll
     for (int x = 0; x < BR; ++x) {
-      float pm = 0.f;   // (as in the decode step's kernel)
-#pragma unroll
-      for (int g = 0; g < G; ++g) pm = fmaf(ex2(fmaf(sv[x][g], 1.44269504088896340736f, -m[g])), il[g], pm);
+      const float pm = group_mean(sv[x], m, il);
       if (i0 + x * NTH < n) {
         pb[i0 + x * NTH] = pm;   // (in the place of its own logit, which has been read)
         nucleus_add<NTH>(s_nu, base, pm);
