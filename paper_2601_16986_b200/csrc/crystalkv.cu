@@ -683,11 +683,10 @@ static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, cons
     p.store = last;
     attn<<<dim3((p.W * p.G + WA_ROWS - 1) / WA_ROWS, h->U), WA_WARPS * 32, WA_SMEM, s>>>(h->st, p);
     CK(h, cudaGetLastError());
-    // (the plan is for the heads' lengths after the last query's step 4, known from their budgets)
-    hits<<<dim3(p.W, h->U + 1), small ? 64 : NT, std::max(sm, PL_SCRATCH * sizeof(int)), s>>>(h->st, p, c.top_p, c.literal_return, sm > 0, h->plans[layer],
-                                                          last ? plan_grid : 0, h->cl[layer], c.evict_every, h->plan_len);
+    hits<<<dim3(p.W, h->U), small ? 64 : NT, sm, s>>>(h->st, p, c.top_p, c.literal_return, sm > 0);
     CK(h, cudaGetLastError());
-    window_apply_kernel<<<h->U, NT, 0, s>>>(h->st, p, last, c.evict_every, reinterpret_cast<int*>(h->sc_pbar[1]), h->cap_s);
+    window_apply_kernel<<<1 + h->U, NT, 0, s>>>(h->st, p, last, c.evict_every, reinterpret_cast<int*>(h->sc_pbar[1]), h->cap_s,
+                                                h->plans[layer], plan_grid, h->cl[layer], h->plan_len);
     CK(h, cudaGetLastError());
   }
   return CRYSTALKV_OK;

@@ -2,8 +2,8 @@
 // already stored.  Which entries a query hits depends on its scores alone, not on what earlier
 // queries of the window marked, so the window is one attention kernel over all (query, head) rows,
 // one threshold search per (head, query), and one kernel that walks an entry through its queries.
-// 128 heads x 1024 tokens, 32 queries of 5 heads: 92 + 41 + 14 us a layer, the pages and the launch plan included (as kernels
-// of their own they took 20 and 9 us, the three others 83 + 49 + 21); a decode-step launch pair
+// 128 heads x 1024 tokens, 32 queries of 5 heads: 95 + 36 + 16 us a layer, the pages and the launch plan included (as kernels
+// of their own they took 20 and 9 us, the three others 85 + 50 + 20); a decode-step launch pair
 // per query, each reading the prompt's rows again, took 720 us.
 #pragma once
 #include "attn_kernel.cuh"
@@ -229,25 +229,19 @@ __global__ void __launch_bounds__(WA_WARPS * 32, 3) window_attn_kernel(const __g
 }
 
 // The hit bits of one (query, head): Algorithm 1 step 1 with the query of time t over its t + 1 entries.
-// grid: (W, U + 1); one CTA of the last row writes the layer's launch plan meanwhile.
+// grid: (W, U).
 // Bound: issue slots (some hundred instructions per warp beside those per entry), three quarters of which are in use:
 // short prompts take CTAs of two warps (WH_SMALL), and the query heads are a template argument.  128 heads x 32 queries over
 // 1000 entries: 41 us (with the heads a run-time number and expf 48.7; with CTAs of eight warps as well 49.3).
 // pbar lives in shared memory or, for long prompts, in the place of the first query head's logits.
 template <int NTH, int G>
 __global__ void __launch_bounds__(NTH) window_hits_kernel(const __grid_constant__ State st, const WindowParams p, float top_p, int literal,
-                                                          int in_smem, const __grid_constant__ Plan plan, int plan_grid, int plan_cl,
-                                                          int shrink, int* plan_len) {
+                                                          int in_smem) {
   constexpr int WARPS = NTH / 32;
-  extern __shared__ __align__(16) float s_pbar[];   // (the planner's scratch in its CTA)
+  extern __shared__ float s_pbar[];
   __shared__ NucleusSmem<NTH> s_nu;
   __shared__ int s_cnt[WARPS];
   const int u = blockIdx.y, q = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  if (u == p.U) {
-    if (q == 0 && plan_grid > 0)
-      write_plan<NTH>(st, plan, p.layer, plan_grid * NW, plan_grid, plan_cl, plan_len, reinterpret_cast<int*>(s_pbar), shrink);
-    return;
-  }
   const int n = p.t0 + q + 1;
   unsigned* bits = p.hits + ((size_t)u * p.W + q) * p.words;
   if (literal) {   // Algorithm 1's first line as printed: nothing runs below the budget
@@ -318,7 +312,7 @@ __global__ void __launch_bounds__(NTH) window_hits_kernel(const __grid_constant_
   }
 }
 
-using WindowHits = void (*)(State, WindowParams, float, int, int, Plan, int, int, int, int*);
+using WindowHits = void (*)(State, WindowParams, float, int, int);
 template <int NTH>
 WindowHits window_hits_of(int G) {
   switch (G) {
@@ -335,12 +329,21 @@ WindowHits window_hits_of(int G) {
 
 // Steps 2-3 of the launch's W queries for every entry in turn (an entry takes part from its own time
 // on; its CRF and tau only depend on its own hits), and after the last query (last != 0) step 4: the
-// head comes down to its budget.  One CTA per head; tmp: U x tmp_stride ints.
-// Bound: latency (W dependent multiply-adds per entry).
-__global__ void __launch_bounds__(NT) window_apply_kernel(State st, const WindowParams p, int last, int evict_every,
-                                                          int* tmp, int tmp_stride) {
-  __shared__ int sh[300];
-  const int u = blockIdx.x, seq = u / st.H, tid = threadIdx.x;
+// head comes down to its budget.  One CTA per head behind CTA 0, which writes the layer's launch plan meanwhile (last):
+// from a head's length or, where that is evict_every or more over its budget, from the budget it comes down to, so that it
+// does not matter whether the head's CTA has been there.  tmp: U x tmp_stride ints.
+// Bound: latency (W dependent multiply-adds per entry; with many heads the plan).  The three kernels of a window with the plan
+// written here, and by one CTA of the threshold searches, which starts last and has two warps: 128 heads x 1024 tokens, 32
+// queries 151 us and 155, 1024 heads x 300 tokens, 2 queries 144 and 193, 1024 heads x 256 tokens, 32 queries 241 and 292.
+__global__ void __launch_bounds__(NT) window_apply_kernel(const __grid_constant__ State st, const WindowParams p, int last, int evict_every,
+                                                          int* tmp, int tmp_stride, const __grid_constant__ Plan plan, int plan_grid,
+                                                          int plan_cl, int* plan_len) {
+  __shared__ __align__(16) int sh[PL_SCRATCH];
+  if (blockIdx.x == 0) {
+    if (last) write_plan<NT>(st, plan, p.layer, plan_grid * NW, plan_grid, plan_cl, plan_len, sh, evict_every);
+    return;
+  }
+  const int u = blockIdx.x - 1, seq = u / st.H, tid = threadIdx.x;
   const int uid = (seq * st.L + p.layer) * st.H + u % st.H;
   if (st.n_cur[uid] != p.P) return;   // the prompt found no pages: the head is empty
   const size_t mb = (size_t)uid * st.cap;
