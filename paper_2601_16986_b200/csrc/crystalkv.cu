@@ -647,12 +647,29 @@ int crystalkv_time(crystalkv_t* h, int layer) {
   return h->t_layer[layer];
 }
 
+// Queries of a window over P tokens that one launch replays: what the logit sets, the partials and the pbar area have room for.
+static int window_queries(const crystalkv_t* h, int P) {
+  const long long rows = (P + 7) / 8 * 8, words = (P + 31) / 32;
+  return (int)std::max<long long>(1, std::min({(long long)NSETS * h->cap_s * QH / (h->G * rows),
+                                               (long long)h->pmax * (16 + h->G * HD) / 16, h->cap_s / words, 1ll << 30}));
+}
+
+// Whether a window's attention kernel also fills the pages, from the tiles it reads: where its last launch has a CTA for four
+// fifths of the SMs at least.  With fewer CTAs a copy kernel over the whole chip is the faster one.  The window's kernels of a
+// layer, pages from the tiles and copied: one CTA a head, 6 queries over 4096 tokens, 16 heads 289 us and 233, 64 heads
+// 311 and 282, 96 heads 319 and 312, 128 heads 336 and 344; 160 heads, 2 queries, 366 and 382; 128 heads of 1024 tokens, 2 queries
+// 106 and 105; three CTAs a head, 32 queries over 1024 tokens, 16 heads 84 and 84, 40 heads 90 and 92.5.
+static bool window_fills_pages(const crystalkv_t* h, int P, int W) {
+  const int last = (W - 1) % window_queries(h, P) + 1;
+  return 5ll * h->U * ((last * h->G + WA_ROWS - 1) / WA_ROWS) >= 4ll * h->num_sms;
+}
+
 // Algorithm 1 with the queries of the prompt's last W tokens, in as many launches as the scratch
 // asks for (usually one): steps 1-3 for every query, step 4 after the last one.  Everything runs on
 // `s`, which has joined the internal streams: the logit sets, one block of the arena, hold the
 // window's logits, the partials its softmax references, the first pbar area the hit bits.
 static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, const unsigned char* v, const unsigned char* q,
-                         int P, int W, __nv_bfloat16* out, cudaStream_t s) {
+                         int P, int W, __nv_bfloat16* out, bool fill_pages, cudaStream_t s) {
   const crystalkv_config_t& c = h->cfg;
   WindowParams p{};
   p.k = k; p.v = v;
@@ -664,9 +681,7 @@ static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, cons
   p.words = (P + 31) / 32;
   p.scale = c.sm_scale;
   p.scale_log2 = c.sm_scale * 1.44269504088896340736f;
-  // queries of one launch: what the logit sets, the partials and the pbar area have room for
-  const long long fit = std::min<long long>((long long)NSETS * h->cap_s * QH / ((long long)h->G * p.Ps),
-                                            std::min<long long>((long long)h->pmax * (16 + h->G * HD) / 16, h->cap_s / p.words));
+  const int fit = window_queries(h, P);
   const size_t sm = (size_t)P * sizeof(float) <= WIN_SMEM ? (size_t)P * sizeof(float) : 0;
   const auto attn = out ? window_attn_kernel<true> : window_attn_kernel<false>;
   const bool small = P <= WH_SMALL;
@@ -675,12 +690,12 @@ static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, cons
   CK(h, cudaFuncSetAttribute(attn, cudaFuncAttributeMaxDynamicSharedMemorySize, WA_SMEM));
   const size_t qn = (size_t)c.batch * c.n_q_heads * HD;
   for (int w0 = 0; w0 < W; w0 += p.W) {
-    p.W = (int)std::min<long long>(W - w0, std::max<long long>(1, fit));
+    p.W = std::min(W - w0, fit);
     p.t0 = P - W + w0;
     p.q = q + (size_t)w0 * qn * sizeof(__nv_bfloat16);
     p.out = out ? out + (size_t)w0 * qn : nullptr;
     const bool last = w0 + p.W == W;
-    p.store = last;
+    p.store = last && fill_pages;
     attn<<<dim3((p.W * p.G + WA_ROWS - 1) / WA_ROWS, h->U), WA_WARPS * 32, WA_SMEM, s>>>(h->st, p);
     CK(h, cudaGetLastError());
     hits<<<dim3(p.W, h->U), small ? 64 : NT, sm, s>>>(h->st, p, c.top_p, c.literal_return, sm > 0);
@@ -746,16 +761,17 @@ static int prefill_common(crystalkv_t* h, int layer, const void* k, const void* 
     CK(h, cudaGetLastError());
   }
   // the whole prompt is stored; in full-cache mode the first step's plan is written beside the copy, and a replayed window
-  // copies the rows in its attention kernel where that reads all of them (it has outputs)
+  // copies the rows in its attention kernel where that reads all of them (it has outputs) and is wide enough
+  const bool fill_pages = evict && out_window && window_fills_pages(h, P, W);
   prefill_take_kernel<<<h->U, NT, 0, s>>>(h->st, layer, P, W > 0 ? 1 : 0);
   CK(h, cudaGetLastError());
-  if (!evict || !out_window) {
+  if (!fill_pages) {
     prefill_rows_kernel<<<1 + h->U * per_head, NT, 0, s>>>(h->st, h->plans[layer], layer, kb, vb, P, W > 0 ? ROWS_ALL : ROWS_ALL_LAST,
                                                            per_head, evict ? 0 : plan_grid * NW, plan_grid, h->cl[layer]);
     CK(h, cudaGetLastError());
   }
   if (evict) {
-    rc = replay_window(h, layer, kb, vb, static_cast<const unsigned char*>(q), P, W, static_cast<__nv_bfloat16*>(out_window), s);
+    rc = replay_window(h, layer, kb, vb, static_cast<const unsigned char*>(q), P, W, static_cast<__nv_bfloat16*>(out_window), fill_pages, s);
     if (rc) return rc;
   }
   h->t_layer[layer] = P - 1;

@@ -48,7 +48,7 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
 // of 64 keys in two cp.async stages; three CTAs fit an SM.  (Two CTAs of five warps for 160 rows, without idle rows but with
 // ten warps an SM instead of twelve: 92 us instead of 82.)
 // The tiles are also what the heads' pages are filled from (store): the CTAs of a head take its tiles in turn, a tile that
-// only the last one sees in full falls to that one.  (A copy kernel of its own read the prompt again: 20 us.)
+// only the last one sees in full falls to that one.  (A copy kernel of its own reads the prompt again: 20 us.)
 template <bool OUT>
 __global__ void __launch_bounds__(WA_WARPS * 32, 3) window_attn_kernel(const __grid_constant__ State st, const WindowParams p) {
   extern __shared__ __align__(1024) unsigned char smem[];
