@@ -684,8 +684,6 @@ static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, cons
   const int fit = window_queries(h, P);
   const size_t sm = (size_t)P * sizeof(float) <= WIN_SMEM ? (size_t)P * sizeof(float) : 0;
   const auto attn = out ? window_attn_kernel<true> : window_attn_kernel<false>;
-  const bool small = P <= WH_SMALL;
-  const WindowHits hits = small ? window_hits_of<64>(h->G) : window_hits_of<NT>(h->G);
   const int plan_grid = h->plan_grid(layer);
   CK(h, cudaFuncSetAttribute(attn, cudaFuncAttributeMaxDynamicSharedMemorySize, WA_SMEM));
   const size_t qn = (size_t)c.batch * c.n_q_heads * HD;
@@ -698,7 +696,8 @@ static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, cons
     p.store = last && fill_pages;
     attn<<<dim3((p.W * p.G + WA_ROWS - 1) / WA_ROWS, h->U), WA_WARPS * 32, WA_SMEM, s>>>(h->st, p);
     CK(h, cudaGetLastError());
-    hits<<<dim3(p.W, h->U), small ? 64 : NT, sm, s>>>(h->st, p, c.top_p, c.literal_return, sm > 0);
+    const bool small = P <= WH_SMALL && (long long)p.W * h->U >= P + h->num_sms;
+    (small ? window_hits_of<64>(h->G) : window_hits_of<NT>(h->G))<<<dim3(p.W, h->U), small ? 64 : NT, sm, s>>>(h->st, p, c.top_p, c.literal_return, sm > 0);
     CK(h, cudaGetLastError());
     window_apply_kernel<<<1 + h->U, NT, 0, s>>>(h->st, p, last, c.evict_every, reinterpret_cast<int*>(h->sc_pbar[1]), h->cap_s,
                                                 h->plans[layer], plan_grid, h->cl[layer], h->plan_len);

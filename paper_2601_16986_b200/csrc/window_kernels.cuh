@@ -19,7 +19,7 @@ constexpr int WA_KEYS = 64;                   // keys per tile
 constexpr int WA_TILE = WA_KEYS * ROW_BYTES;  // bytes of a K (or V) tile
 constexpr int WA_SMEM = 4 * WA_TILE;          // K and V, two stages
 constexpr int WIN_SMEM = 32 * 1024;           // pbar of up to this many bytes stays in shared memory
-constexpr int WH_SMALL = 1280;                // entries up to which window_hits_kernel takes CTAs of two warps
+constexpr int WH_SMALL = 1280;                // entries up to which window_hits_kernel may take CTAs of two warps
 
 struct WindowParams {
   const unsigned char* k;      // [batch][P][H][128]
@@ -231,8 +231,12 @@ __global__ void __launch_bounds__(WA_WARPS * 32, 3) window_attn_kernel(const __g
 // The hit bits of one (query, head): Algorithm 1 step 1 with the query of time t over its t + 1 entries.
 // grid: (W, U).
 // Bound: issue slots (some hundred instructions per warp beside those per entry), three quarters of which are in use:
-// short prompts take CTAs of two warps (WH_SMALL), and the query heads are a template argument.  128 heads x 32 queries over
-// 1000 entries: 41 us (with the heads a run-time number and expf 48.7; with CTAs of eight warps as well 49.3).
+// many searches of short prompts take CTAs of two warps, and the query heads are a template argument.  Few searches are bound by
+// the latency of one: the line is as many searches as entries and SMs, and WH_SMALL entries.  us with two warps and with
+// eight: 64 heads, 300 entries, 512 searches 6.4 and 6.7, 1024 7.7 and 10.7; 16 heads, 128 searches 6.0 and 4.5; 1024 entries, 128
+// searches 10.7 and 5.0, 512 12.0 and 7.7, 1024 13.3 and 12.8, 1536 15.6 and 17.3; 1280 entries, 512 searches 14.7 and 10.1, 2048 23.6
+// and 28.5, 4096 45.4 and 54.3; 1600 entries, 4096 searches 61.2 and 60.2, 2048 entries 74.7 and 65.4.
+// 128 heads x 32 queries over 1000 entries: 36 us.
 // pbar lives in shared memory or, for long prompts, in the place of the first query head's logits.
 template <int NTH, int G>
 __global__ void __launch_bounds__(NTH) window_hits_kernel(const __grid_constant__ State st, const WindowParams p, float top_p, int literal,
