@@ -655,13 +655,15 @@ static int window_queries(const crystalkv_t* h, int P) {
 }
 
 // Whether a window's attention kernel also fills the pages, from the tiles it reads: where its last launch has a CTA for four
-// fifths of the SMs at least.  With fewer CTAs a copy kernel over the whole chip is the faster one.  The window's kernels of a
+// fifths of the SMs at least, or the prompt is so short that a launch more costs what it saves.  With fewer CTAs a copy kernel
+// over the whole chip is the faster one.  The window's kernels of a
 // layer, pages from the tiles and copied: one CTA a head, 6 queries over 4096 tokens, 16 heads 289 us and 233, 64 heads
 // 311 and 282, 96 heads 319 and 312, 128 heads 336 and 344; 160 heads, 2 queries, 366 and 382; 128 heads of 1024 tokens, 2 queries
-// 106 and 105; three CTAs a head, 32 queries over 1024 tokens, 16 heads 84 and 84, 40 heads 90 and 92.5.
+// 106 and 105; three CTAs a head, 32 queries over 1024 tokens, 16 heads 84 and 84, 40 heads 90 and 92.5.  8 queries, 16 heads of 300 tokens 43 and 47, 64 heads 47
+// and 51.5, 2 heads of 512 tokens, 4 queries, 51.5 and 51.6, 16 heads of 1024 tokens, 8 queries, 86 and 74.
 static bool window_fills_pages(const crystalkv_t* h, int P, int W) {
   const int last = (W - 1) % window_queries(h, P) + 1;
-  return 5ll * h->U * ((last * h->G + WA_ROWS - 1) / WA_ROWS) >= 4ll * h->num_sms;
+  return P <= 512 || 5ll * h->U * ((last * h->G + WA_ROWS - 1) / WA_ROWS) >= 4ll * h->num_sms;
 }
 
 // Algorithm 1 with the queries of the prompt's last W tokens, in as many launches as the scratch
