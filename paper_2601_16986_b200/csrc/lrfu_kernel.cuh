@@ -186,6 +186,21 @@ __device__ __forceinline__ int lrfu_unit(const DecodeParams& p, int u, int uid, 
       });
   const uint32_t theta = nu.theta;
   const unsigned long long w_theta = mass_of(__uint_as_float(theta));
+  // The earliest of the entries that carry the threshold's value are hits: their positions are listed in the histogram's
+  // place.  (Among 4097 random entries every seven thousandth search meets two.  Each of them going through all entries' values
+  // held the CTA, and with it the layers that wait for it, for 290 us: 16 heads of 4097 entries took 13.9 us a layer in
+  // ten passes without such a pair, 15.1, 16.3 and 17.5 with one, two and three.)
+  constexpr int LISTED = 256;
+  int* eq_pos = reinterpret_cast<int*>(sh.nu.hist_lo);
+  static_assert(LISTED <= fine_bins(NTH), "the list takes the histogram's place");
+  const bool listed = nu.cnt_eq > 1 && nu.cnt_eq <= LISTED;
+  if (listed) {
+    if (tid == 0) sh.nu.ncand = 0;
+    __syncthreads();
+    for (int i = tid; i < n; i += NTH)
+      if (__float_as_uint(pb[i]) == theta) eq_pos[atomicAdd(&sh.nu.ncand, 1)] = st.meta_pos[mb + i];
+    __syncthreads();
+  }
 
   // ---- steps 2-3: CRF/tau update; step 4 candidates
   // step 4 runs once the head is evict_every entries over its budget, and then for all of them
@@ -200,10 +215,14 @@ __device__ __forceinline__ int lrfu_unit(const DecodeParams& p, int u, int uid, 
     bool hit = key > theta && nu.found;
     if (key == theta && nu.found) {
       unsigned long long before = 0;
-      if (nu.cnt_eq > 1)
-#pragma unroll 1
+      if (listed) {
+#pragma unroll 4
+        for (int x = 0; x < nu.cnt_eq; ++x) before += eq_pos[x] < pos_i;
+      } else if (nu.cnt_eq > 1) {
+#pragma unroll 4
         for (int x = 0; x < n; ++x)
           before += (__float_as_uint(pb[x]) == theta) && (st.meta_pos[mb + x] < pos_i);
+      }
       hit = (nu.A + before * w_theta) < nu.Pthr;
     }
     float ct = __fmul_rn(dec, crf);
