@@ -291,16 +291,19 @@ int find_clusters(crystalkv_t* h) {
 // groups 7.9 and 6.65, of 41 groups 8.1 and 8.8, of 65 groups 9.9 and 11.2; 64 heads, two CTAs: of 41 groups 9.3 and
 // 9.3, of 57 groups 10.5 and 12.0.  One layer of 2 heads, four CTAs: of 29 groups 10.8 and 10.95, of 33 groups 10.7 and
 // 11.4.
-// Longer heads of one length gain from two CTAs where one could not hold them without pieces twice as long
-// as a chain-bound launch takes: their other choice is more than eight pieces and a merge through global memory
-// at the end of the launch (4 us for 64 heads of 257 groups).  64 heads of 193 groups 24.3 and 28.2, of 257 32.5 and
-// 32.4; 72 of 257 34.9 and 39.7; 60 of 257 30.7 and 30.9; 48 of 257 27.3 and 27.8.
+// Longer heads of one length (from 193 groups, where they no longer fit a CTA in pieces of 2 GLAT) gain from two CTAs where their
+// other choice is more than eight pieces and a merge through global memory at the end of the launch. The longer the pieces,
+// the more the CTAs that then have nothing to stream count: up to 14 groups a piece from 45 heads on, up to 24 from 52.  us a
+// layer, shared and not, of 193, 225, 257, 288, 313, 345 and 376 groups: 48 heads 19.8 22.2 24.2 25.9 27.8 30.0 31.9 and 21.9 22.3 23.6
+// 25.4 27.5 29.8 32.0; 52 heads 20.3 22.8 25.1 27.1 29.1 31.2 34.1 and 22.6 22.9 25.5 27.9 29.9 32.4 35.5; 64 heads 22.4 25.9 28.5 31.3
+// 33.5 36.7 39.9 and 27.3 31.2 29.6 32.3 34.5 37.3 40.2; 72 heads 23.8 27.5 30.5 33.5 36.2 39.3 42.8 and 28.7 32.4 36.4 39.6 43.0 46.5 50.2.
 int share_heads(crystalkv_t* h, int entries) {
   const int g = (entries + GRP - 1) / GRP, alone = (g + NW - 1) / NW;
   for (int cl = MAX_CLUSTER; cl > 1; cl /= 2) {
     const int per = (g + NW * cl - 1) / (NW * cl);
-    const bool chain = per <= GLAT, merge = cl == 2 && h->uniform && 10 * h->U >= 3 * h->num_sms && alone > 2 * GLAT && per <= 2 * GLAT;
-    if (h->share_ok[cl] && (chain || merge) && alone - per >= (h->cfg.n_layers > 1 ? 4 : 3)) return cl;
+    const int most = 20 * h->U >= 7 * h->num_sms ? 2 * GLAT : GLAT + 2;
+    const bool merge = cl == 2 && h->uniform && 10 * h->U >= 3 * h->num_sms && alone > 2 * GLAT && per <= most;
+    if (h->share_ok[cl] && (per <= GLAT || merge) && alone - per >= (h->cfg.n_layers > 1 ? 4 : 3)) return cl;
   }
   return 1;
 }
