@@ -48,23 +48,17 @@ struct crystalkv {
   float* sc_mfin[NSETS] = {};
   float* sc_partials[2] = {};
   int* sc_ticket[2] = {};
-  // The LRFU kernels of consecutive layers do not depend on one another and run on internal streams taken in turn, so that
-  // the next may fill SM room as one's CTAs finish.  Three: an LRFU kernel of few long heads takes 33 to 40 us beside the
-  // attention kernels, and with two streams a layer took half of that where its attention kernel takes less.  us a layer with
-  // two and with three: 32 heads of 4097 entries 21.6 and 19.7, of 3001 15.2 and 14.0, 48 heads of 4097 27.0 and 26.0, 64 31.3 and
-  // 30.4, 66 of 3001 23.8 and 23.3, 128 heads of 1024 .. 3072 28.8 and 28.35; many short heads and launches bound by the
-  // host do not change.  (A fourth stream gains nothing more.)
-  static constexpr int NSIDE = 3;
-  float* sc_pbar[NSIDE] = {};      // one per internal stream
+  float* sc_pbar[2] = {};          // one per internal stream
   int cap_s = 0, pmax = 0;
   long long nA = 0;                // attention launches so far
   std::vector<int> t_layer;        // per layer: time of the last step
   // LRFU launches are numbered; launch k uses scratch set k % NSETS and event k % EV_RING
   static constexpr int EV_RING = 32;
-  cudaStream_t side[NSIDE] = {};
+  // two internal streams taken in turn: the LRFU kernels of consecutive layers do not depend on
+  // one another, so the second may fill SM room as the first one's CTAs finish
+  cudaStream_t side[2] = {};
   cudaEvent_t evA[EV_RING] = {}, evF[EV_RING] = {};
-  long long kF = 0, joined = -1;   // launches up to `joined` have been waited for on the stream joined_on
-  cudaStream_t joined_on = nullptr;
+  long long kF = 0, joined = -1;
   std::vector<long long> lastF;    // per layer: number of its latest LRFU launch, -1 = none
   int prev_layer = -1;             // layer of the launch pair issued last, -1 after any other call
   int stage = CRYSTALKV_STAGE_THINK;
@@ -341,20 +335,12 @@ int shrink_layers(crystalkv_t* h, int layer0, int count, int t_last, cudaStream_
   return CRYSTALKV_OK;
 }
 
-// Makes `s` wait for the LRFU kernels up to launch `target`: an internal stream runs in order, so its newest launch covers
-// the ones before.
-int wait_lrfu(crystalkv_t* h, long long target, cudaStream_t s) {
-  const long long from = std::max(s == h->joined_on ? h->joined : -1ll, target - crystalkv::NSIDE);
-  for (long long k = target; k > from; --k) CK(h, cudaStreamWaitEvent(s, h->evF[k % crystalkv::EV_RING], 0));
-  h->joined = target;
-  h->joined_on = s;
-  return CRYSTALKV_OK;
-}
-
 // Makes `s` wait for every LRFU kernel launched so far.
 int join_side(crystalkv_t* h, cudaStream_t s) {
   h->prev_layer = -1;
-  if (int rc = wait_lrfu(h, h->kF - 1, s)) return rc;
+  if (h->kF > 0) CK(h, cudaStreamWaitEvent(s, h->evF[(h->kF - 1) % crystalkv::EV_RING], 0));
+  if (h->kF > 1) CK(h, cudaStreamWaitEvent(s, h->evF[(h->kF - 2) % crystalkv::EV_RING], 0));   // the other internal stream
+  h->joined = h->kF - 1;
   if (h->nHost > 0) CK(h, cudaStreamWaitEvent(s, h->evOut[(h->nHost - 1) % crystalkv::HOST_RING], 0));   // copies back run in order
   return CRYSTALKV_OK;
 }
@@ -374,13 +360,17 @@ int launch_step(crystalkv_t* h, DecodeParams& p, int layer, cudaStream_t s) {
   const long long k = h->kF;
   {
     // launch k reuses the scratch of launch k - NSETS and continues the state its layer's
-    // previous LRFU launch wrote
+    // previous LRFU launch wrote; each internal stream runs in order, so the events of two
+    // consecutive launches cover everything before them
     // A wait on the caller's stream costs several microseconds (the attention kernel behind it
     // no longer starts early), so one wait covers as many launches as the sets allow: it targets
     // the newest LRFU launch that has had two attention kernels' time to finish.
     const long long need = std::max(k - NSETS, h->lastF[layer]);
     if (need >= 0 && need > h->joined) {
-      if (int rc = wait_lrfu(h, std::max(need, k - 1 - crystalkv::NSIDE), s)) return rc;
+      const long long target = std::max(need, k - 3);
+      CK(h, cudaStreamWaitEvent(s, h->evF[target % crystalkv::EV_RING], 0));
+      if (target > 0) CK(h, cudaStreamWaitEvent(s, h->evF[(target - 1) % crystalkv::EV_RING], 0));   // the other internal stream
+      h->joined = target;
     }
     p.sc.logits = h->sc_logits[k % NSETS];
     p.sc.mfin = h->sc_mfin[k % NSETS];
@@ -408,7 +398,7 @@ int launch_step(crystalkv_t* h, DecodeParams& p, int layer, cudaStream_t s) {
   }
   h->prev_layer = layer;
   {
-    const int si = (int)(k % crystalkv::NSIDE);
+    const int si = (int)(k & 1);
     cudaEvent_t ea = h->evA[k % crystalkv::EV_RING];
     p.sc.pbar = h->sc_pbar[si];
     p.done_ctr = h->done_ctr + 2 * si;
@@ -582,8 +572,8 @@ int crystalkv_create(const crystalkv_config_t* cfg, crystalkv_t** out) {
     a.add(&gpl, (size_t)c.n_layers * h->U);
     a.add(&hdr, (size_t)c.n_layers * 4);
     a.add(&h->d_plans, c.n_layers);
-    a.add(&h->done_ctr, 2 * crystalkv::NSIDE);   // per internal stream: finished CTAs of its running LRFU kernel; whether the layer's plan went stale
-    a.add(&h->plan_len, (size_t)crystalkv::NSIDE * (h->U + 1));
+    a.add(&h->done_ctr, 4);   // per internal stream: finished CTAs of its running LRFU kernel; whether the layer's plan went stale
+    a.add(&h->plan_len, (size_t)2 * (h->U + 1));
     a.add(&h->tab, (size_t)c.max_context + 1);
     a.add(&st.errword, 1);
     a.add(&st.counters, 4);
@@ -594,8 +584,8 @@ int crystalkv_create(const crystalkv_config_t* cfg, crystalkv_t** out) {
     for (int i = 0; i < 2; ++i) {
       a.add(&h->sc_partials[i], (size_t)h->U * h->pmax * (16 + h->G * HD));
       a.add(&h->sc_ticket[i], h->U);
+      a.add(&h->sc_pbar[i], (size_t)h->U * h->cap_s);
     }
-    for (float*& x : h->sc_pbar) a.add(&x, (size_t)h->U * h->cap_s);
     for (int i = 0; i < crystalkv::HOST_RING; ++i) {
       a.add(&h->dq[i], qn); a.add(&h->dout[i], qn); a.add(&h->dk[i], kn); a.add(&h->dv[i], kn);
     }
@@ -607,7 +597,7 @@ int crystalkv_create(const crystalkv_config_t* cfg, crystalkv_t** out) {
   }
   st.tab = h->tab;
   CKC(cudaMemset(hdr, 0, (size_t)c.n_layers * 4 * sizeof(int)));
-  CKC(cudaMemset(h->done_ctr, 0, 2 * crystalkv::NSIDE * sizeof(int)));
+  CKC(cudaMemset(h->done_ctr, 0, 4 * sizeof(int)));
   for (int i = 0; i < 2; ++i) CKC(cudaMemset(h->sc_ticket[i], 0, (size_t)h->U * sizeof(int)));
   h->plans.resize(c.n_layers);
   for (int l = 0; l < c.n_layers; ++l)
