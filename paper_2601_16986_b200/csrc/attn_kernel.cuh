@@ -221,7 +221,10 @@ __device__ __forceinline__ void merge_head(const DecodeParams& p, int u, int npi
 // SHARED: the launch consists of clusters that share a head each (plan.cuh).  Two instantiations: with both kinds in
 // one kernel the launches without clusters were slower (14B shape with unequal budgets 27.95 us a layer instead of
 // 27.74, 64 heads of 4097 entries 31.5 instead of 31.2, a short full cache 8.05 instead of 7.75).
-template <bool SHARED>
+// TRACK: Algorithm 1 follows, the step's logits and softmax references are left for it.  An instantiation of its own each way:
+// with the question asked at every group of keys a full cache of 128 heads of 9350 entries took 98.7 us a layer instead of 98.35, and steps
+// that track took 28.6 (64 heads of 4097 entries), 27.25 (8B shape with unequal budgets) and 26.45 (14B) instead of 28.3, 27.0 and 26.3.
+template <bool SHARED, bool TRACK>
 __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 registers: two LRFU CTAs fit beside it on an SM)
   extern __shared__ __align__(1024) unsigned char smem[];
   const State& st = p.st;
@@ -419,7 +422,7 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
         for (int x = 0; x < 4; ++x) s[x] += s2[x];
       }
       const bool v0 = gid < valid, v1 = gid + 8 < valid;
-      if (p.track) {
+      if (TRACK) {
         float* lrow = lrow0 + (size_t)base * QH;
         const uint64_t pol_keep = policy_evict_last();   // (one instruction: kept over the loop it cost a spilled register)
         if (v0) st_f32x2_hint(lrow, __fmul_rn(s[0], p.scale), __fmul_rn(s[1], p.scale), pol_keep);
@@ -495,7 +498,7 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
           ob[h1 * HD + 16 * mt + 8] = __float2bfloat16_rn(o[mt][3] * i1);
         }
       }
-      if (gid == 0 && p.track) {   // reference point and normaliser of the step's softmax, for the LRFU kernel
+      if (gid == 0 && TRACK) {   // reference point and normaliser of the step's softmax, for the LRFU kernel
         if (h0 < G) { p.sc.mfin[u * (2 * QH) + h0] = m0; p.sc.mfin[u * (2 * QH) + QH + h0] = ls0; }
         if (h1 < G) { p.sc.mfin[u * (2 * QH) + h1] = m1; p.sc.mfin[u * (2 * QH) + QH + h1] = ls1; }
       }
@@ -561,7 +564,7 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
         pk.x = pack_bf16(a.x * iv, a.y * iv);
         pk.y = pack_bf16(a.z * iv, a.w * iv);
         *reinterpret_cast<uint2*>(p.out + ((size_t)(u * G + g)) * HD + lane * 4) = pk;
-        if (lane == 0 && p.track) {
+        if (lane == 0 && TRACK) {
           p.sc.mfin[u * (2 * QH) + g] = m;
           p.sc.mfin[u * (2 * QH) + QH + g] = L;
         }
@@ -601,7 +604,7 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
           pk.x = pack_bf16(a.x * iv, a.y * iv);
           pk.y = pack_bf16(a.z * iv, a.w * iv);
           *reinterpret_cast<uint2*>(p.out + ((size_t)(u * G + g)) * HD + lane * 4) = pk;
-          if (lane == 0 && p.track) {
+          if (lane == 0 && TRACK) {
             p.sc.mfin[u * (2 * QH) + g] = m;
             p.sc.mfin[u * (2 * QH) + QH + g] = L;
           }

@@ -271,7 +271,7 @@ int find_clusters(crystalkv_t* h) {
     lc.attrs = at;
     lc.numAttrs = 1;
     int n = 0;
-    CK(h, cudaOccupancyMaxActiveClusters(&n, attn_kernel<true>, &lc));
+    CK(h, cudaOccupancyMaxActiveClusters(&n, attn_kernel<true, true>, &lc));
     h->share_ok[cl] = n >= h->U;
   }
   return CRYSTALKV_OK;
@@ -394,7 +394,9 @@ int launch_step(crystalkv_t* h, DecodeParams& p, int layer, cudaStream_t s) {
     at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
     lc.attrs = at;
     lc.numAttrs = p.cl > 1 ? 2 : 1;
-    CK(h, cudaLaunchKernelEx(&lc, p.cl > 1 ? attn_kernel<true> : attn_kernel<false>, p));
+    const auto attn = p.track ? (p.cl > 1 ? attn_kernel<true, true> : attn_kernel<false, true>)
+                              : (p.cl > 1 ? attn_kernel<true, false> : attn_kernel<false, false>);
+    CK(h, cudaLaunchKernelEx(&lc, attn, p));
   }
   h->prev_layer = layer;
   {
@@ -512,13 +514,13 @@ int crystalkv_create(const crystalkv_config_t* cfg, crystalkv_t** out) {
   // handle (the attribute belongs to the function, so no handle may lower it under another)
   h->smem = RING_BYTES + NW * STAGES * 8 + NW * FIFO * sizeof(int);
   int bps = 0;
-  for (auto attn : {attn_kernel<false>, attn_kernel<true>}) {
+  for (auto attn : {attn_kernel<false, false>, attn_kernel<true, false>, attn_kernel<false, true>, attn_kernel<true, true>}) {
     CKC(cudaFuncSetAttribute(attn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->smem));
     // The largest shared-memory carve-out, although the ring alone would fit a smaller one: the CTAs
     // of the LRFU kernel have to find room beside an attention CTA on the same SM.
     CKC(cudaFuncSetAttribute(attn, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
   }
-  CKC(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, attn_kernel<false>, NT, h->smem));
+  CKC(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, attn_kernel<false, true>, NT, h->smem));
   if (bps < 1) { h->err = "attention kernel does not fit on an SM"; CREATE_FAIL(CRYSTALKV_ECUDA); }
   h->grid = h->num_sms * bps;
   h->cl.assign(c.n_layers, 1);
