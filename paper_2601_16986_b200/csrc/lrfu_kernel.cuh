@@ -329,9 +329,9 @@ __global__ void __maxnreg__(48) lrfu_kernel(const __grid_constant__ DecodeParams
     }
   }
   if (!settled && threadIdx.x == NTH - 32) {   // no Algorithm 1: the head keeps its new entry
+    sh.is_last = settle_length(p, uid, seq, n, 0, g_plan);
     if (n > 1) count_unit(st, uid, n, 0, 0);
     else atomicOr(st.errword, ERR_EMPTY);   // the head has no entries and no page: nothing was attended
-    sh.is_last = settle_length(p, uid, seq, n, 0, g_plan);
   }
   __syncthreads();
   if (!sh.is_last) return;
