@@ -225,7 +225,7 @@ int crystalkv_time(crystalkv_t* h, int layer);
 /*
  * Bytes the Section 2.2 / Algorithm 1 data flow must move for the steps run so far:
  * *kv_bytes = sum over steps and heads of entries attended * 512 (K and V rows).
- * Synchronises `stream`; counters are kept on the device and cost one atomic per head.
+ * Synchronises `stream`; counters are kept on the device, per head, and cost a few additions without a result.
  */
 int crystalkv_get_counters(crystalkv_t* h, uint64_t* entries_attended, uint64_t* hits,
                            uint64_t* evictions, void* stream);

@@ -254,14 +254,4 @@ __device__ __forceinline__ Nucleus nucleus_find(int base, float top_p, NucleusSm
   return r;
 }
 
-template <int NTH, class Each>
-__device__ __forceinline__ Nucleus nucleus_search(int n, float top_p, NucleusSmem<NTH>& sh, int* errword, Each each) {
-  const int base = nucleus_base<NTH>(n);
-  nucleus_clear<NTH>(sh);
-  __syncthreads();
-  each([&](float pm) { nucleus_add<NTH>(sh, base, pm); });
-  __syncthreads();
-  return nucleus_find<NTH>(base, top_p, sh, errword, each, [] {});
-}
-
 }  // namespace ckv
