@@ -15,8 +15,8 @@
 //
 // Bound: latency, a chain of a dozen block-wide steps and dependent reads beside an attention kernel
 // that saturates HBM; the attention warps of the same SM feel its issue slots and loads.  256 heads of 512 .. 1536
-// entries: 22 us beside the attention kernel and 26.6 us a layer; with pbar in register arrays, a spilling path for
-// heads of more than ten entries per thread, counters shared by all heads and the heads counted last, 28 and 27.3.
+// entries: 22 us beside the attention kernel and 26.3 us a layer; with pbar in register arrays, a spilling path for
+// heads of more than ten entries per thread, counters shared by all heads and the heads counted last, 28 and 27.4.
 // (Sharing long heads among the CTAs of a cluster did not help: two to four
 // CTAs for heads of 4097 entries took 48 us beside the attention kernel instead of 56, and the layer
 // 36.3 us instead of 34.4; for heads of 1025 entries 17 us instead of 11.  Nor did fewer instructions by predicated loads at

@@ -15,9 +15,10 @@ constexpr int LRFU_SMALL = 64;   // threads of the CTAs for short heads
 //    of them fit beside an attention CTA instead of two of eight warps, most of which idle in the
 //    block-wide steps.  128 sequences of 8 heads of 257 entries: 27.8 us a layer instead of 38.7.
 //  * All other heads take CTAs of eight warps, two of which fit beside an attention CTA.  (Sixteen for heads of more than
-//    1280 entries make the kernel shorter and the layer longer, 64 heads of 4097 entries 33.0 us instead of 32.4,
-//    128 heads of 1024 .. 3072 entries 29.1 instead of 28.85: what counts is how hard a CTA presses on the attention
-//    warps of its SM.)
+//    1280 entries where every head finds an SM make the kernel shorter and the layer longer: what counts is how hard a CTA
+//    presses on the attention warps of its SM.  us a layer with sixteen and with eight, heads of 4097 entries: 16 heads 13.8 and
+//    13.7, 32 17.4 and 18.2, 44 23.1 and 22.4, 48 24.0 and 23.4, 64 29.9 and 28.2, 72 31.4 and 30.3, 96 43.1 and 42.4; 128 heads of 1024 ..
+//    3072 27.7 and 27.0, 64 of 1300 .. 3900 21.9 and 20.4, 32 of 2049 12.0 and 11.5.)
 inline int lrfu_threads(int U, int hint, bool uniform, int num_sms) {
   return uniform && hint <= FRONT * LRFU_SMALL && U > num_sms ? LRFU_SMALL : NT;
 }
