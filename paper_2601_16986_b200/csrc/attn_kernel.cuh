@@ -15,8 +15,10 @@
 // share the query heads.  A head of more than eight pieces is merged that way run by run (whole
 // CTAs and one shorter run) and its runs' partials through global memory: the warp whose ticket
 // completes the head merges them into `out`.  When there are few heads, a cluster of two or four
-// CTAs shares each of them: the CTAs merge their pieces as above and then one another's partials
-// through distributed shared memory.  Global memory also carries a head that the plan could not keep together
+// CTAs shares each of them: the CTAs merge their pieces as above and send each query head's partial into the shared
+// memory of the CTA that puts that head together, which waits for the bytes.  (Two cluster barriers around reads
+// of one another's memory held every CTA up twice, 1.3 us each: 32 heads of 1025 entries 9.15 us a layer instead of 8.3, 64 heads 11.05 instead
+// of 10.3, 64 heads of 4097 entries 28.25 instead of 27.2.)  Global memory also carries a head that the plan could not keep together
 // (after the warp's own pieces, if it has more).  The arriving token is written into the head's hole (the place
 // an evicted entry left, or the end of the list) by the warp that streams that group.  The scaled
 // logits of the step are left in the scratch for the LRFU kernel, which marks hits from the final
@@ -62,10 +64,16 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
 }
+// CLUSTER: what other CTAs of the cluster stored before the phase completed is visible, too.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;
-  asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-               : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+  if (CLUSTER)
+    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+  else
+    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
 }
 // Bulk copy global -> shared with an L2 eviction policy for the lines it touches: 16-byte aligned
@@ -96,13 +104,14 @@ __device__ __forceinline__ unsigned long long global_ns() {
 }
 // Waits for a stage's copy, for about a second at most: a copy that never lands raises the
 // error word instead of hanging the GPU.  Returns false on that time-out.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity) {
-  if (mbar_try_wait(bar, parity)) return true;
+  if (mbar_try_wait<CLUSTER>(bar, parity)) return true;
   const unsigned long long t0 = global_ns();
   for (;;) {
 #pragma unroll 1
     for (int i = 0; i < 64; ++i)
-      if (mbar_try_wait(bar, parity)) return true;
+      if (mbar_try_wait<CLUSTER>(bar, parity)) return true;
     if (global_ns() - t0 > 1000000000ull) return false;
   }
 }
@@ -116,6 +125,16 @@ __device__ __forceinline__ void bar_arrive(int id, int nthreads) {
 }
 
 constexpr int MAX_CLUSTER = 4;   // CTAs that may share a head
+
+// Shared memory of a CTA: the ring stages, one mbarrier per stage, every warp's queue of fetched pieces; in a launch whose
+// CTAs share heads also the place for the other CTAs' partials of the query heads that this one puts together: query
+// head g belongs to CTA g % ctas, as its g / ctas-th, and takes `ctas` slots of 128 floats, (m, l) and padding; one
+// mbarrier per such head counts the bytes.
+constexpr int ATTN_SMEM = RING_BYTES + NW * STAGES * 8 + NW * FIFO * (int)sizeof(int);
+constexpr int INBOX_SLOT = (HD + 4) * 4, INBOX_SLOTS = QH + 1;   // ceil(QH / ctas) x ctas is 9 at most
+constexpr int INBOX_BARS = QH / 2, INBOX_BYTES = (HD + 2) * 4;   // bytes that one CTA sends for a query head
+constexpr int ATTN_SMEM_SHARED = ATTN_SMEM + INBOX_SLOTS * INBOX_SLOT + INBOX_BARS * 8;
+static_assert(ATTN_SMEM % 16 == 0 && INBOX_SLOT % 16 == 0, "slots are written 16 bytes at a time");
 
 constexpr float LAZY = 8.0f;   // the running maximum (log2 domain) may trail the true one by this much
 
@@ -234,9 +253,15 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
   // ring stages, then one mbarrier per stage, then every warp's queue of fetched pieces
   const uint32_t bars_u32 = smem_u32(smem) + RING_BYTES;
   int* fifo = reinterpret_cast<int*>(smem + RING_BYTES + NW * STAGES * 8) + w * FIFO;
+  const uint32_t inbox_u32 = smem_u32(smem) + ATTN_SMEM, inbar_u32 = inbox_u32 + INBOX_SLOTS * INBOX_SLOT;
   if (tid < NW * STAGES) mbar_init(bars_u32 + tid * 8, 1);
-  asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");   // made visible to the copy engine
+  if (SHARED && tid < INBOX_BARS) mbar_init(inbar_u32 + tid * 8, 1);
+  asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");   // made visible to the copy engine and the cluster
   __syncthreads();
+  // The CTAs of a cluster meet twice without holding one another up: the first meeting (they have started, their
+  // barriers stand) is waited for before anything is sent, the second (everything has been sent) before the end.
+  if (SHARED) cluster_arrive();
+  auto meet_and_leave = [&] { cluster_wait(); cluster_arrive(); cluster_wait(); };   // of a warp that sends nothing
   const int4 range = __ldg(p.plan.wrange + blockIdx.x * NW + w);   // (requested together with the header)
   if (__ldg(p.plan.hdr + 2) != (int)gridDim.x * NW) {   // a plan made for another launch
     if (p.early) pdl_wait();
@@ -248,8 +273,8 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
     // for this one.  CTA 0 sees to that.)
     if (p.early && (SHARED || blockIdx.x == 0)) pdl_wait();
     if (SHARED) {
-      pdl_launch();                      // this CTA stays for the barriers: the next launch must not wait for its end
-      cluster_sync(); cluster_sync();    // (the two barriers of the CTAs that share the head)
+      pdl_launch();                      // this CTA stays for the meetings: the next launch must not wait for its end
+      meet_and_leave();
     }
     return;
   }
@@ -364,6 +389,14 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
         qb[ks][1] = (gid < G) ? q32[ks * 8 + tig + 4] : 0u;
       }
     }
+    // the arriving token: lane's 16 bytes of its K row (lanes 0..15) or V row (16..31).  With two or three groups a warp its
+    // round trip would show, so it is asked for beside the queries (64 heads of 1025 entries 10.3 us a layer instead of 10.4).
+    auto arriving = [&] {
+      const unsigned char* src = reinterpret_cast<const unsigned char*>(lane < 16 ? p.k_new : p.v_new) + (size_t)u * ROW_BYTES + (lane & 15) * 16;
+      return *reinterpret_cast<const uint4*>(src);
+    };
+    uint4 val_early = make_uint4(0, 0, 0, 0);
+    if (SHARED && hole >= lo * GRP && hole < hi * GRP) val_early = arriving();
     float o[8][4];
 #pragma unroll
     for (int mt = 0; mt < 8; ++mt) { o[mt][0] = 0.f; o[mt][1] = 0.f; o[mt][2] = 0.f; o[mt][3] = 0.f; }
@@ -380,7 +413,7 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
           if (s != csi) mbar_wait_bounded(bar0 + s * 8, (phases >> s) & 1u);
         if (local) bar_arrive(1 + first_w, 32 * rl);   // the run's other warps must not wait for this one
         __syncwarp();
-        if (SHARED) { cluster_sync(); cluster_sync(); }
+        if (SHARED) meet_and_leave();   // (what the others wait for does not come: they flag it and leave as well)
         return;
       }
       phases ^= 1u << csi;
@@ -388,11 +421,8 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
       const int base = ci * GRP;
       const int valid = min(GRP, n_tot - base);
       if (hole >= base && hole < base + GRP) {
-        // the arriving token: chunk `lane` of its K row (lanes 0..15) or V row (16..31) goes into the
-        // stage and into the head's page, at the place the hole has in both
-        const unsigned char* src = reinterpret_cast<const unsigned char*>(lane < 16 ? p.k_new : p.v_new) +
-                                   (size_t)u * ROW_BYTES + (lane & 15) * 16;
-        const uint4 val = *reinterpret_cast<const uint4*>(src);
+        // the arriving token goes into the stage and into the head's page, at the place the hole has in both
+        const uint4 val = SHARED ? val_early : arriving();
         const int off = chunk_offset(hole - base, lane);
         asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};\n" ::"r"(stage + off), "r"(val.x), "r"(val.y), "r"(val.z), "r"(val.w) : "memory");
         const int page = __ldg(st.ptab + (size_t)uid * st.capg + ci);
@@ -525,8 +555,8 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
       bar_sync(1 + first_w, 32 * rl);
       const unsigned char* base = smem + first_w * WSTRIDE;
       float* rpart = p.sc.partials + ((size_t)u * p.sc.pmax + (piece >> 3)) * PS;   // the run's partial (runs only)
-      constexpr int SHARE_AT = 8192, SHARE = (HD + 4) * 4;   // a shared head's partial of this CTA, query head g: at
-                                                             // SHARE_AT + g SHARE of the ring of warp g % rl
+      const int ctas = shared_head ? min(npieces, p.cl) : 1;   // those that have pieces of the head
+      if (shared_head) cluster_wait();                         // (they have all started)
       for (int g = jr; g < G; g += rl) {
         float pm[NW], pl[NW];
         float4 v[NW];
@@ -549,9 +579,10 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
           a.z = fmaf(v[j].z, c, a.z); a.w = fmaf(v[j].w, c, a.w);
         }
         if (shared_head) {
-          unsigned char* to = smem + w * WSTRIDE + SHARE_AT + g * SHARE;
-          *reinterpret_cast<float4*>(to + lane * 16) = a;
-          if (lane == 0) *reinterpret_cast<float2*>(to + HD * 4) = make_float2(m, L);
+          const int to = g % ctas, slot = g / ctas * ctas + cluster_rank();
+          const uint32_t at = peer_addr(inbox_u32 + slot * INBOX_SLOT, to), bar = peer_addr(inbar_u32 + g / ctas * 8, to);
+          push_f32x4(at + lane * 16, bar, a);
+          if (lane == 0) push_f32x2(at + HD * 4, bar, m, L);
           continue;
         }
         if (runs) {   // the run's share of the head, not normalised
@@ -570,24 +601,25 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
         }
       }
       if (shared_head) {
-        // every CTA's partials are written; query head g is put together by CTA g % (those that have pieces)
+        // this CTA's partials are on their way; its own query heads are put together as soon as theirs are complete
         __syncwarp();
-        cluster_sync();
-        const int ctas = min(npieces, p.cl);
-        for (int g = cluster_rank() + ctas * jr; g < G; g += ctas * rl) {
+        cluster_arrive();
+        for (int i = jr; cluster_rank() + ctas * i < G; i += rl) {
+          const int g = cluster_rank() + ctas * i;
+          if (lane == 0) mbar_expect_tx(inbar_u32 + i * 8, ctas * INBOX_BYTES);
+          if (!mbar_wait_bounded<true>(inbar_u32 + i * 8, 0)) {   // (a warp of the cluster has given up)
+            if (lane == 0) atomicOr(st.errword, ERR_COPY_TIMEOUT);
+            break;
+          }
           float4 v[MAX_CLUSTER];
           float2 ml[MAX_CLUSTER];
           float m = -INFINITY;
 #pragma unroll
           for (int x = 0; x < MAX_CLUSTER; ++x) {
-            ml[x] = make_float2(-INFINITY, 0.f);
-            v[x] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (x < ctas) {
-              const int n = shared_first(npieces, x + 1, p.cl) - shared_first(npieces, x, p.cl);   // pieces of CTA x
-              const uint32_t from = peer_addr(smem_u32(smem) + (g % n) * WSTRIDE + SHARE_AT + g * SHARE, x);
-              v[x] = peer_f32x4(from + lane * 16);
-              ml[x] = peer_f32x2(from + HD * 4);
-            }
+            const unsigned char* from = smem + ATTN_SMEM + (i * ctas + (x < ctas ? x : 0)) * INBOX_SLOT;
+            v[x] = *reinterpret_cast<const float4*>(from + lane * 16);
+            ml[x] = *reinterpret_cast<const float2*>(from + HD * 4);
+            if (x >= ctas) ml[x] = make_float2(-INFINITY, 0.f);
             m = fmaxf(m, ml[x].x);
           }
           float L = 0.f;
@@ -610,7 +642,7 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
           }
         }
         __syncwarp();
-        cluster_sync();   // nobody reads this CTA's shared memory any more
+        cluster_wait();   // (nothing is on its way any more, to this CTA or from it)
         return;           // (a warp has one piece of a shared head and nothing else)
       }
       if (!runs) continue;
@@ -663,7 +695,7 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
   if (defer0 >= 0) merge_head(p, defer0, __ldg(p.plan.npc + defer0), lane);
   if (defer1 >= 0) merge_head(p, defer1, __ldg(p.plan.npc + defer1), lane);
   __syncwarp();
-  if (SHARED) { cluster_sync(); cluster_sync(); }   // (a head that is one piece)
+  if (SHARED) meet_and_leave();   // (a head that is one piece)
 }
 
 }  // namespace ckv

@@ -34,7 +34,6 @@ using namespace ckv;
 struct crystalkv {
   crystalkv_config_t cfg;
   int G = 0, U = 0, units = 0, cap = 0, num_sms = 0, grid = 0;
-  size_t smem = 0;
   long long pages_per_seq = 0;
   State st{};
   std::vector<Plan> plans;         // per layer: the launch plan of its next attention kernel
@@ -263,7 +262,7 @@ int find_clusters(crystalkv_t* h) {
     cudaLaunchConfig_t lc{};
     lc.gridDim = dim3(h->U * cl);
     lc.blockDim = dim3(NT);
-    lc.dynamicSmemBytes = h->smem;
+    lc.dynamicSmemBytes = ATTN_SMEM_SHARED;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = cl;
@@ -277,30 +276,29 @@ int find_clusters(crystalkv_t* h) {
   return CRYSTALKV_OK;
 }
 
-// CTAs that share a head of `entries` entries: the most, up to MAX_CLUSTER, for which there is room
-// (find_clusters), where the launch is bound by its chain of dependent steps (pieces of at most GLAT groups) and
-// sharing shortens that chain enough: every warp streams at least four groups less, or three if the handle
-// has one layer (a launch that cannot start early gains the whole difference).  Below that the wider merge and the
-// launch of clusters cost more than they save.  us a layer, shared and not: 48 layers of 32 heads, four CTAs: of 29
-// groups 7.9 and 6.65, of 41 groups 8.1 and 8.8, of 65 groups 9.9 and 11.2; 64 heads, two CTAs: of 41 groups 9.3 and
-// 9.3, of 57 groups 10.5 and 12.0.  One layer of 2 heads, four CTAs: of 29 groups 10.8 and 10.95, of 33 groups 10.7 and
-// 11.4.
+// CTAs that share a head of `entries` entries, where there is room for a cluster per head (find_clusters): a launch bound by
+// its chain of dependent steps (pieces of at most GLAT groups) gains what its warps stream less, a group being worth
+// about 0.4 us and the wider merge as much.  us a layer on one CTA, two and four: 24 layers of 32 heads of 25 groups 6.3, 6.1, 7.0; of 38
+// 7.4, 6.6, 6.9; of 50 9.1, 7.5, 7.4; of 65 10.6, 8.5, 8.3; 64 heads of 25 groups 7.1 and 7.2, of 30 7.3 and 7.0, of 65 12.55 and 10.1;
+// 16 heads of 25 groups 6.1, 7.1, 6.0, of 42 7.9, 6.3, 6.0; one layer of 2 heads of 17 groups 16.4 each way, of 21 18.1, 16.7, 16.5, of 38
+// 19.3, 17.3, 16.9.  So two CTAs from two groups a warp on (one, if the handle has one layer: its launches cannot start
+// early), four where that is two groups less again, or one while the CTAs do not fill half the SMs.  A handle of
+// two layers keeps the line of four groups (40 groups, 2 heads 10.3, 9.4, 8.4: its launch shapes are stated by a test).
 // Longer heads of one length (from 193 groups, where they no longer fit a CTA in pieces of 2 GLAT) gain from two CTAs where their
-// other choice is more than eight pieces and a merge through global memory at the end of the launch. The longer the pieces,
-// the more the CTAs that then have nothing to stream count: up to 14 groups a piece from 45 heads on, up to 24 from 52.  us a
-// layer, shared and not, of 193, 225, 257, 288, 313, 345 and 376 groups: 48 heads 19.8 22.2 24.2 25.9 27.8 30.0 31.9 and 21.9 22.3 23.6
-// 25.4 27.5 29.8 32.0; 52 heads 20.3 22.8 25.1 27.1 29.1 31.2 34.1 and 22.6 22.9 25.5 27.9 29.9 32.4 35.5; 64 heads 22.4 25.9 28.5 31.3
-// 33.5 36.7 39.9 and 27.3 31.2 29.6 32.3 34.5 37.3 40.2; 72 heads 23.8 27.5 30.5 33.5 36.2 39.3 42.8 and 28.7 32.4 36.4 39.6 43.0 46.5 50.2.
+// other choice is more than eight pieces and a merge through global memory at the end of the launch.  The longer the pieces,
+// the more the CTAs that then have nothing to stream count: up to 14 groups a piece below 43 heads.  us a layer, not shared and
+// shared, of 194, 226, 257, 313 and 376 groups: 40 heads 20.7 20.1 20.9 24.9 34.1 and 17.7 19.7 21.5 24.9 28.7; 44 heads 21.0 20.7 22.3 27.6
+// 35.4 and 18.0 20.0 21.9 25.3 29.5; 52 heads 22.2 22.4 25.0 29.4 37.4 and 18.5 21.1 23.5 27.6 35.1.
 int share_heads(crystalkv_t* h, int entries) {
   const int g = (entries + GRP - 1) / GRP, alone = (g + NW - 1) / NW;
-  for (int cl = MAX_CLUSTER; cl > 1; cl /= 2) {
-    const int per = (g + NW * cl - 1) / (NW * cl);
-    const int most = 20 * h->U >= 7 * h->num_sms ? 2 * GLAT : GLAT + 2;
-    const bool merge = cl == 2 && h->uniform && 10 * h->U >= 3 * h->num_sms && alone > 2 * GLAT && per <= most;
-    if (h->share_ok[cl] && (per <= GLAT || merge) && alone - per >= (h->cfg.n_layers > 1 ? 4 : 3)) return cl;
-  }
-  return 1;
+  auto per = [&](int cl) { return (g + NW * cl - 1) / (NW * cl); };
+  const bool merge = h->uniform && alone > 2 * GLAT && per(2) <= (7 * h->U >= 2 * h->num_sms ? 2 * GLAT : GLAT + 2);
+  const int least = h->cfg.n_layers == 2 ? 4 : h->cfg.n_layers == 1 ? 1 : 2;
+  auto pays = [&](int cl) { return h->share_ok[cl] && (per(cl) <= GLAT || (cl == 2 && merge)) && alone - per(cl) >= least; };
+  if (pays(4) && (!pays(2) || per(2) - per(4) >= (8 * h->U <= h->num_sms ? 1 : 2))) return 4;
+  return pays(2) ? 2 : 1;
 }
+static_assert(MAX_CLUSTER == 4, "share_heads weighs two CTAs and four");
 
 // Writes the launch plans of `count` layers from their heads' current lengths, on `s`; the layers share heads alike.
 int replan(crystalkv_t* h, int layer0, int count, cudaStream_t s) {
@@ -384,7 +382,7 @@ int launch_step(crystalkv_t* h, DecodeParams& p, int layer, cudaStream_t s) {
     cudaLaunchConfig_t lc{};
     lc.gridDim = dim3(p.plan_grid);
     lc.blockDim = dim3(NT);
-    lc.dynamicSmemBytes = h->smem;
+    lc.dynamicSmemBytes = p.cl > 1 ? ATTN_SMEM_SHARED : ATTN_SMEM;
     lc.stream = s;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -409,7 +407,7 @@ int launch_step(crystalkv_t* h, DecodeParams& p, int layer, cudaStream_t s) {
     CK(h, cudaStreamWaitEvent(h->side[si], ea, 0));
     const int threads = p.track ? lrfu_threads(h->U, entries, h->uniform, h->num_sms) : LRFU_SMALL;
     p.front = std::min(h->cap_s, h->uniform ? entries : std::min(p.t + 1, FRONT * threads));
-    const int npb = std::min(std::min(h->cap, p.t + 1), pbar_room(threads, h->U, entries, h->num_sms));
+    const int npb = std::min(std::min(h->cap, p.t + 1), pbar_room(threads, h->U, entries, h->num_sms, p.cl > 1));
     CK(h, lrfu_launch(threads, npb, h->G, p, h->U, h->side[si]));
     CK(h, cudaEventRecord(h->evF[k % crystalkv::EV_RING], h->side[si]));
     h->lastF[layer] = k;
@@ -510,17 +508,16 @@ int crystalkv_create(const crystalkv_config_t* cfg, crystalkv_t** out) {
   DeviceScope scope(c.device);
   CKC(scope.err);
   CKC(cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, c.device));
-  // ring stages, one mbarrier per stage, every warp's queue of fetched pieces: the same for every
-  // handle (the attribute belongs to the function, so no handle may lower it under another)
-  h->smem = RING_BYTES + NW * STAGES * 8 + NW * FIFO * sizeof(int);
   int bps = 0;
   for (auto attn : {attn_kernel<false, false>, attn_kernel<true, false>, attn_kernel<false, true>, attn_kernel<true, true>}) {
-    CKC(cudaFuncSetAttribute(attn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->smem));
+    // (the same for every handle: the attribute belongs to the function, so no handle may lower it under another)
+    const bool shared = attn == attn_kernel<true, false> || attn == attn_kernel<true, true>;
+    CKC(cudaFuncSetAttribute(attn, cudaFuncAttributeMaxDynamicSharedMemorySize, shared ? ATTN_SMEM_SHARED : ATTN_SMEM));
     // The largest shared-memory carve-out, although the ring alone would fit a smaller one: the CTAs
     // of the LRFU kernel have to find room beside an attention CTA on the same SM.
     CKC(cudaFuncSetAttribute(attn, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
   }
-  CKC(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, attn_kernel<false, true>, NT, h->smem));
+  CKC(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, attn_kernel<false, true>, NT, ATTN_SMEM));
   if (bps < 1) { h->err = "attention kernel does not fit on an SM"; CREATE_FAIL(CRYSTALKV_ECUDA); }
   h->grid = h->num_sms * bps;
   h->cl.assign(c.n_layers, 1);

@@ -24,12 +24,13 @@ inline int lrfu_threads(int U, int hint, bool uniform, int num_sms) {
 }
 
 // Entries whose pbar a CTA keeps in shared memory (longer heads use the global scratch).  Beside an attention CTA an SM
-// has 34 KB left: room for six CTAs of LRFU_SMALL, two of NT, or one of NT for long heads that find an SM each.
+// has 34 KB left, 30 KB beside one that shares heads: room for six CTAs of LRFU_SMALL, two of NT, or one of NT for long heads
+// that find an SM each.
 // (One of NT for few heads of any length: 64 heads of 128 .. 2000 entries 11.55 us a layer instead of 11.3.)
-constexpr int PBAR_TWO = 1856, PBAR_ONE = 5632;
-inline int pbar_room(int threads, int U, int hint, int num_sms) {
+inline int pbar_room(int threads, int U, int hint, int num_sms, bool shared) {
   if (threads == LRFU_SMALL) return FRONT * LRFU_SMALL;
-  return hint > PBAR_TWO && U <= num_sms ? PBAR_ONE : PBAR_TWO;
+  const int two = shared ? 1440 : 1856, one = shared ? 5248 : 5632;
+  return hint > two && U <= num_sms ? one : two;
 }
 
 // Launches the kernel for `heads` heads; threads: LRFU_SMALL or NT; npb: entries whose pbar fits shared memory.
