@@ -83,8 +83,16 @@ typedef struct {
  */
 int crystalkv_create(const crystalkv_config_t* cfg, crystalkv_t** out);
 
-/* Frees everything the handle owns.  NULL is accepted. */
+/*
+ * Frees the handle, once its device is idle.  NULL is accepted.  What the handle had of its device (memory, streams, events)
+ * may be kept for the next handle on it: one set per device, of at most 8 GiB, and only while a
+ * quarter of the device's memory is free.  A later handle that it does not fit, a failing allocation of this library, or
+ * crystalkv_trim gives it back.
+ */
 int crystalkv_destroy(crystalkv_t* h);
+
+/* Gives back what destroyed handles left on the device.  May be called from any thread.  Errors: EINVAL, ECUDA. */
+int crystalkv_trim(int device);
 
 /*
  * Loads a prompt into one layer (Algorithm 1 inputs K/V, Q^last) and runs one

@@ -81,6 +81,7 @@ def load_library():
     vp, i32, p32 = C.c_void_p, C.c_int, C.POINTER(C.c_int32)
     lib.crystalkv_create.argtypes = [C.POINTER(_Cfg), C.POINTER(vp)]
     lib.crystalkv_destroy.argtypes = [vp]
+    lib.crystalkv_trim.argtypes = [i32]
     lib.crystalkv_prefill.argtypes = [vp, i32, vp, vp, vp, i32, vp]
     lib.crystalkv_prefill_window.argtypes = [vp, i32, vp, vp, vp, i32, i32, vp, vp]
     lib.crystalkv_decode_step.argtypes = [vp, i32, vp, vp, vp, vp, vp]
@@ -109,6 +110,13 @@ def load_library():
     lib.crystalkv_last_error.restype = C.c_char_p
     _lib = lib
     return lib
+
+
+def trim(device: int = 0):
+    """Gives back the device memory that closed handles left for the next one."""
+    rc = load_library().crystalkv_trim(device)
+    if rc:
+        raise CrystalKVError(rc, load_library().crystalkv_strerror(rc).decode())
 
 
 def _stream():

@@ -11,6 +11,8 @@
 // event.  Everything else (prefill, reallocation, inspection) first joins the internal stream.
 #include "../../include/crystalkv.h"
 
+#include <cuda.h>
+
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -31,7 +33,24 @@
 
 using namespace ckv;
 
-struct crystalkv {
+// What a handle has of its device: its memory, streams and events.
+struct DeviceKit {
+  void* arena = nullptr;           // the one device allocation that all arrays of the handle lie in
+  size_t arena_bytes = 0;
+  // LRFU launches are numbered; launch k uses scratch set k % NSETS and event k % EV_RING
+  static constexpr int EV_RING = 32;
+  // two internal streams taken in turn: the LRFU kernels of consecutive layers do not depend on
+  // one another, so the second may fill SM room as the first one's CTAs finish
+  cudaStream_t side[2] = {};
+  cudaEvent_t evA[EV_RING] = {}, evF[EV_RING] = {};
+  // host I/O: HOST_RING staging sets; inputs go up on one internal stream and results come
+  // down on another, so the copies of other layers run beside the attention kernels
+  static constexpr int HOST_RING = 64;
+  cudaStream_t copy_in = nullptr, copy_out = nullptr;
+  cudaEvent_t evIn[HOST_RING] = {}, evUse[HOST_RING] = {}, evOut[HOST_RING] = {};
+};
+
+struct crystalkv : DeviceKit {
   crystalkv_config_t cfg;
   int G = 0, U = 0, units = 0, cap = 0, num_sms = 0, grid = 0;
   long long pages_per_seq = 0;
@@ -51,13 +70,7 @@ struct crystalkv {
   int cap_s = 0, pmax = 0;
   long long nA = 0;                // attention launches so far
   std::vector<int> t_layer;        // per layer: time of the last step
-  // LRFU launches are numbered; launch k uses scratch set k % NSETS and event k % EV_RING
-  static constexpr int EV_RING = 32;
-  // two internal streams taken in turn: the LRFU kernels of consecutive layers do not depend on
-  // one another, so the second may fill SM room as the first one's CTAs finish
-  cudaStream_t side[2] = {};
-  cudaEvent_t evA[EV_RING] = {}, evF[EV_RING] = {};
-  long long kF = 0, joined = -1;
+  long long kF = 0, joined = -1;   // LRFU launches so far
   std::vector<long long> lastF;    // per layer: number of its latest LRFU launch, -1 = none
   int prev_layer = -1;             // layer of the launch pair issued last, -1 after any other call
   int stage = CRYSTALKV_STAGE_THINK;
@@ -71,12 +84,7 @@ struct crystalkv {
   // Entries of a head in a decode step of the layer (as len_cap) that brings the tokens so far to `tokens`.
   int entries(int layer, int tokens) const { return cfg.mode == CRYSTALKV_MODE_EVICT ? std::min(len_cap[layer], tokens) : tokens; }
   long long* Asum = nullptr;
-  // host I/O: HOST_RING staging sets; inputs go up on one internal stream and results come
-  // down on another, so the copies of other layers run beside the attention kernels
-  static constexpr int HOST_RING = 64;
   __nv_bfloat16 *dq[HOST_RING] = {}, *dk[HOST_RING] = {}, *dv[HOST_RING] = {}, *dout[HOST_RING] = {};
-  cudaStream_t copy_in = nullptr, copy_out = nullptr;
-  cudaEvent_t evIn[HOST_RING] = {}, evUse[HOST_RING] = {}, evOut[HOST_RING] = {};
   long long outJoined = -1;   // newest host step whose copy back the caller's stream has waited for
   long long nHost = 0;             // host-buffer steps so far
   int* io_rec = nullptr;           // staging for export / import of one head: records, rows, count
@@ -84,7 +92,6 @@ struct crystalkv {
   int* io_n = nullptr;
   unsigned long long* io_sum = nullptr;   // ... and for the counters
   float* tab = nullptr;
-  void* arena = nullptr;           // the one device allocation all of the above point into
   std::string err;
   bool cuda_dead = false;
 };
@@ -135,6 +142,83 @@ struct DeviceScope {
   DeviceScope dev_scope_((h)->cfg.device); \
   CK((h), dev_scope_.err)
 
+// ---- what a destroyed handle leaves for the next one
+// A server makes a handle for a new batch and frees it again and again.  Taking and giving back 5.5 GB costs 1.05 and 3.2 ms,
+// the streams and events another half, as much as all else: a new batch of 16 prompts of 512 tokens in the 8B shape, 1.9 ms of
+// kernels, took 6.7 ms and takes 1.8 to 2.0 with them kept (8 prompts of 9350 tokens 5.6 and 3.4 to 3.9, windows of 32 12.4 and 8.4 to 9.2).  So a device keeps at most one kit, of at most KEEP_BYTES, and that only
+// while a quarter of its memory is free; crystalkv_trim, a handle that it does not fit and an allocation
+// that fails for want of memory give it back.  (A pool of the driver's gives back by itself, but its first 5.5 GB took 34 to 280 ms.)
+constexpr size_t KEEP_BYTES = size_t(8) << 30;
+struct Kept {
+  DeviceKit kit;
+  unsigned long long context = 0;   // of the CUDA context that the kit belongs to (a device reset ends it); 0: nothing is kept
+};
+Kept g_kept[MAX_DEVICES];
+std::mutex g_kept_mu;
+
+unsigned long long context_id() {   // of the current context, 0: unknown
+  using Fn = CUresult (*)(CUcontext, unsigned long long*);
+  static const Fn fn = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult r;
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &r) != cudaSuccess || r != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      p = nullptr;
+    }
+    return reinterpret_cast<Fn>(p);
+  }();
+  unsigned long long id = 0;
+  return fn && fn(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+void free_kit(DeviceKit& k) {
+  for (cudaStream_t x : {k.side[0], k.side[1], k.copy_in, k.copy_out})
+    if (x) cudaStreamDestroy(x);
+  for (auto* ring : {k.evIn, k.evUse, k.evOut})
+    for (int i = 0; i < DeviceKit::HOST_RING; ++i)
+      if (ring[i]) cudaEventDestroy(ring[i]);
+  for (auto* ring : {k.evA, k.evF})
+    for (int i = 0; i < DeviceKit::EV_RING; ++i)
+      if (ring[i]) cudaEventDestroy(ring[i]);
+  if (k.arena) cudaFree(k.arena);
+  k = DeviceKit{};
+}
+
+// The kit that the current device keeps, if it belongs to the current context, taken out; an empty one else.
+DeviceKit take_kept(int device) {
+  std::lock_guard<std::mutex> lock(g_kept_mu);
+  Kept& k = g_kept[device];
+  DeviceKit kit;
+  if (k.context && k.context == context_id()) std::swap(kit, k.kit), k.context = 0;
+  return kit;
+}
+
+// Keeps a complete kit that no work on the device uses any more.  False: it is the caller's to free.
+bool keep_kit(int device, const DeviceKit& kit) {
+  if (!kit.arena || kit.arena_bytes > KEEP_BYTES || !kit.evF[DeviceKit::EV_RING - 1]) return false;   // (the last to be made)
+  size_t room = 0, total = 0;
+  if (cudaMemGetInfo(&room, &total) != cudaSuccess) { cudaGetLastError(); return false; }
+  if (room < total / 4) return false;
+  std::lock_guard<std::mutex> lock(g_kept_mu);
+  Kept& k = g_kept[device];
+  const unsigned long long id = context_id();
+  if (k.context || !id) return false;
+  k.kit = kit;
+  k.context = id;
+  return true;
+}
+
+// cudaMalloc that gives back what the device keeps if there is not enough memory.
+cudaError_t device_malloc(int device, void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaErrorMemoryAllocation) return e;
+  DeviceKit kit = take_kept(device);
+  if (!kit.arena) return e;
+  cudaGetLastError();
+  free_kit(kit);
+  return cudaMalloc(p, bytes);
+}
+
 // A handle's device arrays are parts of one allocation.  Some 330 separate ones (staging sets, logit
 // sets, lists) cost a handle of the 8B shape (5.5 GB) 16 ms to take and 16 ms to give back, against
 // 0.5 and 2.3 ms for one of the same total size.
@@ -147,19 +231,42 @@ struct Arena {
     parts.push_back({reinterpret_cast<void**>(p), bytes});
     bytes += (std::max<size_t>(count, 1) * sizeof(T) + 255) / 256 * 256;   // every array starts on a 256-byte boundary
   }
+  // The handle's kit: the kept one if its memory is enough and at most twice as much, else a new one.
   int take(crystalkv_t* h) {
-    void* base = nullptr;
-    cudaError_t e = cudaMalloc(&base, bytes);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      return fail(h, e == cudaErrorMemoryAllocation ? CRYSTALKV_ENOMEM : CRYSTALKV_ECUDA,
-                  std::string("cudaMalloc: ") + cudaGetErrorString(e));
+    DeviceKit& kit = *h;
+    kit = take_kept(h->cfg.device);
+    if (kit.arena && (kit.arena_bytes < bytes || kit.arena_bytes / 2 > bytes)) free_kit(kit);
+    if (!kit.arena) {
+      const cudaError_t e = device_malloc(h->cfg.device, &kit.arena, bytes);
+      if (e != cudaSuccess) {
+        cudaGetLastError();
+        return fail(h, e == cudaErrorMemoryAllocation ? CRYSTALKV_ENOMEM : CRYSTALKV_ECUDA,
+                    std::string("cudaMalloc: ") + cudaGetErrorString(e));
+      }
+      kit.arena_bytes = bytes;
     }
-    h->arena = base;
-    for (const Part& x : parts) *x.where = static_cast<unsigned char*>(base) + x.at;
+    for (const Part& x : parts) *x.where = static_cast<unsigned char*>(kit.arena) + x.at;
     return CRYSTALKV_OK;
   }
 };
+
+// Streams and events of a kit that has none yet.
+cudaError_t make_streams(DeviceKit& k) {
+  if (k.side[0]) return cudaSuccess;
+  // The LRFU kernels run at the highest stream priority: the attention kernel of the layer after
+  // next is already queued when one of them becomes ready (it was released early and waits for
+  // shared memory), and at equal priority its CTAs, which cannot be placed yet, are served first.
+  int least = 0, greatest = 0;
+  cudaError_t e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
+  for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = cudaStreamCreateWithPriority(&k.side[i], cudaStreamNonBlocking, greatest);
+  for (cudaStream_t* x : {&k.copy_in, &k.copy_out})
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(x, cudaStreamNonBlocking);
+  for (auto* ring : {k.evIn, k.evUse, k.evOut})
+    for (int i = 0; i < DeviceKit::HOST_RING && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&ring[i], cudaEventDisableTiming);
+  for (auto* ring : {k.evA, k.evF})
+    for (int i = 0; i < DeviceKit::EV_RING && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&ring[i], cudaEventDisableTiming);
+  return e;
+}
 
 __global__ void init_free_stack_kernel(int* stack, int* top, long long pages_per_seq, int batch) {
   const long long total = pages_per_seq * batch;
@@ -437,22 +544,18 @@ const char* crystalkv_last_error(crystalkv_t* h) { return h ? h->err.c_str() : g
 int crystalkv_destroy(crystalkv_t* h) {
   if (!h) return CRYSTALKV_OK;
   DeviceScope scope(h->cfg.device);
-  cudaDeviceSynchronize();
-  for (cudaStream_t x : h->side)
-    if (x) cudaStreamDestroy(x);
-  if (h->copy_in) cudaStreamDestroy(h->copy_in);
-  if (h->copy_out) cudaStreamDestroy(h->copy_out);
-  for (int i = 0; i < crystalkv::HOST_RING; ++i) {
-    if (h->evIn[i]) cudaEventDestroy(h->evIn[i]);
-    if (h->evUse[i]) cudaEventDestroy(h->evUse[i]);
-    if (h->evOut[i]) cudaEventDestroy(h->evOut[i]);
-  }
-  for (cudaEvent_t e : h->evA)
-    if (e) cudaEventDestroy(e);
-  for (cudaEvent_t e : h->evF)
-    if (e) cudaEventDestroy(e);
-  if (h->arena) cudaFree(h->arena);
+  const bool idle = cudaDeviceSynchronize() == cudaSuccess && !h->cuda_dead;
+  if (!idle || !keep_kit(h->cfg.device, *h)) free_kit(*h);
   delete h;
+  return CRYSTALKV_OK;
+}
+
+int crystalkv_trim(int device) {
+  if (device < 0 || device >= MAX_DEVICES) return CRYSTALKV_EINVAL;
+  DeviceScope scope(device);
+  if (scope.err != cudaSuccess) return CRYSTALKV_ECUDA;
+  DeviceKit kit = take_kept(device);
+  free_kit(kit);
   return CRYSTALKV_OK;
 }
 
@@ -523,24 +626,6 @@ int crystalkv_create(const crystalkv_config_t* cfg, crystalkv_t** out) {
   h->cl.assign(c.n_layers, 1);
   h->len_cap.assign(c.n_layers, c.budget_per_head + c.evict_every);
   if (int r = find_clusters(h)) CREATE_FAIL(r);
-  {
-    // The LRFU kernels run at the highest stream priority: the attention kernel of the layer after
-    // next is already queued when one of them becomes ready (it was released early and waits for
-    // shared memory), and at equal priority its CTAs, which cannot be placed yet, are served first.
-    int least = 0, greatest = 0;
-    CKC(cudaDeviceGetStreamPriorityRange(&least, &greatest));
-    for (cudaStream_t& x : h->side) CKC(cudaStreamCreateWithPriority(&x, cudaStreamNonBlocking, greatest));
-  }
-  CKC(cudaStreamCreateWithFlags(&h->copy_in, cudaStreamNonBlocking));
-  CKC(cudaStreamCreateWithFlags(&h->copy_out, cudaStreamNonBlocking));
-  for (int i = 0; i < crystalkv::HOST_RING; ++i) {
-    CKC(cudaEventCreateWithFlags(&h->evIn[i], cudaEventDisableTiming));
-    CKC(cudaEventCreateWithFlags(&h->evUse[i], cudaEventDisableTiming));
-    CKC(cudaEventCreateWithFlags(&h->evOut[i], cudaEventDisableTiming));
-  }
-  for (cudaEvent_t& e : h->evA) CKC(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-  for (cudaEvent_t& e : h->evF) CKC(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-
   State& st = h->st;
   st.batch = c.batch; st.L = c.n_layers; st.H = c.n_kv_heads; st.cap = h->cap; st.capg = h->cap / GRP;
   st.pages_per_seq = h->pages_per_seq;
@@ -593,6 +678,7 @@ int crystalkv_create(const crystalkv_config_t* cfg, crystalkv_t** out) {
     a.add(&h->io_n, 1);
     a.add(&h->io_sum, 4);
     if (int r = a.take(h)) CREATE_FAIL(r);
+    CKC(make_streams(*h));
   }
   st.tab = h->tab;
   CKC(cudaMemset(hdr, 0, (size_t)c.n_layers * 4 * sizeof(int)));
@@ -1099,7 +1185,7 @@ int crystalkv_validate(crystalkv_t* h, void* stream) {
   if (int jr = join_side(h, s)) return jr;
   const long long total = (long long)c.batch * h->pages_per_seq;
   int* seen = nullptr;
-  CK(h, cudaMalloc(&seen, (size_t)(total + 2) * sizeof(int)));
+  CK(h, device_malloc(c.device, reinterpret_cast<void**>(&seen), (size_t)(total + 2) * sizeof(int)));
   cudaError_t e = cudaMemsetAsync(seen, 0, (size_t)(total + 2) * sizeof(int), s);
   if (e == cudaSuccess) {
     mark_free_kernel<<<dim3(256, c.batch), 256, 0, s>>>(h->st, seen);
