@@ -450,6 +450,37 @@ int join_side(crystalkv_t* h, cudaStream_t s) {
   return CRYSTALKV_OK;
 }
 
+// A tensor map of bf16 in boxes of `box`, zeros beyond the ends.
+bool tensor_map(CUtensorMap* m, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box,
+                CUtensorMapSwizzle swizzle) {
+  using Fn = decltype(&cuTensorMapEncodeTiled);
+  static const Fn encode = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult r;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &r) != cudaSuccess || r != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      p = nullptr;
+    }
+    return reinterpret_cast<Fn>(p);
+  }();
+  const cuuint32_t step[4] = {1, 1, 1, 1};
+  return encode && encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(base), dims, strides, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                          swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+// The tokens of a prompt as tiles: [batch][P][H][128] in boxes of 64 channels x WA_KEYS tokens of one head.
+bool tile_map(CUtensorMap* m, const void* base, int batch, int P, int H) {
+  const cuuint64_t dims[4] = {HD, (cuuint64_t)H, (cuuint64_t)P, (cuuint64_t)batch};
+  const cuuint64_t strides[3] = {ROW_BYTES, (cuuint64_t)H * ROW_BYTES, (cuuint64_t)P * H * ROW_BYTES};
+  const cuuint32_t box[4] = {HD / 2, 1, WA_KEYS, 1};
+  return tensor_map(m, base, 4, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
+}
+// The pool as quarters of entries, in boxes of a page's.
+bool pool_map(CUtensorMap* m, const crystalkv_t* h) {
+  const cuuint64_t dims[3] = {HD / 2, 4, (cuuint64_t)h->cfg.batch * h->pages_per_seq * GRP}, strides[2] = {SLOT_BYTES / 4, SLOT_BYTES};
+  const cuuint32_t box[3] = {HD / 2, 1, GRP};
+  return tensor_map(m, h->st.pool, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE);
+}
+
 // One attention launch on `s` and its follow-up (Algorithm 1 when it runs, the heads' new lengths
 // and the layer's next plan) on the internal stream.
 int launch_step(crystalkv_t* h, DecodeParams& p, int layer, cudaStream_t s) {
@@ -735,11 +766,10 @@ int crystalkv_time(crystalkv_t* h, int layer) {
   return h->t_layer[layer];
 }
 
-// Queries of a window over P tokens that one launch replays: what the logit sets, the partials and the pbar area have room for.
+// Queries of a window over P tokens that one launch replays: what the logit sets and the pbar area have room for.
 static int window_queries(const crystalkv_t* h, int P) {
   const long long rows = (P + 7) / 8 * 8, words = (P + 31) / 32;
-  return (int)std::max<long long>(1, std::min({(long long)NSETS * h->cap_s * QH / (h->G * rows),
-                                               (long long)h->pmax * (16 + h->G * HD) / 16, h->cap_s / words, 1ll << 30}));
+  return (int)std::max<long long>(1, std::min({(long long)NSETS * h->cap_s * QH / rows, h->cap_s / words, 1ll << 30}));
 }
 
 // Whether a window's attention kernel also fills the pages, from the tiles it reads: where its last launch has a CTA for four
@@ -751,31 +781,31 @@ static int window_queries(const crystalkv_t* h, int P) {
 // and 51.5, 2 heads of 512 tokens, 4 queries, 51.5 and 51.6, 16 heads of 1024 tokens, 8 queries, 86 and 74.
 static bool window_fills_pages(const crystalkv_t* h, int P, int W) {
   const int last = (W - 1) % window_queries(h, P) + 1;
-  return P <= 512 || 5ll * h->U * ((last * h->G + WA_ROWS - 1) / WA_ROWS) >= 4ll * h->num_sms;
+  return P <= 512 || 5ll * h->U * window_blocks(last, h->G) >= 4ll * h->num_sms;
 }
 
 // Algorithm 1 with the queries of the prompt's last W tokens, in as many launches as the scratch
 // asks for (usually one): steps 1-3 for every query, step 4 after the last one.  Everything runs on
 // `s`, which has joined the internal streams: the logit sets, one block of the arena, hold the
-// window's logits, the partials its softmax references, the first pbar area the hit bits.
+// window's group means, the first pbar area the hit bits.
 static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, const unsigned char* v, const unsigned char* q,
                          int P, int W, __nv_bfloat16* out, bool fill_pages, cudaStream_t s) {
   const crystalkv_config_t& c = h->cfg;
   WindowParams p{};
   p.k = k; p.v = v;
-  p.logits = h->sc_logits[0];
-  p.ml = h->sc_partials[0];
+  p.pbar = h->sc_logits[0];
   p.hits = reinterpret_cast<unsigned*>(h->sc_pbar[0]);
   p.H = c.n_kv_heads; p.G = h->G; p.U = h->U; p.P = P; p.layer = layer;
-  p.Ps = (P + 7) / 8 * 8;   // rows of logits start on 32-byte sectors
+  p.Ps = (P + 7) / 8 * 8;   // rows of group means start on 32-byte sectors
   p.words = (P + 31) / 32;
   p.scale = c.sm_scale;
   p.scale_log2 = c.sm_scale * 1.44269504088896340736f;
   const int fit = window_queries(h, P);
   const size_t sm = (size_t)P * sizeof(float) <= WIN_SMEM ? (size_t)P * sizeof(float) : 0;
-  const auto attn = out ? window_attn_kernel<true> : window_attn_kernel<false>;
   const int plan_grid = h->plan_grid(layer);
-  CK(h, cudaFuncSetAttribute(attn, cudaFuncAttributeMaxDynamicSharedMemorySize, WA_SMEM));
+  CUtensorMap mk, mv, mp;
+  if (!tile_map(&mk, k, c.batch, P, c.n_kv_heads) || !tile_map(&mv, v, c.batch, P, c.n_kv_heads) || !pool_map(&mp, h))
+    return fail(h, CRYSTALKV_EINVAL, "k and v must be 16-byte aligned");
   const size_t qn = (size_t)c.batch * c.n_q_heads * HD;
   for (int w0 = 0; w0 < W; w0 += p.W) {
     p.W = std::min(W - w0, fit);
@@ -784,10 +814,15 @@ static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, cons
     p.out = out ? out + (size_t)w0 * qn : nullptr;
     const bool last = w0 + p.W == W;
     p.store = last && fill_pages;
-    attn<<<dim3((p.W * p.G + WA_ROWS - 1) / WA_ROWS, h->U), WA_WARPS * 32, WA_SMEM, s>>>(h->st, p);
+    const int blocks = window_blocks(p.W, p.G);
+    p.rows = window_rows(p.W, p.G);
+    const auto attn = window_attn_of(p.rows, out != nullptr);
+    const int smem = wa_smem(p.rows, out != nullptr);
+    CK(h, cudaFuncSetAttribute(attn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    attn<<<dim3(blocks, h->U), WA_THREADS, smem, s>>>(h->st, p, mk, mv, mp);
     CK(h, cudaGetLastError());
     const bool small = P <= WH_SMALL && (long long)p.W * h->U >= P + h->num_sms;
-    (small ? window_hits_of<64>(h->G) : window_hits_of<NT>(h->G))<<<dim3(p.W, h->U), small ? 64 : NT, sm, s>>>(h->st, p, c.top_p, c.literal_return, sm > 0);
+    (small ? window_hits_kernel<64> : window_hits_kernel<NT>)<<<dim3(p.W, h->U), small ? 64 : NT, sm, s>>>(h->st, p, c.top_p, c.literal_return, sm > 0);
     CK(h, cudaGetLastError());
     window_apply_kernel<<<1 + h->U, NT, 0, s>>>(h->st, p, last, c.evict_every, reinterpret_cast<int*>(h->sc_pbar[1]), h->cap_s,
                                                 h->plans[layer], plan_grid, h->cl[layer], h->plan_len);
