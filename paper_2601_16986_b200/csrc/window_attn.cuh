@@ -8,10 +8,8 @@
 // the third the group means of the probabilities, all that Algorithm 1 needs of the queries (a fifth of the bytes of the
 // logits of five heads).  So nothing is ever rescaled, and a thread, which holds one key of every tile, keeps its share of
 // the maxima and sums in registers until a pass ends.  The weights go in as a bf16 head plus a bf16 remainder, like in the decode kernel.
-// One warp brings the tiles by TMA into three stages (in the second pass one of them holds keys and two hold values) and issues the
-// products; it and the others meet at mbarriers only.  (With these done by a thread of the sixteen between barriers
-// of the CTA, every step's latency showed: 94 us instead of WA_NOW for 128 heads x 1024 tokens, 32 queries of 5 heads.)
-// The tiles are also what the heads' pages are filled from (store): a key's 64 channels in a stage are, byte for byte, a quarter
+// A warp brings the tiles of all passes by TMA into a ring of stages, another issues the products; these and the sixteen meet at
+// mbarriers only.// The tiles are also what the heads' pages are filled from (store): a key's 64 channels in a stage are, byte for byte, a quarter
 // of an entry in a page, so another warp has TMA store them as they are.  The CTAs of a head take its tiles in turn, a tile that
 // only the last one sees in full falls to that one.  (A copy kernel of its own reads the prompt again: 20 us.)
 #pragma once
@@ -23,16 +21,19 @@
 namespace ckv {
 
 constexpr int WA_WARPS = 16;                  // warp w: keys 32 (w % 4) .. + 31 of every tile, the (w / 4)-th quarter of the rows
-constexpr int WA_THREADS = (WA_WARPS + 2) * 32;   // ... one warp that brings the tiles and issues the products, one that fills the pages
+constexpr int WA_THREADS = (WA_WARPS + 3) * 32;   // ... one warp brings the tiles, one issues the products, one fills the pages
 constexpr int WA_KEYS = 128;                  // keys per tile
 constexpr int WA_HALF = WA_KEYS * 128;        // bytes of a tile's 64 first (last) channels: 128-byte rows, 128-byte swizzle
 constexpr int WA_TILE = 2 * WA_HALF;
-constexpr int WA_STAGES = 3;
 constexpr int WA_MAX_ROWS = 160;              // rows of a CTA: 3 N <= 512 columns of tensor memory, and shared memory
 constexpr int WA_TMEM = 512;
-constexpr int wa_smem(int rows, bool out) {   // stages, rows (the swizzled layouts start on multiples of 1024), weights
-  return 1024 + WA_STAGES * WA_TILE + (out ? 3 : 1) * rows * 256 + (4 + 4 + 1) * rows * 4 + 128;
+// Stages of tiles: what the rows (the swizzled layouts start on multiples of 1024), the weights and the small arrays leave room for.
+__host__ __device__ constexpr int wa_stages(int rows, bool out) { return rows <= 32 ? 6 : rows <= 64 || !out ? 5 : rows <= 96 ? 4 : 3; }
+constexpr int wa_smem(int rows, bool out) {
+  return 1024 + wa_stages(rows, out) * WA_TILE + (out ? 3 : 1) * rows * 256 + (4 + 4 + 1 + 1) * rows * 4 + 192;
 }
+static_assert(wa_smem(32, true) <= 232448 && wa_smem(64, true) <= 232448 && wa_smem(96, true) <= 232448 && wa_smem(128, true) <= 232448 &&
+              wa_smem(160, true) <= 232448 && wa_smem(160, false) <= 232448, "shared memory of an SM");
 // Queries that a quarter of a CTA of `rows` rows takes: whole ones, so that a thread has all heads of a key's group mean.
 __host__ __device__ constexpr int wa_queries(int rows, int G) { return rows / 4 / G; }
 
@@ -121,22 +122,23 @@ template <int CW, bool OUT>
 __global__ void __launch_bounds__(WA_THREADS, 1) window_attn_kernel(const __grid_constant__ State st, const WindowParams p,
                                                                     const __grid_constant__ CUtensorMap mk, const __grid_constant__ CUtensorMap mv,
                                                                     const __grid_constant__ CUtensorMap mp) {
-  constexpr int N = 4 * CW;
+  constexpr int N = 4 * CW, S = wa_stages(N, OUT);
   extern __shared__ unsigned char smem_raw[];
   const uint32_t s0 = (smem_u32(smem_raw) + 1023) & ~1023u;
   unsigned char* sm = smem_raw + (s0 - smem_u32(smem_raw));
-  const uint32_t s_q = s0 + WA_STAGES * WA_TILE, s_p = s_q + N * 256;   // weights: heads, then remainders
-  float* s_m = reinterpret_cast<float*>(sm + WA_STAGES * WA_TILE + (OUT ? 3 : 1) * N * 256);   // reference points (log2 domain)
+  const uint32_t s_q = s0 + S * WA_TILE, s_p = s_q + N * 256;   // weights: heads, then remainders
+  float* s_m = reinterpret_cast<float*>(sm + S * WA_TILE + (OUT ? 3 : 1) * N * 256);   // reference points (log2 domain)
   float* s_l = s_m + N;                                                                          // 1 / normaliser
   float2* s_ml = reinterpret_cast<float2*>(s_l + N);                                             // reference point (natural), 1 / (normaliser x query heads)
   float* s_red = reinterpret_cast<float*>(s_ml + N);                                             // [4][N]
   int* s_t = reinterpret_cast<int*>(s_red + 4 * N);                                              // times of the rows
-  const uint32_t bar_ld = smem_u32(s_t + N);            // a load's bytes, per stage
-  const uint32_t bar_s = bar_ld + 8 * WA_STAGES;        // S is there, per buffer
+  int* s_row = s_t + N;                                                                          // rows: query x G + head, -1 for none
+  const uint32_t bar_ld = smem_u32(s_row + N);          // a load's bytes, per stage
+  const uint32_t bar_e = bar_ld + 8 * S;                // a stage has been used
+  const uint32_t bar_s = bar_e + 8 * S;                 // S is there, per buffer
   const uint32_t bar_free = bar_s + 16;                 // S has been read, per buffer
-  const uint32_t bar_p = bar_free + 16, bar_o = bar_p + 8;   // the weights are there; O is
-  const uint32_t bar_pg = bar_o + 8, tm_at = bar_pg + 8 * WA_STAGES;   // a tile has gone to its pages, per stage; the tensor memory's address
-  volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(reinterpret_cast<unsigned char*>(s_t + N) + (tm_at - bar_ld));
+  const uint32_t bar_p = bar_free + 16, bar_o = bar_p + 8, tm_at = bar_o + 8;   // the weights are there; O is; the tensor memory's address
+  volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(reinterpret_cast<unsigned char*>(s_row + N) + (tm_at - bar_ld));
 
   const int u = blockIdx.y, seq = u / p.H, head = u % p.H;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -149,69 +151,85 @@ __global__ void __launch_bounds__(WA_THREADS, 1) window_attn_kernel(const __grid
   // A wait gives up after about a second; from then on the thread waits for nothing, and nothing more is issued.
   bool dead = false;
   auto wait = [&](uint32_t bar, int n) { if (!dead) dead = !mbar_wait_bounded(bar, (uint32_t)n & 1u); };   // for its n-th phase
-  auto load = [&](const CUtensorMap& map, int tile, int stage) {
+  const int uid = (seq * st.L + p.layer) * st.H + head;
+  const bool store = OUT && p.store && st.n_cur[uid] == p.P;   // (a head that found no pages stays empty)
+  // The loads of all passes in the order in which the products use them, load i into stage i % S: the keys; the keys with every tile's
+  // values behind the next tile's keys (or the keys alone); the keys once more.  (-1 - tile: values)
+  const int n_mid = OUT ? 2 * nt : nt, n_loads = 2 * nt + n_mid;
+  auto what = [&](int i) {
+    if (i < nt) return i;
+    i -= nt;
+    if (i >= n_mid) return i - n_mid;
+    if (!OUT) return i;
+    return i == 2 * nt - 1 ? -nt : i & 1 ? (i + 1) / 2 : i ? -(i / 2) : 0;
+  };
+  auto load = [&](int i) {
+    const int x = what(i), stage = i % S, tile = x < 0 ? -1 - x : x;
     mbar_expect_tx(bar_ld + 8 * stage, WA_TILE);
-    for (int x = 0; x < 2; ++x) tma_tile(s0 + stage * WA_TILE + x * WA_HALF, &map, 64 * x, head, tile * WA_KEYS, seq, bar_ld + 8 * stage);
+    for (int y = 0; y < 2; ++y)
+      tma_tile(s0 + stage * WA_TILE + y * WA_HALF, x < 0 ? &mv : &mk, 64 * y, head, tile * WA_KEYS, seq, bar_ld + 8 * stage);
   };
   if (w == WA_WARPS) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(tm_at), "n"(WA_TMEM) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+  } else if (w == WA_WARPS + 1) {
     if (lane == 0) {
-      for (int x = 0; x < WA_STAGES + 2; ++x) mbar_init(bar_ld + 8 * x, 1);
+      for (int x = 0; x < S; ++x) {
+        mbar_init(bar_ld + 8 * x, 1);
+        mbar_init(bar_e + 8 * x, 2);   // by the products, and by the warp that fills the pages
+      }
+      for (int x = 0; x < 2; ++x) mbar_init(bar_s + 8 * x, 1);
       for (int x = 0; x < 3; ++x) mbar_init(bar_free + 8 * x, WA_WARPS);   // (bar_p as well)
-      for (int x = 0; x < 1 + WA_STAGES; ++x) mbar_init(bar_o + 8 * x, 1);   // (and bar_pg)
+      mbar_init(bar_o, 1);
       asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
       asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-      for (int x = 0; x < min(2, nt); ++x) load(mk, x, x);
+      for (int i = 0; i < min(S, n_loads); ++i) load(i);
     }
   } else if (w < WA_WARPS) {
     // row r of the CTA: column c of quarter x is head c % G of query q_lo + x qq + c / G; the others are zeros.
     // 64 channels per 128-byte row, 16-byte piece c of row r at c ^ (r & 7)
     constexpr int PER = N * 16 / (WA_WARPS * 32);
+    if (tid < N) {
+      const int c = tid % CW, q = q_lo + tid / CW * qq + c / p.G;
+      const bool there = c < cols && q < p.W;
+      s_row[tid] = there ? q * p.G + c % p.G : -1;
+      s_t[tid] = p.t0 + (there ? q : 0);
+    }
+    bar_sync(1, WA_WARPS * 32);
     uint4 v[PER];
-    auto query_of = [&](int r) {
-      const int x = r / CW, c = r % CW, q = q_lo + x * qq + c / p.G;
-      return c < cols && q < p.W ? q : -1;
-    };
 #pragma unroll
     for (int x = 0; x < PER; ++x) {
-      const int i = tid + x * (WA_WARPS * 32), r = i >> 4, q = query_of(r);
-      const uint32_t* src = reinterpret_cast<const uint32_t*>(p.q + (size_t)max(q, 0) * qstride + ((size_t)u * p.G + r % CW % p.G) * ROW_BYTES + (i & 15) * 16);
+      const int i = tid + x * (WA_WARPS * 32), row = s_row[i >> 4], q = max(s_t[i >> 4] - p.t0, 0);
+      const uint32_t* src = reinterpret_cast<const uint32_t*>(p.q + (size_t)q * qstride + ((size_t)u * p.G + max(row - q * p.G, 0)) * ROW_BYTES + (i & 15) * 16);
       v[x] = make_uint4(src[0], src[1], src[2], src[3]);
-      if (q < 0) v[x] = make_uint4(0, 0, 0, 0);
+      if (row < 0) v[x] = make_uint4(0, 0, 0, 0);
     }
 #pragma unroll
     for (int x = 0; x < PER; ++x) {
       const int i = tid + x * (WA_WARPS * 32), r = i >> 4, c = i & 15;
       *reinterpret_cast<uint4*>(sm + (s_q - s0) + (c >> 3) * (N * 128) + r * 128 + (((c & 7) ^ (r & 7)) << 4)) = v[x];
     }
-    if (tid < N) s_t[tid] = p.t0 + max(query_of(tid), 0);
   }
   asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // what was stored is read by the tensor cores
   tmem_before_sync();
   __syncthreads();
   tmem_after_sync();
   const uint32_t tm = *s_tmem;
-  const int uid = (seq * st.L + p.layer) * st.H + head;
-  const bool store = OUT && p.store && st.n_cur[uid] == p.P;   // (a head that found no pages stays empty)
-  const int ld1 = (nt + 1) / WA_STAGES, ld2 = nt / WA_STAGES;   // loads of the first pass into stages 1 and 2
 
   if (w == WA_WARPS) {
     if (lane == 0) {
-      // ---- tiles and products.  S of position i (tiles of all passes counted) goes to buffer i % 2.
+      // ---- the products.  S of position i (tiles of all passes counted) goes to buffer i % 2.
       const uint64_t dk = umma_desc(s0, 16, 1024, 2), dq = umma_desc(s_q, 16, 1024, 2);
       const uint64_t dv = umma_desc(s0, WA_HALF, 1024, 2), dp = umma_desc(s_p, WA_KEYS * 64, 512, 4);
-      int loads[WA_STAGES] = {0, 0, 0};
-      for (int x = 0; x < min(2, nt); ++x) loads[x] = 1;
-      auto next = [&](const CUtensorMap& map, int tile, int stage) {
-        if (dead) return;
-        load(map, tile, stage);
-        ++loads[stage];
+      int at = 0, stage = 0;   // the next load and its stage
+      auto landed = [&] { wait(bar_ld + 8 * stage, at / S); };
+      auto used = [&] {        // by the products issued so far
+        umma_commit(bar_e + 8 * stage);
+        ++at;
+        stage = stage + 1 == S ? 0 : stage + 1;
       };
-      auto landed = [&](int stage) { wait(bar_ld + 8 * stage, loads[stage] - 1); };
-      auto s_done = [&](int pos) { wait(bar_s + 8 * (pos & 1), pos >> 1); };
-      auto issue_s = [&](int stage, int pos) {
-        landed(stage);
+      auto issue_s = [&](int pos) {
+        landed();
         if (pos > 1) wait(bar_free + 8 * (pos & 1), (pos >> 1) - 1);
         tmem_after_sync();
         if (dead) return;
@@ -221,97 +239,75 @@ __global__ void __launch_bounds__(WA_THREADS, 1) window_attn_kernel(const __grid
           umma(tm + (pos & 1) * N, a + ((x >> 2) * (WA_HALF >> 4) + (x & 3) * 2), dq + ((x >> 2) * (N * 128 >> 4) + (x & 3) * 2),
                umma_instr(N, false), x > 0);
         umma_commit(bar_s + 8 * (pos & 1));
+        used();
       };
-      // a pass over keys alone, from position pos on, whose first two tiles are under way
-      auto ring = [&](int pos, bool pages) {
-        for (int x = 0; x < nt; ++x) {
-          issue_s(x % WA_STAGES, pos + x);
-          if (x + 2 < nt) {
-            if (x > 0) {   // the stage that tile x + 2 takes has been used
-              s_done(pos + x - 1);
-              if (pages) wait(bar_pg + 8 * ((x - 1) % WA_STAGES), (x - 1) / WA_STAGES);
-            }
-            next(mk, x + 2, (x + 2) % WA_STAGES);
-          }
-        }
-        s_done(pos + nt - 1);
-        if (pages)
-          for (int x = max(0, nt - 3); x < nt; ++x) wait(bar_pg + 8 * (x % WA_STAGES), x / WA_STAGES);
-      };
-      ring(0, store);
-      if (OUT) {
-        next(mk, 0, 0);
-        next(mv, 0, 1);
-        if (nt > 1) next(mv, 1, 2);
-        issue_s(0, nt);
-        for (int t = 0; t < nt; ++t) {
-          const int vs = 1 + (t & 1);
-          if (t + 1 < nt) {
-            s_done(nt + t);
-            next(mk, t + 1, 0);
-          }
-          if (t + 1 < nt) issue_s(0, nt + t + 1);
-          if (t > 0) {   // the other stage of values has been used
-            wait(bar_o, t - 1);
-            if (t + 1 < nt) {
-              const int o = 1 + ((t + 1) & 1);
-              if (store) wait(bar_pg + 8 * o, (o == 1 ? ld1 : ld2) + ((t - 1) >> 1));
-              next(mv, t + 1, o);
-            }
-          }
-          landed(vs);
-          wait(bar_p, t);
-          tmem_after_sync();
-          if (!dead) {
+      auto issue_o = [&](int t) {
+        landed();
+        wait(bar_p, t);
+        tmem_after_sync();
+        if (dead) return;
 #pragma unroll
-            for (int x = 0; x < 8; ++x) {   // 16 keys at a time
-              const uint64_t a = dv + (vs * (WA_TILE >> 4) + x * 128), b = dp + x * 64;
-              umma(tm + 2 * N, a, b, umma_instr(N, true), t > 0 || x > 0);
-              umma(tm + 2 * N, a, b + (N * 256 >> 4), umma_instr(N, true), true);
-            }
-            umma_commit(bar_o);
-          }
+        for (int x = 0; x < 8; ++x) {   // 16 keys at a time
+          const uint64_t a = dv + (stage * (WA_TILE >> 4) + x * 128), b = dp + x * 64;
+          umma(tm + 2 * N, a, b, umma_instr(N, true), t > 0 || x > 0);
+          umma(tm + 2 * N, a, b + (N * 256 >> 4), umma_instr(N, true), true);
         }
-        wait(bar_o, nt - 1);
-        if (store)
-          for (int t = max(0, nt - 2); t < nt; ++t) wait(bar_pg + 8 * (1 + (t & 1)), (t & 1 ? ld2 : ld1) + (t >> 1));
+        umma_commit(bar_o);
+        used();
+      };
+#pragma unroll 1
+      for (int x = 0; x < nt; ++x) issue_s(x);
+      if (OUT) {   // (the next tile's S goes ahead of a tile's O: the other warps wait for it)
+        issue_s(nt);
+#pragma unroll 1
+        for (int t = 0; t < nt; ++t) {
+          if (t + 1 < nt) issue_s(nt + t + 1);
+          issue_o(t);
+        }
       } else {
-        for (int x = 0; x < min(2, nt); ++x) next(mk, x, x);
-        ring(nt, false);
+#pragma unroll 1
+        for (int x = 0; x < nt; ++x) issue_s(nt + x);
       }
-      for (int x = 0; x < min(2, nt); ++x) next(mk, x, x);
-      ring(2 * nt, false);
-      if (dead) {   // copies that are still on their way must land in memory that is this CTA's
-        atomicOr(st.errword, ERR_COPY_TIMEOUT);
-        for (int x = 0; x < WA_STAGES; ++x)
-          if (loads[x] > 0) mbar_wait_bounded(bar_ld + 8 * x, (uint32_t)(loads[x] - 1) & 1u);
-      }
+#pragma unroll 1
+      for (int x = 0; x < nt; ++x) issue_s(2 * nt + x);
+      if (dead) atomicOr(st.errword, ERR_COPY_TIMEOUT);
     }
     __syncwarp();
   } else if (w == WA_WARPS + 1) {
-    // ---- the prompt's rows go to the head's pages: keys in the first pass, values in the second; lane x takes the tile's page x
-    if (store) {
-      const int last = gridDim.x - 1;
-      auto fill = [&](int tile, int stage, int n, int v) {   // n: which of the stage's loads it is
-        const int turn = tile % gridDim.x, at = tile * WA_KEYS + lane * GRP;
-        const bool mine = blockIdx.x == ((tile + 1) * WA_KEYS <= keys_of(turn) ? turn : last) && lane < WA_KEYS / GRP && at < p.P;
-        const int page = mine ? __ldg(st.ptab + (size_t)uid * st.capg + at / GRP) : 0;
-        wait(bar_ld + 8 * stage, n);
-        if (mine && !dead) {   // (rows past the prompt's end are zeros and go to places without an entry)
-          for (int y = 0; y < 2; ++y)
-            tma_store(&mp, 0, 2 * v + y, ((int)(seq * st.pages_per_seq) + page) * GRP, s0 + stage * WA_TILE + y * WA_HALF + lane * GRP * 128);
-          asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
-          asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar_pg + 8 * stage);
-      };
+    if (lane == 0) {
+      // ---- the tiles
 #pragma unroll 1
-      for (int x = 0; x < nt; ++x) fill(x, x % WA_STAGES, x / WA_STAGES, 0);
-#pragma unroll 1
-      for (int t = 0; t < nt; ++t) fill(t, 1 + (t & 1), (t & 1 ? ld2 : ld1) + (t >> 1), 1);
-      asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");
+      for (int i = S; i < n_loads; ++i) {
+        wait(bar_e + 8 * (i % S), i / S - 1);
+        if (dead) break;
+        load(i);
+      }
+      if (dead) {   // what is still on its way must land in memory that is this CTA's
+        atomicOr(st.errword, ERR_COPY_TIMEOUT);
+        for (int x = 0; x < S; ++x) mbar_wait_bounded(bar_ld + 8 * x, 0), mbar_wait_bounded(bar_ld + 8 * x, 1);
+      }
     }
+    __syncwarp();
+  } else if (w == WA_WARPS + 2) {
+    // ---- the prompt's rows go to the head's pages: keys in the first pass, values in the second; lane x takes the tile's page x
+    const int last = gridDim.x - 1;
+#pragma unroll 1
+    for (int i = 0; i < n_loads; ++i) {
+      const int x = what(i), tile = x < 0 ? -1 - x : x, stage = i % S, turn = tile % gridDim.x, at = tile * WA_KEYS + lane * GRP;
+      const bool mine = store && (i < nt || x < 0) && blockIdx.x == ((tile + 1) * WA_KEYS <= keys_of(turn) ? turn : last) &&
+                        lane < WA_KEYS / GRP && at < p.P;
+      const int page = mine ? __ldg(st.ptab + (size_t)uid * st.capg + at / GRP) : 0;
+      wait(bar_ld + 8 * stage, i / S);
+      if (mine && !dead) {   // (rows past the prompt's end are zeros and go to places without an entry)
+        for (int y = 0; y < 2; ++y)
+          tma_store(&mp, 0, (x < 0 ? 2 : 0) + y, ((int)(seq * st.pages_per_seq) + page) * GRP, s0 + stage * WA_TILE + y * WA_HALF + lane * GRP * 128);
+        asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+        asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_e + 8 * stage);
+    }
+    asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");
     __syncwarp();
   } else {
     const int quarter = w >> 2, c_lo = quarter * CW, key_w = (w & 3) * 32 + lane;
