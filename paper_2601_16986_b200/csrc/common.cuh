@@ -150,6 +150,13 @@ __device__ __forceinline__ int warp_sum_i(int v) {
 // first (the first min(k, cl) CTAs get at least one).
 __host__ __device__ __forceinline__ int shared_first(int k, int x, int cl) { return k / cl * x + (x < k % cl ? x : k % cl); }
 
+// Programmatic dependent launch: a kernel launched with the stream-serialisation attribute may
+// start while the kernel before it in the stream still runs; pdl_wait() returns once that
+// kernel has completed and its writes are visible, pdl_launch() lets the kernel after this
+// one start.  Both are no-ops for a launch without the attribute.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+
 // ---- thread-block clusters (a launch without the attribute is a cluster of one)
 __device__ __forceinline__ int cluster_rank() {
   int r;

@@ -450,6 +450,24 @@ int join_side(crystalkv_t* h, cudaStream_t s) {
   return CRYSTALKV_OK;
 }
 
+// A launch that may start before the kernel ahead of it in the stream has ended; the kernel waits for that (griddepcontrol.wait).
+// The kernels of a prompt let the next one start once they have themselves waited, so everything before the kernel ahead has ended by then.
+// Ordinary launches leave 1 to 2 us between two of them: a new batch of 16 prompts of 512 tokens 1.75 ms and 1.62, windows of 32 queries 6.1 and 5.8.
+template <class... P, class... A>
+cudaError_t launch_next(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = grid;
+  lc.blockDim = dim3(threads);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  return cudaLaunchKernelEx(&lc, kernel, static_cast<P>(args)...);
+}
+
 // A tensor map of bf16 in boxes of `box`, zeros beyond the ends.
 bool tensor_map(CUtensorMap* m, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box,
                 CUtensorMapSwizzle swizzle) {
@@ -772,16 +790,14 @@ static int window_queries(const crystalkv_t* h, int P) {
   return (int)std::max<long long>(1, std::min({(long long)NSETS * h->cap_s * QH / rows, h->cap_s / words, 1ll << 30}));
 }
 
-// Whether a window's attention kernel also fills the pages, from the tiles it reads: where its last launch has a CTA for four
-// fifths of the SMs at least, or the prompt is so short that a launch more costs what it saves.  With fewer CTAs a copy kernel
-// over the whole chip is the faster one.  The window's kernels of a
-// layer, pages from the tiles and copied: one CTA a head, 6 queries over 4096 tokens, 16 heads 289 us and 233, 64 heads
-// 311 and 282, 96 heads 319 and 312, 128 heads 336 and 344; 160 heads, 2 queries, 366 and 382; 128 heads of 1024 tokens, 2 queries
-// 106 and 105; three CTAs a head, 32 queries over 1024 tokens, 16 heads 84 and 84, 40 heads 90 and 92.5.  8 queries, 16 heads of 300 tokens 43 and 47, 64 heads 47
-// and 51.5, 2 heads of 512 tokens, 4 queries, 51.5 and 51.6, 16 heads of 1024 tokens, 8 queries, 86 and 74.
+// Whether a window's attention kernel also fills the pages, from the tiles it reads: a tile's pages hold up one of a head's
+// CTAs, which take the tiles in turn, 0.6 us, a copy kernel over the whole chip takes 4.5 us and the time of the bytes.  The window's kernels of a layer,
+// pages from the tiles and copied: 2 heads x 4096 tokens, 1 query 120 us and 105; 16 heads x 4096, 6 queries 140 and 133, x 12000, 8 queries 416
+// and 380, x 1024, 8 queries 43.5 and 45; 32 heads x 2048, 8 queries 79 and 82; 40 heads x 1024, 32 queries 75 and 82; 64 heads x
+// 1024, 2 queries 43 and 50, x 4096, 6 queries 141 and 161.
 static bool window_fills_pages(const crystalkv_t* h, int P, int W) {
-  const int last = (W - 1) % window_queries(h, P) + 1;
-  return P <= 512 || 5ll * h->U * window_blocks(last, h->G) >= 4ll * h->num_sms;
+  const long long blocks = window_blocks((W - 1) % window_queries(h, P) + 1, h->G);   // of the last launch
+  return 470ll * P < blocks * (450000 + 17ll * h->U * P);
 }
 
 // Algorithm 1 with the queries of the prompt's last W tokens, in as many launches as the scratch
@@ -819,14 +835,12 @@ static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, cons
     const auto attn = window_attn_of(p.rows, out != nullptr);
     const int smem = wa_smem(p.rows, out != nullptr);
     CK(h, cudaFuncSetAttribute(attn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    attn<<<dim3(blocks, h->U), WA_THREADS, smem, s>>>(h->st, p, mk, mv, mp);
-    CK(h, cudaGetLastError());
+    CK(h, launch_next(attn, dim3(blocks, h->U), WA_THREADS, smem, s, h->st, p, mk, mv, mp));
     const bool small = P <= WH_SMALL && (long long)p.W * h->U >= P + h->num_sms;
-    (small ? window_hits_kernel<64> : window_hits_kernel<NT>)<<<dim3(p.W, h->U), small ? 64 : NT, sm, s>>>(h->st, p, c.top_p, c.literal_return, sm > 0);
-    CK(h, cudaGetLastError());
-    window_apply_kernel<<<1 + h->U, NT, 0, s>>>(h->st, p, last, c.evict_every, reinterpret_cast<int*>(h->sc_pbar[1]), h->cap_s,
-                                                h->plans[layer], plan_grid, h->cl[layer], h->plan_len);
-    CK(h, cudaGetLastError());
+    CK(h, launch_next(small ? window_hits_kernel<64> : window_hits_kernel<NT>, dim3(p.W, h->U), small ? 64 : NT, sm, s, h->st, p, c.top_p,
+                      c.literal_return, sm > 0));
+    CK(h, launch_next(window_apply_kernel, dim3(1 + h->U), NT, 0, s, h->st, p, last, c.evict_every, reinterpret_cast<int*>(h->sc_pbar[1]),
+                      h->cap_s, h->plans[layer], plan_grid, h->cl[layer], h->plan_len));
   }
   return CRYSTALKV_OK;
 }
@@ -871,12 +885,10 @@ static int prefill_common(crystalkv_t* h, int layer, const void* k, const void* 
       CK(h, cudaFuncSetAttribute(prefill_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SEL_SMEM));
     CK(h, score_dispatch(h->G, p.sc, static_cast<const __nv_bfloat16*>(k), static_cast<const __nv_bfloat16*>(q), h->U,
                          c.n_kv_heads, P, p.scale, p.scale_log2, s));
-    prefill_select_kernel<<<h->U, SEL_NT, sm, s>>>(h->st, p.sc, layer, P, h->G, chunks, p.scale_log2 / p.scale, c.top_p, c.evict_every,
-                                                   c.literal_return, c.budget_ratio > 0.f ? ratio_budget(c, P) : 0, sm > 0);
-    CK(h, cudaGetLastError());
-    prefill_rows_kernel<<<1 + h->U * per_head, NT, 0, s>>>(h->st, h->plans[layer], layer, kb, vb, P, ROWS_SURVIVORS, per_head,
-                                                           plan_grid * NW, plan_grid, h->cl[layer]);
-    CK(h, cudaGetLastError());
+    CK(h, launch_next(prefill_select_kernel, dim3(h->U), SEL_NT, sm, s, h->st, p.sc, layer, P, h->G, chunks, p.scale_log2 / p.scale, c.top_p,
+                      c.evict_every, c.literal_return, c.budget_ratio > 0.f ? ratio_budget(c, P) : 0, sm > 0));
+    CK(h, launch_next(prefill_rows_kernel, dim3(1 + h->U * per_head), NT, 0, s, h->st, h->plans[layer], layer, kb, vb, P, ROWS_SURVIVORS,
+                      per_head, plan_grid * NW, plan_grid, h->cl[layer]));
     h->t_layer[layer] = P - 1;
     return CRYSTALKV_OK;
   }
@@ -890,9 +902,8 @@ static int prefill_common(crystalkv_t* h, int layer, const void* k, const void* 
   prefill_take_kernel<<<h->U, NT, 0, s>>>(h->st, layer, P, W > 0 ? 1 : 0);
   CK(h, cudaGetLastError());
   if (!fill_pages) {
-    prefill_rows_kernel<<<1 + h->U * per_head, NT, 0, s>>>(h->st, h->plans[layer], layer, kb, vb, P, W > 0 ? ROWS_ALL : ROWS_ALL_LAST,
-                                                           per_head, evict ? 0 : plan_grid * NW, plan_grid, h->cl[layer]);
-    CK(h, cudaGetLastError());
+    CK(h, launch_next(prefill_rows_kernel, dim3(1 + h->U * per_head), NT, 0, s, h->st, h->plans[layer], layer, kb, vb, P,
+                      W > 0 ? ROWS_ALL : ROWS_ALL_LAST, per_head, evict ? 0 : plan_grid * NW, plan_grid, h->cl[layer]));
   }
   if (evict) {
     rc = replay_window(h, layer, kb, vb, static_cast<const unsigned char*>(q), P, W, static_cast<__nv_bfloat16*>(out_window), fill_pages, s);

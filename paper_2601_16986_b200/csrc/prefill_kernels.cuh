@@ -43,6 +43,7 @@ __global__ void __launch_bounds__(SCORE_NT, 3) prefill_score_kernel(Scratch sc, 
   extern __shared__ __align__(128) unsigned char s_keys[];
   __shared__ __align__(16) float s_q[G * HD];
   __shared__ float s_m[SCORE_NT / 32][G];
+  pdl_launch();   // (an ordinary launch: what was queued before it has ended)
   const int u = blockIdx.y, seq = u / H, head = u % H;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int i0 = blockIdx.x * SCORE_KEYS, n = min(SCORE_KEYS, P - i0);
@@ -199,6 +200,8 @@ __global__ void __launch_bounds__(SEL_NT) prefill_select_kernel(State st, Scratc
   const size_t mb = (size_t)uid * st.cap;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   nucleus_clear<SEL_NT>(s_nu);   // (a barrier follows long before the histogram is filled)
+  pdl_wait();
+  pdl_launch();
   const int B = fixed_budget > 0 ? fixed_budget : st.budget[uid];
   if (fixed_budget > 0 && tid == 0) st.budget[uid] = fixed_budget;
   const float* S = sc.logits + (size_t)u * sc.cap_s * QH;
@@ -325,6 +328,7 @@ __global__ void __launch_bounds__(SEL_NT) prefill_select_kernel(State st, Scratc
 // time (its queries are replayed).
 __global__ void __launch_bounds__(NT) prefill_take_kernel(State st, int layer, int P, int meta) {
   __shared__ int s_top;
+  pdl_launch();   // (an ordinary launch: what was queued before it has ended)
   const int u = blockIdx.x, seq = u / st.H, uid = (seq * st.L + layer) * st.H + u % st.H;
   if (meta) {
     const size_t mb = (size_t)uid * st.cap;
@@ -352,6 +356,8 @@ __global__ void __launch_bounds__(NT) prefill_rows_kernel(const __grid_constant_
                                                           int plan_warps, int plan_grid, int plan_cl) {
   __shared__ int s_gs[MAX_UNITS_PER_CALL + 1];
   __shared__ int s_red[320];
+  pdl_wait();
+  pdl_launch();
   if (blockIdx.x == 0) {
     if (plan_warps > 0) write_plan(st, plan, layer, plan_warps, plan_grid, plan_cl, s_gs, s_red);
     return;

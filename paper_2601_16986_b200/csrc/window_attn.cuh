@@ -152,7 +152,6 @@ __global__ void __launch_bounds__(WA_THREADS, 1) window_attn_kernel(const __grid
   bool dead = false;
   auto wait = [&](uint32_t bar, int n) { if (!dead) dead = !mbar_wait_bounded(bar, (uint32_t)n & 1u); };   // for its n-th phase
   const int uid = (seq * st.L + p.layer) * st.H + head;
-  const bool store = OUT && p.store && st.n_cur[uid] == p.P;   // (a head that found no pages stays empty)
   // The loads of all passes in the order in which the products use them, load i into stage i % S: the keys; the keys with every tile's
   // values behind the next tile's keys (or the keys alone); the keys once more.  (-1 - tile: values)
   const int n_mid = OUT ? 2 * nt : nt, n_loads = 2 * nt + n_mid;
@@ -290,6 +289,9 @@ __global__ void __launch_bounds__(WA_THREADS, 1) window_attn_kernel(const __grid
     __syncwarp();
   } else if (w == WA_WARPS + 2) {
     // ---- the prompt's rows go to the head's pages: keys in the first pass, values in the second; lane x takes the tile's page x
+    // (Only here the kernel ahead, which takes the pages, has to have ended; what was queued before that one has.)
+    pdl_wait();
+    const bool store = OUT && p.store && st.n_cur[uid] == p.P;   // (a head that found no pages stays empty)
     const int last = gridDim.x - 1;
 #pragma unroll 1
     for (int i = 0; i < n_loads; ++i) {
@@ -309,6 +311,7 @@ __global__ void __launch_bounds__(WA_THREADS, 1) window_attn_kernel(const __grid
     }
     asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");
     __syncwarp();
+    pdl_launch();
   } else {
     const int quarter = w >> 2, c_lo = quarter * CW, key_w = (w & 3) * 32 + lane;
     const int nq = max(0, min(qq, p.W - (q_lo + quarter * qq)));   // queries of this warp's quarter
@@ -339,16 +342,20 @@ __global__ void __launch_bounds__(WA_THREADS, 1) window_attn_kernel(const __grid
     for (int i = 0; i < nt; ++i) {
       s_ready(i);
       const int key = i * WA_KEYS + key_w;
-      const bool all_see = (i + 1) * WA_KEYS - 1 <= t_first;
       float s[CW / 8][8];
 #pragma unroll
       for (int c = 0; c < CW / 8; ++c) tmem_ld8(s[c], tm_warp + (i & 1) * N + c * 8);
 #pragma unroll
       for (int c = 0; c < CW / 8; ++c) tmem_wait(s[c]);
       s_read(i);
+      if ((i + 1) * WA_KEYS - 1 <= t_first) {   // all rows see all of the tile
 #pragma unroll
-      for (int c = 0; c < CW; ++c)
-        if (all_see || key <= s_t[c_lo + c]) acc[c] = fmaxf(acc[c], s[c / 8][c % 8]);
+        for (int c = 0; c < CW; ++c) acc[c] = fmaxf(acc[c], s[c / 8][c % 8]);
+      } else {
+#pragma unroll
+        for (int c = 0; c < CW; ++c)
+          if (key <= s_t[c_lo + c]) acc[c] = fmaxf(acc[c], s[c / 8][c % 8]);
+      }
     }
     reduce_columns(acc, lane, [](float a, float b) { return fmaxf(a, b); });
     put_columns(acc);

@@ -30,6 +30,8 @@ template <int NTH>
 __global__ void __launch_bounds__(NTH) window_hits_kernel(const __grid_constant__ State st, const WindowParams p, float top_p, int literal,
                                                           int in_smem) {
   constexpr int WARPS = NTH / 32;
+  pdl_wait();
+  pdl_launch();
   extern __shared__ float s_pbar[];
   __shared__ NucleusSmem<NTH> s_nu;
   __shared__ int s_cnt[WARPS];
@@ -103,6 +105,8 @@ __global__ void __launch_bounds__(NT) window_apply_kernel(const __grid_constant_
                                                           int* tmp, int tmp_stride, const __grid_constant__ Plan plan, int plan_grid,
                                                           int plan_cl, int* plan_len) {
   __shared__ __align__(16) int sh[PL_SCRATCH];
+  pdl_wait();
+  pdl_launch();
   if (blockIdx.x == 0) {
     if (last) write_plan<NT>(st, plan, p.layer, plan_grid * NW, plan_grid, plan_cl, plan_len, sh, evict_every);
     return;
