@@ -485,11 +485,11 @@ bool tensor_map(CUtensorMap* m, const void* base, int rank, const cuuint64_t* di
   return encode && encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(base), dims, strides, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE,
                           swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
-// The tokens of a prompt as tiles: [batch][P][H][128] in boxes of 64 channels x WA_KEYS tokens of one head.
-bool tile_map(CUtensorMap* m, const void* base, int batch, int P, int H) {
+// The tokens of a prompt as tiles: [batch][P][H][128] in boxes of 64 channels x `tokens` tokens of one head.
+bool tile_map(CUtensorMap* m, const void* base, int batch, int P, int H, int tokens) {
   const cuuint64_t dims[4] = {HD, (cuuint64_t)H, (cuuint64_t)P, (cuuint64_t)batch};
   const cuuint64_t strides[3] = {ROW_BYTES, (cuuint64_t)H * ROW_BYTES, (cuuint64_t)P * H * ROW_BYTES};
-  const cuuint32_t box[4] = {HD / 2, 1, WA_KEYS, 1};
+  const cuuint32_t box[4] = {HD / 2, 1, (cuuint32_t)tokens, 1};
   return tensor_map(m, base, 4, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 // The pool as quarters of entries, in boxes of a page's.
@@ -820,7 +820,7 @@ static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, cons
   const size_t sm = (size_t)P * sizeof(float) <= WIN_SMEM ? (size_t)P * sizeof(float) : 0;
   const int plan_grid = h->plan_grid(layer);
   CUtensorMap mk, mv, mp;
-  if (!tile_map(&mk, k, c.batch, P, c.n_kv_heads) || !tile_map(&mv, v, c.batch, P, c.n_kv_heads) || !pool_map(&mp, h))
+  if (!tile_map(&mk, k, c.batch, P, c.n_kv_heads, WA_KEYS) || !tile_map(&mv, v, c.batch, P, c.n_kv_heads, WA_KEYS) || !pool_map(&mp, h))
     return fail(h, CRYSTALKV_EINVAL, "k and v must be 16-byte aligned");
   const size_t qn = (size_t)c.batch * c.n_q_heads * HD;
   for (int w0 = 0; w0 < W; w0 += p.W) {
@@ -883,8 +883,15 @@ static int prefill_common(crystalkv_t* h, int layer, const void* k, const void* 
     const size_t sm = (size_t)P * sizeof(float) <= SEL_SMEM ? (size_t)P * sizeof(float) : 0;
     if (sm > 32 * 1024)
       CK(h, cudaFuncSetAttribute(prefill_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SEL_SMEM));
-    CK(h, score_dispatch(h->G, p.sc, static_cast<const __nv_bfloat16*>(k), static_cast<const __nv_bfloat16*>(q), h->U,
-                         c.n_kv_heads, P, p.scale, p.scale_log2, s));
+    CUtensorMap mk;
+    if (!tile_map(&mk, k, c.batch, P, c.n_kv_heads, SCORE_KEYS)) return fail(h, CRYSTALKV_EINVAL, "k must be 16-byte aligned");
+    const long long items = (long long)c.batch * chunks * c.n_kv_heads;
+    const int ctas = (int)std::min<long long>(h->num_sms, (items + NW - 1) / NW);
+    const int warps = ctas * NW < c.n_kv_heads ? ctas * NW : ctas * NW / c.n_kv_heads * c.n_kv_heads;
+    CK(h, cudaFuncSetAttribute(prefill_score_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SCORE_SMEM));
+    prefill_score_kernel<<<ctas, NT, SCORE_SMEM, s>>>(p.sc, mk, static_cast<const __nv_bfloat16*>(q), c.batch, c.n_kv_heads, h->G, P, warps,
+                                                      p.scale, p.scale_log2, h->st.errword);
+    CK(h, cudaGetLastError());
     CK(h, launch_next(prefill_select_kernel, dim3(h->U), SEL_NT, sm, s, h->st, p.sc, layer, P, h->G, chunks, p.scale_log2 / p.scale, c.top_p,
                       c.evict_every, c.literal_return, c.budget_ratio > 0.f ? ratio_budget(c, P) : 0, sm > 0));
     CK(h, launch_next(prefill_rows_kernel, dim3(1 + h->U * per_head), NT, 0, s, h->st, h->plans[layer], layer, kb, vb, P, ROWS_SURVIVORS,

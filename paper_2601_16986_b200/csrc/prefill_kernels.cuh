@@ -4,9 +4,10 @@
 // layer's launch plan beside the copying).  The pool never holds more than the budget.  A prompt
 // that is kept as it is (full cache, observation window) only takes its pages and copies its rows.
 #pragma once
-#include "common.cuh"
+#include "attn_kernel.cuh"
 #include "nucleus.cuh"
 #include "plan.cuh"
+#include "tma.cuh"
 
 namespace ckv {
 
@@ -21,113 +22,101 @@ __global__ void __launch_bounds__(NT) plan_kernel(const __grid_constant__ State 
 constexpr int SEL_NT = 1024;            // threads of prefill_select_kernel
 constexpr int SEL_SMEM = 160 * 1024;    // pbar of up to this many bytes stays in shared memory
 
-constexpr int SCORE_NT = 256;           // threads of prefill_score_kernel, one key each
-constexpr int SCORE_KEYS = SCORE_NT;
+constexpr int SCORE_KEYS = 32;          // keys of an item of prefill_score_kernel: two tiles of 64 channels
+constexpr int SCORE_HALF = SCORE_KEYS * 128, SCORE_ITEM = 2 * SCORE_HALF;
+constexpr int SCORE_STAGES = 3;
+constexpr int SCORE_SMEM = 1024 + NW * SCORE_STAGES * (SCORE_ITEM + 8);
 
-// The scaled logits of the last query's G heads against the prompt's keys, and per CTA the softmax
-// reference point (log2 domain) of its keys.  grid: (chunks of SCORE_KEYS keys, U).
-//   k: [batch][P][H][128]   q_last: [batch][Hq][128]   partials: [U][chunks][8] = m
-// Every logit is one chain of fp32 multiply-adds over the channels in order, by one thread: which
-// entries of a prompt survive hangs on the last bits of the logits, so their rounding is part of the
-// result.  Bound: HBM and, close behind, the multiply-adds (G x 128 per key).  A CTA brings its 64 KB
-// of keys into shared memory with 16-byte asynchronous copies (chunk c of key i at c ^ (i & 7): the
-// threads of a quarter warp read eight different bank groups) and then computes; three CTAs share an
-// SM, so that the others' copies run beside one's arithmetic.  64 heads x 9350 tokens (153 MB): 46 us,
-// 3.3 TB/s (two keys a thread, half the warps: 55 us; one CTA per head with a thread per row of
-// global memory: 252 us; MMA fragments straight from global memory: 38 us, but other roundings, and a
-// head in some thousands then kept another entry at the hit boundary).  128 heads x 512 tokens: 9.6 us.
-template <int G>
-__global__ void __launch_bounds__(SCORE_NT, 3) prefill_score_kernel(Scratch sc, const __nv_bfloat16* __restrict__ k,
-                                                                    const __nv_bfloat16* __restrict__ q_last, int H, int P,
-                                                                    float scale, float scale_log2) {
-  extern __shared__ __align__(128) unsigned char s_keys[];
-  __shared__ __align__(16) float s_q[G * HD];
-  __shared__ float s_m[SCORE_NT / 32][G];
+// The scaled logits of the last query's G heads against the prompt's keys, and per item the softmax
+// reference point (log2 domain) of its keys.  Items are (sequence, 32 tokens, head), head fastest, and a warp takes every
+// `warps`-th (a multiple of H where that is 1, 2, 4 or 8: its queries then only change with the sequence).
+//   mk: k [batch][P][H][128], boxes of 64 channels x 32 tokens of a head   q_last: [batch][Hq][128]   partials: [U][chunks][8] = m
+// Bound: HBM.  Every warp keeps a ring of three items full by TMA, like the attention kernel's of pages, and eight warps that
+// read the heads of the same tokens keep to the same DRAM pages; the products are mma.sync with keys on M and the (padded) query
+// heads on N, 16 per item.  64 heads x 9350 tokens (153 MB): SCORE_NOW (a thread per key with fp32 multiply-adds from shared memory, three
+// CTAs of 64 KB an SM: 45.5 us, half of its cycles spent on 16-byte broadcasts of the queries).
+__global__ void __launch_bounds__(NT, 1) prefill_score_kernel(Scratch sc, const __grid_constant__ CUtensorMap mk, const __nv_bfloat16* __restrict__ q_last,
+                                                              int batch, int H, int G, int P, int warps, float scale, float scale_log2, int* errword) {
+  extern __shared__ unsigned char s_raw[];
   pdl_launch();   // (an ordinary launch: what was queued before it has ended)
-  const int u = blockIdx.y, seq = u / H, head = u % H;
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int i0 = blockIdx.x * SCORE_KEYS, n = min(SCORE_KEYS, P - i0);
-  {
-    const size_t row = (size_t)H * ROW_BYTES;
-    const unsigned char* src = reinterpret_cast<const unsigned char*>(k) + (((size_t)seq * P + i0) * H + head) * ROW_BYTES + (tid & 15) * 16;
-    const uint32_t dst = smem_u32(s_keys);
-    for (int i = tid >> 4; i < n; i += SCORE_NT / 16)
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n"
-                   ::"r"(dst + i * ROW_BYTES + (((tid & 15) ^ (i & 7)) << 4)), "l"(src + (size_t)i * row) : "memory");
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-  }
-  for (int x = tid; x < G * HD; x += SCORE_NT) s_q[x] = __bfloat162float(q_last[(size_t)u * G * HD + x]);
-  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-  __syncthreads();
-  float acc[G];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, gid = lane >> 2, tig = lane & 3, mi = lane >> 3, r8 = lane & 7;
+  const uint32_t s0 = (smem_u32(s_raw) + 1023) & ~1023u, ring = s0 + w * (SCORE_STAGES * SCORE_ITEM);
+  const uint32_t bars = s0 + NW * SCORE_STAGES * SCORE_ITEM + w * (SCORE_STAGES * 8);
+  if (lane < SCORE_STAGES) mbar_init(bars + lane * 8, 1);
+  asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  __syncwarp();
+  const int chunks = (P + SCORE_KEYS - 1) / SCORE_KEYS, items = batch * chunks * H, first = blockIdx.x * NW + w;
+  auto fetch = [&](int i, int stage) {   // by lane 0
+    const int head = i % H, at = i / H;
+    mbar_expect_tx(bars + stage * 8, SCORE_ITEM);
+    for (int x = 0; x < 2; ++x)
+      tma_tile(ring + stage * SCORE_ITEM + x * SCORE_HALF, &mk, 64 * x, head, at % chunks * SCORE_KEYS, at / chunks, bars + stage * 8);
+  };
+  if (first >= warps) return;
+  if (lane == 0)
+    for (int x = 0; x < SCORE_STAGES; ++x)
+      if (first + x * warps < items) fetch(first + x * warps, x);
+  uint32_t qb[8][2];
+  int have = -1;   // the head whose queries qb holds
+  const uint32_t krow = (uint32_t)(((mi & 1) * 8 + r8) * 128), khalf = (uint32_t)(mi >> 1);
+  int stage = 0;
+  uint32_t phase = 0;
+#pragma unroll 1
+  for (int i = first; i < items; i += warps) {
+    const int head = i % H, at = i / H, chunk = at % chunks, u = at / chunks * H + head;
+    if (u != have) {   // the G queries as B fragments
+      have = u;
+      const unsigned short* q = reinterpret_cast<const unsigned short*>(q_last) + ((size_t)u * G + gid) * HD;
 #pragma unroll
-  for (int g = 0; g < G; ++g) acc[g] = 0.f;
-  const unsigned char* ra = s_keys + tid * ROW_BYTES;   // (rows past the prompt's end hold anything; their results are dropped)
-#pragma unroll 2
-  for (int c = 0; c < HD / 8; ++c) {
-    const uint4 va = *reinterpret_cast<const uint4*>(ra + ((c ^ (tid & 7)) << 4));
-    const uint32_t ua[4] = {va.x, va.y, va.z, va.w};
-    float ka[8];
+      for (int ks = 0; ks < 8; ++ks)
 #pragma unroll
-    for (int x = 0; x < 4; ++x) {   // a bf16 is the upper half of its fp32
-      ka[2 * x] = __uint_as_float(ua[x] << 16); ka[2 * x + 1] = __uint_as_float(ua[x] & 0xffff0000u);
+        for (int x = 0; x < 2; ++x) {
+          const int c = ks * 16 + x * 8 + tig * 2;
+          qb[ks][x] = gid < G ? (uint32_t)__ldg(q + c) | ((uint32_t)__ldg(q + c + 1) << 16) : 0u;
+        }
     }
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-      const float4 q0 = *reinterpret_cast<const float4*>(s_q + g * HD + c * 8), q1 = *reinterpret_cast<const float4*>(s_q + g * HD + c * 8 + 4);
-      const float q[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
-#pragma unroll
-      for (int x = 0; x < 8; ++x) acc[g] = fmaf(q[x], ka[x], acc[g]);
+    if (!mbar_wait_bounded(bars + stage * 8, phase)) {
+      if (lane == 0) atomicOr(errword, ERR_COPY_TIMEOUT);
+      for (int x = 0; x < SCORE_STAGES; ++x) mbar_wait_bounded(bars + x * 8, x < stage ? phase ^ 1u : phase);   // what else is on its way
+      return;
     }
-  }
-  float* S = sc.logits + ((size_t)u * sc.cap_s + i0) * QH;
-  float mx[G];
+    const uint32_t tile = ring + stage * SCORE_ITEM;
+    float* S = sc.logits + ((size_t)u * sc.cap_s + chunk * SCORE_KEYS) * QH;
+    float c0 = -INFINITY, c1 = -INFINITY;
 #pragma unroll
-  for (int g = 0; g < G; ++g) mx[g] = -INFINITY;
-  if (tid < n) {
-    float out[QH];
+    for (int m = 0; m < SCORE_KEYS / 16; ++m) {
+      float s[4] = {0.f, 0.f, 0.f, 0.f}, s2[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int g = 0; g < QH; ++g) out[g] = g < G ? __fmul_rn(acc[g < G ? g : 0], scale) : 0.f;
-    *reinterpret_cast<float4*>(S + (size_t)tid * QH) = make_float4(out[0], out[1], out[2], out[3]);
-    if (G > 4) *reinterpret_cast<float4*>(S + (size_t)tid * QH + 4) = make_float4(out[4], out[5], out[6], out[7]);
+      for (int ks = 0; ks < 8; ks += 2) {   // two chains of four
+        uint32_t a[4], a2[4];
+        const uint32_t ka = tile + (ks >> 2) * SCORE_HALF + m * 16 * 128 + krow;
+        ldsm_x4(a, ka + ((((ks & 3) * 2 + khalf) ^ r8) << 4));
+        ldsm_x4(a2, ka + ((((ks & 3) * 2 + 2 + khalf) ^ r8) << 4));
+        mma_bf16(s, a, qb[ks][0], qb[ks][1]);
+        mma_bf16(s2, a2, qb[ks + 1][0], qb[ks + 1][1]);
+      }
 #pragma unroll
-    for (int g = 0; g < G; ++g) mx[g] = acc[g] * scale_log2;
-  }
+      for (int x = 0; x < 2; ++x) {
+        const int key = m * 16 + x * 8 + gid;
+        const float a = s[2 * x] + s2[2 * x], b = s[2 * x + 1] + s2[2 * x + 1];
+        if (chunk * SCORE_KEYS + key < P) {
+          *reinterpret_cast<float2*>(S + (size_t)key * QH + 2 * tig) = make_float2(__fmul_rn(a, scale), __fmul_rn(b, scale));
+          c0 = fmaxf(c0, a);
+          c1 = fmaxf(c1, b);
+        }
+      }
+    }
+    __syncwarp();   // the stage has been read
+    if (lane == 0 && i + SCORE_STAGES * warps < items) fetch(i + SCORE_STAGES * warps, stage);
+    if (++stage == SCORE_STAGES) { stage = 0; phase ^= 1u; }
 #pragma unroll
-  for (int g = 0; g < G; ++g) {
-    const float m = warp_max(mx[g]);
-    if (lane == 0) s_m[w][g] = m;
+    for (int x = 4; x < 32; x <<= 1) {
+      c0 = fmaxf(c0, __shfl_xor_sync(0xffffffffu, c0, x));
+      c1 = fmaxf(c1, __shfl_xor_sync(0xffffffffu, c1, x));
+    }
+    if (gid == 0)
+      *reinterpret_cast<float2*>(sc.partials + ((size_t)u * chunks + chunk) * QH + 2 * tig) = make_float2(c0 * scale_log2, c1 * scale_log2);
   }
-  __syncthreads();
-  if (tid < G) {
-    float m = s_m[0][tid];
-    for (int x = 1; x < SCORE_NT / 32; ++x) m = fmaxf(m, s_m[x][tid]);
-    sc.partials[((size_t)u * gridDim.x + blockIdx.x) * QH + tid] = m;
-  }
-}
-
-template <int G>
-cudaError_t launch_score(const Scratch& sc, const __nv_bfloat16* k, const __nv_bfloat16* q, int U, int H, int P, float scale,
-                         float scale_log2, cudaStream_t s) {
-  const int sm = SCORE_KEYS * ROW_BYTES;
-  cudaError_t e = cudaFuncSetAttribute(prefill_score_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  if (e != cudaSuccess) return e;
-  prefill_score_kernel<G><<<dim3((P + SCORE_KEYS - 1) / SCORE_KEYS, U), SCORE_NT, sm, s>>>(sc, k, q, H, P, scale, scale_log2);
-  return cudaGetLastError();
-}
-inline cudaError_t score_dispatch(int G, const Scratch& sc, const __nv_bfloat16* k, const __nv_bfloat16* q, int U, int H, int P,
-                                  float scale, float scale_log2, cudaStream_t s) {
-  switch (G) {
-    case 1: return launch_score<1>(sc, k, q, U, H, P, scale, scale_log2, s);
-    case 2: return launch_score<2>(sc, k, q, U, H, P, scale, scale_log2, s);
-    case 3: return launch_score<3>(sc, k, q, U, H, P, scale, scale_log2, s);
-    case 4: return launch_score<4>(sc, k, q, U, H, P, scale, scale_log2, s);
-    case 5: return launch_score<5>(sc, k, q, U, H, P, scale, scale_log2, s);
-    case 6: return launch_score<6>(sc, k, q, U, H, P, scale, scale_log2, s);
-    case 7: return launch_score<7>(sc, k, q, U, H, P, scale, scale_log2, s);
-    case 8: return launch_score<8>(sc, k, q, U, H, P, scale, scale_log2, s);
-  }
-  return cudaErrorInvalidValue;
 }
 
 // Exclusive scan of one int per thread over the SEL_NT threads; red: SEL_NT / 32 ints.

@@ -13,10 +13,9 @@
 // of an entry in a page, so another warp has TMA store them as they are.  The CTAs of a head take its tiles in turn, a tile that
 // only the last one sees in full falls to that one.  (A copy kernel of its own reads the prompt again: 20 us.)
 #pragma once
-#include <cuda.h>
-
 #include "attn_kernel.cuh"
 #include "nucleus.cuh"
+#include "tma.cuh"
 
 namespace ckv {
 
@@ -82,15 +81,6 @@ __device__ __forceinline__ void tmem_wait(float (&r)[8]) {
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void tma_store(const CUtensorMap* map, int c0, int c1, int c2, uint32_t src) {
-  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3}], [%4];\n"
-               ::"l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(src) : "memory");
-}
-__device__ __forceinline__ void tma_tile(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3, uint32_t bar) {
-  asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];\n"
-               ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar) : "memory");
-}
-
 template <int X>
 struct Const { static constexpr int value = X; };
 
