@@ -892,7 +892,7 @@ static int prefill_common(crystalkv_t* h, int layer, const void* k, const void* 
     prefill_score_kernel<<<ctas, NT, SCORE_SMEM, s>>>(p.sc, mk, static_cast<const __nv_bfloat16*>(q), c.batch, c.n_kv_heads, h->G, P, warps,
                                                       p.scale, p.scale_log2, h->st.errword);
     CK(h, cudaGetLastError());
-    CK(h, launch_next(prefill_select_kernel, dim3(h->U), SEL_NT, sm, s, h->st, p.sc, layer, P, h->G, chunks, p.scale_log2 / p.scale, c.top_p,
+    CK(h, launch_next(prefill_select_kernel, dim3(h->U), SEL_NT, sm, s, h->st, p.sc, layer, P, h->G, chunks, c.top_p,
                       c.evict_every, c.literal_return, c.budget_ratio > 0.f ? ratio_budget(c, P) : 0, sm > 0));
     CK(h, launch_next(prefill_rows_kernel, dim3(1 + h->U * per_head), NT, 0, s, h->st, h->plans[layer], layer, kb, vb, P, ROWS_SURVIVORS,
                       per_head, plan_grid * NW, plan_grid, h->cl[layer]));

@@ -28,9 +28,9 @@ constexpr int SCORE_STAGES = 3;
 constexpr int SCORE_SMEM = 1024 + NW * SCORE_STAGES * (SCORE_ITEM + 8);
 
 // The scaled logits of the last query's G heads against the prompt's keys, and per item the softmax
-// reference point (log2 domain) of its keys.  Items are (sequence, 32 tokens, head), head fastest, and a warp takes every
+// reference point (log2 domain) and normaliser of its keys.  Items are (sequence, 32 tokens, head), head fastest, and a warp takes every
 // `warps`-th (a multiple of H where that is 1, 2, 4 or 8: its queries then only change with the sequence).
-//   mk: k [batch][P][H][128], boxes of 64 channels x 32 tokens of a head   q_last: [batch][Hq][128]   partials: [U][chunks][8] = m
+//   mk: k [batch][P][H][128], boxes of 64 channels x 32 tokens of a head   q_last: [batch][Hq][128]   partials: [U][chunks][16] = m, l
 // Bound: HBM.  Every warp keeps a ring of three items full by TMA, like the attention kernel's of pages, and eight warps that
 // read the heads of the same tokens keep to the same DRAM pages; the products are mma.sync with keys on M and the (padded) query
 // heads on N, 16 per item.  64 heads x 9350 tokens (153 MB): SCORE_NOW (a thread per key with fp32 multiply-adds from shared memory, three
@@ -82,6 +82,7 @@ __global__ void __launch_bounds__(NT, 1) prefill_score_kernel(Scratch sc, const 
     }
     const uint32_t tile = ring + stage * SCORE_ITEM;
     float* S = sc.logits + ((size_t)u * sc.cap_s + chunk * SCORE_KEYS) * QH;
+    float t[SCORE_KEYS / 16][4];   // logits in the log2 domain
     float c0 = -INFINITY, c1 = -INFINITY;
 #pragma unroll
     for (int m = 0; m < SCORE_KEYS / 16; ++m) {
@@ -99,11 +100,12 @@ __global__ void __launch_bounds__(NT, 1) prefill_score_kernel(Scratch sc, const 
       for (int x = 0; x < 2; ++x) {
         const int key = m * 16 + x * 8 + gid;
         const float a = s[2 * x] + s2[2 * x], b = s[2 * x + 1] + s2[2 * x + 1];
-        if (chunk * SCORE_KEYS + key < P) {
-          *reinterpret_cast<float2*>(S + (size_t)key * QH + 2 * tig) = make_float2(__fmul_rn(a, scale), __fmul_rn(b, scale));
-          c0 = fmaxf(c0, a);
-          c1 = fmaxf(c1, b);
-        }
+        const bool there = chunk * SCORE_KEYS + key < P;
+        if (there) *reinterpret_cast<float2*>(S + (size_t)key * QH + 2 * tig) = make_float2(__fmul_rn(a, scale), __fmul_rn(b, scale));
+        t[m][2 * x] = there ? a * scale_log2 : -INFINITY;
+        t[m][2 * x + 1] = there ? b * scale_log2 : -INFINITY;
+        c0 = fmaxf(c0, t[m][2 * x]);
+        c1 = fmaxf(c1, t[m][2 * x + 1]);
       }
     }
     __syncwarp();   // the stage has been read
@@ -114,8 +116,22 @@ __global__ void __launch_bounds__(NT, 1) prefill_score_kernel(Scratch sc, const 
       c0 = fmaxf(c0, __shfl_xor_sync(0xffffffffu, c0, x));
       c1 = fmaxf(c1, __shfl_xor_sync(0xffffffffu, c1, x));
     }
-    if (gid == 0)
-      *reinterpret_cast<float2*>(sc.partials + ((size_t)u * chunks + chunk) * QH + 2 * tig) = make_float2(c0 * scale_log2, c1 * scale_log2);
+    float l0 = 0.f, l1 = 0.f;   // (an item has a key, so the reference points are finite)
+#pragma unroll
+    for (int m = 0; m < SCORE_KEYS / 16; ++m) {
+      l0 += ex2(t[m][0] - c0) + ex2(t[m][2] - c0);
+      l1 += ex2(t[m][1] - c1) + ex2(t[m][3] - c1);
+    }
+#pragma unroll
+    for (int x = 4; x < 32; x <<= 1) {
+      l0 += __shfl_xor_sync(0xffffffffu, l0, x);
+      l1 += __shfl_xor_sync(0xffffffffu, l1, x);
+    }
+    if (gid == 0) {
+      float* ml = sc.partials + ((size_t)u * chunks + chunk) * (2 * QH) + 2 * tig;
+      *reinterpret_cast<float2*>(ml) = make_float2(c0, c1);
+      *reinterpret_cast<float2*>(ml + QH) = make_float2(l0, l1);
+    }
   }
 }
 
@@ -177,11 +193,11 @@ __device__ __forceinline__ bool take_pages(const State& st, int uid, int seq, in
 // the decode step's Algorithm 1 kernel with its radix
 // select over 96-bit keys in global memory took 286 us.  128 heads x 512 tokens: 10.9 us.
 __global__ void __launch_bounds__(SEL_NT) prefill_select_kernel(State st, Scratch sc, int layer, int P, int G, int chunks,
-                                                                float to_log2, float top_p, int evict_every, int literal,
+                                                                float top_p, int evict_every, int literal,
                                                                 int fixed_budget, int in_smem) {
   extern __shared__ float s_pbar[];
   __shared__ NucleusSmem<SEL_NT> s_nu;
-  __shared__ float s_m[QH], s_il[QH], s_l[8][QH];
+  __shared__ float s_m[QH], s_il[QH];
   __shared__ int s_red[SEL_NT / 32];
   __shared__ int s_top;
   const int u = blockIdx.x, seq = u / st.H, head = u % st.H;
@@ -194,37 +210,18 @@ __global__ void __launch_bounds__(SEL_NT) prefill_select_kernel(State st, Scratc
   const int B = fixed_budget > 0 ? fixed_budget : st.budget[uid];
   if (fixed_budget > 0 && tid == 0) st.budget[uid] = fixed_budget;
   const float* S = sc.logits + (size_t)u * sc.cap_s * QH;
-  if (w < G) {   // warp g: query head g's reference point
-    const float* pp = sc.partials + (size_t)u * chunks * QH;
-    float m = -INFINITY;
-    for (int c = lane; c < chunks; c += 32) m = fmaxf(m, pp[c * QH + w]);
+  if (w < G) {   // warp g: query head g's reference point and normaliser
+    const float* pp = sc.partials + (size_t)u * chunks * (2 * QH) + w;
+    float m = -INFINITY, l = 0.f;
+    for (int c = lane; c < chunks; c += 32) m = fmaxf(m, pp[c * (2 * QH)]);
     m = warp_max(m);
-    if (lane == 0) s_m[w] = m;
-  }
-  __syncthreads();
-  // normalisers: 256 threads to a pair of query heads, thread t over tokens t, t + 256, ..; then the
-  // lanes of a warp, then the eight warps in order (an order the results hang on, like the logits')
-  {
-    const int g = 2 * (tid >> 8), t = tid & 255;
-    float s0 = 0.f, s1 = 0.f;
-    if (g < G) {
-      const float m0 = s_m[g], m1 = s_m[min(g + 1, G - 1)];
-#pragma unroll 8
-      for (int i = t; i < P; i += 256) {
-        const float2 x = *reinterpret_cast<const float2*>(S + (size_t)i * QH + g);
-        s0 += ex2(x.x * to_log2 - m0);
-        s1 += ex2(x.y * to_log2 - m1);
-      }
+#pragma unroll 4
+    for (int c = lane; c < chunks; c += 32) l = fmaf(pp[c * (2 * QH) + QH], ex2(pp[c * (2 * QH)] - m), l);
+    l = warp_sum(l);
+    if (lane == 0) {
+      s_m[w] = m;
+      s_il[w] = 1.0f / (l * (float)G);
     }
-    s0 = warp_sum(s0);
-    s1 = warp_sum(s1);
-    if (lane == 0) { s_l[w & 7][g] = s0; s_l[w & 7][g + 1] = s1; }
-  }
-  __syncthreads();
-  if (tid < G) {
-    float l = 0.f;
-    for (int x = 0; x < 8; ++x) l += s_l[x][tid];
-    s_il[tid] = 1.0f / (l * (float)G);
   }
   __syncthreads();
   // ---- step 1: pbar_i = mean_g exp(s_gi - m_g) / l_g
