@@ -129,6 +129,8 @@ constexpr int INBOX_BARS = QH / 2, INBOX_BYTES = (HD + 2) * 4;   // bytes that o
 constexpr int ATTN_SMEM_SHARED = ATTN_SMEM + INBOX_SLOTS * INBOX_SLOT + INBOX_BARS * 8;
 static_assert(ATTN_SMEM % 16 == 0 && INBOX_SLOT % 16 == 0, "slots are written 16 bytes at a time");
 
+constexpr int HEAD_BITS = 11;
+static_assert(MAX_UNITS_PER_CALL <= 1 << HEAD_BITS, "a head's number and its count of partials share a word");
 constexpr float LAZY = 8.0f;   // the running maximum (log2 domain) may trail the true one by this much
 
 // The merge of HB heads over at most PB pieces in one round of loads: every lane loads the
@@ -196,7 +198,8 @@ __device__ __forceinline__ void merge_head(const DecodeParams& p, int u, int npi
 #pragma unroll
       for (int h = 0; h < 5; ++h) put(h, mm[h], L[h], acc[h]);
     } else {
-      for (int g0 = 0; g0 < G; g0 += 4) {
+#pragma unroll
+      for (int g0 = 0; g0 < QH; g0 += 4) {
         float mm[4], L[4];
         float4 acc[4];
         merge_small<4, 4>(pbase, PS, npieces, g0, G, lane, mm, L, acc);
@@ -205,11 +208,13 @@ __device__ __forceinline__ void merge_head(const DecodeParams& p, int u, int npi
       }
     }
   } else {   // four heads x four pieces per round of loads, rounds chained by the usual rescale
+#pragma unroll 1
     for (int g0 = 0; g0 < G; g0 += 4) {
       float mg[4], Lg[4];
       float4 acc[4];
 #pragma unroll
       for (int h = 0; h < 4; ++h) { mg[h] = -INFINITY; Lg[h] = 0.f; acc[h] = make_float4(0.f, 0.f, 0.f, 0.f); }
+#pragma unroll 1
       for (int pc0 = 0; pc0 < npieces; pc0 += 4) {
         float mm[4], L[4];
         float4 a2[4];
@@ -282,9 +287,9 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
   const uint32_t vrow = (uint32_t)(((mi >> 1) * 8 + r8) * SLOT_BYTES), vhalf = (uint32_t)(mi & 1);
   bool waited = p.early == 0;
   uint32_t phases = 0;      // bit s: parity of the next completion of stage s
-  int fsi = 0, csi = 0;     // stage the next copy fills / the next compute reads
+  int csi = 0;              // stage the next compute reads
   int fq_head = 0, fq_tail = 0;
-  int defer0 = -1, defer1 = -1;   // heads this warp completed and merges after its own run
+  int defer0 = -1, defer1 = -1;   // heads this warp completed and has yet to merge, and how many partials << HEAD_BITS
 
   // ---- fetching side: the piece whose groups are being requested
   int f_pi = range.x, f_next = 0, f_hi = 0, f_ntot = 0, f_seq = 0, ids = 0, idbase = 0;
@@ -313,17 +318,17 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
     ++fq_tail;
     __syncwarp();
   };
-  auto fetch_next = [&]() -> bool {
-    if (f_pi < 0) return false;
+  auto fetch_next = [&](int s) {   // the next group of this run into stage s, if there is one
+    if (f_pi < 0) return;
     if (f_next == f_hi) {
       f_pi = (f_pi + 1 < range.y) ? f_pi + 1 : -1;
-      if (f_pi < 0) return false;
+      if (f_pi < 0) return;
       open_piece(f_pi, __ldg(p.plan.desc + f_pi));
     }
     if (f_next - idbase >= 32) { idbase = f_next; ids = (f_next + lane < f_hi) ? __ldg(pt + f_next + lane) : 0; }
     const int page = __shfl_sync(0xffffffffu, ids, f_next - idbase);
     const int valid = min(GRP, f_ntot - f_next * GRP);
-    const uint32_t stage = ring_u32 + fsi * PAGE_BYTES;
+    const uint32_t stage = ring_u32 + s * PAGE_BYTES;
     if (valid < GRP) {   // rows past the head's end must not feed stale bits into the MMAs
       for (int e = valid; e < GRP; ++e)
         asm volatile("st.shared.v4.b32 [%0], {%1,%1,%1,%1};\n" ::"r"(stage + e * SLOT_BYTES + lane * 16), "r"(0) : "memory");
@@ -331,18 +336,16 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
       __syncwarp();
     }
     if (lane == 0) {
-      const uint32_t bar = bar0 + fsi * 8;
+      const uint32_t bar = bar0 + s * 8;
       mbar_expect_tx(bar, (uint32_t)valid * SLOT_BYTES);
       bulk_g2s_hint(stage, st.pool + ((size_t)f_seq * st.pages_per_seq + (unsigned)page) * PAGE_BYTES,
                     (uint32_t)valid * SLOT_BYTES, bar, pol_stream);
     }
     ++f_next;
-    fsi = (fsi + 1 == STAGES) ? 0 : fsi + 1;
-    return true;
   };
   open_piece(f_pi, dd_first);
 #pragma unroll 1
-  for (int s = 0; s < STAGES; ++s) fetch_next();
+  for (int s = 0; s < STAGES; ++s) fetch_next(s);
   // everything above reads only the cache, its lists and the plan; the call's inputs (q, the
   // arriving rows) may come from the kernel ahead in the stream
   if (!waited) { pdl_wait(); waited = true; }
@@ -382,14 +385,13 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
         qb[ks][1] = (gid < G) ? q32[ks * 8 + tig + 4] : 0u;
       }
     }
-    // the arriving token: lane's 16 bytes of its K row (lanes 0..15) or V row (16..31).  With two or three groups a warp its
-    // round trip would show, so it is asked for beside the queries (64 heads of 1025 entries 10.3 us a layer instead of 10.4).
-    auto arriving = [&] {
-      const unsigned char* src = reinterpret_cast<const unsigned char*>(lane < 16 ? p.k_new : p.v_new) + (size_t)u * ROW_BYTES + (lane & 15) * 16;
-      return *reinterpret_cast<const uint4*>(src);
-    };
-    uint4 val_early = make_uint4(0, 0, 0, 0);
-    if (SHARED && hole >= lo * GRP && hole < hi * GRP) val_early = arriving();
+    // With two or three groups a warp the round trip for the arriving token's rows would show, so they are asked for beside
+    // the queries (64 heads of 1025 entries 10.3 us a layer instead of 10.4).
+    [[maybe_unused]] uint4 val_early = make_uint4(0, 0, 0, 0);
+    if constexpr (SHARED)
+      if (hole >= lo * GRP && hole < hi * GRP)
+        val_early = *reinterpret_cast<const uint4*>(reinterpret_cast<const unsigned char*>(lane < 16 ? p.k_new : p.v_new) +
+                                                    (size_t)u * ROW_BYTES + (lane & 15) * 16);
     float o[8][4];
 #pragma unroll
     for (int mt = 0; mt < 8; ++mt) { o[mt][0] = 0.f; o[mt][1] = 0.f; o[mt][2] = 0.f; o[mt][3] = 0.f; }
@@ -414,8 +416,16 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
       const int base = ci * GRP;
       const int valid = min(GRP, n_tot - base);
       if (hole >= base && hole < base + GRP) {
-        // the arriving token goes into the stage and into the head's page, at the place the hole has in both
-        const uint4 val = SHARED ? val_early : arriving();
+        // the arriving token: chunk `lane` of its K row (lanes 0..15) or V row (16..31) goes into the
+        // stage and into the head's page, at the place the hole has in both
+        uint4 val;
+        if constexpr (SHARED) {
+          val = val_early;
+        } else {
+          const unsigned char* src = reinterpret_cast<const unsigned char*>(lane < 16 ? p.k_new : p.v_new) +
+                                     (size_t)u * ROW_BYTES + (lane & 15) * 16;
+          val = *reinterpret_cast<const uint4*>(src);
+        }
         const int off = chunk_offset(hole - base, lane);
         asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};\n" ::"r"(stage + off), "r"(val.x), "r"(val.y), "r"(val.z), "r"(val.w) : "memory");
         const int page = __ldg(st.ptab + (size_t)uid * st.capg + ci);
@@ -493,9 +503,9 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
           mma_bf16(o[mt + 1], a2, rr0, rr1);
         }
       }
+      __syncwarp();      // the stage is free again
+      fetch_next(csi);   // and is refilled at once, with the next group of this run
       csi = (csi + 1 == STAGES) ? 0 : csi + 1;
-      __syncwarp();   // the stage is free again
-      fetch_next();   // and is refilled at once, with the next group of this run
     }
 
     // l over the keys of all lanes that hold the same heads
@@ -650,7 +660,7 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
         if (last) p.sc.ticket[u] = 0;
       }
       last = __shfl_sync(0xffffffffu, last, 0);
-      if (last) merge_head(p, u, (npieces + NW - 1) / NW, lane);
+      if (last) (defer0 < 0 ? defer0 : defer1) = u | ((npieces + NW - 1) / NW) << HEAD_BITS;
       continue;
     }
     // ---- publish the piece's partial and take a ticket
@@ -678,17 +688,24 @@ __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 r
       if (last) p.sc.ticket[u] = 0;   // ready for the next launch that uses this scratch set
     }
     last = __shfl_sync(0xffffffffu, last, 0);
-    if (!last) continue;
-    // the head is complete.  Merging it now would stall this warp's stream for a round trip to L2,
-    // so a warp with more of its run ahead merges afterwards (a run cuts at most two heads).
-    if (fq_head != fq_tail && defer0 < 0) defer0 = u;
-    else if (fq_head != fq_tail && defer1 < 0) defer1 = u;
-    else merge_head(p, u, npieces, lane);
+    if (last) (defer0 < 0 ? defer0 : defer1) = u | npieces << HEAD_BITS;
   }
-  if (defer0 >= 0) merge_head(p, defer0, __ldg(p.plan.npc + defer0), lane);
-  if (defer1 >= 0) merge_head(p, defer1, __ldg(p.plan.npc + defer1), lane);
+  // Heads completed on the way (a run cuts at most two): merging one there would stall this warp's stream for a round trip to L2.
+  // The one place of the merge, where nothing of the stream is live any more: with one at each of the four places that find a
+  // head complete the kernel had 141 KB of code instead of 55, and a launch ended on instructions yet to be fetched (14B shape with
+  // unequal budgets 26.35 us a layer instead of 25.8).
+#pragma unroll 1
+  for (int x = 0; x < 2; ++x) {
+    const int d = x ? defer1 : defer0;
+    if (d >= 0) merge_head(p, d & ((1 << HEAD_BITS) - 1), d >> HEAD_BITS, lane);
+  }
   __syncwarp();
   if (SHARED) meet_and_leave();   // (a head that is one piece)
 }
+
+// The instantiations are compiled in a unit of their own (attn.cu): beside others in one unit, registers and schedule of this
+// kernel changed with theirs (40 heads of 5001 entries 20.8 us a layer, and 22.1 once a kernel of prompts used the same helpers).
+using AttnKernel = void (*)(DecodeParams);
+AttnKernel attn_of(bool shared, bool track);
 
 }  // namespace ckv

@@ -377,7 +377,7 @@ int find_clusters(crystalkv_t* h) {
     lc.attrs = at;
     lc.numAttrs = 1;
     int n = 0;
-    CK(h, cudaOccupancyMaxActiveClusters(&n, attn_kernel<true, true>, &lc));
+    CK(h, cudaOccupancyMaxActiveClusters(&n, attn_of(true, true), &lc));
     h->share_ok[cl] = n >= h->U;
   }
   return CRYSTALKV_OK;
@@ -393,13 +393,15 @@ int find_clusters(crystalkv_t* h) {
 // two layers keeps the line of four groups (40 groups, 2 heads 10.3, 9.4, 8.4: its launch shapes are stated by a test).
 // Longer heads of one length (from 193 groups, where they no longer fit a CTA in pieces of 2 GLAT) gain from two CTAs where their
 // other choice is more than eight pieces and a merge through global memory at the end of the launch.  The longer the pieces,
-// the more the CTAs that then have nothing to stream count: up to 14 groups a piece below 43 heads.  us a layer, not shared and
-// shared, of 194, 226, 257, 313 and 376 groups: 40 heads 20.7 20.1 20.9 24.9 34.1 and 17.7 19.7 21.5 24.9 28.7; 44 heads 21.0 20.7 22.3 27.6
-// 35.4 and 18.0 20.0 21.9 25.3 29.5; 52 heads 22.2 22.4 25.0 29.4 37.4 and 18.5 21.1 23.5 27.6 35.1.
+// the more the CTAs that then have nothing to stream count: up to 14 groups a piece from 45 heads on, up to 24 from 52.  us a
+// layer, not shared and shared, of 194, 226, 257, 313 and 376 groups: 48 heads 21.7 21.4 23.3 27.5 37.1 and 18.2 20.6 22.8 26.5 31.6; 52 heads 22.2
+// 22.4 25.0 29.4 37.4 and 18.5 21.1 23.5 27.6 35.1; 64 heads of 257 28.2 and 27.1.  (The lines are older than these figures, by which 40 heads of
+// 194 groups, 20.7 and 17.7, and 48 of 376 would share as well; tests state the lines.)
 int share_heads(crystalkv_t* h, int entries) {
   const int g = (entries + GRP - 1) / GRP, alone = (g + NW - 1) / NW;
   auto per = [&](int cl) { return (g + NW * cl - 1) / (NW * cl); };
-  const bool merge = h->uniform && alone > 2 * GLAT && per(2) <= (7 * h->U >= 2 * h->num_sms ? 2 * GLAT : GLAT + 2);
+  const bool merge = h->uniform && 10 * h->U >= 3 * h->num_sms && alone > 2 * GLAT &&
+                     per(2) <= (20 * h->U >= 7 * h->num_sms ? 2 * GLAT : GLAT + 2);
   const int least = h->cfg.n_layers == 2 ? 4 : h->cfg.n_layers == 1 ? 1 : 2;
   auto pays = [&](int cl) { return h->share_ok[cl] && (per(cl) <= GLAT || (cl == 2 && merge)) && alone - per(cl) >= least; };
   if (pays(4) && (!pays(2) || per(2) - per(4) >= (8 * h->U <= h->num_sms ? 1 : 2))) return 4;
@@ -548,9 +550,7 @@ int launch_step(crystalkv_t* h, DecodeParams& p, int layer, cudaStream_t s) {
     at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
     lc.attrs = at;
     lc.numAttrs = p.cl > 1 ? 2 : 1;
-    const auto attn = p.track ? (p.cl > 1 ? attn_kernel<true, true> : attn_kernel<false, true>)
-                              : (p.cl > 1 ? attn_kernel<true, false> : attn_kernel<false, false>);
-    CK(h, cudaLaunchKernelEx(&lc, attn, p));
+    CK(h, cudaLaunchKernelEx(&lc, attn_of(p.cl > 1, p.track != 0), p));
   }
   h->prev_layer = layer;
   {
@@ -661,15 +661,16 @@ int crystalkv_create(const crystalkv_config_t* cfg, crystalkv_t** out) {
   CKC(scope.err);
   CKC(cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, c.device));
   int bps = 0;
-  for (auto attn : {attn_kernel<false, false>, attn_kernel<true, false>, attn_kernel<false, true>, attn_kernel<true, true>}) {
+  for (int x = 0; x < 4; ++x) {
     // (the same for every handle: the attribute belongs to the function, so no handle may lower it under another)
-    const bool shared = attn == attn_kernel<true, false> || attn == attn_kernel<true, true>;
+    const bool shared = x & 1;
+    const AttnKernel attn = attn_of(shared, x >> 1);
     CKC(cudaFuncSetAttribute(attn, cudaFuncAttributeMaxDynamicSharedMemorySize, shared ? ATTN_SMEM_SHARED : ATTN_SMEM));
     // The largest shared-memory carve-out, although the ring alone would fit a smaller one: the CTAs
     // of the LRFU kernel have to find room beside an attention CTA on the same SM.
     CKC(cudaFuncSetAttribute(attn, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared));
   }
-  CKC(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, attn_kernel<false, true>, NT, ATTN_SMEM));
+  CKC(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, attn_of(false, true), NT, ATTN_SMEM));
   if (bps < 1) { h->err = "attention kernel does not fit on an SM"; CREATE_FAIL(CRYSTALKV_ECUDA); }
   h->grid = h->num_sms * bps;
   h->cl.assign(c.n_layers, 1);
