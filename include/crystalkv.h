@@ -320,7 +320,7 @@ int crystalkv_debug_ctas_needed(int32_t whole_ctas, const int32_t* runs_by_lengt
 
 /*
  * Test hook for the placement itself (no GPU, no handle): where the planner puts those runs on a grid of
- * `grid` CTAs.  first_warp receives, for the runs of length 7, then 6, .. 1, the warp (CTA x 8 + place in
+ * `grid` CTAs if they belong to heads of one length.  first_warp receives, for the runs of length 7, then 6, .. 1, the warp (CTA x 8 + place in
  * the CTA) each starts at; cap is its room.  Returns the number of runs, ESTATE if they do not fit, or EINVAL
  * for a NULL array, a negative number or too little room.
  */

@@ -1347,7 +1347,7 @@ int crystalkv_debug_place_runs(int32_t whole_ctas, const int32_t* runs_by_length
   }
   if (total > cap) return CRYSTALKV_EINVAL;
   Placement p{};
-  if (whole_ctas > grid || !place_runs(whole_ctas, cnt, grid, p)) return CRYSTALKV_ESTATE;
+  if (ctas_needed(whole_ctas, cnt) > grid || !place_runs(whole_ctas, cnt, grid, true, p)) return CRYSTALKV_ESTATE;   // (as the planner asks first)
   int at = 0;
   for (int s = 7; s >= 1; --s)
     for (int r = 0; r < cnt[s]; ++r) first_warp[at++] = run_warp(p, s, r);

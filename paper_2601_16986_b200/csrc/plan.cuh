@@ -22,7 +22,7 @@ namespace ckv {
 // pieces are packed best fit, longest first.  A run goes to the open CTA with the fewest free
 // warps that still holds it, so a CTA with c free warps takes c / s runs of length s one after the
 // other: the loop below moves whole classes of CTAs at once and counts exactly what the
-// run-by-run placement does; place_runs() below walks the same classes and says where each run goes.
+// run-by-run placement does.
 __host__ __device__ __forceinline__ int ctas_needed(int full, const int (&cnt)[8]) {
   int open[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};   // open[c]: CTAs with c free warps
   int ctas = full;
@@ -50,10 +50,17 @@ __host__ __device__ __forceinline__ int ctas_needed(int full, const int (&cnt)[8
   return ctas;
 }
 
-// Where the runs go: the same walk as ctas_needed() over ranges of consecutive CTAs instead of counts.
+// Where the runs go.  Heads of one length are spread where there are 33 groups a CTA or more: a run goes to a fresh CTA while there is
+// one and then to an open CTA with the most free warps, longest runs first, so that no SM idles while another one's CTA streams eight
+// pieces.  us a layer, spread and with CTAs filled up one after the other: 150 heads of 76 groups 19.8 and 22.1, 320 of 20 13.0 and 15.2, 160 of 44 14.4
+// and 16.1, 160 of 32 11.9 and 13.1, 256 of 65 25.5 and 26.0, 1024 of 17 25.9 and 26.2, 96 of 51 (33 a CTA) 11.65 and 11.7; but 480 of 10 (32) 11.4 and 10.8, 192 of 19 (25)
+// 9.9 and 9.55.  Heads of unequal lengths gain in some launches (96 of 512 .. 1536 entries 15.9 and 16.2) and lose in others (720 of 150 .. 450
+// 25.9 and 25.4: Algorithm 1's kernels then run on SMs without an attention CTA).  All these, and runs that do not fit the other
+// way, are placed by the walk of ctas_needed(), which fits them whenever that counts no more CTAs than there are.  Both walk over
+// ranges of consecutive CTAs instead of CTAs, class by class of free warps.
 // An entry says: the runs [r0, r0 + n) of length s (in head order) fill CTAs base, base + 1, ... with q
 // runs each, from warp `off` on.  A range of CTAs visited for a length is cut into at most a consumed, a
-// partly consumed and an untouched part, so no more than 13 ranges and 35 entries arise.
+// partly consumed and an untouched part.
 constexpr int PL_SCRATCH = 320;   // ints of shared scratch that write_plan() wants
 constexpr int PL_ENTRIES = 40, PL_RANGES = 16;
 struct Placement {
@@ -63,19 +70,23 @@ struct Placement {
 };
 static_assert(sizeof(Placement) <= (PL_SCRATCH - 64) * sizeof(int), "the placement lives in the planner's scratch");
 // cnt[s]: runs of length s; full: CTAs taken whole (the first ones).  One thread.  False if they do not fit.
-__host__ __device__ inline bool place_runs(int full, const int* cnt, int grid, Placement& p) {
+template <bool SPREAD>
+__host__ __device__ inline bool place_runs_by(int full, const int* cnt, int grid, Placement& p) {
   int ne = 0, nr = 0, fresh = full;
   p.first[8] = p.first[7] = 0;
   for (int s = 7; s >= 1; --s) {
     p.first[s] = ne;
     int todo = cnt[s], done = 0;
-    for (int c = s; c <= 8 && todo > 0; ++c) {
-      const int q = c / s, live = nr;   // (ranges made while this length is placed have fewer than s warps left or one run's)
+    for (int k = s; k <= 8 && todo > 0; ++k) {
+      const int c = SPREAD ? 8 + s - k : k;             // free warps of the CTAs visited: most first, or fewest
+      const int q = SPREAD ? 1 : c / s, live = nr;      // runs one such CTA takes now
       for (int x = 0; x < (c == 8 ? 1 : live) && todo > 0; ++x) {
         int base, have;
         if (c == 8) {
           base = fresh; have = (todo + q - 1) / q;
+          if (SPREAD) have = have < grid - fresh ? have : grid - fresh;
           if (fresh + have > grid) return false;
+          if (have <= 0) continue;
           fresh += have;
         } else {
           if (p.rc[x] != c || p.rn[x] == 0) continue;
@@ -102,6 +113,9 @@ __host__ __device__ inline bool place_runs(int full, const int* cnt, int grid, P
   }
   p.first[0] = ne;
   return true;
+}
+__host__ __device__ inline bool place_runs(int full, const int* cnt, int grid, bool spread, Placement& p) {
+  return (spread && place_runs_by<true>(full, cnt, grid, p)) || place_runs_by<false>(full, cnt, grid, p);
 }
 
 // The first warp (CTA x NW + its place in the CTA) of run r of length s.
@@ -276,7 +290,7 @@ __device__ __noinline__ void write_plan(const State& st, const Plan& pl, int lay
     // One thread walks the classes of CTAs, then every head looks its run up.  (A
     // plan of 128 heads takes 9 us; one warp placing the runs one by one took it to 26.)
     if (tid == 0) {
-      const bool ok = wholes <= grid && place_runs(wholes, runs, grid, place);
+      const bool ok = wholes <= grid && place_runs(wholes, runs, grid, Gtot == gmax * U && Gtot >= 33 * grid, place);
       place.first[8] = ok;
       if (!ok) atomicOr(st.errword, ERR_PLAN);   // cannot happen while ctas_needed() counts the same walk
     }

@@ -105,6 +105,33 @@ def test_the_planners_count_equals_placing_the_runs_one_by_one(lib):
     assert lib.crystalkv_debug_ctas_needed(-1, (C.c_int32 * 8)()) == -1
 
 
+def test_placed_runs_are_spread_over_the_grid(lib):
+    """With more CTAs than the runs need, every CTA gets a run before one gets two (where ranges of like CTAs allow to say
+    so in the planner's memory: always for runs of up to three lengths)."""
+    rng = np.random.RandomState(11)
+    where = np.zeros(1200, dtype=np.int32)
+    for trial in range(2000):
+        runs, grid, whole = [0] * 8, int(rng.randint(1, 149)), int(rng.randint(0, 5))
+        for s in rng.choice(np.arange(1, 8), int(rng.randint(1, 4)), replace=False):
+            runs[s] = int(rng.randint(0, 60))
+        arr = (C.c_int32 * 8)(*runs)
+        if lib.crystalkv_debug_ctas_needed(whole, arr) > grid or whole + sum(runs) == 0:
+            continue
+        got = lib.crystalkv_debug_place_runs(whole, arr, grid, where.ctypes.data_as(C.c_void_p), len(where))
+        assert got == sum(runs)
+        ctas = set((where[:got] // 8).tolist())
+        taken, at = np.zeros(8 * grid, dtype=np.int32), 0
+        taken[:8 * whole] = 1
+        for s in range(7, 0, -1):
+            for _ in range(runs[s]):
+                assert where[at] % 8 + s <= 8
+                taken[where[at]:where[at] + s] += 1
+                at += 1
+        assert taken.max(initial=0) <= 1
+        if whole + sum(runs) <= grid:
+            assert len(ctas) == got
+
+
 def test_placed_runs_fit_their_ctas_and_do_not_overlap(lib):
     """The planner's placement: every run sits inside one CTA, no two share a warp, none touches the CTAs taken
     whole, and it fits a grid exactly when the counting rule says so."""
