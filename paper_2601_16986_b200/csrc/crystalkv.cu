@@ -840,7 +840,8 @@ static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, cons
     const bool small = P <= WH_SMALL && (long long)p.W * h->U >= P + h->num_sms;
     CK(h, launch_next(small ? window_hits_kernel<64> : window_hits_kernel<NT>, dim3(p.W, h->U), small ? 64 : NT, sm, s, h->st, p, c.top_p,
                       c.literal_return, sm > 0));
-    CK(h, launch_next(window_apply_kernel, dim3(1 + h->U), NT, 0, s, h->st, p, last, c.evict_every, reinterpret_cast<int*>(h->sc_pbar[1]),
+    const bool wide = P > APPLY_LINE && 2 * h->U <= h->num_sms;
+    CK(h, launch_next(wide ? window_apply_kernel<APPLY_WIDE> : window_apply_kernel<NT>, dim3(1 + h->U), wide ? APPLY_WIDE : NT, 0, s, h->st, p, last, c.evict_every, reinterpret_cast<int*>(h->sc_pbar[1]),
                       h->cap_s, h->plans[layer], plan_grid, h->cl[layer], h->plan_len));
   }
   return CRYSTALKV_OK;

@@ -33,8 +33,10 @@ constexpr int SCORE_SMEM = 1024 + NW * SCORE_STAGES * (SCORE_ITEM + 8);
 //   mk: k [batch][P][H][128], boxes of 64 channels x 32 tokens of a head   q_last: [batch][Hq][128]   partials: [U][chunks][16] = m, l
 // Bound: HBM.  Every warp keeps a ring of three items full by TMA, like the attention kernel's of pages, and eight warps that
 // read the heads of the same tokens keep to the same DRAM pages; the products are mma.sync with keys on M and the (padded) query
-// heads on N, 16 per item.  64 heads x 9350 tokens (153 MB): SCORE_NOW (a thread per key with fp32 multiply-adds from shared memory, three
-// CTAs of 64 KB an SM: 45.5 us, half of its cycles spent on 16-byte broadcasts of the queries).
+// heads on N, 16 per item.  64 heads x 9350 tokens (153 MB of keys, 19 MB of
+// logits): 35.5 us (a thread per key with fp32 multiply-adds from shared memory, three
+// CTAs of 64 KB an SM: 45.5 us, half of its cycles spent on 16-byte broadcasts of the queries), 128 heads x 512 tokens 8.0 (9.3).  Error of a scaled
+// logit against 64 bits, keys N(0, 1): rms 6.95e-8, largest of 524288 8.8e-7 (7.25e-8 and 1.1e-6 with one chain of multiply-adds).
 __global__ void __launch_bounds__(NT, 1) prefill_score_kernel(Scratch sc, const __grid_constant__ CUtensorMap mk, const __nv_bfloat16* __restrict__ q_last,
                                                               int batch, int H, int G, int P, int warps, float scale, float scale_log2, int* errword) {
   extern __shared__ unsigned char s_raw[];
@@ -189,7 +191,7 @@ __device__ __forceinline__ bool take_pages(const State& st, int uid, int seq, in
 // fixed_budget > 0 sets the heads' budget first.
 // Bound: latency (a few block-wide steps over 36 bytes per token); 1024 threads keep a prompt of
 // 10 000 tokens at ten entries per thread, pbar in shared memory up to SEL_SMEM bytes.
-// 64 heads x 9350 tokens cut to 935: 25.9 us (40.6 while the threshold search fell back to its radix passes);
+// 64 heads x 9350 tokens cut to 935: 22 us (25.9 with a pass over the logits for the normalisers, which the items bring now);
 // the decode step's Algorithm 1 kernel with its radix
 // select over 96-bit keys in global memory took 286 us.  128 heads x 512 tokens: 10.9 us.
 __global__ void __launch_bounds__(SEL_NT) prefill_select_kernel(State st, Scratch sc, int layer, int P, int G, int chunks,

@@ -2,8 +2,7 @@
 // already stored.  Which entries a query hits depends on its scores alone, not on what earlier
 // queries of the window marked, so the window is one attention kernel over all (query, head) rows,
 // one threshold search per (head, query), and one kernel that walks an entry through its queries.
-// 128 heads x 1024 tokens, 32 queries of 5 heads: 95 + 36 + 16 us a layer, the pages and the launch plan included (as kernels
-// of their own they took 20 and 9 us, the three others 85 + 50 + 20); a decode-step launch pair
+// 128 heads x 1024 tokens, 32 queries of 5 heads: 59 + 20 + 16 us a layer, the pages and the launch plan included; a decode-step launch pair
 // per query, each reading the prompt's rows again, took 720 us.
 #pragma once
 #include "evict.cuh"
@@ -14,18 +13,20 @@
 namespace ckv {
 
 constexpr int WIN_SMEM = 32 * 1024;           // pbar of up to this many bytes stays in shared memory
+constexpr int APPLY_WIDE = 1024;              // threads of window_apply_kernel for few heads' prompts of more than APPLY_LINE tokens
+constexpr int APPLY_LINE = 2048;
 constexpr int WH_SMALL = 1280;                // entries up to which window_hits_kernel may take CTAs of two warps
 
 // The hit bits of one (query, head): Algorithm 1 step 1 with the query of time t over its t + 1 entries.
 // grid: (W, U).
-// Bound: issue slots (some hundred instructions per warp beside those per entry), three quarters of which are in use:
-// many searches of short prompts take CTAs of two warps, and the query heads are a template argument.  Few searches are bound by
+// Bound: issue slots (some hundred instructions per warp beside those per entry):
+// many searches of short prompts take CTAs of two warps.  Few searches are bound by
 // the latency of one: the line is as many searches as entries and SMs, and WH_SMALL entries.  us with two warps and with
-// eight: 64 heads, 300 entries, 512 searches 6.4 and 6.7, 1024 7.7 and 10.7; 16 heads, 128 searches 6.0 and 4.5; 1024 entries, 128
-// searches 10.7 and 5.0, 512 12.0 and 7.7, 1024 13.3 and 12.8, 1536 15.6 and 17.3; 1280 entries, 512 searches 14.7 and 10.1, 2048 23.6
-// and 28.5, 4096 45.4 and 54.3; 1600 entries, 4096 searches 61.2 and 60.2, 2048 entries 74.7 and 65.4.
-// 128 heads x 32 queries over 1000 entries: 36 us.
-// pbar lives in shared memory or, for long prompts, in the place of the first query head's logits.
+// eight, while the searches still took the means themselves: 64 heads, 300 entries, 512 searches 6.4 and 6.7, 1024 7.7 and 10.7; 16 heads, 128
+// searches 6.0 and 4.5; 1024 entries, 128 searches 10.7 and 5.0, 512 12.0 and 7.7, 1024 13.3 and 12.8, 1536 15.6 and 17.3; 1280 entries, 2048 23.6
+// and 28.5; 1600 entries, 4096 searches 61.2 and 60.2.
+// 128 heads x 32 queries over 1000 entries: 20 us (36 with the logits of five heads to read and weigh).
+// pbar lives in shared memory or, for long prompts, where it is.
 template <int NTH>
 __global__ void __launch_bounds__(NTH) window_hits_kernel(const __grid_constant__ State st, const WindowParams p, float top_p, int literal,
                                                           int in_smem) {
@@ -101,14 +102,18 @@ __global__ void __launch_bounds__(NTH) window_hits_kernel(const __grid_constant_
 // Bound: latency (W dependent multiply-adds per entry; with many heads the plan).  The three kernels of a window with the plan
 // written here, and by one CTA of the threshold searches, which starts last and has two warps: 128 heads x 1024 tokens, 32
 // queries 151 us and 155, 1024 heads x 300 tokens, 2 queries 144 and 193, 1024 heads x 256 tokens, 32 queries 241 and 292.
-__global__ void __launch_bounds__(NT) window_apply_kernel(const __grid_constant__ State st, const WindowParams p, int last, int evict_every,
+// Heads that fill half of the SMs at most take CTAs of 1024 threads for long prompts; with more heads the plan is what takes long, and that
+// takes longer with more warps.  us a layer of windows with 1024 threads and with 256: 16 heads x 3000 tokens 96 and 102, x 6000 174 and 197, x
+// 12000 338 and 377, 64 heads x 4096 129 and 143, 2 heads x 2100 60.5 and 61; but 128 heads x 2100 119 and 113, x 3000 151 and 146.
+template <int NTH>
+__global__ void __launch_bounds__(NTH) window_apply_kernel(const __grid_constant__ State st, const WindowParams p, int last, int evict_every,
                                                           int* tmp, int tmp_stride, const __grid_constant__ Plan plan, int plan_grid,
                                                           int plan_cl, int* plan_len) {
   __shared__ __align__(16) int sh[PL_SCRATCH];
   pdl_wait();
   pdl_launch();
   if (blockIdx.x == 0) {
-    if (last) write_plan<NT>(st, plan, p.layer, plan_grid * NW, plan_grid, plan_cl, plan_len, sh, evict_every);
+    if (last) write_plan<NTH>(st, plan, p.layer, plan_grid * NW, plan_grid, plan_cl, plan_len, sh, evict_every);
     return;
   }
   const int u = blockIdx.x - 1, seq = u / st.H, tid = threadIdx.x;
@@ -117,7 +122,7 @@ __global__ void __launch_bounds__(NT) window_apply_kernel(const __grid_constant_
   const size_t mb = (size_t)uid * st.cap;
   int nhit = 0;
   const int lane = tid & 31;
-  for (int i0 = tid - lane; i0 < p.P; i0 += NT) {   // a warp takes 32 entries: one word of hit bits per query, a word per lane
+  for (int i0 = tid - lane; i0 < p.P; i0 += NTH) {   // a warp takes 32 entries: one word of hit bits per query, a word per lane
     const int i = i0 + lane, e = min(i, p.P - 1);
     float crf = st.meta_crf[mb + e];
     int tau = st.meta_tau[mb + e];
@@ -148,7 +153,7 @@ __global__ void __launch_bounds__(NT) window_apply_kernel(const __grid_constant_
   const int B = st.budget[uid];
   __syncthreads();
   if (p.P - B >= evict_every && p.P > 1)
-    evict_many(st, uid, seq, p.P, min(p.P - B, p.P - 1), p.t0 + p.W - 1, true, sh, tmp + (size_t)u * tmp_stride);
+    evict_many<NTH>(st, uid, seq, p.P, min(p.P - B, p.P - 1), p.t0 + p.W - 1, true, sh, tmp + (size_t)u * tmp_stride);
 }
 
 }  // namespace ckv
