@@ -1,7 +1,7 @@
 // C ABI of the Crystal-KV decode hot path (see include/crystalkv.h).  Host code only
 // validates, keeps the per-layer clocks and launches; every step of the path runs in the
 // kernels of attn_kernel.cuh and lrfu_kernel.cuh (a decode step; its launch plan: plan.cuh),
-// prefill_kernels.cuh and window_kernels.cuh (prompts) and aux_kernels.cuh (reallocations, exports).
+// prefill_kernels.cuh, window_attn.cuh and window_kernels.cuh (prompts) and aux_kernels.cuh (reallocations, exports).
 //
 // Stream plan of a tracked decode step of layer l: the attention kernel runs on the caller's
 // stream (so `out` is ready in stream order), the LRFU kernel of the same layer on an
@@ -37,6 +37,7 @@ using namespace ckv;
 struct DeviceKit {
   void* arena = nullptr;           // the one device allocation that all arrays of the handle lie in
   size_t arena_bytes = 0;
+  unsigned long long context = 0;  // of the CUDA context that all of this belongs to (a device reset ends it); 0: unknown
   // LRFU launches are numbered; launch k uses scratch set k % NSETS and event k % EV_RING
   static constexpr int EV_RING = 32;
   // two internal streams taken in turn: the LRFU kernels of consecutive layers do not depend on
@@ -149,11 +150,7 @@ struct DeviceScope {
 // while a quarter of its memory is free; crystalkv_trim, a handle that it does not fit and an allocation
 // that fails for want of memory give it back.  (A pool of the driver's gives back by itself, but its first 5.5 GB took 34 to 280 ms.)
 constexpr size_t KEEP_BYTES = size_t(8) << 30;
-struct Kept {
-  DeviceKit kit;
-  unsigned long long context = 0;   // of the CUDA context that the kit belongs to (a device reset ends it); 0: nothing is kept
-};
-Kept g_kept[MAX_DEVICES];
+DeviceKit g_kept[MAX_DEVICES];   // (context 0: nothing is kept)
 std::mutex g_kept_mu;
 
 unsigned long long context_id() {   // of the current context, 0: unknown
@@ -187,9 +184,8 @@ void free_kit(DeviceKit& k) {
 // The kit that the current device keeps, if it belongs to the current context, taken out; an empty one else.
 DeviceKit take_kept(int device) {
   std::lock_guard<std::mutex> lock(g_kept_mu);
-  Kept& k = g_kept[device];
   DeviceKit kit;
-  if (k.context && k.context == context_id()) std::swap(kit, k.kit), k.context = 0;
+  if (g_kept[device].context && g_kept[device].context == context_id()) std::swap(kit, g_kept[device]);
   return kit;
 }
 
@@ -200,11 +196,8 @@ bool keep_kit(int device, const DeviceKit& kit) {
   if (cudaMemGetInfo(&room, &total) != cudaSuccess) { cudaGetLastError(); return false; }
   if (room < total / 4) return false;
   std::lock_guard<std::mutex> lock(g_kept_mu);
-  Kept& k = g_kept[device];
-  const unsigned long long id = context_id();
-  if (k.context || !id) return false;
-  k.kit = kit;
-  k.context = id;
+  if (g_kept[device].context || !kit.context || kit.context != context_id()) return false;
+  g_kept[device] = kit;
   return true;
 }
 
@@ -244,6 +237,7 @@ struct Arena {
                     std::string("cudaMalloc: ") + cudaGetErrorString(e));
       }
       kit.arena_bytes = bytes;
+      kit.context = context_id();
     }
     for (const Part& x : parts) *x.where = static_cast<unsigned char*>(kit.arena) + x.at;
     return CRYSTALKV_OK;
