@@ -245,8 +245,7 @@ template <bool SHARED, bool TRACK>
 __global__ void __maxnreg__(160) attn_kernel(const DecodeParams p) {   // (160 registers: two LRFU CTAs fit beside it on an SM)
   extern __shared__ __align__(1024) unsigned char smem[];
   const State& st = p.st;
-  // Without `early` the kernel before this one may still be writing the lists this one reads.
-  if (!p.early) pdl_wait();
+  // Without `early` this is an ordinary launch: the kernel ahead, which may have written the lists that this one reads, has ended.
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   // ring stages, then one mbarrier per stage, then every warp's queue of fetched pieces
   const uint32_t bars_u32 = smem_u32(smem) + RING_BYTES;

@@ -447,7 +447,8 @@ int join_side(crystalkv_t* h, cudaStream_t s) {
 }
 
 // A launch that may start before the kernel ahead of it in the stream has ended; the kernel waits for that (griddepcontrol.wait).
-// The kernels of a prompt let the next one start once they have themselves waited, so everything before the kernel ahead has ended by then.
+// The kernels of a prompt let the next one start once they have themselves waited, so everything before the kernel ahead has ended by then;
+// what the kernel ahead writes is read with ordinary loads, after the wait.  The last one lets nothing start: what follows it is none of them.
 // Ordinary launches leave 1 to 2 us between two of them: a new batch of 16 prompts of 512 tokens 1.75 ms and 1.62, windows of 32 queries 6.1 and 5.8.
 template <class... P, class... A>
 cudaError_t launch_next(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A... args) {
@@ -527,8 +528,9 @@ int launch_step(crystalkv_t* h, DecodeParams& p, int layer, cudaStream_t s) {
   }
   // The attention kernel may start while the kernel ahead of it still runs: it first fills its
   // pipeline from the cache and waits for that kernel before it touches the call's inputs.
-  // That is only sound if the kernel ahead cannot be writing this layer's lists, which holds
-  // when it is the attention kernel of another layer.
+  // That is only sound if the kernel ahead cannot be writing this layer's lists or plan, which holds
+  // when it is the attention kernel of another layer.  Else the launch is an ordinary one: it is not enough to wait
+  // inside, because the kernel reads them through the read-only path, which wants them final when it starts.
   p.early = (h->prev_layer >= 0 && h->prev_layer != layer) ? 1 : 0;
   {
     cudaLaunchConfig_t lc{};
@@ -538,7 +540,7 @@ int launch_step(crystalkv_t* h, DecodeParams& p, int layer, cudaStream_t s) {
     lc.stream = s;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[0].val.programmaticStreamSerializationAllowed = p.early;
     at[1].id = cudaLaunchAttributeClusterDimension;
     at[1].val.clusterDim.x = p.cl;
     at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;

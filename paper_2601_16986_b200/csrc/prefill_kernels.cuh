@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(NT) prefill_rows_kernel(const __grid_constant_
   __shared__ int s_gs[MAX_UNITS_PER_CALL + 1];
   __shared__ int s_red[320];
   pdl_wait();
-  pdl_launch();
+  if (plan_warps == 0) pdl_launch();   // (a window's kernels follow; else this is the prompt's last)
   if (blockIdx.x == 0) {
     if (plan_warps > 0) write_plan(st, plan, layer, plan_warps, plan_grid, plan_cl, s_gs, s_red);
     return;

@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(WA_THREADS, 1) window_attn_kernel(const __grid
       const int x = what(i), tile = x < 0 ? -1 - x : x, stage = i % S, turn = tile % gridDim.x, at = tile * WA_KEYS + lane * GRP;
       const bool mine = store && (i < nt || x < 0) && blockIdx.x == ((tile + 1) * WA_KEYS <= keys_of(turn) ? turn : last) &&
                         lane < WA_KEYS / GRP && at < p.P;
-      const int page = mine ? __ldg(st.ptab + (size_t)uid * st.capg + at / GRP) : 0;
+      const int page = mine ? __ldcg(st.ptab + (size_t)uid * st.capg + at / GRP) : 0;
       wait(bar_ld + 8 * stage, i / S);
       if (mine && !dead) {   // (rows past the prompt's end are zeros and go to places without an entry)
         for (int y = 0; y < 2; ++y)

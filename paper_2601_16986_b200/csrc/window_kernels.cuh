@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(NTH) window_apply_kernel(const __grid_constant
                                                           int plan_cl, int* plan_len) {
   __shared__ __align__(16) int sh[PL_SCRATCH];
   pdl_wait();
-  pdl_launch();
+  if (!last) pdl_launch();
   if (blockIdx.x == 0) {
     if (last) write_plan<NTH>(st, plan, p.layer, plan_grid * NW, plan_grid, plan_cl, plan_len, sh, evict_every);
     return;
