@@ -102,7 +102,8 @@ int crystalkv_trim(int device);
  * A prompt longer than the budget is scored from k and q_last as they are, and only the rows
  * of the entries Algorithm 1 retains are stored, so the pool never holds more than the budget.
  * P must satisfy 1 <= P < max_context and P <= max_budget + evict_every + max_answer_tokens (the
- * heads' list capacity).  Errors: EINVAL; ESTATE if the layer was prefilled.
+ * heads' list capacity); k and v must be 16-byte aligned.  Errors: EINVAL; ESTATE if the layer was prefilled;
+ * ECUDA.  A call refused with EINVAL or ESTATE has changed nothing: the layer is still to be loaded.
  */
 int crystalkv_prefill(crystalkv_t* h, int layer, const void* k, const void* v,
                       const void* q_last, int P, void* stream);
@@ -121,7 +122,8 @@ int crystalkv_prefill(crystalkv_t* h, int layer, const void* k, const void* v,
  * has run.  1 <= W <= P, and P <= budget_per_head + max_answer_tokens in evict mode (the window's
  * outputs need every token's values, so the whole prompt is stored before the one eviction).
  * FullKV mode: only the insertion
- * (and out_window, if asked for, stays untouched).  Errors: EINVAL; ESTATE if the layer was prefilled.
+ * (and out_window, if asked for, stays untouched).  k and v must be 16-byte aligned, q_window and out_window
+ * 4-byte aligned (not looked at in FullKV mode).  Errors: as crystalkv_prefill.
  */
 int crystalkv_prefill_window(crystalkv_t* h, int layer, const void* k, const void* v,
                              const void* q_window, int P, int W, void* out_window, void* stream);

@@ -801,8 +801,9 @@ static bool window_fills_pages(const crystalkv_t* h, int P, int W) {
 // asks for (usually one): steps 1-3 for every query, step 4 after the last one.  Everything runs on
 // `s`, which has joined the internal streams: the logit sets, one block of the arena, hold the
 // window's group means, the first pbar area the hit bits.
-static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, const unsigned char* v, const unsigned char* q,
-                         int P, int W, __nv_bfloat16* out, bool fill_pages, cudaStream_t s) {
+// mk, mv, mp: tiles of the prompt's keys and values, the pool.
+static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, const unsigned char* v, const unsigned char* q, int P, int W,
+                         __nv_bfloat16* out, bool fill_pages, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mp, cudaStream_t s) {
   const crystalkv_config_t& c = h->cfg;
   WindowParams p{};
   p.k = k; p.v = v;
@@ -816,9 +817,6 @@ static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, cons
   const int fit = window_queries(h, P);
   const size_t sm = (size_t)P * sizeof(float) <= WIN_SMEM ? (size_t)P * sizeof(float) : 0;
   const int plan_grid = h->plan_grid(layer);
-  CUtensorMap mk, mv, mp;
-  if (!tile_map(&mk, k, c.batch, P, c.n_kv_heads, WA_KEYS) || !tile_map(&mv, v, c.batch, P, c.n_kv_heads, WA_KEYS) || !pool_map(&mp, h))
-    return fail(h, CRYSTALKV_EINVAL, "k and v must be 16-byte aligned");
   const size_t qn = (size_t)c.batch * c.n_q_heads * HD;
   for (int w0 = 0; w0 < W; w0 += p.W) {
     p.W = std::min(W - w0, fit);
@@ -860,9 +858,20 @@ static int prefill_common(crystalkv_t* h, int layer, const void* k, const void* 
     return fail(h, CRYSTALKV_EINVAL, "prompt with an observation window longer than budget_per_head + max_answer_tokens");
   if (evict && P + 1 > h->cap) return fail(h, CRYSTALKV_EINVAL, "prompt longer than the heads' list capacity (max_budget + evict_every + max_answer_tokens)");
   if (P >= c.max_context) return fail(h, CRYSTALKV_EINVAL, "prompt reaches max_context");
+  const auto misaligned = [](const void* x, uintptr_t bytes) { return reinterpret_cast<uintptr_t>(x) % bytes != 0; };
+  if (misaligned(k, 16) || misaligned(v, 16)) return fail(h, CRYSTALKV_EINVAL, "k and v must be 16-byte aligned");
+  if (evict && W > 0 && (misaligned(q, 4) || misaligned(out_window, 4)))
+    return fail(h, CRYSTALKV_EINVAL, "q_window and out_window must be 4-byte aligned");
   if (h->t_layer[layer] >= 0) return fail(h, CRYSTALKV_ESTATE, "layer already prefilled");
   ON_DEVICE(h);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  // All that a call may be refused for comes before the first launch and the first change: a refused layer is still to be loaded.
+  CUtensorMap mk{}, mv{}, mp{};
+  if (evict) {
+    bool ok = tile_map(&mk, k, c.batch, P, c.n_kv_heads, W > 0 ? WA_KEYS : SCORE_KEYS);
+    if (W > 0) ok = ok && tile_map(&mv, v, c.batch, P, c.n_kv_heads, WA_KEYS) && pool_map(&mp, h);
+    if (!ok) return fail(h, CRYSTALKV_ECUDA, "the driver makes no tensor maps (cuTensorMapEncodeTiled)");
+  }
   rc = join_side(h, s);   // the insertion takes pages; no LRFU kernel may take or return any meanwhile
   if (rc) return rc;
   const auto* kb = static_cast<const unsigned char*>(k);
@@ -881,8 +890,6 @@ static int prefill_common(crystalkv_t* h, int layer, const void* k, const void* 
     const size_t sm = (size_t)P * sizeof(float) <= SEL_SMEM ? (size_t)P * sizeof(float) : 0;
     if (sm > 32 * 1024)
       CK(h, cudaFuncSetAttribute(prefill_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SEL_SMEM));
-    CUtensorMap mk;
-    if (!tile_map(&mk, k, c.batch, P, c.n_kv_heads, SCORE_KEYS)) return fail(h, CRYSTALKV_EINVAL, "k must be 16-byte aligned");
     const long long items = (long long)c.batch * chunks * c.n_kv_heads;
     const int ctas = (int)std::min<long long>(h->num_sms, (items + NW - 1) / NW);
     const int warps = ctas * NW < c.n_kv_heads ? ctas * NW : ctas * NW / c.n_kv_heads * c.n_kv_heads;
@@ -911,7 +918,8 @@ static int prefill_common(crystalkv_t* h, int layer, const void* k, const void* 
                       W > 0 ? ROWS_ALL : ROWS_ALL_LAST, per_head, evict ? 0 : plan_grid * NW, plan_grid, h->cl[layer]));
   }
   if (evict) {
-    rc = replay_window(h, layer, kb, vb, static_cast<const unsigned char*>(q), P, W, static_cast<__nv_bfloat16*>(out_window), fill_pages, s);
+    rc = replay_window(h, layer, kb, vb, static_cast<const unsigned char*>(q), P, W, static_cast<__nv_bfloat16*>(out_window), fill_pages,
+                       mk, mv, mp, s);
     if (rc) return rc;
   }
   h->t_layer[layer] = P - 1;
