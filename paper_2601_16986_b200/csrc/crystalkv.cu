@@ -379,26 +379,40 @@ int find_clusters(crystalkv_t* h) {
 
 // CTAs that share a head of `entries` entries, where there is room for a cluster per head (find_clusters): a launch bound by
 // its chain of dependent steps (pieces of at most GLAT groups) gains what its warps stream less, a group being worth
-// about 0.4 us and the wider merge as much.  us a layer on one CTA, two and four: 24 layers of 32 heads of 25 groups 6.3, 6.1, 7.0; of 38
-// 7.4, 6.6, 6.9; of 50 9.1, 7.5, 7.4; of 65 10.6, 8.5, 8.3; 64 heads of 25 groups 7.1 and 7.2, of 30 7.3 and 7.0, of 65 12.55 and 10.1;
-// 16 heads of 25 groups 6.1, 7.1, 6.0, of 42 7.9, 6.3, 6.0; one layer of 2 heads of 17 groups 16.4 each way, of 21 18.1, 16.7, 16.5, of 38
-// 19.3, 17.3, 16.9.  So two CTAs from two groups a warp on (one, if the handle has one layer: its launches cannot start
-// early), four where that is two groups less again, or one while the CTAs do not fill half the SMs.  A handle of
-// two layers keeps the line of four groups (40 groups, 2 heads 10.3, 9.4, 8.4: its launch shapes are stated by a test).
+// about 0.4 us and the wider merge as much, and loses where the clusters leave Algorithm 1's kernels no SM without an attention CTA.
+//
+// Two CTAs, by the groups a warp streams without sharing.  us a layer on one CTA and on two (24 layers where nothing else is said):
+//  * one layer, whose launches cannot start early: from two.  2 heads of 17 groups 17.8 and 16.3, 64 of 33 20.5 and 18.4; 1 head of 12 16.4
+//    and 15.0, 74 of 16 18.8 and 17.7 (of 9 groups 17.0 and 17.4).
+//  * two layers: from four groups less with sharing than without.  The line is older than these figures and higher than it need be.
+//  * from three while two CTAs a head fill half of the SMs at most: 1 head of 17 groups 5.95 and 5.15, 16 of 17 6.3 and 5.55, 32 of 17 6.35 and 5.75 (on
+//    four, which make pieces of two groups as well, 6.85); of 24 6.8 and 5.8.
+//  * else from four: 50 heads of 41 groups 8.4 and 7.0, 60 of 33 7.6 and 7.2, 64 of 25 6.7 and 6.75, of 30 7.05 and 6.9, of 33 7.75 and 7.5;
+//    68 of 30 7.3 and 7.4, of 33 8.0 and 7.85; three layers, 70 of 25 10.25 and 9.05.
+//  * from five where fewer than twelve SMs are left (70 of 25 6.9 and 7.2, of 33 8.1 and 8.0, of 40 8.8 and 8.5; 72 of 30 7.4 and 7.75),
+//    from six for heads of one length where fewer than four are (74 of 25 7.1 and 7.8, of 33 8.25 and 8.75, of 40 9.05 and 9.15, of 41 9.55 and 9.3; with unequal budgets of
+//    33 groups on average 8.85 and 8.85, of 40 10.15 and 9.3).  Not with three layers: 74 of 25 10.3 and 8.95 (but of 40 11.4 and 12.1).
+// Four CTAs where their pieces are two groups shorter again, and from four groups a warp without sharing on while they fill half of the SMs at
+// most (below, the plan makes pieces of two groups either way): 32 heads of 41 groups 6.5 on two and 6.95 on four, of 50 7.5 and 7.4, of 65 8.5 and
+// 8.3; 16 of 17 5.55 and 5.7, of 30 5.75 and 5.75, of 33 6.15 and 5.7, of 41 6.3 and 5.85; three layers with unequal budgets, 4 of 30 on average 9.35 and 8.25.
+//
 // Longer heads of one length (from 193 groups, where they no longer fit a CTA in pieces of 2 GLAT) gain from two CTAs where their
 // other choice is more than eight pieces and a merge through global memory at the end of the launch.  The longer the pieces,
 // the more the CTAs that then have nothing to stream count: up to 14 groups a piece from 45 heads on, up to 24 from 52.  us a
 // layer, not shared and shared, of 194, 226, 257, 313 and 376 groups: 48 heads 21.7 21.4 23.3 27.5 37.1 and 18.2 20.6 22.8 26.5 31.6; 52 heads 22.2
-// 22.4 25.0 29.4 37.4 and 18.5 21.1 23.5 27.6 35.1; 64 heads of 257 28.2 and 27.1.  (The lines are older than these figures, by which 40 heads of
-// 194 groups, 20.7 and 17.7, and 48 of 376 would share as well; tests state the lines.)
+// 22.4 25.0 29.4 37.4 and 18.5 21.1 23.5 27.6 35.1; 64 heads of 257 28.2 and 27.1.  (These lines, too, are older than the figures, by which 40 heads of
+// 194 groups, 20.7 and 17.7, and 48 of 376 would share as well.)
 int share_heads(crystalkv_t* h, int entries) {
   const int g = (entries + GRP - 1) / GRP, alone = (g + NW - 1) / NW;
+  const int layers = h->cfg.n_layers, left = h->num_sms - 2 * h->U;   // SMs that two CTAs a head leave
   auto per = [&](int cl) { return (g + NW * cl - 1) / (NW * cl); };
   const bool merge = h->uniform && 10 * h->U >= 3 * h->num_sms && alone > 2 * GLAT &&
                      per(2) <= (20 * h->U >= 7 * h->num_sms ? 2 * GLAT : GLAT + 2);
-  const int least = h->cfg.n_layers == 2 ? 4 : h->cfg.n_layers == 1 ? 1 : 2;
-  auto pays = [&](int cl) { return h->share_ok[cl] && (per(cl) <= GLAT || (cl == 2 && merge)) && alone - per(cl) >= least; };
-  if (pays(4) && (!pays(2) || per(2) - per(4) >= (8 * h->U <= h->num_sms ? 1 : 2))) return 4;
+  const int from = layers == 1 ? 2 : 4 * h->U <= h->num_sms ? 3 : layers == 3 || left >= 12 ? 4 : left >= 4 || !h->uniform ? 5 : 6;
+  auto pays = [&](int cl) {
+    return h->share_ok[cl] && (per(cl) <= GLAT || (cl == 2 && merge)) && (layers == 2 ? alone - per(cl) >= 4 : alone >= from);
+  };
+  if (pays(4) && (!pays(2) || (8 * h->U <= h->num_sms ? alone >= 4 : per(2) - per(4) >= 2))) return 4;
   return pays(2) ? 2 : 1;
 }
 static_assert(MAX_CLUSTER == 4, "share_heads weighs two CTAs and four");
