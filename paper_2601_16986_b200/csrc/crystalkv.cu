@@ -795,19 +795,42 @@ int crystalkv_time(crystalkv_t* h, int layer) {
   return h->t_layer[layer];
 }
 
-// Queries of a window over P tokens that one launch replays: what the logit sets and the pbar area have room for.
-static int window_queries(const crystalkv_t* h, int P) {
+// Queries of a window over P tokens that one launch replays: what the logit sets, the pbar area and, for mma.sync, which keeps the logits
+// of every query head, the partials have room for.
+static int window_queries(const crystalkv_t* h, int P, bool tc) {
   const long long rows = (P + 7) / 8 * 8, words = (P + 31) / 32;
-  return (int)std::max<long long>(1, std::min({(long long)NSETS * h->cap_s * QH / rows, h->cap_s / words, 1ll << 30}));
+  return (int)std::max<long long>(1, std::min({(long long)NSETS * h->cap_s * QH / (tc ? rows : h->G * rows),
+                                               tc ? 1ll << 30 : (long long)h->pmax * (16 + h->G * HD) / 16, h->cap_s / words, 1ll << 30}));
 }
+
+// Whether the attention of a window runs on tcgen05 (window_attn.cuh: one CTA an SM, three passes over the keys) or on mma.sync
+// (window_mma.cuh: three CTAs an SM, one pass).  us a layer, all kernels of the window, on tcgen05 and on mma.sync:
+//  * With outputs the products decide, except for prompts of one tile, whose CTAs are all start and end, with more heads than SMs (8 queries
+//    of 5 heads: 1024 heads x 40 tokens 100 and 79; 1 query of 5: 512 x 64 50 and 45; but 160 x 100 33 and 37) or more than 128 rows (32 of 5: 48 x 64 36 and 31), and for
+//    very many heads with many queries over little more (64 of 1: 1024 x 129 292 and 271; but 64 of 5: 512 x 300 307 and 412).
+//  * Without outputs there is half the work for the tensor cores, and the three passes show: with more heads than SMs (1 query of 5: 1024 x 300 159 and
+//    134; 8 of 2: 256 x 1000 126 and 117) unless the logits of all heads, which mma.sync leaves in memory, cost more (32 of 5: 256 x 1000 182
+//    and 249), and with one query head over long prompts (64 of 1: 32 x 2048 163 and 153, 8 of 1: 128 x 4096 222 and 207; but 64 of 1: 16 x 129 47 and 55).
+//  * Where the scratch holds the logits of all heads of fewer queries than it holds means, another launch costs more than all of this (64 of 8
+//    with outputs: 32 x 64 50 and 78), but for very many heads.
+static bool window_tcgen05(const crystalkv_t* h, int P, int W, bool out) {
+  auto launches = [&](bool tc) { return (W - 1) / window_queries(h, P, tc); };
+  const bool very = h->U > 4 * h->num_sms, once = launches(false) == launches(true), many = h->U > h->num_sms && (once || very);
+  if (out) return !(P <= 64 && (many || (once && (long long)W * h->G > 128))) && !(very && P <= 192 && W >= 32);
+  return !(many && !(h->G >= 5 && W >= 16 && P >= 256)) && !(h->G == 1 && W >= 8 && P >= 1000);
+}
+// Row blocks of a head on tcgen05.  Without outputs small ones for few heads, from 512 tokens on: 16 heads x 4096 tokens, 16 queries of 8 heads
+// 104 us a layer instead of 128; but 32 heads x 300, 16 of 5 34 and 32.
+static int window_blocks_of(const crystalkv_t* h, int P, int W, bool out) { return window_blocks(W, h->G, out || P < 512 ? 0 : h->num_sms / h->U); }
 
 // Whether a window's attention kernel also fills the pages, from the tiles it reads: a tile's pages hold up one of a head's
 // CTAs, which take the tiles in turn, 0.6 us, a copy kernel over the whole chip takes 4.5 us and the time of the bytes.  The window's kernels of a layer,
 // pages from the tiles and copied: 2 heads x 4096 tokens, 1 query 120 us and 105; 16 heads x 4096, 6 queries 140 and 133, x 12000, 8 queries 416
 // and 380, x 1024, 8 queries 43.5 and 45; 32 heads x 2048, 8 queries 79 and 82; 40 heads x 1024, 32 queries 75 and 82; 64 heads x
 // 1024, 2 queries 43 and 50, x 4096, 6 queries 141 and 161.
-static bool window_fills_pages(const crystalkv_t* h, int P, int W) {
-  const long long blocks = window_blocks((W - 1) % window_queries(h, P) + 1, h->G);   // of the last launch
+static bool window_fills_pages(const crystalkv_t* h, int P, int W, bool tc) {
+  if (!tc) return true;   // (short prompts, for which a launch more costs what it saves)
+  const long long blocks = window_blocks_of(h, P, (W - 1) % window_queries(h, P, tc) + 1, true);   // of the last launch
   return 470ll * P < blocks * (450000 + 17ll * h->U * P);
 }
 
@@ -817,18 +840,19 @@ static bool window_fills_pages(const crystalkv_t* h, int P, int W) {
 // window's group means, the first pbar area the hit bits.
 // mk, mv, mp: tiles of the prompt's keys and values, the pool.
 static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, const unsigned char* v, const unsigned char* q, int P, int W,
-                         __nv_bfloat16* out, bool fill_pages, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mp, cudaStream_t s) {
+                         __nv_bfloat16* out, bool tc, bool fill_pages, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mp, cudaStream_t s) {
   const crystalkv_config_t& c = h->cfg;
   WindowParams p{};
   p.k = k; p.v = v;
-  p.pbar = h->sc_logits[0];
+  p.pbar = p.logits = h->sc_logits[0];
+  p.ml = h->sc_partials[0];
   p.hits = reinterpret_cast<unsigned*>(h->sc_pbar[0]);
   p.H = c.n_kv_heads; p.G = h->G; p.U = h->U; p.P = P; p.layer = layer;
   p.Ps = (P + 7) / 8 * 8;   // rows of group means start on 32-byte sectors
   p.words = (P + 31) / 32;
   p.scale = c.sm_scale;
   p.scale_log2 = c.sm_scale * 1.44269504088896340736f;
-  const int fit = window_queries(h, P);
+  const int fit = window_queries(h, P, tc);
   const size_t sm = (size_t)P * sizeof(float) <= WIN_SMEM ? (size_t)P * sizeof(float) : 0;
   const int plan_grid = h->plan_grid(layer);
   const size_t qn = (size_t)c.batch * c.n_q_heads * HD;
@@ -839,15 +863,24 @@ static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, cons
     p.out = out ? out + (size_t)w0 * qn : nullptr;
     const bool last = w0 + p.W == W;
     p.store = last && fill_pages;
-    const int blocks = window_blocks(p.W, p.G);
-    p.rows = window_rows(p.W, p.G);
-    const auto attn = window_attn_of(p.rows, out != nullptr);
-    const int smem = wa_smem(p.rows, out != nullptr);
-    CK(h, cudaFuncSetAttribute(attn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    CK(h, launch_next(attn, dim3(blocks, h->U), WA_THREADS, smem, s, h->st, p, mk, mv, mp));
+    if (tc) {
+      const int blocks = window_blocks_of(h, P, p.W, out != nullptr);
+      p.rows = window_rows(p.W, p.G, blocks);
+      const auto attn = window_attn_of(p.rows, out != nullptr);
+      const int smem = wa_smem(p.rows, out != nullptr);
+      CK(h, cudaFuncSetAttribute(attn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+      CK(h, launch_next(attn, dim3(blocks, h->U), WA_THREADS, smem, s, h->st, p, mk, mv, mp));
+    } else {
+      const auto attn = out ? window_mma_kernel<true> : window_mma_kernel<false>;
+      CK(h, cudaFuncSetAttribute(attn, cudaFuncAttributeMaxDynamicSharedMemorySize, WM_SMEM));
+      // (An ordinary launch: early CTAs gather, three to an SM, on the SMs that are free first.  32 heads x 2048 tokens, 32 queries of 2 heads 133 us
+      // a layer instead of 89.)
+      attn<<<dim3((p.W * p.G + WM_ROWS - 1) / WM_ROWS, h->U), WM_WARPS * 32, WM_SMEM, s>>>(h->st, p);
+      CK(h, cudaGetLastError());
+    }
     const bool small = P <= WH_SMALL && (long long)p.W * h->U >= P + h->num_sms;
-    CK(h, launch_next(small ? window_hits_kernel<64> : window_hits_kernel<NT>, dim3(p.W, h->U), small ? 64 : NT, sm, s, h->st, p, c.top_p,
-                      c.literal_return, sm > 0));
+    CK(h, launch_next(small ? window_hits_of<64>(tc ? 0 : p.G) : window_hits_of<NT>(tc ? 0 : p.G), dim3(p.W, h->U), small ? 64 : NT, sm, s,
+                      h->st, p, c.top_p, c.literal_return, sm > 0));
     const bool wide = P > APPLY_LINE && 2 * h->U <= h->num_sms;
     CK(h, launch_next(wide ? window_apply_kernel<APPLY_WIDE> : window_apply_kernel<NT>, dim3(1 + h->U), wide ? APPLY_WIDE : NT, 0, s, h->st, p, last, c.evict_every, reinterpret_cast<int*>(h->sc_pbar[1]),
                       h->cap_s, h->plans[layer], plan_grid, h->cl[layer], h->plan_len));
@@ -924,7 +957,7 @@ static int prefill_common(crystalkv_t* h, int layer, const void* k, const void* 
   }
   // the whole prompt is stored; in full-cache mode the first step's plan is written beside the copy, and a replayed window
   // copies the rows in its attention kernel where that reads all of them (it has outputs) and is wide enough
-  const bool fill_pages = evict && out_window && window_fills_pages(h, P, W);
+  const bool tc = evict && window_tcgen05(h, P, W, out_window != nullptr), fill_pages = evict && out_window && window_fills_pages(h, P, W, tc);
   prefill_take_kernel<<<h->U, NT, 0, s>>>(h->st, layer, P, W > 0 ? 1 : 0);
   CK(h, cudaGetLastError());
   if (!fill_pages) {
@@ -932,7 +965,7 @@ static int prefill_common(crystalkv_t* h, int layer, const void* k, const void* 
                       W > 0 ? ROWS_ALL : ROWS_ALL_LAST, per_head, evict ? 0 : plan_grid * NW, plan_grid, h->cl[layer]));
   }
   if (evict) {
-    rc = replay_window(h, layer, kb, vb, static_cast<const unsigned char*>(q), P, W, static_cast<__nv_bfloat16*>(out_window), fill_pages,
+    rc = replay_window(h, layer, kb, vb, static_cast<const unsigned char*>(q), P, W, static_cast<__nv_bfloat16*>(out_window), tc, fill_pages,
                        mk, mv, mp, s);
     if (rc) return rc;
   }

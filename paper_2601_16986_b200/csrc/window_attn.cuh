@@ -42,6 +42,8 @@ struct WindowParams {
   const unsigned char* q;      // [W][batch][Hq][128], from the first query of this launch
   __nv_bfloat16* out;          // the same shape
   float* pbar;                 // [U][W][Ps] group means of the probabilities
+  float* logits;               // mma.sync: [U][W][G][Ps] scaled logits instead
+  float* ml;                   //           [U][W][16] reference point (log2 domain) [8], normaliser [8]
   unsigned* hits;              // [U][W][words] hit bits, bit i % 32 of word i / 32
   int H, G, U, P, Ps, words;
   int W, t0;                   // queries of this launch, time of the first
@@ -290,7 +292,7 @@ __global__ void __launch_bounds__(WA_THREADS, 1) window_attn_kernel(const __grid
       const int x = what(i), tile = x < 0 ? -1 - x : x, stage = i % S, turn = tile % gridDim.x, at = tile * WA_KEYS + lane * GRP;
       const bool mine = store && (i < nt || x < 0) && blockIdx.x == ((tile + 1) * WA_KEYS <= keys_of(turn) ? turn : last) &&
                         lane < WA_KEYS / GRP && at < p.P;
-      const int page = mine ? __ldcg(st.ptab + (size_t)uid * st.capg + at / GRP) : 0;
+      const int page = mine ? st.ptab[(size_t)uid * st.capg + at / GRP] : 0;
       wait(bar_ld + 8 * stage, i / S);
       if (mine && !dead) {   // (rows past the prompt's end are zeros and go to places without an entry)
         for (int y = 0; y < 2; ++y)
@@ -501,10 +503,14 @@ __global__ void __launch_bounds__(WA_THREADS, 1) window_attn_kernel(const __grid
   if (w == WA_WARPS) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tm), "n"(WA_TMEM) : "memory");
 }
 
-// Row blocks of a head for W queries of G heads each, as few as there can be, and the rows of each, a multiple of 32.
-inline int window_blocks(int W, int G) { const int most = 4 * wa_queries(WA_MAX_ROWS, G); return (W + most - 1) / most; }
-inline int window_rows(int W, int G) {
-  const int each = (W + window_blocks(W, G) - 1) / window_blocks(W, G);   // queries of a block
+// Row blocks of a head for W queries of G query heads: as few as there can be, or of 32 rows each if those are no more than `room`; and the
+// rows of each, a multiple of 32.
+inline int window_blocks(int W, int G, int room) {
+  const int most = 4 * wa_queries(WA_MAX_ROWS, G), least = 4 * wa_queries(32, G);   // queries of a block
+  return (W + least - 1) / least <= room ? (W + least - 1) / least : (W + most - 1) / most;
+}
+inline int window_rows(int W, int G, int blocks) {
+  const int each = (W + blocks - 1) / blocks;   // queries of a block
   int rows = 32;
   while (4 * wa_queries(rows, G) < each) rows += 32;
   return rows;

@@ -9,6 +9,7 @@
 #include "nucleus.cuh"
 #include "plan.cuh"
 #include "window_attn.cuh"
+#include "window_mma.cuh"
 
 namespace ckv {
 
@@ -27,7 +28,7 @@ constexpr int WH_SMALL = 1280;                // entries up to which window_hits
 // and 28.5; 1600 entries, 4096 searches 61.2 and 60.2.
 // 128 heads x 32 queries over 1000 entries: 20 us (36 with the logits of five heads to read and weigh).
 // pbar lives in shared memory or, for long prompts, where it is.
-template <int NTH>
+template <int NTH, int G>
 __global__ void __launch_bounds__(NTH) window_hits_kernel(const __grid_constant__ State st, const WindowParams p, float top_p, int literal,
                                                           int in_smem) {
   constexpr int WARPS = NTH / 32;
@@ -46,22 +47,38 @@ __global__ void __launch_bounds__(NTH) window_hits_kernel(const __grid_constant_
       return;
     }
   }
-  const float* S = p.pbar + ((size_t)u * p.W + q) * p.Ps;
-  const float* pb = in_smem ? s_pbar : S;
+  float* S = G ? p.logits + ((size_t)u * p.W + q) * G * p.Ps : p.pbar + ((size_t)u * p.W + q) * p.Ps;
+  float* pb = in_smem ? s_pbar : S;
+  float m[G ? G : 1], il[G ? G : 1];   // reference point, 1 / (normaliser x query heads)
+  if constexpr (G > 0) {
+    const float* ml = p.ml + ((size_t)u * p.W + q) * 16;
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      m[g] = to_natural(ml[g]);
+      il[g] = 1.0f / (ml[8 + g] * (float)G);
+    }
+  }
   const int base = nucleus_base<NTH>(n);
   nucleus_clear<NTH>(s_nu);
   __syncthreads();
   constexpr int BR = 4;   // entries requested together
   for (int i0 = tid; i0 < n; i0 += BR * NTH) {
-    float v[BR];
+    float v[BR][G ? G : 1];
 #pragma unroll
-    for (int x = 0; x < BR; ++x) v[x] = S[min(i0 + x * NTH, n - 1)];
+    for (int x = 0; x < BR; ++x) {
+      const float* r = S + min(i0 + x * NTH, n - 1);
 #pragma unroll
-    for (int x = 0; x < BR; ++x)
+      for (int g = 0; g < (G ? G : 1); ++g) v[x][g] = r[(size_t)g * p.Ps];
+    }
+#pragma unroll
+    for (int x = 0; x < BR; ++x) {
+      float pm = v[x][0];
+      if constexpr (G > 0) pm = group_mean(v[x], m, il);
       if (i0 + x * NTH < n) {
-        if (in_smem) s_pbar[i0 + x * NTH] = v[x];
-        nucleus_add<NTH>(s_nu, base, v[x]);
+        if (G > 0 || in_smem) pb[i0 + x * NTH] = pm;   // (mma.sync, long prompt: in the place of its own logit, which has been read)
+        nucleus_add<NTH>(s_nu, base, pm);
       }
+    }
   }
   __syncthreads();
   const Nucleus nu = nucleus_find<NTH>(base, top_p, s_nu, st.errword, [&](auto f) {
@@ -91,6 +108,22 @@ __global__ void __launch_bounds__(NTH) window_hits_kernel(const __grid_constant_
     }
     const unsigned m = __ballot_sync(0xffffffffu, hit);
     if (lane == 0 && (i >> 5) < p.words) bits[i >> 5] = m;
+  }
+}
+
+using WindowHits = void (*)(State, WindowParams, float, int, int);
+template <int NTH>
+WindowHits window_hits_of(int G) {   // 0: the group means are there
+  switch (G) {
+    case 0: return window_hits_kernel<NTH, 0>;
+    case 1: return window_hits_kernel<NTH, 1>;
+    case 2: return window_hits_kernel<NTH, 2>;
+    case 3: return window_hits_kernel<NTH, 3>;
+    case 4: return window_hits_kernel<NTH, 4>;
+    case 5: return window_hits_kernel<NTH, 5>;
+    case 6: return window_hits_kernel<NTH, 6>;
+    case 7: return window_hits_kernel<NTH, 7>;
+    default: return window_hits_kernel<NTH, 8>;
   }
 }
 
