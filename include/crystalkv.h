@@ -85,13 +85,19 @@ int crystalkv_create(const crystalkv_config_t* cfg, crystalkv_t** out);
 
 /*
  * Frees the handle, once its device is idle.  NULL is accepted.  What the handle had of its device (memory, streams, events)
- * may be kept for the next handle on it: one set per device, of at most 8 GiB, and only while a
- * quarter of the device's memory is free.  A later handle that it does not fit, a failing allocation of this library, or
- * crystalkv_trim gives it back.
+ * may be kept for the next handle on it: one set per device (of its primary context), of at most 8 GiB, and only if a quarter of the
+ * device's memory is free at that moment.  A later handle that it does not fit (one that needs more of it, or less than half), a failing
+ * allocation of this library, or crystalkv_trim gives it back; a handle may thus hold up to twice the memory it needs.
+ * Other allocators of the process do not get the memory back when they run short: a program that wants it for them calls
+ * crystalkv_trim after closing its handles.
  */
 int crystalkv_destroy(crystalkv_t* h);
 
-/* Gives back what destroyed handles left on the device.  May be called from any thread.  Errors: EINVAL, ECUDA. */
+/*
+ * Gives back what destroyed handles left on the device.  May be called from any thread; a device on which nothing is kept is not
+ * touched.  Errors: EINVAL; ECUDA if something is still kept afterwards (the device cannot be made current, or another
+ * thread closed a handle meanwhile).
+ */
 int crystalkv_trim(int device);
 
 /*
@@ -328,6 +334,15 @@ int crystalkv_debug_ctas_needed(int32_t whole_ctas, const int32_t* runs_by_lengt
  */
 int crystalkv_debug_place_runs(int32_t whole_ctas, const int32_t* runs_by_length, int32_t grid, int32_t* first_warp,
                                int32_t cap);
+
+/*
+ * Test hook for the place in which a device's set is kept (no GPU, no handle): n operations on a place of its own, four int32
+ * each: what, the current context's id, the context the set was made in, the set's number.  what = 0: a handle is closed
+ * (found: 1 if its set is kept); 1: a handle is made, or the set given back (found: the number of the set that is taken out, 0 if
+ * none).  An id of 0 stands for a context that is not the device's primary one.  Returns 1 if a set is kept at the end, 0 if none,
+ * or EINVAL for a NULL array, a negative n or an unknown operation.
+ */
+int crystalkv_debug_kept_kit(const int32_t* ops, int32_t n, int32_t* found);
 
 const char* crystalkv_strerror(int code);
 const char* crystalkv_last_error(crystalkv_t* h);

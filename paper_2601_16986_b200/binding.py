@@ -82,6 +82,7 @@ def load_library():
     lib.crystalkv_create.argtypes = [C.POINTER(_Cfg), C.POINTER(vp)]
     lib.crystalkv_destroy.argtypes = [vp]
     lib.crystalkv_trim.argtypes = [i32]
+    lib.crystalkv_debug_kept_kit.argtypes = [p32, i32, p32]
     lib.crystalkv_prefill.argtypes = [vp, i32, vp, vp, vp, i32, vp]
     lib.crystalkv_prefill_window.argtypes = [vp, i32, vp, vp, vp, i32, i32, vp, vp]
     lib.crystalkv_decode_step.argtypes = [vp, i32, vp, vp, vp, vp, vp]

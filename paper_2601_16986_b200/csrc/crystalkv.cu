@@ -37,7 +37,7 @@ using namespace ckv;
 struct DeviceKit {
   void* arena = nullptr;           // the one device allocation that all arrays of the handle lie in
   size_t arena_bytes = 0;
-  unsigned long long context = 0;  // of the CUDA context that all of this belongs to (a device reset ends it); 0: unknown
+  unsigned long long context = 0;  // the primary context that all of this belongs to (a device reset ends it); 0: another context, or unknown
   // LRFU launches are numbered; launch k uses scratch set k % NSETS and event k % EV_RING
   static constexpr int EV_RING = 32;
   // two internal streams taken in turn: the LRFU kernels of consecutive layers do not depend on
@@ -146,26 +146,63 @@ struct DeviceScope {
 // ---- what a destroyed handle leaves for the next one
 // A server makes a handle for a new batch and frees it again and again.  Taking and giving back 5.5 GB costs 1.05 and 3.2 ms,
 // the streams and events another half, as much as all else: a new batch of 16 prompts of 512 tokens in the 8B shape, 1.9 ms of
-// kernels, took 6.7 ms and takes 1.8 to 2.0 with them kept (8 prompts of 9350 tokens 5.6 and 3.4 to 3.9, windows of 32 12.4 and 8.4 to 9.2).  So a device keeps at most one kit, of at most KEEP_BYTES, and that only
+// kernels, took 6.7 ms and takes 1.6 to 2.0 with them kept.  So a device keeps at most one kit, of at most KEEP_BYTES, and that only
 // while a quarter of its memory is free; crystalkv_trim, a handle that it does not fit and an allocation
 // that fails for want of memory give it back.  (A pool of the driver's gives back by itself, but its first 5.5 GB took 34 to 280 ms.)
 constexpr size_t KEEP_BYTES = size_t(8) << 30;
-DeviceKit g_kept[MAX_DEVICES];   // (context 0: nothing is kept)
+
+// The place of a device's kit.  Only kits of the device's primary context are kept, of which there is one at a time: a kit of
+// another one is of a context that has ended (a device reset), and with it all that the kit names.
+struct KeptKit {
+  DeviceKit kit;   // (context 0: nothing is kept)
+  bool empty() const { return !kit.context; }
+  // Whether a kit that was made in the primary context `current` (0: the caller is in another one, or it is unknown) finds room.
+  bool room_for(const DeviceKit& k, unsigned long long current) const { return k.context && k.context == current && kit.context != current; }
+  bool put(const DeviceKit& k, unsigned long long current) {
+    if (!room_for(k, current)) return false;
+    kit = k;
+    return true;
+  }
+  // The kit of the primary context `current`, taken out; an empty one else.
+  DeviceKit take(unsigned long long current) {
+    DeviceKit k;
+    if (current && kit.context && kit.context != current) kit = DeviceKit{};
+    if (current) std::swap(k, kit);
+    return k;
+  }
+};
+KeptKit g_kept[MAX_DEVICES];
 std::mutex g_kept_mu;
 
-unsigned long long context_id() {   // of the current context, 0: unknown
-  using Fn = CUresult (*)(CUcontext, unsigned long long*);
-  static const Fn fn = [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult r;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &r) != cudaSuccess || r != cudaDriverEntryPointSuccess) {
-      cudaGetLastError();
-      p = nullptr;
-    }
-    return reinterpret_cast<Fn>(p);
-  }();
+template <class Fn>
+Fn driver_call(const char* name) {   // a call of the CUDA driver's as of 12.0, null if there is none
+  void* p = nullptr;
+  cudaDriverEntryPointQueryResult r;
+  if (cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &r) != cudaSuccess || r != cudaDriverEntryPointSuccess) {
+    cudaGetLastError();
+    p = nullptr;
+  }
+  return reinterpret_cast<Fn>(p);
+}
+
+// The id of the current context if it is the primary one of its device, else 0.
+unsigned long long primary_id() {
+  static const auto current = driver_call<decltype(&cuCtxGetCurrent)>("cuCtxGetCurrent");
+  static const auto device_of = driver_call<decltype(&cuCtxGetDevice)>("cuCtxGetDevice");
+  static const auto retain = driver_call<decltype(&cuDevicePrimaryCtxRetain)>("cuDevicePrimaryCtxRetain");
+  static const auto release = driver_call<decltype(&cuDevicePrimaryCtxRelease)>("cuDevicePrimaryCtxRelease");
+  static const auto state = driver_call<decltype(&cuDevicePrimaryCtxGetState)>("cuDevicePrimaryCtxGetState");
+  static const auto id_of = driver_call<CUresult (*)(CUcontext, unsigned long long*)>("cuCtxGetId");
+  if (!current || !device_of || !retain || !release || !state || !id_of) return 0;
+  CUcontext ctx = nullptr, primary = nullptr;
+  CUdevice dev = 0;
+  unsigned flags = 0;
+  int active = 0;
   unsigned long long id = 0;
-  return fn && fn(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+  if (current(&ctx) != CUDA_SUCCESS || !ctx || device_of(&dev) != CUDA_SUCCESS) return 0;
+  if (state(dev, &flags, &active) != CUDA_SUCCESS || !active || retain(&primary, dev) != CUDA_SUCCESS) return 0;
+  release(dev);
+  return primary == ctx && id_of(ctx, &id) == CUDA_SUCCESS ? id : 0;
 }
 
 void free_kit(DeviceKit& k) {
@@ -183,32 +220,51 @@ void free_kit(DeviceKit& k) {
 
 // The kit that the current device keeps, if it belongs to the current context, taken out; an empty one else.
 DeviceKit take_kept(int device) {
+  const unsigned long long ctx = primary_id();
   std::lock_guard<std::mutex> lock(g_kept_mu);
-  DeviceKit kit;
-  if (g_kept[device].context && g_kept[device].context == context_id()) std::swap(kit, g_kept[device]);
-  return kit;
+  return g_kept[device].take(ctx);
 }
 
 // Keeps a complete kit that no work on the device uses any more.  False: it is the caller's to free.
 bool keep_kit(int device, const DeviceKit& kit) {
   if (!kit.arena || kit.arena_bytes > KEEP_BYTES || !kit.evF[DeviceKit::EV_RING - 1]) return false;   // (the last to be made)
+  const unsigned long long ctx = primary_id();
+  {
+    std::lock_guard<std::mutex> lock(g_kept_mu);
+    if (!g_kept[device].room_for(kit, ctx)) return false;
+  }
   size_t room = 0, total = 0;
   if (cudaMemGetInfo(&room, &total) != cudaSuccess) { cudaGetLastError(); return false; }
   if (room < total / 4) return false;
   std::lock_guard<std::mutex> lock(g_kept_mu);
-  if (g_kept[device].context || !kit.context || kit.context != context_id()) return false;
-  g_kept[device] = kit;
-  return true;
+  return g_kept[device].put(kit, ctx);
+}
+
+// Gives back what the device keeps, whatever context is current.  True if there was something.
+bool give_back(int device) {
+  {
+    std::lock_guard<std::mutex> lock(g_kept_mu);
+    if (g_kept[device].empty()) return false;   // (a device that was never used gets no context)
+  }
+  static const auto current = driver_call<decltype(&cuCtxGetCurrent)>("cuCtxGetCurrent");
+  static const auto make_current = driver_call<decltype(&cuCtxSetCurrent)>("cuCtxSetCurrent");
+  CUcontext ctx = nullptr;
+  int before = -1;
+  if (!current || !make_current || current(&ctx) != CUDA_SUCCESS || cudaGetDevice(&before) != cudaSuccess) return false;
+  DeviceKit kit;
+  if (cudaSetDevice(device) == cudaSuccess) kit = take_kept(device);   // (the primary context is the current one now)
+  const bool had = kit.arena != nullptr;
+  free_kit(kit);
+  if (before != device) cudaSetDevice(before);
+  if (ctx) make_current(ctx);
+  return had;
 }
 
 // cudaMalloc that gives back what the device keeps if there is not enough memory.
 cudaError_t device_malloc(int device, void** p, size_t bytes) {
   cudaError_t e = cudaMalloc(p, bytes);
-  if (e != cudaErrorMemoryAllocation) return e;
-  DeviceKit kit = take_kept(device);
-  if (!kit.arena) return e;
+  if (e != cudaErrorMemoryAllocation || !give_back(device)) return e;
   cudaGetLastError();
-  free_kit(kit);
   return cudaMalloc(p, bytes);
 }
 
@@ -237,7 +293,7 @@ struct Arena {
                     std::string("cudaMalloc: ") + cudaGetErrorString(e));
       }
       kit.arena_bytes = bytes;
-      kit.context = context_id();
+      kit.context = primary_id();
     }
     for (const Part& x : parts) *x.where = static_cast<unsigned char*>(kit.arena) + x.at;
     return CRYSTALKV_OK;
@@ -482,16 +538,7 @@ cudaError_t launch_next(void (*kernel)(P...), dim3 grid, int threads, size_t sme
 // A tensor map of bf16 in boxes of `box`, zeros beyond the ends.
 bool tensor_map(CUtensorMap* m, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box,
                 CUtensorMapSwizzle swizzle) {
-  using Fn = decltype(&cuTensorMapEncodeTiled);
-  static const Fn encode = [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult r;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &r) != cudaSuccess || r != cudaDriverEntryPointSuccess) {
-      cudaGetLastError();
-      p = nullptr;
-    }
-    return reinterpret_cast<Fn>(p);
-  }();
+  static const auto encode = driver_call<decltype(&cuTensorMapEncodeTiled)>("cuTensorMapEncodeTiled");
   const cuuint32_t step[4] = {1, 1, 1, 1};
   return encode && encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(base), dims, strides, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE,
                           swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -611,11 +658,28 @@ int crystalkv_destroy(crystalkv_t* h) {
 
 int crystalkv_trim(int device) {
   if (device < 0 || device >= MAX_DEVICES) return CRYSTALKV_EINVAL;
-  DeviceScope scope(device);
-  if (scope.err != cudaSuccess) return CRYSTALKV_ECUDA;
-  DeviceKit kit = take_kept(device);
-  free_kit(kit);
-  return CRYSTALKV_OK;
+  give_back(device);
+  std::lock_guard<std::mutex> lock(g_kept_mu);
+  return g_kept[device].empty() ? CRYSTALKV_OK : CRYSTALKV_ECUDA;
+}
+
+int crystalkv_debug_kept_kit(const int32_t* ops, int32_t n, int32_t* found) {
+  if (!ops || !found || n < 0) return CRYSTALKV_EINVAL;
+  KeptKit place;
+  for (int i = 0; i < n; ++i) {
+    const int32_t* op = ops + 4 * i;   // what, current context, the kit's context, the kit's number
+    DeviceKit k;
+    if (op[0] == 0) {
+      k.context = (unsigned long long)op[2];
+      k.arena_bytes = (size_t)op[3];
+      found[i] = place.put(k, (unsigned long long)op[1]);
+    } else if (op[0] == 1) {
+      found[i] = (int32_t)place.take((unsigned long long)op[1]).arena_bytes;
+    } else {
+      return CRYSTALKV_EINVAL;
+    }
+  }
+  return place.empty() ? 0 : 1;
 }
 
 int crystalkv_create(const crystalkv_config_t* cfg, crystalkv_t** out) {

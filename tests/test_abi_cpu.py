@@ -65,6 +65,35 @@ def test_binding_refuses_to_run_without_a_gpu():
         CrystalKV(Config(n_layers=1, n_q_heads=2, n_kv_heads=1, batch=1, budget_per_head=8, max_context=32))
 
 
+def _kept(lib, *ops):
+    """(what each operation found, whether a set is kept at the end)"""
+    arr = (C.c_int32 * (4 * len(ops)))(*[x for op in ops for x in (tuple(op) + (0, 0))[:4]])
+    found = (C.c_int32 * len(ops))()
+    return list(found) if (rc := lib.crystalkv_debug_kept_kit(arr, len(ops), found)) < 0 else (list(found), rc)
+
+
+def test_what_a_closed_handle_leaves_outlives_its_context_only_in_name(lib):
+    """The place that keeps one set per device: taken by the next handle of the same context; after a device reset (another id) the dead
+    set neither serves a handle nor holds the place; a handle of a context that is not the primary one leaves and takes nothing."""
+    CLOSE, MAKE = 0, 1
+    assert _kept(lib, (CLOSE, 7, 7, 1), (MAKE, 7), (MAKE, 7)) == ([1, 1, 0], 0)
+    assert _kept(lib, (CLOSE, 7, 7, 1), (CLOSE, 7, 7, 2), (MAKE, 7)) == ([1, 0, 1], 0)          # one at a time
+    assert _kept(lib, (CLOSE, 7, 7, 1), (MAKE, 8), (CLOSE, 8, 8, 2), (MAKE, 8)) == ([1, 0, 1, 2], 0)
+    assert _kept(lib, (CLOSE, 7, 7, 1), (CLOSE, 8, 8, 2), (MAKE, 8)) == ([1, 1, 2], 0)          # the new set takes the dead one's place
+    assert _kept(lib, (CLOSE, 7, 7, 1), (MAKE, 8)) == ([1, 0], 0)                               # given back: nothing is kept any more
+    assert _kept(lib, (CLOSE, 8, 7, 1)) == ([0], 0)                                             # made before the reset, closed after it
+    assert _kept(lib, (CLOSE, 7, 7, 1), (MAKE, 0), (CLOSE, 0, 0, 2), (MAKE, 7)) == ([1, 0, 0, 1], 0)
+    assert _kept(lib, (CLOSE, 7, 0, 1), (CLOSE, 0, 7, 1)) == ([0, 0], 0)
+    assert lib.crystalkv_debug_kept_kit(None, 1, None) == -1 and _kept(lib, (2, 7)) == [0]
+
+
+def test_trim_of_a_device_that_keeps_nothing_touches_none(lib):
+    """No context is made for it: the call works where there is no GPU at all."""
+    for device in (0, 1, 63):
+        assert lib.crystalkv_trim(device) == 0
+    assert lib.crystalkv_trim(-1) == -1 and lib.crystalkv_trim(64) == -1
+
+
 def _place_runs_one_by_one(whole, runs):
     """Best fit, longest first, one run at a time: the placement the planner performs."""
     free = []            # free warps of every open CTA
