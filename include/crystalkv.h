@@ -327,13 +327,16 @@ int crystalkv_debug_get_plan(crystalkv_t* h, int layer, int32_t* hdr_host, int32
 int crystalkv_debug_ctas_needed(int32_t whole_ctas, const int32_t* runs_by_length);
 
 /*
- * Test hook for the placement itself (no GPU, no handle): where the planner puts those runs on a grid of
- * `grid` CTAs if they belong to heads of one length.  first_warp receives, for the runs of length 7, then 6, .. 1, the warp (CTA x 8 + place in
- * the CTA) each starts at; cap is its room.  Returns the number of runs, ESTATE if they do not fit, or EINVAL
- * for a NULL array, a negative number or too little room.
+ * Test hooks for the placement itself (no GPU, no handle): where the planner puts those runs on a grid of
+ * `grid` CTAs, by the walk that crystalkv_debug_ctas_needed counts, and (spread) as it does with heads of one length.  first_warp
+ * receives, for the runs of length 7, then 6, .. 1, the warp (CTA x 8 + place in the CTA) each starts at; cap is
+ * its room.  Return the number of runs, ESTATE if they do not fit, or EINVAL for a NULL array, a
+ * negative number or too little room.
  */
 int crystalkv_debug_place_runs(int32_t whole_ctas, const int32_t* runs_by_length, int32_t grid, int32_t* first_warp,
                                int32_t cap);
+int crystalkv_debug_spread_runs(int32_t whole_ctas, const int32_t* runs_by_length, int32_t grid, int32_t* first_warp,
+                                int32_t cap);
 
 /*
  * Test hook for the place in which a device's set is kept (no GPU, no handle): n operations on a place of its own, four int32

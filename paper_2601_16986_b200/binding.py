@@ -104,7 +104,8 @@ def load_library():
     lib.crystalkv_debug_set_page.argtypes = [vp, i32, i32, i32, C.c_int32, C.c_int32, vp]
     lib.crystalkv_debug_get_plan.argtypes = [vp, i32, vp, vp, C.c_int32, vp, C.c_int32, vp]
     lib.crystalkv_debug_ctas_needed.argtypes = [C.c_int32, vp]
-    lib.crystalkv_debug_place_runs.argtypes = [C.c_int32, vp, C.c_int32, vp, C.c_int32]
+    for f in (lib.crystalkv_debug_place_runs, lib.crystalkv_debug_spread_runs):
+        f.argtypes = [C.c_int32, vp, C.c_int32, vp, C.c_int32]
     lib.crystalkv_strerror.argtypes = [i32]
     lib.crystalkv_strerror.restype = C.c_char_p
     lib.crystalkv_last_error.argtypes = [vp]

@@ -1452,7 +1452,7 @@ int crystalkv_debug_ctas_needed(int32_t whole_ctas, const int32_t* runs_by_lengt
   return ctas_needed(whole_ctas, cnt);
 }
 
-int crystalkv_debug_place_runs(int32_t whole_ctas, const int32_t* runs_by_length, int32_t grid, int32_t* first_warp, int32_t cap) {
+static int place_runs_hook(int32_t whole_ctas, const int32_t* runs_by_length, int32_t grid, int32_t spread, int32_t* first_warp, int32_t cap) {
   if (!runs_by_length || !first_warp || whole_ctas < 0 || grid < 0) return CRYSTALKV_EINVAL;
   int cnt[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   long long total = 0;
@@ -1463,11 +1463,19 @@ int crystalkv_debug_place_runs(int32_t whole_ctas, const int32_t* runs_by_length
   }
   if (total > cap) return CRYSTALKV_EINVAL;
   Placement p{};
-  if (ctas_needed(whole_ctas, cnt) > grid || !place_runs(whole_ctas, cnt, grid, true, p)) return CRYSTALKV_ESTATE;   // (as the planner asks first)
+  if (whole_ctas > grid || !place_runs(whole_ctas, cnt, grid, spread != 0, p)) return CRYSTALKV_ESTATE;
   int at = 0;
   for (int s = 7; s >= 1; --s)
     for (int r = 0; r < cnt[s]; ++r) first_warp[at++] = run_warp(p, s, r);
   return at;
+}
+
+int crystalkv_debug_place_runs(int32_t whole_ctas, const int32_t* runs_by_length, int32_t grid, int32_t* first_warp, int32_t cap) {
+  return place_runs_hook(whole_ctas, runs_by_length, grid, 0, first_warp, cap);
+}
+
+int crystalkv_debug_spread_runs(int32_t whole_ctas, const int32_t* runs_by_length, int32_t grid, int32_t* first_warp, int32_t cap) {
+  return place_runs_hook(whole_ctas, runs_by_length, grid, 1, first_warp, cap);
 }
 
 int crystalkv_debug_get_plan(crystalkv_t* h, int layer, int32_t* hdr_host, int32_t* wrange_host, int32_t warps_cap,

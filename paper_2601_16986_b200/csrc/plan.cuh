@@ -60,7 +60,8 @@ __host__ __device__ __forceinline__ int ctas_needed(int full, const int (&cnt)[8
 // ranges of consecutive CTAs instead of CTAs, class by class of free warps.
 // An entry says: the runs [r0, r0 + n) of length s (in head order) fill CTAs base, base + 1, ... with q
 // runs each, from warp `off` on.  A range of CTAs visited for a length is cut into at most a consumed, a
-// partly consumed and an untouched part.
+// partly consumed and an untouched part, so no more than 13 ranges and 35 entries arise in the walk of ctas_needed(); a spread
+// that runs out of either is one that does not fit.
 constexpr int PL_SCRATCH = 320;   // ints of shared scratch that write_plan() wants
 constexpr int PL_ENTRIES = 40, PL_RANGES = 16;
 struct Placement {

@@ -135,8 +135,8 @@ def test_the_planners_count_equals_placing_the_runs_one_by_one(lib):
 
 
 def test_placed_runs_are_spread_over_the_grid(lib):
-    """With more CTAs than the runs need, every CTA gets a run before one gets two (where ranges of like CTAs allow to say
-    so in the planner's memory: always for runs of up to three lengths)."""
+    """Heads of one length: with more CTAs than the runs need, every CTA gets a run before one gets two (where ranges of like CTAs allow to say
+    so in the planner's memory: always for runs of up to three lengths; heads of one length have one)."""
     rng = np.random.RandomState(11)
     where = np.zeros(1200, dtype=np.int32)
     for trial in range(2000):
@@ -146,7 +146,7 @@ def test_placed_runs_are_spread_over_the_grid(lib):
         arr = (C.c_int32 * 8)(*runs)
         if lib.crystalkv_debug_ctas_needed(whole, arr) > grid or whole + sum(runs) == 0:
             continue
-        got = lib.crystalkv_debug_place_runs(whole, arr, grid, where.ctypes.data_as(C.c_void_p), len(where))
+        got = lib.crystalkv_debug_spread_runs(whole, arr, grid, where.ctypes.data_as(C.c_void_p), len(where))
         assert got == sum(runs)
         ctas = set((where[:got] // 8).tolist())
         taken, at = np.zeros(8 * grid, dtype=np.int32), 0
@@ -183,6 +183,8 @@ def test_placed_runs_fit_their_ctas_and_do_not_overlap(lib):
                 taken[w:w + s] += 1
                 at += 1
         assert taken.max(initial=0) <= 1
+        # spread, too, whatever the mix: what does not fit that way falls back to the other walk
+        assert lib.crystalkv_debug_spread_runs(whole, arr, need, where.ctypes.data_as(C.c_void_p), len(where)) == sum(runs)
         if need > 0:
             assert lib.crystalkv_debug_place_runs(whole, arr, need - 1, where.ctypes.data_as(C.c_void_p), len(where)) == -2
     assert lib.crystalkv_debug_place_runs(0, None, 1, where.ctypes.data_as(C.c_void_p), 1) == -1
