@@ -117,17 +117,19 @@ __host__ __device__ inline bool place_runs(int full, const int* cnt, int grid, b
   return (spread && place_runs_by<true>(full, cnt, grid, p)) || place_runs_by<false>(full, cnt, grid, p);
 }
 
-// Whether U heads of g groups each, `full` and cnt their CTAs taken whole and runs, are spread: from 33 groups a CTA on, unless Algorithm 1's kernel
+// Whether U heads of g groups each, in k pieces, are spread: from 33 groups a CTA on, unless Algorithm 1's kernel
 // then misses the SMs without an attention CTA: its CTAs of eight warps (heads of more than 20 groups), of which two fit beside an attention CTA, come in
 // several waves with more than two heads an SM, and they show while the streams are short.  us a layer, spread and with CTAs filled up one after the other:
 // 150 heads of 76 groups 19.8 and 22.1, 160 of 44 14.4 and 16.1, 160 of 32 11.9 and 13.1, 256 of 65 25.0 and 25.6, 1024 of 17 26.3 and 26.8, 96 of 51 (33 a CTA) 11.65
 // and 11.7; but 480 of 10 (32) 11.4 and 10.8, 192 of 19 (25) 9.9 and 9.55.  More than 296 heads that would fill 128 CTAs: 512 of 20 17.3 and 17.7, of 25 23.8 and 21.3,
 // of 37 31.2 and 29.2, of 44 33.5 and 33.7, 1024 of 21 38.4 and 34.5, of 34 51.1 and 50.4; 104 CTAs: 832 of 26 36.0 and 33.0, of 34 41.0 and 42.5; 92 CTAs: 736 of 22 28.8 and 27.1, of
 // 26 30.6 and 31.8; 90 CTAs: 360 of 22 15.0 and 16.7; 80 CTAs: 640 of 25 25.2 and 29.0.
-__host__ __device__ inline bool spread_pays(int U, int g, int grid, int full, const int (&cnt)[8]) {
-  if (U * g < 33 * grid) return false;
-  if (U <= 2 * grid || g <= 20 || g > 40) return true;
-  return 100 * ctas_needed(full, cnt) <= (g <= 22 ? 61 : g <= 32 ? 70 : 80) * grid;
+// (So many heads are in one or two pieces.  The planner is part of Algorithm 1's kernels, whose launches got slower by 0.3 per cent with a second
+// count of the CTAs, or branches, here.)
+__host__ __device__ __forceinline__ bool spread_pays(int U, int g, int k, int grid) {
+  const int filled = (U * k + NW - 1) / NW;   // CTAs, filled up one after the other
+  const int line = U > 2 * grid && (unsigned)(g - 21) < 20u ? (g <= 22 ? 61 : g <= 32 ? 70 : 80) : 100;   // hundredths of the grid
+  return U * g >= 33 * grid && 100 * filled <= line * grid;
 }
 
 // The first warp (CTA x NW + its place in the CTA) of run r of length s.
@@ -302,7 +304,7 @@ __device__ __noinline__ void write_plan(const State& st, const Plan& pl, int lay
     // One thread walks the classes of CTAs, then every head looks its run up.  (A
     // plan of 128 heads takes 9 us; one warp placing the runs one by one took it to 26.)
     if (tid == 0) {
-      const bool ok = wholes <= grid && place_runs(wholes, runs, grid, Gtot == gmax * U && spread_pays(U, gmax, grid, wholes, runs), place);
+      const bool ok = wholes <= grid && place_runs(wholes, runs, grid, Gtot == gmax * U && spread_pays(U, gmax, (gmax + T - 1) / T, grid), place);
       place.first[8] = ok;
       if (!ok) atomicOr(st.errword, ERR_PLAN);   // cannot happen while ctas_needed() counts the same walk
     }
