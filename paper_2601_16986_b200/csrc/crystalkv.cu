@@ -1,7 +1,7 @@
 // C ABI of the Crystal-KV decode hot path (see include/crystalkv.h).  Host code only
 // validates, keeps the per-layer clocks and launches; every step of the path runs in the
 // kernels of attn_kernel.cuh and lrfu_kernel.cuh (a decode step; its launch plan: plan.cuh),
-// prefill_kernels.cuh, window_attn.cuh and window_kernels.cuh (prompts) and aux_kernels.cuh (reallocations, exports).
+// prefill_kernels.cuh, window_attn.cuh, window_mma.cuh and window_kernels.cuh (prompts) and aux_kernels.cuh (reallocations, exports).
 //
 // Stream plan of a tracked decode step of layer l: the attention kernel runs on the caller's
 // stream (so `out` is ready in stream order), the LRFU kernel of the same layer on an
@@ -946,8 +946,8 @@ static int replay_window(crystalkv_t* h, int layer, const unsigned char* k, cons
     CK(h, launch_next(small ? window_hits_of<64>(tc ? 0 : p.G) : window_hits_of<NT>(tc ? 0 : p.G), dim3(p.W, h->U), small ? 64 : NT, sm, s,
                       h->st, p, c.top_p, c.literal_return, sm > 0));
     const bool wide = P > APPLY_LINE && 2 * h->U <= h->num_sms;
-    CK(h, launch_next(wide ? window_apply_kernel<APPLY_WIDE> : window_apply_kernel<NT>, dim3(1 + h->U), wide ? APPLY_WIDE : NT, 0, s, h->st, p, last, c.evict_every, reinterpret_cast<int*>(h->sc_pbar[1]),
-                      h->cap_s, h->plans[layer], plan_grid, h->cl[layer], h->plan_len));
+    CK(h, launch_next(wide ? window_apply_kernel<APPLY_WIDE> : window_apply_kernel<NT>, dim3(1 + h->U), wide ? APPLY_WIDE : NT, 0, s, h->st, p,
+                      last, c.evict_every, reinterpret_cast<int*>(h->sc_pbar[1]), h->cap_s, h->plans[layer], plan_grid, h->cl[layer], h->plan_len));
   }
   return CRYSTALKV_OK;
 }

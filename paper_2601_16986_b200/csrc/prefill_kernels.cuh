@@ -35,8 +35,11 @@ constexpr int SCORE_SMEM = 1024 + NW * SCORE_STAGES * (SCORE_ITEM + 8);
 // read the heads of the same tokens keep to the same DRAM pages; the products are mma.sync with keys on M and the (padded) query
 // heads on N, 16 per item.  64 heads x 9350 tokens (153 MB of keys, 19 MB of
 // logits): 35.5 us (a thread per key with fp32 multiply-adds from shared memory, three
-// CTAs of 64 KB an SM: 45.5 us, half of its cycles spent on 16-byte broadcasts of the queries), 128 heads x 512 tokens 8.0 (9.3).  Error of a scaled
-// logit against 64 bits, keys N(0, 1): rms 6.95e-8, largest of 524288 8.8e-7 (7.25e-8 and 1.1e-6 with one chain of multiply-adds).
+// CTAs of 64 KB an SM: 45.5 us, half of its cycles spent on 16-byte broadcasts of the queries), 128 heads x 512 tokens 8.0 (9.3).
+// Which entries survive hangs on the last bits of the logits where an entry lies at the threshold.  Errors of a scaled logit against 64 bits, rms and largest
+// of 524288, and of one chain of multiply-adds: keys N(0, 1) 6.95e-8, 8.8e-7 (7.25e-8, 1.1e-6), times 3 (outliers) 2.15e-7, 2.3e-6
+// (2.2e-7, 3.7e-6), times 8 (sinks) 5.85e-7, 6.6e-6 (6e-7, 9.6e-6).  Of 17408 heads of prompts with sinks and outliers (2000 tokens to 400, 9350 to
+// 2400; 1, 4 and 8 query heads) two keep another entry than in 64 bits, with either kernel.
 __global__ void __launch_bounds__(NT, 1) prefill_score_kernel(Scratch sc, const __grid_constant__ CUtensorMap mk, const __nv_bfloat16* __restrict__ q_last,
                                                               int batch, int H, int G, int P, int warps, float scale, float scale_log2, int* errword) {
   extern __shared__ unsigned char s_raw[];

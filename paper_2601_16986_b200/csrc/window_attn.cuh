@@ -9,7 +9,8 @@
 // logits of five heads).  So nothing is ever rescaled, and a thread, which holds one key of every tile, keeps its share of
 // the maxima and sums in registers until a pass ends.  The weights go in as a bf16 head plus a bf16 remainder, like in the decode kernel.
 // A warp brings the tiles of all passes by TMA into a ring of stages, another issues the products; these and the sixteen meet at
-// mbarriers only.// The tiles are also what the heads' pages are filled from (store): a key's 64 channels in a stage are, byte for byte, a quarter
+// mbarriers only.
+// The tiles are also what the heads' pages are filled from (store): a key's 64 channels in a stage are, byte for byte, a quarter
 // of an entry in a page, so another warp has TMA store them as they are.  The CTAs of a head take its tiles in turn, a tile that
 // only the last one sees in full falls to that one.  (A copy kernel of its own reads the prompt again: 20 us.)
 #pragma once

@@ -19,7 +19,7 @@ constexpr int APPLY_LINE = 2048;
 constexpr int WH_SMALL = 1280;                // entries up to which window_hits_kernel may take CTAs of two warps
 
 // The hit bits of one (query, head): Algorithm 1 step 1 with the query of time t over its t + 1 entries.
-// grid: (W, U).
+// grid: (W, U).  G: the query heads whose logits the attention kernel left, 0 if it left their group means.
 // Bound: issue slots (some hundred instructions per warp beside those per entry):
 // many searches of short prompts take CTAs of two warps.  Few searches are bound by
 // the latency of one: the line is as many searches as entries and SMs, and WH_SMALL entries.  us with two warps and with
